@@ -138,8 +138,6 @@ __device__ __forceinline__ int next_item(const volatile unsigned long long *queu
     return 1;
 }
 
-__device__ __forceinline__ float swiglu(float g, float u) { return __fdividef(g * u, 1.f + __expf(-g)); }
-
 // A tile of at most DBL_ROWS pair rows takes two blocks of weight rows per item ("double item"): a
 // k-step of such a tile costs the pipeline the same time whether it carries one block or two (the
 // tensor pipe is idle most of it: an MMA of N <= 128 columns takes about 70 cycles however narrow it

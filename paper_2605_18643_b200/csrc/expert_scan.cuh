@@ -12,6 +12,7 @@ struct ScanShared {
     int32_t cnt[kMaxCand];
     int32_t off[kMaxCand + 1];
     int32_t ptile[kMaxCand + 1];  // exclusive scan of the experts' tile counts
+    int4 chunk[kMaxCand / 32];    // per 32 experts: pairs, tiles, active experts, most pairs of one expert
 };
 
 // From per-expert pair counts in sh.cnt: exclusive offsets, P, U, and the tile list of the expert
@@ -23,45 +24,54 @@ __device__ __forceinline__ void finish_expert_scan(ScanShared &sh, int n_real, i
                                                    int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                                                    const WorkLists &wl, bool write_global = true,
                                                    int list_part = 0, int list_parts = 1, int tile_rows = kPairTileM) {
-    if (threadIdx.x < 32) {
-        // warp 0 scans the per-expert sequences in steps of 32 with shuffle prefix sums
-        int base_off = 0, base_ptile = 0, active = 0, max_rows = 0;
-        for (int e0 = 0; e0 < n_real; e0 += 32) {
-            const int i = e0 + threadIdx.x;
-            const int c = (i < n_real) ? sh.cnt[i] : 0;
-            const int pt = (c + tile_rows - 1) / tile_rows;
-            int so = c, sp = pt;
+    // every warp scans chunks of 32 experts with shuffle prefix sums (a single warp walking all chunks is a
+    // chain of 4 x 17 dependent shuffles for 128 experts); the chunk totals are then added up by every thread
+    const int lane = threadIdx.x & 31, n_chunks = (n_real + 31) / 32;
+    for (int ch = threadIdx.x >> 5; ch < n_chunks; ch += blockDim.x >> 5) {
+        const int i = 32 * ch + lane;
+        const int c = (i < n_real) ? sh.cnt[i] : 0;
+        const int pt = (c + tile_rows - 1) / tile_rows;
+        int so = c, sp = pt;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int a = __shfl_up_sync(kFull, so, o);
-                const int q = __shfl_up_sync(kFull, sp, o);
-                if ((int)threadIdx.x >= o) { so += a; sp += q; }
-            }
-            if (i < n_real) {
-                sh.off[i] = base_off + so - c;
-                sh.ptile[i] = base_ptile + sp - pt;
-            }
-            base_off += __shfl_sync(kFull, so, 31);
-            base_ptile += __shfl_sync(kFull, sp, 31);
-            active += __popc(__ballot_sync(kFull, c > 0));
-            int mx = c;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, o));
-            max_rows = max(max_rows, mx);
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(kFull, so, o);
+            const int q = __shfl_up_sync(kFull, sp, o);
+            if (lane >= o) { so += a; sp += q; }
         }
-        if (threadIdx.x == 0) {
-            sh.off[n_real] = base_off;
-            sh.ptile[n_real] = base_ptile;
+        const int active = __popc(__ballot_sync(kFull, c > 0)), mx = __reduce_max_sync(kFull, c);
+        if (i < n_real) {
+            sh.off[i] = so - c;
+            sh.ptile[i] = sp - pt;
         }
-        if (threadIdx.x == 0 && write_global) {
-            meta[kMetaPairs] = base_off;
-            meta[kMetaActive] = active;
-            meta[kMetaZeroSlots] = total_slots - base_off;
-            meta[kMetaPairTiles] = base_ptile;
-            meta[kMetaMaxRows] = max_rows;
-            meta[kMetaNextItem1] = 0;
-            meta[kMetaNextItem2] = 0;
-            if (n_pairs_out) *n_pairs_out = base_off;
+        if (lane == 31) sh.chunk[ch] = make_int4(so, sp, active, mx);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= n_real; i += blockDim.x) {  // entry n_real: the totals
+        int off = 0, tiles = 0, active = 0, max_rows = 0;
+        const int before = i < n_real ? i >> 5 : n_chunks;
+        for (int ch = 0; ch < before; ++ch) {
+            const int4 v = sh.chunk[ch];
+            off += v.x;
+            tiles += v.y;
+            active += v.z;
+            max_rows = max(max_rows, v.w);
+        }
+        if (i < n_real) {
+            sh.off[i] += off;
+            sh.ptile[i] += tiles;
+        } else {
+            sh.off[n_real] = off;
+            sh.ptile[n_real] = tiles;
+            if (write_global) {
+                meta[kMetaPairs] = off;
+                meta[kMetaActive] = active;
+                meta[kMetaZeroSlots] = total_slots - off;
+                meta[kMetaPairTiles] = tiles;
+                meta[kMetaMaxRows] = max_rows;
+                meta[kMetaNextItem1] = 0;
+                meta[kMetaNextItem2] = 0;
+                if (n_pairs_out) *n_pairs_out = off;
+            }
         }
     }
     __syncthreads();

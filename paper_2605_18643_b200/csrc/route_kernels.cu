@@ -91,6 +91,65 @@ router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restric
     }
 }
 
+// Few tokens: one candidate row per CTA, so that the rows (1.5 MB for 192 candidates of 2048) are read by
+// 192 SM-wide bursts instead of 24; the reduction axis is split over four warps.  NT tokens per CTA, all
+// of their loads in flight at once.  The row is asked into L2 before the wait for the kernel in front (a
+// prefetch only: its values are read after the wait).
+constexpr int kFewTokens = 32;  // calls of at most this many tokens
+constexpr int kFewThreads = 128;
+constexpr int kFewUnroll = 4;
+
+template <int NT>
+__global__ void __launch_bounds__(kFewThreads)
+router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w,
+                         const float *__restrict__ router_bias, int T, int d, int n_cand, float *__restrict__ logits) {
+    pdl_launch_dependents();
+    const int j = blockIdx.x, t0 = blockIdx.y * NT;
+    const float *wrow = router_w + (size_t)j * d;
+    for (int i = threadIdx.x; i < d / 32; i += kFewThreads) asm volatile("prefetch.global.L2 [%0];" ::"l"(wrow + 32 * i));
+    pdl_wait();
+    float acc[NT];
+#pragma unroll
+    for (int r = 0; r < NT; ++r) acc[r] = 0.f;
+    for (int c0 = threadIdx.x; c0 < d / 4; c0 += kFewThreads * kFewUnroll) {
+        float4 w[kFewUnroll];
+        uint2 xv[NT][kFewUnroll];
+#pragma unroll
+        for (int u = 0; u < kFewUnroll; ++u) {
+            const int c = c0 + kFewThreads * u;
+            const bool in = c < d / 4;
+            w[u] = in ? __ldg(reinterpret_cast<const float4 *>(wrow) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < NT; ++r)
+                xv[r][u] = in && t0 + r < T ? __ldg(reinterpret_cast<const uint2 *>(x + (size_t)(t0 + r) * d) + c) : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int r = 0; r < NT; ++r) {
+#pragma unroll
+            for (int u = 0; u < kFewUnroll; ++u) {
+                acc[r] = fmaf(w[u].x, __uint_as_float(xv[r][u].x << 16), acc[r]);
+                acc[r] = fmaf(w[u].y, __uint_as_float(xv[r][u].x & 0xffff0000u), acc[r]);
+                acc[r] = fmaf(w[u].z, __uint_as_float(xv[r][u].y << 16), acc[r]);
+                acc[r] = fmaf(w[u].w, __uint_as_float(xv[r][u].y & 0xffff0000u), acc[r]);
+            }
+        }
+    }
+    __shared__ float red[kFewThreads / 32][NT];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int r = 0; r < NT; ++r) {
+        const float s = warp_sum(acc[r]);
+        if (lane == 0) red[warp][r] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < NT && t0 + (int)threadIdx.x < T) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < kFewThreads / 32; ++q) s += red[q][threadIdx.x];
+        logits[(size_t)(t0 + threadIdx.x) * n_cand + j] = s + (router_bias ? __ldg(router_bias + j) : 0.f);
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Softmax, top-K and routing weights: one warp per token, logits held in registers (candidate
 // j lives in lane j % 32, register j / 32).  K rounds of warp arg-max; equal logits go to the
@@ -290,8 +349,9 @@ constexpr int kSmallTokens = 128;
 constexpr int kSmallCluster = 8;
 constexpr int kSmallThreads = 32 * (kSmallTokens / kSmallCluster);  // one warp per token
 
-template <int RPL>
-__global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallThreads)
+// CLUSTER = 1: up to 16 tokens fit one CTA, which saves the cluster's launch and barriers.
+template <int RPL, int CLUSTER>
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kSmallThreads)
 route_small_kernel(const float *__restrict__ logits, int T, int n_real, int n_cand, int K, int gate_mode,
                    int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ counts,
                    int32_t *__restrict__ offsets, int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
@@ -304,11 +364,11 @@ route_small_kernel(const float *__restrict__ logits, int T, int n_real, int n_ca
     __shared__ ScanShared sh;
     __shared__ uint32_t sel[kMaxCand][kSmallTokens / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned rank = cluster.block_rank();
+    const unsigned rank = CLUSTER > 1 ? cluster.block_rank() : 0u;
     if (rank == 0)
         for (int i = threadIdx.x; i < n_real * (kSmallTokens / 32); i += blockDim.x) (&sel[0][0])[i] = 0u;
-    cluster.sync();
-    uint32_t *sel0 = cluster.map_shared_rank(&sel[0][0], 0);
+    if (CLUSTER > 1) cluster.sync(); else __syncthreads();
+    uint32_t *sel0 = CLUSTER > 1 ? cluster.map_shared_rank(&sel[0][0], 0) : &sel[0][0];
     const int t = rank * (kSmallThreads / 32) + warp;
     if (t < T) {
         int my_idx;
@@ -320,7 +380,8 @@ route_small_kernel(const float *__restrict__ logits, int T, int n_real, int n_ca
             if (my_idx < n_real) atomicOr(sel0 + my_idx * (kSmallTokens / 32) + (t >> 5), 1u << (t & 31));
         }
     }
-    cluster.sync();  // release/acquire at cluster scope: masks and topk_idx of every CTA are visible
+    // release/acquire at cluster (CTA) scope: masks and topk_idx of every CTA are visible
+    if (CLUSTER > 1) cluster.sync(); else __syncthreads();
     if (rank != 0) return;
     if ((int)threadIdx.x < n_real) {
         int c = 0;
@@ -640,6 +701,17 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
     }
     const int d = h->cfg.d_model, n_cand = h->cfg.n_real + h->cfg.n_zero;
     const int tiles = (T + kTok - 1) / kTok;
+    if (T <= kFewTokens) {
+        auto go = [&](auto kernel, int per_cta) {
+            return launch_kernel(h->pdl, kernel, dim3(n_cand, (T + per_cta - 1) / per_cta), dim3(kFewThreads), 0, s, x, h->router_w,
+                                 h->router_bias, T, d, n_cand, logits);
+        };
+        const cudaError_t e = T == 1   ? go(router_logits_few_kernel<1>, 1)
+                              : T == 2 ? go(router_logits_few_kernel<2>, 2)
+                              : T <= 4 ? go(router_logits_few_kernel<4>, 4)
+                                       : go(router_logits_few_kernel<8>, 8);
+        return e == cudaSuccess ? 1 : -1;
+    }
     // split the candidates over grid.y until the grid covers the SMs about twice
     int splits = 1;
     const int max_splits = (n_cand + 7) / 8;
@@ -669,9 +741,10 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         else { CALL(16); }                             \
     } while (0)
     if (T <= kSmallTokens && c.n_real <= kSmallThreads) {
+        const bool one_cta = T <= kSmallTokens / kSmallCluster;
 #define ZEDA_CALL_SMALL(R)                                                                                         \
-    launch_kernel(h->pdl, route_small_kernel<R>, dim3(kSmallCluster), dim3(kSmallThreads), 0, s,                    \
-        logits, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
+    launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1> : route_small_kernel<R, kSmallCluster>,                \
+        dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
         ws.meta, wl, tile_rows, ws.perm, out.perm, ws.inv, ws.pair_token)
         ZEDA_RPL_DISPATCH(ZEDA_CALL_SMALL);
 #undef ZEDA_CALL_SMALL

@@ -1,0 +1,313 @@
+// Expert kernels for the smallest batches (a few decoding sequences): weight streams without a ring.
+//
+// With T tokens a call reads at most T * K experts, each for one or a few pair rows: 2 x 6.3 + 3.1 MB
+// of weights per active expert at d = 2048, H_e = 768 and next to no arithmetic.  What bounds such a
+// call is how evenly that read spreads over the SMs and how long the chain of dependent steps is.  The
+// tensor-memory kernels of expert_pair.cu hand out work in items of 256 or 512 weight rows (one token:
+// 12 items for 74 CTA pairs), so here the work is cut into blocks of 16 weight rows, the M of the
+// warp-level MMA, and the weights go from global memory straight into its A fragments.
+//
+// Fragment trick: the sum over k may be taken in any order, so lane (g, t) of a warp reads 16
+// consecutive bytes of weight row g (k = 32 b + 8 t ..) as the A operands of two m16n8k16 MMAs and the
+// same 16 bytes of the pair row of column g as their B operands.  Every load is a full 16 bytes, four
+// lanes cover 64 consecutive bytes of a row, and nothing goes through shared memory.
+#include "zeda_internal.h"
+
+namespace zeda {
+
+namespace {
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// 32 k of 16 weight rows (lo: row g, hi: row g + 8 of the fragment) times 8 pair rows
+__device__ __forceinline__ void mma_block(float (&c)[4], const uint4 &lo, const uint4 &hi, const uint4 &b) {
+    mma_bf16(c, lo.x, hi.x, lo.y, hi.y, b.x, b.y);
+    mma_bf16(c, lo.z, hi.z, lo.w, hi.w, b.z, b.w);
+}
+
+// weights are read once per call: past L1
+__device__ __forceinline__ uint4 ld_weights(const __nv_bfloat16 *p) {
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
+// activations come from the kernel before: straight from L2
+__device__ __forceinline__ uint4 ld_rows(const __nv_bfloat16 *p) { return __ldcg(reinterpret_cast<const uint4 *>(p)); }
+
+constexpr uint4 kZero4 = {0u, 0u, 0u, 0u};
+static_assert(kStreamTokens <= 16, "the kernels are instantiated for up to two column tiles of 8 pair rows");
+
+// The routing results of the call, brought into shared memory by independent loads (one round trip)
+// instead of chains of dependent ones.  One tile of the tile list per active expert: an expert has at
+// most one pair per token, and T <= kStreamTokens is below every tile height.
+struct RouteTables {
+    int32_t expert[kStreamSlots];  // active experts in id order
+    int32_t off[kMaxCand + 1];
+    int32_t n_tiles;
+};
+
+__device__ __forceinline__ void load_route_tables(RouteTables &rt, const int32_t *tile_expert, const int32_t *offsets,
+                                                  const int32_t *meta, int slots, int n_real) {
+    for (int i = threadIdx.x; i < min(slots, n_real); i += blockDim.x) rt.expert[i] = __ldcg(tile_expert + i);
+    for (int i = threadIdx.x; i <= n_real; i += blockDim.x) rt.off[i] = __ldcg(offsets + i);
+    if (threadIdx.x == blockDim.x - 1) rt.n_tiles = __ldcg(meta + kMetaPairTiles);
+}
+
+// GEMM1 + SwiGLU.  Unit = (active expert, 8 features): rows g of the fragment are the 8 gate rows, rows
+// g + 8 the 8 up rows, so a lane's accumulators hold gate and up of the same feature and pair and
+// SwiGLU needs no exchange.  The eight warps of a CTA split the reduction axis; their partial sums meet
+// in shared memory (double-buffered: one barrier per unit), added in warp order.  The next unit's
+// weights are requested before the current one is reduced.
+constexpr int kUpWarps = 8;
+constexpr int kUpChunk = 4;  // 32-k blocks a warp keeps in flight: 4 x (2 x 512 B of weights)
+
+template <int NT>
+__global__ void __launch_bounds__(32 * kUpWarps, NT == 1 ? 3 : 2)
+stream_gate_up_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const int32_t *__restrict__ offsets,
+                      const int32_t *__restrict__ tile_expert, const int32_t *__restrict__ pair_token,
+                      const int32_t *__restrict__ meta, int slots, int n_real, int d, int He, __nv_bfloat16 *__restrict__ hmid) {
+    __shared__ RouteTables rt;
+    __shared__ int32_t s_tok[kStreamSlots];
+    __shared__ float part[2][kUpWarps][NT][4][32];
+    pdl_wait();
+    pdl_launch_dependents();  // only now: the down kernel reads the routing results before its own wait
+    load_route_tables(rt, tile_expert, offsets, meta, slots, n_real);
+    for (int i = threadIdx.x; i < slots; i += blockDim.x) s_tok[i] = __ldcg(pair_token + i);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int groups = He / 8, units = rt.n_tiles * groups;
+    const int kblocks = d / 32, batches = (kblocks + kUpWarps * kUpChunk - 1) / (kUpWarps * kUpChunk);
+    uint4 wg[kUpChunk], wu[kUpChunk], xb[kUpChunk];
+    float acc[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
+    auto row_of = [&](int pos0, int n, int col) -> const __nv_bfloat16 * {
+        return col < n ? x + (size_t)s_tok[pos0 + col] * d : nullptr;
+    };
+    auto fetch = [&](int u, int batch) {
+        const int e = rt.expert[u / groups], f0 = (u % groups) * 8;
+        const __nv_bfloat16 *gate = w + ((size_t)e * 2 * He + f0 + g) * d, *up = gate + (size_t)He * d;
+        const __nv_bfloat16 *row = row_of(rt.off[e], rt.off[e + 1] - rt.off[e], g);
+#pragma unroll
+        for (int i = 0; i < kUpChunk; ++i) {
+            const int b = (batch * kUpWarps + warp) * kUpChunk + i, k = b * 32 + t * 8;
+            const bool in = b < kblocks;
+            wg[i] = in ? ld_weights(gate + k) : kZero4;
+            wu[i] = in ? ld_weights(up + k) : kZero4;
+            xb[i] = in && row ? ld_rows(row + k) : kZero4;
+        }
+    };
+    int u = blockIdx.x, batch = 0, buf = 0;
+    if (u < units) fetch(u, 0);
+    while (u < units) {
+        const int e = rt.expert[u / groups], f0 = (u % groups) * 8, pos0 = rt.off[e], n = rt.off[e + 1] - pos0;
+        const bool last = batch + 1 == batches;
+#pragma unroll
+        for (int i = 0; i < kUpChunk; ++i) mma_block(acc[0], wg[i], wu[i], xb[i]);
+#pragma unroll
+        for (int nt = 1; nt < NT; ++nt) {
+            if (8 * nt >= n) break;  // (uniform over the CTA)
+            const __nv_bfloat16 *row = row_of(pos0, n, 8 * nt + g);
+            uint4 xc[kUpChunk];
+#pragma unroll
+            for (int i = 0; i < kUpChunk; ++i) {
+                const int b = (batch * kUpWarps + warp) * kUpChunk + i;
+                xc[i] = b < kblocks && row ? ld_rows(row + b * 32 + t * 8) : kZero4;
+            }
+#pragma unroll
+            for (int i = 0; i < kUpChunk; ++i) mma_block(acc[nt], wg[i], wu[i], xc[i]);
+        }
+        const int nu = last ? u + gridDim.x : u, nb = last ? 0 : batch + 1;
+        if (nu < units) fetch(nu, nb);
+        if (last) {
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (8 * nt < n) part[buf][warp][nt][c][lane] = acc[nt][c];
+                    acc[nt][c] = 0.f;
+                }
+            __syncthreads();
+            if (threadIdx.x < 64 * NT) {
+                const int nt = threadIdx.x >> 6, j = (threadIdx.x >> 5) & 1, col = 8 * nt + 2 * t + j;
+                if (col < n) {
+                    float gs = 0.f, us = 0.f;
+#pragma unroll
+                    for (int q = 0; q < kUpWarps; ++q) { gs += part[buf][q][nt][j][lane]; us += part[buf][q][nt][2 + j][lane]; }
+                    hmid[(size_t)(pos0 + col) * He + f0 + g] = __float2bfloat16_rn(swiglu(gs, us));
+                }
+            }
+            buf ^= 1;
+        }
+        u = nu;
+        batch = nb;
+    }
+}
+
+// GEMM2 with the weighted combine of Eq. 1: CTA b owns output features [16 b, 16 b + 16) of every token
+// and walks all active experts, so the sum over a token's slots never leaves the CTA.  Sixteen warps:
+// four experts at a time, four slices of the reduction axis; each warp keeps its partial sums of every
+// pair in shared memory and no barrier stands in the stream.  W_down does not depend on GEMM1: the
+// first weights are requested before the wait for it.  At the end the slices are added in order, each
+// expert output is rounded to bf16 (as the other expert kernels store it) and the token's slots are
+// summed in slot order in fp32.
+// resid given: r <- bf16(r + bf16(y)) in place of storing y.
+constexpr int kDownWarps = 16, kDownSlices = 4, kDownExperts = kDownWarps / kDownSlices;
+constexpr int kDownChunk = 6;
+constexpr int kDownStride = 20;  // floats per pair and slice: 16 features; 20 keeps the fragment stores free of bank conflicts
+
+template <int NT>
+__global__ void __launch_bounds__(32 * kDownWarps, 1)
+stream_down_combine_kernel(const __nv_bfloat16 *__restrict__ hmid, const __nv_bfloat16 *__restrict__ w, const int32_t *__restrict__ offsets,
+                           const int32_t *__restrict__ tile_expert, const int32_t *__restrict__ inv,
+                           const float *__restrict__ topk_w, const int32_t *__restrict__ meta, const __nv_bfloat16 *__restrict__ x,
+                           int T, int K, int n_real, int d, int He, int copy_experts, __nv_bfloat16 *__restrict__ y,
+                           __nv_bfloat16 *__restrict__ resid) {
+    __shared__ RouteTables rt;
+    __shared__ int32_t s_inv[kStreamSlots];
+    __shared__ float s_w[kStreamSlots];
+    extern __shared__ float part[];  // [kDownSlices][slots][kDownStride]
+    pdl_launch_dependents();
+    const int slots = T * K;
+    load_route_tables(rt, tile_expert, offsets, meta, slots, n_real);
+    for (int i = threadIdx.x; i < slots; i += blockDim.x) { s_inv[i] = __ldcg(inv + i); s_w[i] = __ldcg(topk_w + i); }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int slice = warp % kDownSlices, m0 = blockIdx.x * 16;
+    const int kblocks = He / 32, batches = (kblocks + kDownSlices * kDownChunk - 1) / (kDownSlices * kDownChunk);
+    const int n_tiles = rt.n_tiles;
+    uint4 lo[kDownChunk], hi[kDownChunk], hb[kDownChunk];
+    float acc[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
+    auto fetch_w = [&](int tile, int batch) {
+        const __nv_bfloat16 *row = w + ((size_t)rt.expert[tile] * d + m0 + g) * He;
+#pragma unroll
+        for (int i = 0; i < kDownChunk; ++i) {
+            const int b = (batch * kDownSlices + slice) * kDownChunk + i, k = b * 32 + t * 8;
+            const bool in = b < kblocks;
+            lo[i] = in ? ld_weights(row + k) : kZero4;
+            hi[i] = in ? ld_weights(row + (size_t)8 * He + k) : kZero4;
+        }
+    };
+    auto fetch_h = [&](uint4 (&v)[kDownChunk], int tile, int batch, int col) {
+        const int e = rt.expert[tile], pos0 = rt.off[e];
+        const bool has = pos0 + col < rt.off[e + 1];
+        const __nv_bfloat16 *row = hmid + (size_t)(pos0 + col) * He;
+#pragma unroll
+        for (int i = 0; i < kDownChunk; ++i) {
+            const int b = (batch * kDownSlices + slice) * kDownChunk + i;
+            v[i] = has && b < kblocks ? ld_rows(row + b * 32 + t * 8) : kZero4;
+        }
+    };
+    int tile = warp / kDownSlices, batch = 0;
+    if (tile < n_tiles) fetch_w(tile, 0);
+    pdl_wait();  // hmid is GEMM1's output
+    if (tile < n_tiles) fetch_h(hb, tile, 0, g);
+    while (tile < n_tiles) {
+        const int e = rt.expert[tile], pos0 = rt.off[e], n = rt.off[e + 1] - pos0;
+        const bool last = batch + 1 == batches;
+#pragma unroll
+        for (int i = 0; i < kDownChunk; ++i) mma_block(acc[0], lo[i], hi[i], hb[i]);
+#pragma unroll
+        for (int nt = 1; nt < NT; ++nt) {
+            if (8 * nt >= n) break;  // (uniform over the warp)
+            uint4 hc[kDownChunk];
+            fetch_h(hc, tile, batch, 8 * nt + g);
+#pragma unroll
+            for (int i = 0; i < kDownChunk; ++i) mma_block(acc[nt], lo[i], hi[i], hc[i]);
+        }
+        const int ntile = last ? tile + kDownExperts : tile, nb = last ? 0 : batch + 1;
+        if (ntile < n_tiles) { fetch_w(ntile, nb); fetch_h(hb, ntile, nb, g); }
+        if (last) {
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                float *p = part + ((size_t)slice * slots + pos0 + 8 * nt + 2 * t) * kDownStride;
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    if (8 * nt + 2 * t + j < n) {
+                        p[j * kDownStride + g] = acc[nt][j];
+                        p[j * kDownStride + g + 8] = acc[nt][2 + j];
+                    }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
+            }
+        }
+        tile = ntile;
+        batch = nb;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < T * 16; i += blockDim.x) {
+        const int tok = i >> 4, f = i & 15;
+        const size_t at = (size_t)tok * d + m0 + f;
+        float sum = 0.f, zero_mass = 0.f;
+        for (int k = 0; k < K; ++k) {
+            const int pos = s_inv[tok * K + k];
+            const float wk = s_w[tok * K + k];
+            if (pos < 0) { zero_mass += wk; continue; }
+            float o = 0.f;
+#pragma unroll
+            for (int q = 0; q < kDownSlices; ++q) o += part[((size_t)q * slots + pos) * kDownStride + f];
+            sum = fmaf(wk, __bfloat162float(__float2bfloat16_rn(o)), sum);
+        }
+        if (copy_experts && zero_mass != 0.f) sum = fmaf(zero_mass, __bfloat162float(x[at]), sum);
+        const __nv_bfloat16 out = __float2bfloat16_rn(sum);
+        if (resid) resid[at] = __float2bfloat16_rn(__bfloat162float(resid[at]) + __bfloat162float(out));
+        else y[at] = out;
+    }
+}
+
+int down_smem_bytes(int slots) { return kDownSlices * slots * kDownStride * (int)sizeof(float); }
+
+}  // namespace
+
+bool stream_path(const zeda_moe *h, int T) {
+    const zeda_moe_config_t &c = h->cfg;
+    return c.ep_size < 1 && T <= kStreamTokens && T * c.top_k <= kStreamSlots;
+}
+
+int init_stream_kernels() {
+    const int smem = down_smem_bytes(kStreamSlots);
+    const bool ok = cudaFuncSetAttribute(stream_down_combine_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                    cudaFuncSetAttribute(stream_down_combine_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+    return ok ? 0 : -1;
+}
+
+int launch_stream_gemm1(const zeda_moe *h, const __nv_bfloat16 *x, int T, cudaStream_t s) {
+    const zeda_moe_config_t &c = h->cfg;
+    const Workspace &ws = h->ws;
+    const int slots = T * c.top_k;
+    auto go = [&](auto kernel, int per_sm) {
+        const int units = (slots < c.n_real ? slots : c.n_real) * (c.d_expert / 8);
+        const int grid = units < per_sm * h->sm_count ? units : per_sm * h->sm_count;
+        return launch_kernel(h->pdl, kernel, dim3(grid), dim3(32 * kUpWarps), 0, s, x, h->w_gate_up, (const int32_t *)ws.offsets,
+                             (const int32_t *)ws.ptile_expert, (const int32_t *)ws.pair_token, (const int32_t *)ws.meta, slots,
+                             (int)c.n_real, (int)c.d_model, (int)c.d_expert, ws.hmid);
+    };
+    const cudaError_t e = T <= 8 ? go(stream_gate_up_kernel<1>, 3) : go(stream_gate_up_kernel<2>, 2);
+    return e == cudaSuccess ? 1 : -1;
+}
+
+int launch_stream_down(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y, __nv_bfloat16 *resid, cudaStream_t s) {
+    const zeda_moe_config_t &c = h->cfg;
+    const Workspace &ws = h->ws;
+    auto go = [&](auto kernel) {
+        return launch_kernel(h->pdl, kernel, dim3(c.d_model / 16), dim3(32 * kDownWarps), down_smem_bytes(T * c.top_k), s,
+                             (const __nv_bfloat16 *)ws.hmid, h->w_down, (const int32_t *)ws.offsets, (const int32_t *)ws.ptile_expert,
+                             (const int32_t *)ws.inv, (const float *)ws.topk_w, (const int32_t *)ws.meta, x, T, (int)c.top_k,
+                             (int)c.n_real, (int)c.d_model, (int)c.d_expert, (int)(c.expert_kind == ZEDA_EXPERT_COPY), y, resid);
+    };
+    const cudaError_t e = T <= 8 ? go(stream_down_combine_kernel<1>) : go(stream_down_combine_kernel<2>);
+    return e == cudaSuccess ? 1 : -1;
+}
+
+}  // namespace zeda

@@ -80,6 +80,13 @@ residual_rmsnorm_kernel(__nv_bfloat16 *__restrict__ r, const __nv_bfloat16 *__re
 }
 
 }  // namespace
+
+int launch_residual_rmsnorm(bool pdl, __nv_bfloat16 *r, const __nv_bfloat16 *y, __nv_bfloat16 *h, int T, int d, float eps,
+                            cudaStream_t s) {
+    const cudaError_t e = launch_kernel(pdl, residual_rmsnorm_kernel, dim3(T), dim3(kGlueThreads), 0, s, r, y, h, d, eps);
+    return e == cudaSuccess ? 1 : -1;
+}
+
 }  // namespace zeda
 
 extern "C" zeda_status_t zeda_residual_rmsnorm(void *r, const void *y, void *h, int32_t T, int32_t d_model, float eps,
@@ -97,10 +104,10 @@ extern "C" zeda_status_t zeda_residual_rmsnorm(void *r, const void *y, void *h, 
         return ZEDA_ERR_INVALID_ARG;
     }
     if (!(eps >= 0.f)) { set_error("eps must be >= 0"); return ZEDA_ERR_INVALID_ARG; }
-    const cudaError_t e = launch_kernel(true, residual_rmsnorm_kernel, dim3(T), dim3(kGlueThreads), 0,
-                                        static_cast<cudaStream_t>(stream), static_cast<__nv_bfloat16 *>(r),
-                                        static_cast<const __nv_bfloat16 *>(y), static_cast<__nv_bfloat16 *>(h),
-                                        (int)d_model, eps);
-    if (e != cudaSuccess) { set_error("zeda_residual_rmsnorm launch: %s", cudaGetErrorString(e)); return ZEDA_ERR_CUDA; }
+    if (launch_residual_rmsnorm(true, static_cast<__nv_bfloat16 *>(r), static_cast<const __nv_bfloat16 *>(y),
+                                static_cast<__nv_bfloat16 *>(h), T, d_model, eps, static_cast<cudaStream_t>(stream)) < 0) {
+        set_error("zeda_residual_rmsnorm launch: %s", cudaGetErrorString(cudaGetLastError()));
+        return ZEDA_ERR_CUDA;
+    }
     return ZEDA_OK;
 }

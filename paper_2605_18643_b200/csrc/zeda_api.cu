@@ -162,6 +162,22 @@ zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_
     n += r;
     mark(2);
     const Workspace &ws = h->ws;
+    if (stream_path(h, T)) {  // the down projection and the combine are one kernel: its time counts as GEMM2
+        r = launch_stream_gemm1(h, x, T, s);
+        if (r < 0) return cuda_fail("expert GEMM1 launch", cudaGetLastError());
+        n += r;
+        mark(3);
+        r = launch_stream_down(h, x, T, y, resid, s);
+        if (r < 0) return cuda_fail("expert GEMM2 launch", cudaGetLastError());
+        n += r;
+        mark(4);
+        r = resid ? launch_residual_rmsnorm(h->pdl, resid, nullptr, y, T, h->cfg.d_model, eps, s) : 0;
+        if (r < 0) return cuda_fail("norm launch", cudaGetLastError());
+        mark(5);
+        h->profiled_last = prof;
+        h->last_launches = n + r;
+        return ZEDA_OK;
+    }
     const ExpertWork work = {ws.counts, ws.offsets, ws.ptile_expert, ws.ptile_row0, ws.pair_token, T * h->cfg.top_k, tile_rows_for(h, T)};
     r = launch_experts_gemm1_pair(h, x, work, s);
     if (r < 0) return cuda_fail("expert GEMM1 launch", cudaGetLastError());
@@ -249,6 +265,7 @@ zeda_status_t zeda_moe_create(const zeda_moe_config_t *cfg, const float *router_
     for (auto &ev : h->ev_host) ev = nullptr;
     carve(*cfg, static_cast<unsigned char *>(workspace), &h->ws, &h->max_tiles);
     if (init_route_kernels(h) < 0) { delete h; return cuda_fail("kernel set-up", cudaGetLastError()); }
+    if (init_stream_kernels() < 0) { delete h; return cuda_fail("kernel set-up", cudaGetLastError()); }
     if (init_pair_kernels(h) < 0) { delete h; return ZEDA_ERR_CUDA; }
     if (init_router_tile(h) < 0) {
         if (h->pmaps) free(h->pmaps);

@@ -15,6 +15,8 @@ constexpr int kSortTokens = 128;    // tokens per CTA in the counting sort (hist
 constexpr int kPairTileM = 256;     // most pair rows per tile of the expert kernels (one CTA pair, N <= 256)
 constexpr int kMidTileM = 128;      // tile rows of the geometry for mid-sized batches
 constexpr int kMaxEpRanks = 64;     // expert-parallel group size limit
+constexpr int kStreamTokens = 16;   // calls of at most this many tokens ...
+constexpr int kStreamSlots = 256;   // ... and slots run the expert kernels of small_batch.cu
 
 // Device-resident counters of one call.
 enum MetaSlot {
@@ -138,6 +140,12 @@ int tile_rows_for(const zeda_moe *h, int T);
 int launch_token_zero_share(const zeda_moe *h, int T, float *out, cudaStream_t s);
 int launch_experts_gemm1_pair(const zeda_moe *h, const __nv_bfloat16 *x, const ExpertWork &w, cudaStream_t s);
 int launch_experts_gemm2_pair(const zeda_moe *h, const ExpertWork &w, cudaStream_t s);
+// the smallest batches (small_batch.cu): GEMM1, and GEMM2 with the combine (resid given: with the residual update)
+bool stream_path(const zeda_moe *h, int T);
+int init_stream_kernels();
+int launch_stream_gemm1(const zeda_moe *h, const __nv_bfloat16 *x, int T, cudaStream_t s);
+int launch_stream_down(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y, __nv_bfloat16 *resid, cudaStream_t s);
+int launch_residual_rmsnorm(bool pdl, __nv_bfloat16 *r, const __nv_bfloat16 *y, __nv_bfloat16 *h, int T, int d, float eps, cudaStream_t s);
 // expert-parallel pieces (expert_parallel.cu)
 int launch_ep_pack(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *send_rows, int32_t *send_counts,
                    int32_t *expert_counts, cudaStream_t s);
@@ -167,6 +175,8 @@ void note_launch_error(cudaError_t e);
 #if defined(__CUDACC__)
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ float swiglu(float g, float u) { return __fdividef(g * u, 1.f + __expf(-g)); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

@@ -1,0 +1,56 @@
+"""The expert kernels for the smallest batches (csrc/small_batch.cu) against the CPU oracle, at the edges
+of their tiles: 8 pair rows per column tile, 16 weight rows per block, reduction slices with a remainder,
+the last batch size that takes them and the first that does not."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2605_18643_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+# bf16 results of fp32 sums against 64 bits: three roundings of 2^-9 (Hmid, expert output, y)
+REL_L2, MAX_ABS_RMS = 1e-2, 5e-2
+
+
+def layer(T, d=256, He=128, E=8, Z=4, K=2, seed=5, zero_fraction=0.5):
+    return inputs.make_layer("small", T=T, d=d, He=He, E=E, Z=Z, K=K, seed=seed,
+                             zero_fraction=zero_fraction if Z else None)
+
+
+@pytest.mark.parametrize("T,shape,kind", [
+    (1, {}, 0), (2, {}, 1), (5, {}, 0), (8, {}, 0), (9, {}, 1), (16, {}, 0), (17, {}, 0), (32, {}, 0), (33, {}, 0),
+    (7, dict(d=320, He=192), 0), (16, dict(d=64, He=64), 1), (3, dict(d=1088, He=832), 0),   # slices with remainders
+    (8, dict(E=1, Z=1, K=2), 0), (16, dict(E=1, Z=0, K=1), 0),                               # every token on one expert
+    (16, dict(E=40, Z=8, K=16), 0), (9, dict(E=300, Z=100, K=16), 1),                        # widest slot table, many experts
+    (4, dict(d=2048, He=768, E=16, Z=8, K=8), 0),
+])
+def test_small_batches_match_the_oracle(T, shape, kind):
+    from paper_2605_18643_b200 import zeda
+    wl = layer(T, **shape)
+    dev = torch.device("cuda:0")
+    m = zeda.from_workload(wl, dev, expert_kind=kind)
+    x = wl.x.to(dev)
+    y = m.forward(x)
+    r = torch.randn(wl.T, wl.d, generator=torch.Generator().manual_seed(3)).to(torch.bfloat16).to(dev)
+    want_r = (r.float() + y.float()).to(torch.bfloat16)
+    want_h = zeda.residual_rmsnorm(want_r.clone(), None)
+    h = torch.empty_like(r)
+    m.forward_residual(x, r, h)
+    torch.cuda.synchronize()
+    bias = None if wl.router_bias is None else wl.router_bias.numpy()
+    y_ref, idx, _ = oracle.forward(inputs.bits(wl.x), wl.router_w.numpy(), bias, inputs.bits(wl.w_gate_up),
+                                   inputs.bits(wl.w_down), wl.E, wl.Z, wl.K, expert_kind=kind)
+    got = y.float().cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - y_ref) <= REL_L2 * np.linalg.norm(y_ref)
+    assert np.max(np.abs(got - y_ref)) <= MAX_ABS_RMS * max(np.sqrt(np.mean(y_ref ** 2)), 1e-30)
+    assert torch.equal(r.view(torch.int16), want_r.view(torch.int16))
+    assert torch.equal(h.view(torch.int16), want_h.view(torch.int16))
+    if kind == 0:
+        dead = np.nonzero((idx >= wl.E).all(axis=1))[0]
+        if dead.size:
+            assert int(y[torch.as_tensor(dead, device=dev)].view(torch.int16).abs().max().item()) == 0
+    P = m.last_counters()[0]
+    assert P == int((idx < wl.E).sum())
+    m.close()
