@@ -157,33 +157,42 @@ router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__res
 // ---------------------------------------------------------------------------------------------
 constexpr int kRegsPerLane = kMaxCand / 32;
 
-// Top-K and routing weights of one token by one warp.  On return lane k < K holds slot k.
+// Top-K and routing weights of one token by one warp.  On return lane k < K holds slot k, and v, m, den
+// the logits (-inf beyond n_cand), their maximum and the softmax denominator.
 // RPL = logits per lane (32 * RPL >= n_cand).
-// The row may arrive as n_parts partial sums, part_stride floats apart; they are added in order.
+// The row may arrive as n_parts partial sums, part_stride floats apart; they are added in order, three
+// slices requested at a time (one slice after another is a chain of L2 round trips).
 template <int RPL>
 __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, int n_parts, size_t part_stride,
-                                                int n_real, int n_cand, int K,
-                                                int gate_mode, int lane, int &my_idx, float &my_w) {
-    float v[RPL];
+                                                int n_real, int n_cand, int K, int gate_mode, int lane,
+                                                float (&v)[RPL], float &m, float &den, int &my_idx, float &my_w) {
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
         const int j = r * 32 + lane;
         v[r] = (j < n_cand) ? row[j] : -INFINITY;
     }
-    for (int p = 1; p < n_parts; ++p) {
+    for (int p = 1; p < n_parts; p += 3) {
+        float a[3][RPL];
 #pragma unroll
-        for (int r = 0; r < RPL; ++r) {
-            const int j = r * 32 + lane;
-            if (j < n_cand) v[r] += row[p * part_stride + j];
-        }
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) {
+                const int j = r * 32 + lane;
+                a[q][r] = p + q < n_parts && j < n_cand ? row[(p + q) * part_stride + j] : 0.f;
+            }
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int r = 0; r < RPL; ++r)
+                if (p + q < n_parts) v[r] += a[q][r];
     }
     // row maximum and softmax denominator over all candidates
-    float m = v[0];
+    m = v[0];
 #pragma unroll
     for (int r = 1; r < RPL; ++r) m = fmaxf(m, v[r]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
-    float den = 0.f;
+    den = 0.f;
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
         const int j = r * 32 + lane;
@@ -244,9 +253,9 @@ topk_gate_kernel(const float *__restrict__ logits, int n_parts, int T, int n_rea
     const int t = blockIdx.x * (blockDim.x >> 5) + warp;
     if (t >= T) return;
     int my_idx;
-    float my_w;
+    float my_w, v[RPL], m, den;
     topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
-                         my_idx, my_w);
+                         v, m, den, my_idx, my_w);
     if (lane < K) {
         topk_idx[(size_t)t * K + lane] = my_idx;
         topk_w[(size_t)t * K + lane] = my_w;
@@ -372,8 +381,8 @@ route_small_kernel(const float *__restrict__ logits, int T, int n_real, int n_ca
     const int t = rank * (kSmallThreads / 32) + warp;
     if (t < T) {
         int my_idx;
-        float my_w;
-        topk_gate_token<RPL>(logits + (size_t)t * n_cand, 1, 0, n_real, n_cand, K, gate_mode, lane, my_idx, my_w);
+        float my_w, v[RPL], m, den;
+        topk_gate_token<RPL>(logits + (size_t)t * n_cand, 1, 0, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
             topk_w[(size_t)t * K + lane] = my_w;
@@ -509,40 +518,29 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
     for (int i = threadIdx.x; i < kPlaceWarps * n_real; i += blockDim.x) pos[i] = 0;
     for (int e = threadIdx.x; e < n_real; e += blockDim.x) { base[e] = 0; sh.cnt[e] = 0; }
     // column sums of the CTA histograms: staged slab by slab with independent coalesced loads (a
-    // per-thread loop over global memory would be one L2 round trip after another)
+    // per-thread loop over global memory would be one L2 round trip after another); with fewer experts
+    // than threads, several threads share a column
     const int slab_blocks = max(1, kScanSlabInts / n_real);
+    const int col_parts = max(1, (int)blockDim.x / n_real);
     for (int b0 = 0; b0 < nblk; b0 += slab_blocks) {
         const int nb = min(slab_blocks, nblk - b0);
         const int32_t *g = block_hist + (size_t)b0 * n_real;
         __syncthreads();
         stage_ints(slab, g, nb * n_real);
         __syncthreads();
-        for (int e = threadIdx.x; e < n_real; e += blockDim.x) {
+        for (int i = threadIdx.x; i < n_real * col_parts; i += blockDim.x) {
+            const int e = i % n_real;
             int before = 0, total = 0;
-            for (int b = 0; b < nb; ++b) {
+#pragma unroll 4
+            for (int b = i / n_real; b < nb; b += col_parts) {
                 const int c = slab[b * n_real + e];
                 total += c;
                 if (b0 + b < (int)blockIdx.x) before += c;
             }
-            base[e] += before;
-            sh.cnt[e] += total;
+            atomicAdd(&base[e], before);
+            atomicAdd(&sh.cnt[e], total);
         }
     }
-    __syncthreads();
-    // The histograms go back to zero for the next call's top-K kernel: the CTA that is last to have
-    // read them (a ticket, nobody waits) clears them and the ticket counter.
-    __shared__ int s_ticket;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_ticket = atomicAdd(meta + kMetaHistTicket, 1);
-    }
-    __syncthreads();
-    if (s_ticket == (int)gridDim.x - 1) {
-        for (int i = threadIdx.x; i < nblk * n_real; i += blockDim.x) block_hist[i] = 0;
-        if (threadIdx.x == 0) meta[kMetaHistTicket] = 0;
-    }
-    finish_expert_scan(sh, n_real, T * K, counts, offsets, n_pairs_out, meta, wl, blockIdx.x == 0, blockIdx.x, gridDim.x, tile_rows);
-    __syncthreads();
     int32_t *mine = pos + warp * n_real;
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
@@ -553,6 +551,16 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
         if (e >= 0 && (grp & lt) == 0) mine[e] += __popc(grp);
         __syncwarp();
     }
+    __syncthreads();
+    // The histograms go back to zero for the next call's top-K kernel: the CTA that is last to have
+    // read them (a ticket, nobody waits; looked at only when this CTA's own work is done) clears them
+    // and the ticket counter.
+    __shared__ int s_ticket;
+    if (threadIdx.x == blockDim.x - 1) {
+        __threadfence();
+        s_ticket = atomicAdd(meta + kMetaHistTicket, 1);
+    }
+    finish_expert_scan(sh, n_real, T * K, counts, offsets, n_pairs_out, meta, wl, blockIdx.x == 0, blockIdx.x, gridDim.x, tile_rows);
     __syncthreads();
     for (int e = threadIdx.x; e < n_real; e += blockDim.x) {
         int run = sh.off[e] + base[e];
@@ -584,79 +592,118 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
             }
         }
     }
+    __syncthreads();
+    if (s_ticket == (int)gridDim.x - 1) {
+        for (int i = threadIdx.x; i < nblk * n_real; i += blockDim.x) block_hist[i] = 0;
+        if (threadIdx.x == 0) meta[kMetaHistTicket] = 0;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
-// Routing statistics (Eq. 4-6 forward values), two deterministic passes: per-CTA partial sums of
-// the selection indicator and of the softmax probabilities, then a fixed-order final reduction.
+// Routing statistics (Eq. 4-6 forward values), two deterministic passes.  The top-K pass of a statistics
+// call has each token's logits, softmax maximum and denominator in registers already, so it also adds
+// up its CTA's selection counts (integers) and softmax probabilities: every warp in registers over its
+// tokens, then the warps in order.  The final pass adds the CTAs' sums in a fixed order.  (As a kernel
+// of its own, one thread per candidate walking 64 tokens, the first pass took 49 us for 8192 tokens of
+// 192 candidates and the final pass, a chain of loads per candidate, 19 us.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kStatTokens = 64;
+constexpr int kStatWarps = 32;
 
-__global__ void __launch_bounds__(256)
-stats_partial_kernel(const float *__restrict__ logits, const int32_t *__restrict__ topk_idx, int T, int K,
-                     int n_cand, float *__restrict__ part) {
-    extern __shared__ float sm[];  // [2][n_cand]
-    float *sf = sm, *sp = sm + n_cand;
-    for (int i = threadIdx.x; i < 2 * n_cand; i += blockDim.x) sm[i] = 0.f;
+template <int RPL>
+__global__ void __launch_bounds__(32 * kStatWarps)
+topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
+                  int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist, float *__restrict__ part) {
+    pdl_launch_dependents();
+    extern __shared__ float sm[];  // [kStatWarps][n_cand] probabilities, then [n_cand] counts
+    int32_t *cnt = reinterpret_cast<int32_t *>(sm + kStatWarps * n_cand);
+    for (int i = threadIdx.x; i < n_cand; i += blockDim.x) cnt[i] = 0;
     __syncthreads();
-    __shared__ float s_max[kStatTokens], s_den[kStatTokens];
+    pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t0 = blockIdx.x * kStatTokens;
-    const int t1 = min(T, t0 + kStatTokens);
-    // per-token softmax maximum and denominator, one warp per token
-    for (int t = t0 + warp; t < t1; t += (blockDim.x >> 5)) {
-        const float *row = logits + (size_t)t * n_cand;
-        float m = -INFINITY;
-        for (int c = lane; c < n_cand; c += 32) m = fmaxf(m, row[c]);
+    const int t0 = blockIdx.x * kStatTokens, t1 = min(T, t0 + kStatTokens);
+    float acc[RPL];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
-        float den = 0.f;
-        for (int c = lane; c < n_cand; c += 32) den += expf(row[c] - m);
-        den = warp_sum(den);
-        if (lane == 0) { s_max[t - t0] = m; s_den[t - t0] = den; }
-    }
-    __syncthreads();
-    // one thread per candidate, tokens summed in increasing order
-    for (int j = threadIdx.x; j < n_cand; j += blockDim.x) {
-        float accp = 0.f, accf = 0.f;
-        for (int t = t0; t < t1; ++t) {
-            accp += expf(logits[(size_t)t * n_cand + j] - s_max[t - t0]) / s_den[t - t0];
-            for (int k = 0; k < K; ++k) accf += (topk_idx[(size_t)t * K + k] == j) ? 1.f : 0.f;
+    for (int r = 0; r < RPL; ++r) acc[r] = 0.f;
+    for (int t = t0 + warp; t < t1; t += kStatWarps) {
+        int my_idx;
+        float my_w, v[RPL], m, den;
+        topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
+                             v, m, den, my_idx, my_w);
+        if (lane < K) {
+            topk_idx[(size_t)t * K + lane] = my_idx;
+            topk_w[(size_t)t * K + lane] = my_w;
+            atomicAdd(cnt + my_idx, 1);
         }
-        sf[j] = accf;
-        sp[j] = accp;
+#pragma unroll
+        for (int r = 0; r < RPL; ++r)
+            if (r * 32 + lane < n_cand) acc[r] += expf(v[r] - m) / den;
     }
+#pragma unroll
+    for (int r = 0; r < RPL; ++r)
+        if (r * 32 + lane < n_cand) sm[warp * n_cand + r * 32 + lane] = acc[r];
     __syncthreads();
-    for (int i = threadIdx.x; i < 2 * n_cand; i += blockDim.x) part[(size_t)blockIdx.x * 2 * n_cand + i] = sm[i];
+    for (int j = threadIdx.x; j < n_cand; j += blockDim.x) {
+        float p = 0.f;
+#pragma unroll 8
+        for (int w = 0; w < kStatWarps; ++w) p += sm[w * n_cand + j];
+        part[(size_t)blockIdx.x * 2 * n_cand + j] = (float)cnt[j];
+        part[(size_t)blockIdx.x * 2 * n_cand + n_cand + j] = p;
+        // pass 1 of the counting sort, as in the top-K kernel above
+        if (block_hist && j < n_real && cnt[j]) atomicAdd(block_hist + (size_t)(t0 / kSortTokens) * n_real + j, cnt[j]);
+    }
 }
 
-__global__ void __launch_bounds__(512)
+// One CTA.  Column c of the partial sums (n_cand counts, then n_cand probabilities) is shared by as many
+// threads as fit, each adding every n-th CTA's value.
+constexpr int kStatFinalThreads = 1024;
+
+__global__ void __launch_bounds__(kStatFinalThreads)
 stats_final_kernel(const float *__restrict__ part, int nblk, int T, int K, int n_real, int n_cand,
                    float *__restrict__ f, float *__restrict__ p_mean, float *__restrict__ out) {
-    __shared__ float sf[kMaxCand], sp[kMaxCand];
-    const int j = threadIdx.x;
-    if (j < n_cand) {
-        float af = 0.f, ap = 0.f;
-        for (int b = 0; b < nblk; ++b) {
-            af += part[(size_t)b * 2 * n_cand + j];
-            ap += part[(size_t)b * 2 * n_cand + n_cand + j];
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ float seg[kStatFinalThreads], col[2 * kMaxCand], red[5][kStatFinalThreads / 32];
+    const int cols = 2 * n_cand, segs = max(1, kStatFinalThreads / cols);
+    {
+        const int c = threadIdx.x % cols, s = threadIdx.x / cols;  // (at most 1024 columns)
+        float a = 0.f;
+        if (s < segs) {
+#pragma unroll 16
+            for (int b = s; b < nblk; b += segs) a += __ldcg(part + (size_t)b * cols + c);
         }
-        sf[j] = af / T;
-        sp[j] = ap / T;
-        if (f) f[j] = sf[j];
-        if (p_mean) p_mean[j] = sp[j];
+        seg[threadIdx.x] = a;
     }
     __syncthreads();
-    if (threadIdx.x == 0 && out) {
-        float la = 0.f, fE = 0.f, pE = 0.f, fZ = 0.f, pZ = 0.f;
-        for (int i = 0; i < n_cand; ++i) {
-            la += sf[i] * sp[i];
-            if (i < n_real) { fE += sf[i]; pE += sp[i]; } else { fZ += sf[i]; pZ += sp[i]; }
+    for (int c = threadIdx.x; c < cols; c += kStatFinalThreads) {
+        float a = 0.f;
+        for (int s = 0; s < segs; ++s) a += seg[s * cols + c];
+        col[c] = a / T;
+        if (c < n_cand) { if (f) f[c] = col[c]; }
+        else if (p_mean) p_mean[c - n_cand] = col[c];
+    }
+    __syncthreads();
+    if (!out) return;
+    const int j = threadIdx.x;
+    const float fj = j < n_cand ? col[j] : 0.f, pj = j < n_cand ? col[n_cand + j] : 0.f;
+    const bool real = j < n_real;
+    const float sums[5] = {fj * pj, real ? fj : 0.f, real ? pj : 0.f, real ? 0.f : fj, real ? 0.f : pj};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const float s = warp_sum(sums[i]);
+        if ((j & 31) == 0) red[i][j >> 5] = s;
+    }
+    __syncthreads();
+    if (j < 32) {
+        float tot[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) tot[i] = warp_sum(red[i][j]);
+        if (j == 0) {
+            out[0] = tot[3] / K;
+            out[1] = tot[0];
+            out[2] = tot[1] * tot[2];
+            out[3] = tot[3] * tot[4];
         }
-        out[0] = fZ / K;
-        out[1] = la;
-        out[2] = fE * pE;
-        out[3] = fZ * pZ;
     }
 }
 
@@ -664,6 +711,8 @@ stats_final_kernel(const float *__restrict__ part, int nblk, int T, int K, int n
 // token's K slots that selected a zero expert.
 __global__ void __launch_bounds__(256)
 token_zero_share_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real, float *__restrict__ out) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     int zero = 0;
@@ -674,8 +723,9 @@ token_zero_share_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int 
 }  // namespace
 
 int launch_token_zero_share(const zeda_moe *h, int T, float *out, cudaStream_t s) {
-    token_zero_share_kernel<<<(T + 255) / 256, 256, 0, s>>>(h->ws.topk_idx, T, h->cfg.top_k, h->cfg.n_real, out);
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+    const cudaError_t e = launch_kernel(h->pdl, token_zero_share_kernel, dim3((T + 255) / 256), dim3(256), 0, s,
+                                        (const int32_t *)h->ws.topk_idx, T, (int)h->cfg.top_k, (int)h->cfg.n_real, out);
+    return e == cudaSuccess ? 1 : -1;
 }
 
 int init_route_kernels(const zeda_moe *h) {
@@ -685,6 +735,13 @@ int init_route_kernels(const zeda_moe *h) {
         return -1;
     // placement CTAs: static scan state plus (per-warp positions, bases, a histogram slab) pass 48 KB
     // together when there are many experts
+    const int stats_smem = (int)sizeof(float) * (kStatWarps + 1) * kMaxCand;
+    bool ok = cudaFuncSetAttribute(topk_stats_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
+    if (!ok) return -1;
     const int place_smem = (int)sizeof(int32_t) * ((kPlaceWarps + 1) * kMaxCand + kScanSlabInts);
     if (cudaFuncSetAttribute(slot_scan_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem) != cudaSuccess)
         return -1;
@@ -724,7 +781,8 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
     return e == cudaSuccess ? 1 : -1;
 }
 
-int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s, int n_parts) {
+int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s, int n_parts,
+                             float *stat_part) {
     const zeda_moe_config_t &c = h->cfg;
     const int n_cand = c.n_real + c.n_zero, K = c.top_k;
     const Workspace &ws = h->ws;
@@ -740,7 +798,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         else if (n_cand <= 256) { CALL(8); }           \
         else { CALL(16); }                             \
     } while (0)
-    if (T <= kSmallTokens && c.n_real <= kSmallThreads) {
+    if (!stat_part && T <= kSmallTokens && c.n_real <= kSmallThreads) {
         const bool one_cta = T <= kSmallTokens / kSmallCluster;
 #define ZEDA_CALL_SMALL(R)                                                                                         \
     launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1> : route_small_kernel<R, kSmallCluster>,                \
@@ -757,8 +815,14 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
 #define ZEDA_CALL_TOPK(R) \
     launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + 7) / 8), dim3(256), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
                   c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
-        ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);
+#define ZEDA_CALL_STATS(R) \
+    launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps), \
+                  sizeof(float) * (kStatWarps + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
+                  ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
+        if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
+        else ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);
 #undef ZEDA_CALL_TOPK
+#undef ZEDA_CALL_STATS
         if (fold) {
             launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk), dim3(kPlaceWarps * 32),
                           sizeof(int32_t) * ((kPlaceWarps + 1) * c.n_real + kScanSlabInts), s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
@@ -784,15 +848,12 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
-int launch_stats(const zeda_moe *h, const float *logits, const int32_t *topk_idx, int T, float *f,
-                 float *p_mean, float *out, cudaStream_t s) {
+int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s) {
     const zeda_moe_config_t &c = h->cfg;
-    const int n_cand = c.n_real + c.n_zero;
-    const int nblk = (T + kStatTokens - 1) / kStatTokens;
-    stats_partial_kernel<<<nblk, 256, sizeof(float) * 2 * n_cand, s>>>(logits, topk_idx, T, c.top_k, n_cand,
-                                                                      h->ws.stat_part);
-    stats_final_kernel<<<1, 512, 0, s>>>(h->ws.stat_part, nblk, T, c.top_k, c.n_real, n_cand, f, p_mean, out);
-    return cudaGetLastError() == cudaSuccess ? 2 : -1;
+    const cudaError_t e = launch_kernel(h->pdl, stats_final_kernel, dim3(1), dim3(kStatFinalThreads), 0, s, (const float *)h->ws.stat_part,
+                                        (T + kStatTokens - 1) / kStatTokens, T, (int)c.top_k, (int)c.n_real, (int)(c.n_real + c.n_zero),
+                                        f, p_mean, out);
+    return e == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace zeda

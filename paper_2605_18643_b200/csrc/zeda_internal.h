@@ -119,9 +119,9 @@ int init_route_kernels(const zeda_moe *h);
 int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s,
                          int *n_parts = nullptr);
 int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s,
-                             int n_parts = 1);
-int launch_stats(const zeda_moe *h, const float *logits, const int32_t *topk_idx, int T, float *f,
-                 float *p_mean, float *out, cudaStream_t s);
+                             int n_parts = 1, float *stat_part = nullptr);
+// The statistics of the last routing pass, which was given ws.stat_part to leave its partial sums in.
+int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s);
 int router_split_pad(int n_cand);
 int init_router_tile(zeda_moe *h);
 constexpr int kRouterMaxSplit = 4;
