@@ -149,11 +149,14 @@ __device__ __forceinline__ bool double_item(int dbl_rows, int n, int mb, int m_b
 }
 
 // MODE 1: GEMM1 + SwiGLU -> Hmid[pos, f].   MODE 2: GEMM2 -> O[pos, row].
+// SCATTER (GEMM2 of an expert-parallel rank): row pos goes to O[pair_token[pos], row], the order in which
+// the rows were received; a lane fetches the target of one row of the next 32 while the current 32 are
+// stored, so the map costs one coalesced load per 32 rows and no pass over the results.
 // HALF_MAX: most B rows one CTA loads per k-step (the tile's column count is at most 2 * HALF_MAX).
 // DBL_ROWS: tiles of at most this many pair rows run as double items (0: none; at most 128).
 // One CTA per SM with two accumulator buffers in TMEM: the epilogue of a tile runs under the MMAs of
 // the CTA's next tile.
-template <int MODE, int HALF_MAX, int STAGES, int DBL_ROWS>
+template <int MODE, int HALF_MAX, int STAGES, int DBL_ROWS, bool SCATTER = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MODE == 1 ? kThreadsGather : kThreads, 1)
 expert_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowMaps maps_b,
                         const __nv_bfloat16 *__restrict__ x, int x_ld, const int32_t *__restrict__ counts,
@@ -544,8 +547,11 @@ expert_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             } else {
                 const int row0 = 256 * mb + 128 * (int)rank + 32 * q;  // first of this warp's 32 output features
                 const bool r_ok = row0 < out_rows;
+                int target = SCATTER && lane < it.n ? pair_token[it.pos0 + lane] : 0;  // of row c0 + lane
                 for (int c0 = 0; c0 < it.n; c0 += 32) {
                     float v[32];
+                    const int target_now = target;
+                    if (SCATTER) target = c0 + 32 + lane < it.n ? pair_token[it.pos0 + c0 + 32 + lane] : 0;
                     tmem_ld32(t0 + c0, v);
                     if (last_sub && c0 + 32 >= it.n) {
                         tc_fence_before();
@@ -559,8 +565,9 @@ expert_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                     for (int i = 0; i < 4; ++i) {
                         const int r = prow + 8 * i;
                         const uint4 val = *reinterpret_cast<const uint4 *>(patch + r * 32 + pch * 8);
+                        const int orow = SCATTER ? __shfl_sync(0xffffffffu, target_now, r) : it.pos0 + c0 + r;
                         if (r_ok && c0 + r < it.n)
-                            *reinterpret_cast<uint4 *>(out + (size_t)(it.pos0 + c0 + r) * out_ld + row0 + pch * 8) = val;
+                            *reinterpret_cast<uint4 *>(out + (size_t)orow * out_ld + row0 + pch * 8) = val;
                     }
                     __syncwarp();
                 }
@@ -593,17 +600,17 @@ constexpr int pair_smem_bytes() {
 }
 
 // One configuration of the kernel: its attribute set-up and its launch.
-template <int MODE, int HALF_MAX, int STAGES, int DBL_ROWS>
+template <int MODE, int HALF_MAX, int STAGES, int DBL_ROWS, bool SCATTER = false>
 struct PairKernel {
     static constexpr int kSmem = pair_smem_bytes<MODE, HALF_MAX, STAGES, DBL_ROWS>();
     static bool prepare() {
-        return cudaFuncSetAttribute(expert_gemm_pair_kernel<MODE, HALF_MAX, STAGES, DBL_ROWS>,
+        return cudaFuncSetAttribute(expert_gemm_pair_kernel<MODE, HALF_MAX, STAGES, DBL_ROWS, SCATTER>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) == cudaSuccess;
     }
     template <typename... Args>
     static cudaError_t launch(const zeda_moe *h, cudaStream_t s, Args &&...args) {
         const int grid = (h->sm_count / 2) * 2;
-        return launch_kernel(h->pdl, expert_gemm_pair_kernel<MODE, HALF_MAX, STAGES, DBL_ROWS>, dim3(grid),
+        return launch_kernel(h->pdl, expert_gemm_pair_kernel<MODE, HALF_MAX, STAGES, DBL_ROWS, SCATTER>, dim3(grid),
                              dim3(MODE == 1 ? kThreadsGather : kThreads), kSmem, s, std::forward<Args>(args)...);
     }
 };
@@ -620,8 +627,13 @@ using Gemm2Mid = PairKernel<2, 64, 9, 0>;
 using Gemm1Big = PairKernel<1, 128, 6, 64>;
 using Gemm1Wide = PairKernel<1, 128, 5, 128>;
 using Gemm2Big = PairKernel<2, 128, 6, 64>;
+// the same three for the received rows of an expert-parallel rank
+using Gemm2SmallEp = PairKernel<2, 32, 10, 0, true>;
+using Gemm2MidEp = PairKernel<2, 64, 9, 0, true>;
+using Gemm2BigEp = PairKernel<2, 128, 6, 64, true>;
 constexpr int kSmallRowsMax = 64;
 constexpr int kMidRowsPerExpert = 100;  // mean slots per candidate (T K / (N + N_Z)) up to which the mid geometry is used
+                                        // (expert parallel: mean received rows per local expert)
 constexpr int kWideRowsPerExpert = 256; // ... and up to which GEMM1 runs tiles of up to 128 rows as double items
 
 // The small geometry holds at most kSmallRowsMax pair rows of one expert.  Without expert parallelism
@@ -640,8 +652,13 @@ bool small_geometry(const zeda_moe *h, const ExpertWork &w) {
 // per candidate.
 int tile_rows_for(const zeda_moe *h, int T) {
     const zeda_moe_config_t &c = h->cfg;
-    if (c.ep_size >= 1) return kPairTileM;
+    if (c.ep_size >= 1) return kPairTileM;  // this list is not used: the received rows have their own
     return (long long)T * c.top_k <= (long long)kMidRowsPerExpert * (c.n_real + c.n_zero) ? kMidTileM : kPairTileM;
+}
+
+// The same for the received rows of an expert-parallel rank, whose number the host knows exactly.
+int ep_tile_rows_for(const zeda_moe *h, int n_rows) {
+    return (long long)n_rows <= (long long)kMidRowsPerExpert * h->n_local ? kMidTileM : kPairTileM;
 }
 
 int init_pair_kernels(zeda_moe *h) {
@@ -672,7 +689,8 @@ int init_pair_kernels(zeda_moe *h) {
         ok = ok && encode_bf16_map(&pm->hmid.m[i], h->ws.hmid, 2, dims, strides, box);
     }
     ok = ok && Gemm1Small::prepare() && Gemm2Small::prepare() && Gemm1Mid::prepare() && Gemm2Mid::prepare() &&
-         Gemm1Big::prepare() && Gemm1Wide::prepare() && Gemm2Big::prepare();
+         Gemm1Big::prepare() && Gemm1Wide::prepare() && Gemm2Big::prepare() && Gemm2SmallEp::prepare() &&
+         Gemm2MidEp::prepare() && Gemm2BigEp::prepare();
     if (!ok) {
         free(pm);
         if (zeda_last_error()[0] == 0) set_error("pair kernel set-up failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -693,13 +711,13 @@ int launch_experts_gemm1_pair(const zeda_moe *h, const __nv_bfloat16 *x, const E
                                    w.tile_rows);
     };
     // an expert cannot hold more pair rows than the call has tokens (a token selects it at most once)
-    // (an expert-parallel rank does not know its load from the call's shape: it takes the form for large batches)
-    const bool wide = c.ep_size < 1 && (long long)w.rows_bound <= (long long)kWideRowsPerExpert * (c.n_real + c.n_zero);
+    const int share = c.ep_size >= 1 ? h->n_local : c.n_real + c.n_zero;
+    const bool wide = (long long)w.rows_bound <= (long long)kWideRowsPerExpert * share;
     const cudaError_t e = small_geometry(h, w) ? go(Gemm1Small{}) : w.tile_rows == kMidTileM ? go(Gemm1Mid{}) : wide ? go(Gemm1Wide{}) : go(Gemm1Big{});
     return e == cudaSuccess ? 1 : -1;
 }
 
-int launch_experts_gemm2_pair(const zeda_moe *h, const ExpertWork &w, cudaStream_t s) {
+int launch_experts_gemm2_pair(const zeda_moe *h, const ExpertWork &w, __nv_bfloat16 *out, cudaStream_t s) {
     const zeda_moe_config_t &c = h->cfg;
     const Workspace &ws = h->ws;
     const PairMaps *pm = static_cast<const PairMaps *>(h->pmaps);
@@ -707,9 +725,11 @@ int launch_experts_gemm2_pair(const zeda_moe *h, const ExpertWork &w, cudaStream
     auto go = [&](auto k) {
         return decltype(k)::launch(h, s, pm->w_down, pm->hmid, (const __nv_bfloat16 *)nullptr, 0, w.counts, w.offsets,
                                    w.tile_expert, w.tile_row0, w.pair_row, ws.meta, c.d_expert, c.d_model, m_blocks,
-                                   ws.obuf, c.d_model, w.tile_rows);
+                                   out, c.d_model, w.tile_rows);
     };
-    const cudaError_t e = small_geometry(h, w) ? go(Gemm2Small{}) : w.tile_rows == kMidTileM ? go(Gemm2Mid{}) : go(Gemm2Big{});
+    const bool small = small_geometry(h, w), mid = w.tile_rows == kMidTileM;
+    const cudaError_t e = c.ep_size >= 1 ? (small ? go(Gemm2SmallEp{}) : mid ? go(Gemm2MidEp{}) : go(Gemm2BigEp{}))
+                                         : (small ? go(Gemm2Small{}) : mid ? go(Gemm2Mid{}) : go(Gemm2Big{}));
     return e == cudaSuccess ? 1 : -1;
 }
 

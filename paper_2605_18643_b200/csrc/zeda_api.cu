@@ -65,7 +65,7 @@ size_t carve(const zeda_moe_config_t &c, unsigned char *base, Workspace *ws, int
     const bool ep = c.ep_size >= 1;
     const size_t n_local = ep ? (size_t)c.n_real / c.ep_size : (size_t)c.n_real;
     const size_t pair_rows = ep ? (size_t)c.max_recv_pairs : slots;
-    const size_t ep_tiles = pair_rows / kPairTileM + n_local + 1;
+    const size_t ep_tiles = pair_rows / kMidTileM + n_local + 1;
     const size_t nblk_stats = (c.max_tokens + 63) / 64;
     Workspace w;
     w.topk_idx = (int32_t *)take(slots * 4);
@@ -83,16 +83,15 @@ size_t carve(const zeda_moe_config_t &c, unsigned char *base, Workspace *ws, int
     w.stat_part = (float *)take(nblk_stats * 2 * n_cand * 4);
     // pair buffers carry one tile of slack rows so that a full tile may be read past the last pair
     w.hmid = (__nv_bfloat16 *)take((pair_rows + kPairTileM) * c.d_expert * 2);
-    w.obuf = (__nv_bfloat16 *)take((pair_rows + kPairTileM) * c.d_model * 2);
+    w.obuf = ep ? nullptr : (__nv_bfloat16 *)take((pair_rows + kPairTileM) * c.d_model * 2);
     w.router_split = (__nv_bfloat16 *)take((size_t)3 * router_split_pad((int)n_cand) * c.d_model * 2);
     w.x_stage = (__nv_bfloat16 *)take((size_t)c.max_tokens * c.d_model * 2);
     w.y_stage = (__nv_bfloat16 *)take((size_t)c.max_tokens * c.d_model * 2);
-    w.ep_counts = w.ep_offsets = w.ep_pair_row = w.ep_row_pos = w.ep_tile_expert = w.ep_tile_row0 = nullptr;
+    w.ep_counts = w.ep_offsets = w.ep_pair_row = w.ep_tile_expert = w.ep_tile_row0 = nullptr;
     if (ep) {
         w.ep_counts = (int32_t *)take(n_local * 4);
         w.ep_offsets = (int32_t *)take((n_local + 1) * 4);
         w.ep_pair_row = (int32_t *)take(pair_rows * 4);
-        w.ep_row_pos = (int32_t *)take(pair_rows * 4);
         w.ep_tile_expert = (int32_t *)take(ep_tiles * 4);
         w.ep_tile_row0 = (int32_t *)take(ep_tiles * 4);
     }
@@ -183,7 +182,7 @@ zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_
     if (r < 0) return cuda_fail("expert GEMM1 launch", cudaGetLastError());
     n += r;
     mark(3);
-    r = launch_experts_gemm2_pair(h, work, s);
+    r = launch_experts_gemm2_pair(h, work, ws.obuf, s);
     if (r < 0) return cuda_fail("expert GEMM2 launch", cudaGetLastError());
     n += r;
     mark(4);
@@ -456,18 +455,16 @@ zeda_status_t zeda_ep_experts(zeda_moe_t *h, const void *recv_rows, const int32_
     cudaError_t e = cudaSetDevice(h->cfg.device);
     if (e != cudaSuccess) return cuda_fail("cudaSetDevice", e);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int n = launch_ep_plan(h, recv_counts, n_rows, s);
+    const int tile_rows = ep_tile_rows_for(h, n_rows);
+    int n = launch_ep_plan(h, recv_counts, n_rows, tile_rows, s);
     if (n < 0) return cuda_fail("plan launch", cudaGetLastError());
     const Workspace &ws = h->ws;
-    const ExpertWork work = {ws.ep_counts, ws.ep_offsets, ws.ep_tile_expert, ws.ep_tile_row0, ws.ep_pair_row, n_rows, kPairTileM};
+    const ExpertWork work = {ws.ep_counts, ws.ep_offsets, ws.ep_tile_expert, ws.ep_tile_row0, ws.ep_pair_row, n_rows, tile_rows};
     int r = launch_experts_gemm1_pair(h, static_cast<const __nv_bfloat16 *>(recv_rows), work, s);
     if (r < 0) return cuda_fail("expert GEMM1 launch", cudaGetLastError());
     n += r;
-    r = launch_experts_gemm2_pair(h, work, s);
+    r = launch_experts_gemm2_pair(h, work, static_cast<__nv_bfloat16 *>(out_rows), s);
     if (r < 0) return cuda_fail("expert GEMM2 launch", cudaGetLastError());
-    n += r;
-    r = launch_ep_unsort(h, n_rows, static_cast<__nv_bfloat16 *>(out_rows), s);
-    if (r < 0) return cuda_fail("unsort launch", cudaGetLastError());
     h->last_launches = n + r;
     return ZEDA_OK;
 }

@@ -47,7 +47,7 @@ struct Workspace {
     float *logits;         // [maxT*(N+N_Z)]
     float *stat_part;      // [nblk_stats * 2 * (N+N_Z)]
     __nv_bfloat16 *hmid;   // [maxT*K, He]
-    __nv_bfloat16 *obuf;   // [maxT*K, d]
+    __nv_bfloat16 *obuf;   // [maxT*K, d] (not on expert-parallel handles: their results go to the caller's buffer)
     __nv_bfloat16 *router_split; // [3][pad128(N+N_Z)][d] bf16 hi/mid/lo pieces of the router rows
     __nv_bfloat16 *x_stage;// [maxT, d]
     __nv_bfloat16 *y_stage;// [maxT, d]
@@ -55,8 +55,7 @@ struct Workspace {
     int32_t *ep_counts;      // [N_local] received pairs per local expert
     int32_t *ep_offsets;     // [N_local + 1]
     int32_t *ep_pair_row;    // [maxR] sorted position -> received row
-    int32_t *ep_row_pos;     // [maxR] received row -> sorted position
-    int32_t *ep_tile_expert; // [maxR / kPairTileM + N_local + 1]
+    int32_t *ep_tile_expert; // [maxR / kMidTileM + N_local + 1]
     int32_t *ep_tile_row0;
 };
 
@@ -137,9 +136,11 @@ int init_pair_kernels(zeda_moe *h);
 // Pair rows per tile for a call of T tokens on this handle: the routing pass builds the tile list with
 // it and the expert kernels of the same call are picked to match.
 int tile_rows_for(const zeda_moe *h, int T);
+int ep_tile_rows_for(const zeda_moe *h, int n_rows);
 int launch_token_zero_share(const zeda_moe *h, int T, float *out, cudaStream_t s);
 int launch_experts_gemm1_pair(const zeda_moe *h, const __nv_bfloat16 *x, const ExpertWork &w, cudaStream_t s);
-int launch_experts_gemm2_pair(const zeda_moe *h, const ExpertWork &w, cudaStream_t s);
+// out: where the results go, in sorted order or (expert-parallel handles) in the order of pair_row
+int launch_experts_gemm2_pair(const zeda_moe *h, const ExpertWork &w, __nv_bfloat16 *out, cudaStream_t s);
 // the smallest batches (small_batch.cu): GEMM1, and GEMM2 with the combine (resid given: with the residual update)
 bool stream_path(const zeda_moe *h, int T);
 int init_stream_kernels();
@@ -149,8 +150,7 @@ int launch_residual_rmsnorm(bool pdl, __nv_bfloat16 *r, const __nv_bfloat16 *y, 
 // expert-parallel pieces (expert_parallel.cu)
 int launch_ep_pack(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *send_rows, int32_t *send_counts,
                    int32_t *expert_counts, cudaStream_t s);
-int launch_ep_plan(const zeda_moe *h, const int32_t *recv_counts, int n_rows, cudaStream_t s);
-int launch_ep_unsort(const zeda_moe *h, int n_rows, __nv_bfloat16 *out_rows, cudaStream_t s);
+int launch_ep_plan(const zeda_moe *h, const int32_t *recv_counts, int n_rows, int tile_rows, cudaStream_t s);
 int launch_combine_rows(const zeda_moe *h, const __nv_bfloat16 *rows, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y,
                         cudaStream_t s);
 int launch_wait_selftest(const zeda_moe *h, long long limit_cycles, cudaStream_t s);

@@ -105,9 +105,11 @@ class ExpertParallelMoE:
         if launches is not None:
             launches.append(m.last_counters()[3])
         recv_counts = self.x.counts(expert_counts)
-        # the one host synchronisation of the call: the all-to-all needs its split sizes on the host
-        send_splits = [int(v) for v in send_counts.tolist()]
-        recv_splits, n_rows = recv_layout(recv_counts)
+        # the one host synchronisation of the call: the all-to-all needs its split sizes on the host (both
+        # directions' counts in one copy)
+        counts = torch.cat((send_counts, recv_counts.reshape(-1))).cpu()
+        send_splits = counts[:self.G].tolist()
+        recv_splits, n_rows = recv_layout(counts[self.G:].view(self.G, -1))
         if n_rows > m.cfg.max_recv_pairs:
             raise RuntimeError("rank receives %d pair rows, handle was sized for %d" % (n_rows, m.cfg.max_recv_pairs))
         recv_rows = self.x.rows(send_rows, send_splits, recv_splits)

@@ -98,6 +98,25 @@ def test_one_rank_group_equals_the_plain_layer_bit_for_bit(zeda):
     ranks[0].moe.close()
 
 
+@pytest.mark.parametrize("T", [30, 300, 700, 2600])
+def test_results_in_received_order_for_every_kernel_form(zeda, T):
+    # two ranks of four experts: a rank receives about T rows, i.e. at most 64 (small form), a mean of up
+    # to 100 and 256 per expert (128-row tiles; wide double items) and more (256-row tiles).  The same sums
+    # in the same order as the plain layer: equal bits
+    dev = torch.device("cuda:0")
+    layer = inputs.tiny(seed=36, T=T)
+    plain = zeda.from_workload(layer, dev)
+    xs = [layer.x.to(dev), layer.x.flip(0).contiguous().to(dev)]
+    ranks = make_group(zeda, layer, 2, T, dev)
+    ys = ep.forward_group_in_one_process(ranks, xs)
+    for x, y in zip(xs, ys):
+        assert torch.equal(plain.forward(x).view(torch.int16), y.view(torch.int16))
+    for r in ranks:
+        r.moe.last_counters()
+        r.moe.close()
+    plain.close()
+
+
 @pytest.mark.parametrize("gate_mode,expert_kind", [(2, 0), (0, 1)])
 def test_group_with_gate_modes_and_copy_experts(zeda, gate_mode, expert_kind):
     dev = torch.device("cuda:0")
