@@ -748,11 +748,11 @@ int init_route_kernels(const zeda_moe *h) {
     return 0;
 }
 
-int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s, int *n_parts) {
+int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s, int *n_parts, int split_T) {
     if (n_parts) *n_parts = 1;
     // large batches: the GEMM goes to the tensor cores (exact three-way bf16 split of the weights)
     if (T >= 256 && h->router_maps) {
-        const int split = n_parts ? router_split_factor(h, T) : 1;
+        const int split = n_parts ? router_split_factor(h, split_T > T ? split_T : T) : 1;
         if (n_parts) *n_parts = split;
         return launch_router_logits_tile(h, x, T, logits, split, s);
     }

@@ -146,13 +146,13 @@ int route_into(zeda_moe_t *h, const __nv_bfloat16 *x, const float *logits_in, in
 // With resid given, the call ends in the fused combine + glue pass: resid <- bf16(resid + y) and
 // the normalised residual goes where y would have gone.
 zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y, cudaStream_t s,
-                             __nv_bfloat16 *resid = nullptr, float eps = 0.f) {
+                             __nv_bfloat16 *resid = nullptr, float eps = 0.f, int split_T = 0) {
     const bool prof = h->profiling;
     auto mark = [&](int i) { if (prof) cudaEventRecord(h->ev[i], s); };
     mark(0);
     h->last_routed_tokens = T;
     int n_parts = 1;
-    int n = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts);
+    int n = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts, split_T);
     if (n < 0) return cuda_fail("router launch", cudaGetLastError());
     mark(1);
     RouteOut none = {};
@@ -346,10 +346,13 @@ zeda_status_t zeda_moe_forward_residual(zeda_moe_t *h, const void *x, int32_t T,
                           static_cast<cudaStream_t>(stream), static_cast<__nv_bfloat16 *>(r), eps);
 }
 
-// Batches of at least this many tokens go through the host-buffer entry point in two chunks, so that
-// the copy of the second chunk runs under the layer of the first and the copy back of the first under
-// the layer of the second.
-static const int kHostSplitMinTokens = 4096;
+// The host-buffer entry point cuts large batches into chunks, so that the copy of a chunk runs under the
+// layer of the one before and the copies back under the layers behind; each chunk reads the experts'
+// weights again.  Below 4096 tokens a second pass over the weights costs more than the copies it hides.
+// A third chunk pays from 8192 tokens on (Zipf load, 75 of 128 experts active: 1211 -> 1068 us a call; an
+// even load, where a third pass over all weights costs most, stands even there and loses 5 % at 7168).
+// Equal chunks: with a quarter, a half and a quarter the copies back queue up behind the half (1216 us).
+static const int kHostSplitMinTokens = 4096, kHostThreeChunksMinTokens = 8192;
 
 zeda_status_t zeda_moe_forward_host(zeda_moe_t *h, const void *x_host, int32_t T, void *y_host, void *stream) {
     if (!h) { set_error("handle is NULL"); return ZEDA_ERR_INVALID_ARG; }
@@ -372,9 +375,8 @@ zeda_status_t zeda_moe_forward_host(zeda_moe_t *h, const void *x_host, int32_t T
         if (e != cudaSuccess) return cuda_fail("cudaStreamSynchronize", e);
         return ZEDA_OK;
     }
-    // Two chunks.  The layer is per token (Eq. 1), so the chunks are two independent calls; their device
-    // work stays on `stream`, one after the other (they share the workspace), the copies run on two
-    // streams of the handle.
+    // The layer is per token (Eq. 1), so the chunks are independent calls; their device work stays on
+    // `stream`, one after the other (they share the workspace), the copies run on two streams of the handle.
     if (!h->copy_in) {
         e = cudaStreamCreateWithFlags(&h->copy_in, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_out, cudaStreamNonBlocking);
@@ -382,34 +384,49 @@ zeda_status_t zeda_moe_forward_host(zeda_moe_t *h, const void *x_host, int32_t T
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
         if (e != cudaSuccess) return cuda_fail("stream / event creation", e);
     }
-    const int T0 = (T / 2 + 255) / 256 * 256, T1 = T - T0;
+    // The result is that of the batch's two halves as calls of their own.  Three chunks give the same bits
+    // where the router slices its reduction axis alike for both halves: the chunks take over that slicing,
+    // and nothing else of a token's result depends on the tokens around it.
+    const int T0 = (T / 2 + 255) / 256 * 256;  // first token of the second half
+    const bool three = T >= kHostThreeChunksMinTokens && router_split_factor(h, T0) == router_split_factor(h, T - T0);
+    const int chunks = three ? kHostMaxChunks : 2;
+    int at[kHostMaxChunks + 1] = {0};  // first token of each chunk
+    for (int i = 1; i < chunks; ++i) at[i] = (int)(((long long)T * i / chunks + 255) / 256 * 256);
+    at[chunks] = T;
     const char *xh = static_cast<const char *>(x_host);
     char *yh = static_cast<char *>(y_host);
     __nv_bfloat16 *xs = h->ws.x_stage, *ys = h->ws.y_stage;
-    cudaEvent_t *ev = h->ev_host;  // 0 start, 1-2 chunk copied in, 3-4 chunk computed, 5 all copied out
-    bool ok = cudaEventRecord(ev[0], s) == cudaSuccess && cudaStreamWaitEvent(h->copy_in, ev[0], 0) == cudaSuccess &&
-              cudaStreamWaitEvent(h->copy_out, ev[0], 0) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(xs, xh, T0 * row, cudaMemcpyHostToDevice, h->copy_in) == cudaSuccess &&
-         cudaEventRecord(ev[1], h->copy_in) == cudaSuccess &&
-         cudaMemcpyAsync(xs + (size_t)T0 * h->cfg.d_model, xh + T0 * row, T1 * row, cudaMemcpyHostToDevice, h->copy_in) == cudaSuccess &&
-         cudaEventRecord(ev[2], h->copy_in) == cudaSuccess;
+    cudaEvent_t start = h->ev_host[0], done = h->ev_host[1], *copied = h->ev_host + 2, *computed = copied + kHostMaxChunks;
+    bool ok = cudaEventRecord(start, s) == cudaSuccess && cudaStreamWaitEvent(h->copy_in, start, 0) == cudaSuccess &&
+              cudaStreamWaitEvent(h->copy_out, start, 0) == cudaSuccess;
+    for (int i = 0; i < chunks; ++i)
+        ok = ok &&
+             cudaMemcpyAsync(xs + (size_t)at[i] * h->cfg.d_model, xh + at[i] * row, (at[i + 1] - at[i]) * row, cudaMemcpyHostToDevice,
+                             h->copy_in) == cudaSuccess &&
+             cudaEventRecord(copied[i], h->copy_in) == cudaSuccess;
     if (!ok) return cuda_fail("copy of x to the device", cudaGetLastError());
-    if (cudaStreamWaitEvent(s, ev[1], 0) != cudaSuccess) return cuda_fail("cudaStreamWaitEvent", cudaGetLastError());
-    zeda_status_t st = forward_device(h, xs, T0, ys, s);
-    if (st != ZEDA_OK) return st;
-    if (cudaEventRecord(ev[3], s) != cudaSuccess || cudaStreamWaitEvent(s, ev[2], 0) != cudaSuccess)
-        return cuda_fail("cudaEventRecord", cudaGetLastError());
-    const int launches0 = h->last_launches;
-    st = forward_device(h, xs + (size_t)T0 * h->cfg.d_model, T1, ys + (size_t)T0 * h->cfg.d_model, s);
-    if (st != ZEDA_OK) return st;
-    h->last_launches += launches0;
-    ok = cudaEventRecord(ev[4], s) == cudaSuccess && cudaStreamWaitEvent(h->copy_out, ev[3], 0) == cudaSuccess &&
-         cudaMemcpyAsync(yh, ys, T0 * row, cudaMemcpyDeviceToHost, h->copy_out) == cudaSuccess &&
-         cudaStreamWaitEvent(h->copy_out, ev[4], 0) == cudaSuccess &&
-         cudaMemcpyAsync(yh + T0 * row, ys + (size_t)T0 * h->cfg.d_model, T1 * row, cudaMemcpyDeviceToHost, h->copy_out) == cudaSuccess &&
-         cudaEventRecord(ev[5], h->copy_out) == cudaSuccess;
-    if (!ok) return cuda_fail("copy of y to the host", cudaGetLastError());
-    e = cudaEventSynchronize(ev[5]);
+    int launches = 0;
+    for (int i = 0; i < chunks; ++i) {
+        const size_t off = (size_t)at[i] * h->cfg.d_model;
+        if (cudaStreamWaitEvent(s, copied[i], 0) != cudaSuccess) return cuda_fail("cudaStreamWaitEvent", cudaGetLastError());
+        const zeda_status_t st = forward_device(h, xs + off, at[i + 1] - at[i], ys + off, s, nullptr, 0.f, three ? T0 : 0);
+        if (st != ZEDA_OK) return st;
+        launches += h->last_launches;
+        if (cudaEventRecord(computed[i], s) != cudaSuccess) return cuda_fail("cudaEventRecord", cudaGetLastError());
+    }
+    h->last_launches = launches;
+    for (int i = 0; i < chunks; ++i)  // behind all launches: a copy into pageable memory holds the host up
+        ok = ok && cudaStreamWaitEvent(h->copy_out, computed[i], 0) == cudaSuccess &&
+             cudaMemcpyAsync(yh + at[i] * row, ys + (size_t)at[i] * h->cfg.d_model, (at[i + 1] - at[i]) * row, cudaMemcpyDeviceToHost,
+                             h->copy_out) == cudaSuccess;
+    if (!ok || cudaEventRecord(done, h->copy_out) != cudaSuccess) return cuda_fail("copy of y to the host", cudaGetLastError());
+    if (three) {  // the handle keeps the second half's routing: routed again under the copies back
+        RouteOut none = {};
+        const int n = route_into(h, xs + (size_t)T0 * h->cfg.d_model, nullptr, T - T0, none, s);
+        if (n < 0) return cuda_fail("routing launch", cudaGetLastError());
+        h->last_launches += n;
+    }
+    e = cudaEventSynchronize(done);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail("cudaStreamSynchronize", e);
     return ZEDA_OK;

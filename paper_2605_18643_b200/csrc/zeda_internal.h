@@ -18,6 +18,8 @@ constexpr int kMaxEpRanks = 64;     // expert-parallel group size limit
 constexpr int kStreamTokens = 16;   // calls of at most this many tokens ...
 constexpr int kStreamSlots = 256;   // ... and slots run the expert kernels of small_batch.cu
 
+constexpr int kHostMaxChunks = 3;   // of the host-buffer entry point
+
 // Device-resident counters of one call.
 enum MetaSlot {
     kMetaPairs = 0,      // P
@@ -103,9 +105,9 @@ struct zeda_moe {
     bool profiled_last;
     int last_routed_tokens;  // T of the most recent routing pass on this handle
     cudaEvent_t ev[ZEDA_STAGE_COUNT + 1];
-    // host-buffer entry point: copy streams and events of its two-chunk pipeline (made on first use)
+    // host-buffer entry point: copy streams and events of its chunk pipeline (made on first use)
     cudaStream_t copy_in, copy_out;
-    cudaEvent_t ev_host[6];
+    cudaEvent_t ev_host[2 + 2 * zeda::kHostMaxChunks];
 };
 
 namespace zeda {
@@ -115,8 +117,10 @@ int init_route_kernels(const zeda_moe *h);
 // With n_parts == nullptr the logits are complete.  Otherwise the router may cut the reduction axis
 // into *n_parts slices (mid-sized batches on the tensor-core path): slice p then lies at
 // logits + p * T * n_cand, and launch_route_from_logits adds the slices in order.
+// split_T: the number of tokens that the slicing is decided by, if not T (a call that is one part of a
+// batch gives the batch's, so that its logits are the batch's bits).
 int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s,
-                         int *n_parts = nullptr);
+                         int *n_parts = nullptr, int split_T = 0);
 int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s,
                              int n_parts = 1, float *stat_part = nullptr);
 // The statistics of the last routing pass, which was given ws.stat_part to leave its partial sums in.

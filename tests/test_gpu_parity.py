@@ -248,6 +248,23 @@ def test_host_buffer_entry_point_in_two_chunks(zeda):
         m.close()
 
 
+@pytest.mark.parametrize("T", [8191, 8192, 8900, 9500])
+def test_host_buffer_entry_point_chunk_counts(zeda, T):
+    # from 8192 tokens three chunks: still, bit for bit, the two halves passed through zeda_moe_forward, and the
+    # routing left in the handle is the second half's
+    wl = inputs.tiny(seed=18, T=T)
+    dev = torch.device("cuda:0")
+    m = zeda.from_workload(wl, dev)
+    x = wl.x.to(dev)
+    T0 = (T // 2 + 255) // 256 * 256
+    want = torch.cat([m.forward(x[:T0].contiguous()), m.forward(x[T0:].contiguous())]).cpu()
+    share, counters = m.token_zero_share(T - T0).cpu(), m.last_counters()[:3]
+    for host in (wl.x.pin_memory(), wl.x):
+        assert torch.equal(want.view(torch.int16), m.forward_host(host).view(torch.int16))
+        assert torch.equal(m.token_zero_share(T - T0).cpu(), share) and m.last_counters()[:3] == counters
+    m.close()
+
+
 def test_routing_statistics(zeda):
     wl = inputs.tiny(seed=9, T=200)
     dev = torch.device("cuda:0")
