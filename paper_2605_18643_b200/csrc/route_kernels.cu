@@ -95,6 +95,8 @@ router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restric
 // 192 SM-wide bursts instead of 24; the reduction axis is split over four warps.  NT tokens per CTA, all
 // of their loads in flight at once.  The row is asked into L2 before the wait for the kernel in front (a
 // prefetch only: its values are read after the wait).
+constexpr int kTileRouterTokens = 160;  // from here on the tensor-core router (128 tokens: 11 us on the CUDA cores, 193: 15; the tensor-core kernel
+                                      // takes 11 and leaves the top-K pass more slices to add)
 constexpr int kFewTokens = 32;  // calls of at most this many tokens
 constexpr int kFewThreads = 128;
 constexpr int kFewUnroll = 4;
@@ -160,9 +162,9 @@ constexpr int kRegsPerLane = kMaxCand / 32;
 // Top-K and routing weights of one token by one warp.  On return lane k < K holds slot k, and v, m, den
 // the logits (-inf beyond n_cand), their maximum and the softmax denominator.
 // RPL = logits per lane (32 * RPL >= n_cand).
-// The row may arrive as n_parts partial sums, part_stride floats apart; they are added in order, three
-// slices requested at a time (one slice after another is a chain of L2 round trips).
-template <int RPL>
+// The row may arrive as n_parts partial sums, part_stride floats apart; they are added in order, PB slices
+// requested at a time (one slice after another is a chain of L2 round trips).
+template <int RPL, int PB = (RPL <= 8 ? 7 : 3)>
 __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, int n_parts, size_t part_stride,
                                                 int n_real, int n_cand, int K, int gate_mode, int lane,
                                                 float (&v)[RPL], float &m, float &den, int &my_idx, float &my_w) {
@@ -171,17 +173,17 @@ __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, i
         const int j = r * 32 + lane;
         v[r] = (j < n_cand) ? row[j] : -INFINITY;
     }
-    for (int p = 1; p < n_parts; p += 3) {
-        float a[3][RPL];
+    for (int p = 1; p < n_parts; p += PB) {
+        float a[PB][RPL];
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
+        for (int q = 0; q < PB; ++q)
 #pragma unroll
             for (int r = 0; r < RPL; ++r) {
                 const int j = r * 32 + lane;
                 a[q][r] = p + q < n_parts && j < n_cand ? row[(p + q) * part_stride + j] : 0.f;
             }
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
+        for (int q = 0; q < PB; ++q)
 #pragma unroll
             for (int r = 0; r < RPL; ++r)
                 if (p + q < n_parts) v[r] += a[q][r];
@@ -207,7 +209,8 @@ __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, i
     for (int r = 0; r < RPL; ++r) {
         unsigned u = __float_as_uint(v[r]);
         if (u == 0x80000000u) u = 0u;  // -0 and +0 are equal logits: the lower id decides between them
-        key[r] = (r * 32 + lane < n_cand) ? ((u & 0x80000000u) ? ~u : (u | 0x80000000u)) : 0u;
+        // (a candidate's key is never 0, not even for the NaN whose key would be: no candidate is taken twice)
+        key[r] = (r * 32 + lane < n_cand) ? max((u & 0x80000000u) ? ~u : (u | 0x80000000u), 1u) : 0u;
     }
     unsigned my_key = 0u;
     my_idx = -1;
@@ -361,7 +364,7 @@ constexpr int kSmallThreads = 32 * (kSmallTokens / kSmallCluster);  // one warp 
 // CLUSTER = 1: up to 16 tokens fit one CTA, which saves the cluster's launch and barriers.
 template <int RPL, int CLUSTER>
 __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kSmallThreads)
-route_small_kernel(const float *__restrict__ logits, int T, int n_real, int n_cand, int K, int gate_mode,
+route_small_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
                    int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ counts,
                    int32_t *__restrict__ offsets, int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                    const WorkLists wl, int tile_rows, int32_t *__restrict__ perm,
@@ -382,7 +385,7 @@ route_small_kernel(const float *__restrict__ logits, int T, int n_real, int n_ca
     if (t < T) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL>(logits + (size_t)t * n_cand, 1, 0, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
+        topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
             topk_w[(size_t)t * K + lane] = my_w;
@@ -483,40 +486,42 @@ slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real
 // ---------------------------------------------------------------------------------------------
 // Counting sort, passes 2 + 3 in one launch (used while the CTA histograms are few): every CTA
 // sums the histogram columns itself (pairs of each expert in earlier CTAs, and in all CTAs), scans
-// the expert totals, and places its slots as above.  CTA 0 also publishes counts, offsets and the
-// counters; the work lists are filled by all CTAs, a share each.  Saves a launch and the single-CTA
-// scan between two short kernels.
+// the expert totals, and places the slots of its kSortTokens tokens.  A token selects an expert at most
+// once, so a slot's rank among its CTA's pairs of the expert is a popcount over a bit mask of the CTA's
+// tokens (one shared-memory atomicOr per slot instead of two passes of match.any over them).  CTA 0
+// also publishes counts, offsets and the counters; the tile list is filled by all CTAs, a share each.
+// What bounds it is the chain of dependent steps, not the data: 7.4 us for 2 CTAs before, as for 64.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kPlaceWarps * 32)
+constexpr int kScanThreads = 256;
+constexpr int kMaskWords = kSortTokens / 32;
+
+__global__ void __launch_bounds__(kScanThreads)
 slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real, int nblk,
                        int32_t *__restrict__ block_hist, int32_t *__restrict__ counts,
                        int32_t *__restrict__ offsets, int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                        const WorkLists wl, int tile_rows, int32_t *__restrict__ perm, int32_t *__restrict__ perm_user,
                        int32_t *__restrict__ inv, int32_t *__restrict__ pair_token) {
-    pdl_launch_dependents();
-    pdl_wait();
     __shared__ ScanShared sh;
-    extern __shared__ int32_t pos[];       // [kPlaceWarps][n_real], then base[n_real], then a histogram slab
-    int32_t *base = pos + kPlaceWarps * n_real;
-    int32_t *slab = base + n_real;         // [kScanSlabInts]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // this warp's slots, fetched now (their latency passes under the histogram sums below): slot
-    // w0 + 32 u + lane in e_reg[u], -1 for zero-expert slots and beyond the end
-    constexpr int kSlotRegs = kSortTokens * kMaxTopK / kPlaceWarps / 32;
-    const int s0 = blockIdx.x * kSortTokens * K;
-    const int s1 = min(T * K, s0 + kSortTokens * K);
-    const int per_warp = ((kSortTokens * K + kPlaceWarps - 1) / kPlaceWarps + 31) / 32 * 32;
-    const int w0 = s0 + warp * per_warp;
-    const int w1 = min(s1, w0 + per_warp);
+    __shared__ int s_ticket;
+    extern __shared__ __align__(16) int32_t place_smem[];  // base[n_real], token masks [n_real][kMaskWords], a histogram slab [kScanSlabInts]
+    int32_t *base = place_smem;
+    const int pad = (n_real + 3) & ~3;  // the masks are read as 16 bytes
+    uint32_t *mask = reinterpret_cast<uint32_t *>(base + pad);
+    int32_t *slab = base + pad + kMaskWords * pad;
+    pdl_launch_dependents();
+    for (int i = threadIdx.x; i < n_real * kMaskWords; i += blockDim.x) mask[i] = 0u;
+    for (int e = threadIdx.x; e < n_real; e += blockDim.x) { base[e] = 0; sh.cnt[e] = 0; }
+    pdl_wait();
+    // slot s0 + threadIdx.x + kScanThreads * u in e_reg[u], -1 for zero-expert slots and beyond the end
+    constexpr int kSlotRegs = kSortTokens * kMaxTopK / kScanThreads;
+    const int s0 = blockIdx.x * kSortTokens * K, n_slots = min(T * K - s0, kSortTokens * K);
     int e_reg[kSlotRegs];
 #pragma unroll
     for (int u = 0; u < kSlotRegs; ++u) {
-        const int s = w0 + 32 * u + lane;
-        int e = (32 * u < per_warp && s < w1) ? __ldg(topk_idx + s) : -1;
+        const int i = threadIdx.x + kScanThreads * u;
+        const int e = i < n_slots ? __ldg(topk_idx + s0 + i) : -1;
         e_reg[u] = (unsigned)e >= (unsigned)n_real ? -1 : e;
     }
-    for (int i = threadIdx.x; i < kPlaceWarps * n_real; i += blockDim.x) pos[i] = 0;
-    for (int e = threadIdx.x; e < n_real; e += blockDim.x) { base[e] = 0; sh.cnt[e] = 0; }
     // column sums of the CTA histograms: staged slab by slab with independent coalesced loads (a
     // per-thread loop over global memory would be one L2 round trip after another); with fewer experts
     // than threads, several threads share a column
@@ -524,9 +529,8 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
     const int col_parts = max(1, (int)blockDim.x / n_real);
     for (int b0 = 0; b0 < nblk; b0 += slab_blocks) {
         const int nb = min(slab_blocks, nblk - b0);
-        const int32_t *g = block_hist + (size_t)b0 * n_real;
         __syncthreads();
-        stage_ints(slab, g, nb * n_real);
+        stage_ints(slab, block_hist + (size_t)b0 * n_real, nb * n_real);
         __syncthreads();
         for (int i = threadIdx.x; i < n_real * col_parts; i += blockDim.x) {
             const int e = i % n_real;
@@ -537,60 +541,44 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
                 total += c;
                 if (b0 + b < (int)blockIdx.x) before += c;
             }
-            atomicAdd(&base[e], before);
-            atomicAdd(&sh.cnt[e], total);
+            if (total) {
+                atomicAdd(&base[e], before);
+                atomicAdd(&sh.cnt[e], total);
+            }
         }
     }
-    int32_t *mine = pos + warp * n_real;
-    const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
     for (int u = 0; u < kSlotRegs; ++u) {
-        if (w0 + 32 * u >= w1 || 32 * u >= per_warp) break;  // (uniform over the warp)
-        const int e = e_reg[u];
-        const unsigned grp = __match_any_sync(kFull, e);
-        if (e >= 0 && (grp & lt) == 0) mine[e] += __popc(grp);
-        __syncwarp();
+        const int tok = (threadIdx.x + kScanThreads * u) / K;
+        if (e_reg[u] >= 0) atomicOr(mask + e_reg[u] * kMaskWords + (tok >> 5), 1u << (tok & 31));
     }
     __syncthreads();
     // The histograms go back to zero for the next call's top-K kernel: the CTA that is last to have
     // read them (a ticket, nobody waits; looked at only when this CTA's own work is done) clears them
     // and the ticket counter.
-    __shared__ int s_ticket;
     if (threadIdx.x == blockDim.x - 1) {
         __threadfence();
         s_ticket = atomicAdd(meta + kMetaHistTicket, 1);
     }
     finish_expert_scan(sh, n_real, T * K, counts, offsets, n_pairs_out, meta, wl, blockIdx.x == 0, blockIdx.x, gridDim.x, tile_rows);
-    __syncthreads();
-    for (int e = threadIdx.x; e < n_real; e += blockDim.x) {
-        int run = sh.off[e] + base[e];
-        for (int w = 0; w < kPlaceWarps; ++w) {
-            const int c = pos[w * n_real + e];
-            pos[w * n_real + e] = run;
-            run += c;
-        }
-    }
-    __syncthreads();
 #pragma unroll
     for (int u = 0; u < kSlotRegs; ++u) {
-        if (w0 + 32 * u >= w1 || 32 * u >= per_warp) break;  // (uniform over the warp)
-        const int s = w0 + 32 * u + lane;
-        const int e = e_reg[u];
-        const bool in_range = s < w1;
-        const unsigned grp = __match_any_sync(kFull, e);
+        const int i = threadIdx.x + kScanThreads * u;
+        if (i >= n_slots) break;
+        const int e = e_reg[u], s = s0 + i, tok = i / K;
         int p = -1;
-        if (e >= 0) p = mine[e] + __popc(grp & lt);
-        __syncwarp();
-        if (e >= 0 && (grp & lt) == 0) mine[e] += __popc(grp);
-        __syncwarp();
-        if (in_range) {
-            inv[s] = p;
-            if (p >= 0) {
-                perm[p] = s;
-                if (perm_user) perm_user[p] = s;
-                pair_token[p] = s / K;
-            }
+        if (e >= 0) {
+            const uint4 m = *reinterpret_cast<const uint4 *>(mask + e * kMaskWords);
+            const uint32_t w[kMaskWords] = {m.x, m.y, m.z, m.w};
+            p = sh.off[e] + base[e];
+#pragma unroll
+            for (int q = 0; q < kMaskWords; ++q)
+                p += __popc(q < (tok >> 5) ? w[q] : q == (tok >> 5) ? w[q] & ((1u << (tok & 31)) - 1u) : 0u);
+            perm[p] = s;
+            if (perm_user) perm_user[p] = s;
+            pair_token[p] = s / K;
         }
+        inv[s] = p;
     }
     __syncthreads();
     if (s_ticket == (int)gridDim.x - 1) {
@@ -628,7 +616,7 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_re
     for (int t = t0 + warp; t < t1; t += kStatWarps) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
+        topk_gate_token<RPL, 3>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
                              v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
@@ -742,7 +730,7 @@ int init_route_kernels(const zeda_moe *h) {
     ok = ok && cudaFuncSetAttribute(topk_stats_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(topk_stats_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
     if (!ok) return -1;
-    const int place_smem = (int)sizeof(int32_t) * ((kPlaceWarps + 1) * kMaxCand + kScanSlabInts);
+    const int place_smem = (int)sizeof(int32_t) * ((kMaskWords + 1) * kMaxCand + kScanSlabInts);
     if (cudaFuncSetAttribute(slot_scan_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem) != cudaSuccess)
         return -1;
     return 0;
@@ -751,7 +739,7 @@ int init_route_kernels(const zeda_moe *h) {
 int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s, int *n_parts, int split_T) {
     if (n_parts) *n_parts = 1;
     // large batches: the GEMM goes to the tensor cores (exact three-way bf16 split of the weights)
-    if (T >= 256 && h->router_maps) {
+    if (T >= kTileRouterTokens && h->router_maps) {
         const int split = n_parts ? router_split_factor(h, split_T > T ? split_T : T) : 1;
         if (n_parts) *n_parts = split;
         return launch_router_logits_tile(h, x, T, logits, split, s);
@@ -802,7 +790,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         const bool one_cta = T <= kSmallTokens / kSmallCluster;
 #define ZEDA_CALL_SMALL(R)                                                                                         \
     launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1> : route_small_kernel<R, kSmallCluster>,                \
-        dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
+        dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
         ws.meta, wl, tile_rows, ws.perm, out.perm, ws.inv, ws.pair_token)
         ZEDA_RPL_DISPATCH(ZEDA_CALL_SMALL);
 #undef ZEDA_CALL_SMALL
@@ -811,6 +799,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         // up to kFoldMaxBlocks sort blocks the top-K kernel counts the slots itself and one more launch
         // scans and places; beyond, histogram, scan and placement are kernels of their own
         const bool fold = nblk <= kFoldMaxBlocks;
+        const int pad = (c.n_real + 3) & ~3;
         int32_t *hist_in_topk = fold ? ws.block_hist : nullptr;
 #define ZEDA_CALL_TOPK(R) \
     launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + 7) / 8), dim3(256), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
@@ -824,8 +813,8 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
 #undef ZEDA_CALL_TOPK
 #undef ZEDA_CALL_STATS
         if (fold) {
-            launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk), dim3(kPlaceWarps * 32),
-                          sizeof(int32_t) * ((kPlaceWarps + 1) * c.n_real + kScanSlabInts), s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
+            launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk), dim3(kScanThreads),
+                          sizeof(int32_t) * ((kMaskWords + 1) * pad + kScanSlabInts), s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
                           nblk, ws.block_hist, ws.counts, ws.offsets, out.n_pairs, ws.meta, wl, tile_rows, ws.perm,
                           out.perm, ws.inv, ws.pair_token);
             launches = 2;

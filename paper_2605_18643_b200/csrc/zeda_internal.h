@@ -127,7 +127,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
 int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s);
 int router_split_pad(int n_cand);
 int init_router_tile(zeda_moe *h);
-constexpr int kRouterMaxSplit = 4;
+constexpr int kRouterMaxSplit = 8;
 // rows of n_cand floats that the workspace holds for router output (complete logits or their slices)
 inline long long router_part_rows(long long max_tokens) {
     const long long cap = 9600;  // past this many tokens the unsplit grid covers the SMs already

@@ -306,6 +306,35 @@ def test_tensor_core_router_path(zeda):
         run_layer(zeda, wl, token_ids=sample_tokens(T, 48, 1))
 
 
+@pytest.mark.parametrize("T,E,Z,K", [(129, 9, 3, 5), (159, 8, 4, 2), (160, 8, 4, 2), (255, 130, 30, 16), (257, 301, 99, 16),
+                                     (700, 3, 2, 1), (1153, 512, 0, 3)])
+def test_routing_at_the_edges_of_its_kernels(zeda, T, E, Z, K):
+    # sort blocks of 128 tokens with one token over, expert counts that are no multiple of 4 or above the
+    # threads of the placement pass, the switch between the two routers at 160 tokens
+    wl = inputs.make_layer("edges", T=T, d=192, He=64, E=E, Z=Z, K=K, seed=21, zero_fraction=0.4 if Z else None)
+    m = zeda.from_workload(wl)
+    l, idx, w, counts, offsets, perm, P = oracle_route(wl)
+    for _ in range(2):  # the second call finds the histograms that the first has cleared
+        check_route(m.route(wl.x.to("cuda:0")), idx, w, counts, offsets, perm, P)
+    m.close()
+
+
+@pytest.mark.parametrize("T", [5, 40, 300])
+def test_no_candidate_is_taken_twice_whatever_the_logits(zeda, T):
+    # NaN of both signs, among them the bit pattern whose order-preserving key would be 0
+    wl = inputs.tiny(seed=22, T=T)
+    m = zeda.from_workload(wl)
+    bits = torch.full((T, wl.E + wl.Z), -1, dtype=torch.int32)          # 0xffffffff
+    bits[1::3] = 0x7fffffff
+    bits[2::3] = torch.tensor(float("-inf")).view(torch.int32)
+    o = m.route_from_logits(bits.view(torch.float32).to("cuda:0"))
+    idx = o["topk_idx"].cpu()
+    assert bool((idx >= 0).all()) and bool((idx < wl.E + wl.Z).all())
+    assert all(len(set(row)) == wl.K for row in idx.tolist())
+    assert int(o["counts"].sum()) == int(o["n_pairs"]) == int((idx < wl.E).sum())
+    m.close()
+
+
 @pytest.mark.parametrize("T,max_tokens", [(300, 300), (2500, 2500), (2500, 9000), (5000, 5000), (300, 20000)])
 def test_router_with_sliced_reduction_axis(zeda, T, max_tokens):
     # mid-sized batches cut the router's reduction axis into 2 or 4 slices (as many as keep the grid
