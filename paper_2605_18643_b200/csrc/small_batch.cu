@@ -11,7 +11,7 @@
 // consecutive bytes of weight row g (k = 32 b + 8 t ..) as the A operands of two m16n8k16 MMAs and the
 // same 16 bytes of the pair row of column g as their B operands.  Every load is a full 16 bytes, four
 // lanes cover 64 consecutive bytes of a row, and nothing goes through shared memory.
-#include "zeda_internal.h"
+#include "route_token.cuh"
 
 namespace zeda {
 
@@ -42,21 +42,140 @@ __device__ __forceinline__ uint4 ld_rows(const __nv_bfloat16 *p) { return __ldcg
 constexpr uint4 kZero4 = {0u, 0u, 0u, 0u};
 static_assert(kStreamTokens <= 16, "the kernels are instantiated for up to two column tiles of 8 pair rows");
 
-// The routing results of the call, brought into shared memory by independent loads (one round trip)
-// instead of chains of dependent ones.  One tile of the tile list per active expert: an expert has at
-// most one pair per token, and T <= kStreamTokens is below every tile height.
+// The routing results of the call in shared memory.  One tile of the tile list per active expert: an
+// expert has at most one pair per token, and T <= kStreamTokens is below every tile height.
+template <int SLOTS>
 struct RouteTables {
-    int32_t expert[kStreamSlots];  // active experts in id order
+    int32_t expert[SLOTS];  // active experts in id order
     int32_t off[kMaxCand + 1];
+    int32_t inv[SLOTS], tok[SLOTS], idx[SLOTS];  // of the slot: position, candidate; of the position: token
+    float w[SLOTS];
     int32_t n_tiles;
+    uint32_t mask[kMaxCand];      // tokens that selected the expert
+    int4 chunk[kMaxCand / 32];    // per 32 experts: pairs, active experts, most pairs of one expert
 };
 
-__device__ __forceinline__ void load_route_tables(RouteTables &rt, const int32_t *tile_expert, const int32_t *offsets,
-                                                  const int32_t *meta, int slots, int n_real) {
-    for (int i = threadIdx.x; i < min(slots, n_real); i += blockDim.x) rt.expert[i] = __ldcg(tile_expert + i);
-    for (int i = threadIdx.x; i <= n_real; i += blockDim.x) rt.off[i] = __ldcg(offsets + i);
-    if (threadIdx.x == blockDim.x - 1) rt.n_tiles = __ldcg(meta + kMetaPairTiles);
+struct RouteArgs {  // the routing pass' buffers in the workspace
+    const float *logits;
+    int32_t *topk_idx;
+    float *topk_w;
+    int32_t *inv, *perm, *pair_token, *counts, *offsets, *tile_expert, *tile_row0, *meta;
+    int T, K, n_real, n_cand, gate_mode;
+};
+
+// Loads what the routing pass left, by independent loads (one round trip).
+template <int SLOTS>
+__device__ __forceinline__ void load_route_tables(RouteTables<SLOTS> &rt, const RouteArgs &ra) {
+    const int slots = ra.T * ra.K;
+    for (int i = threadIdx.x; i < slots; i += blockDim.x) {
+        if (i < ra.n_real) rt.expert[i] = __ldcg(ra.tile_expert + i);
+        rt.inv[i] = __ldcg(ra.inv + i);
+        rt.tok[i] = __ldcg(ra.pair_token + i);
+        rt.w[i] = __ldcg(ra.topk_w + i);
+    }
+    for (int i = threadIdx.x; i <= ra.n_real; i += blockDim.x) rt.off[i] = __ldcg(ra.offsets + i);
+    if (threadIdx.x == blockDim.x - 1) rt.n_tiles = __ldcg(ra.meta + kMetaPairTiles);
+    __syncthreads();
 }
+
+// Up to kRouteHereTokens tokens every CTA routes them itself, from the logits: one warp per token and a
+// scan over bit masks take about as long as fetching another kernel's results, and the call has one
+// kernel fewer in its chain (one token: 24.9 -> 15.7 us a call back to back, 8 tokens: 53.7 -> 52.7).  All
+// CTAs arrive at the same tables.
+constexpr int kRouteHereTokens = 8;
+
+template <int RPL, int SLOTS>
+__device__ __forceinline__ void route_here(RouteTables<SLOTS> &rt, const RouteArgs &ra) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
+    const int n_chunks = (ra.n_real + 31) / 32;
+    for (int t = warp; t < ra.T; t += n_warps) {
+        int my_idx;
+        float my_w, v[RPL], m, den;
+        topk_gate_token<RPL>(ra.logits + (size_t)t * ra.n_cand, 1, 0, ra.n_real, ra.n_cand, ra.K, ra.gate_mode, lane, v, m, den, my_idx, my_w);
+        if (lane < ra.K) {
+            rt.idx[t * ra.K + lane] = my_idx;
+            rt.w[t * ra.K + lane] = my_w;
+            if (my_idx < ra.n_real) atomicOr(rt.mask + my_idx, 1u << t);
+        }
+    }
+    __syncthreads();
+    for (int ch = warp; ch < n_chunks; ch += n_warps) {
+        const int i = 32 * ch + lane, c = i < ra.n_real ? __popc(rt.mask[i]) : 0;
+        int sum = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(kFull, sum, o);
+            if (lane >= o) sum += a;
+        }
+        if (i < ra.n_real) rt.off[i] = sum - c;
+        const unsigned act = __ballot_sync(kFull, c > 0);
+        const int mx = __reduce_max_sync(kFull, c);
+        if (lane == 31) rt.chunk[ch] = make_int4(sum, __popc(act), mx, 0);
+    }
+    __syncthreads();
+    for (int ch = warp; ch <= n_chunks; ch += n_warps) {  // one turn more: the totals
+        int off = 0, tiles = 0;
+        for (int q = 0; q < ch; ++q) { off += rt.chunk[q].x; tiles += rt.chunk[q].y; }
+        if (ch == n_chunks) {
+            if (lane == 0) { rt.off[ra.n_real] = off; rt.n_tiles = tiles; }
+            break;
+        }
+        const int i = 32 * ch + lane;
+        const bool active = i < ra.n_real && rt.mask[i];
+        const unsigned act = __ballot_sync(kFull, active);
+        if (i < ra.n_real) rt.off[i] += off;
+        if (active) rt.expert[tiles + __popc(act & ((1u << lane) - 1u))] = i;
+    }
+    __syncthreads();
+    for (int s = threadIdx.x; s < ra.T * ra.K; s += blockDim.x) {
+        const int e = rt.idx[s], t = s / ra.K;
+        int p = -1;
+        if (e < ra.n_real) {
+            p = rt.off[e] + __popc(rt.mask[e] & ((1u << t) - 1u));
+            rt.tok[p] = t;
+        }
+        rt.inv[s] = p;
+    }
+    __syncthreads();
+}
+
+// What the routing pass leaves in the workspace, by one CTA.
+template <int SLOTS>
+__device__ __forceinline__ void publish_route(const RouteTables<SLOTS> &rt, const RouteArgs &ra) {
+    const int slots = ra.T * ra.K;
+    for (int s = threadIdx.x; s < slots; s += blockDim.x) {
+        const int p = rt.inv[s];
+        ra.topk_idx[s] = rt.idx[s];
+        ra.topk_w[s] = rt.w[s];
+        ra.inv[s] = p;
+        if (p >= 0) {
+            ra.perm[p] = s;
+            ra.pair_token[p] = s / ra.K;
+        }
+    }
+    for (int i = threadIdx.x; i <= ra.n_real; i += blockDim.x) {
+        ra.offsets[i] = rt.off[i];
+        if (i < ra.n_real) ra.counts[i] = rt.off[i + 1] - rt.off[i];
+    }
+    for (int i = threadIdx.x; i < rt.n_tiles; i += blockDim.x) {
+        ra.tile_expert[i] = rt.expert[i];
+        ra.tile_row0[i] = 0;
+    }
+    if (threadIdx.x == 0) {
+        int mx = 0;
+        for (int q = 0; q < (ra.n_real + 31) / 32; ++q) mx = max(mx, rt.chunk[q].z);
+        const int pairs = rt.off[ra.n_real];
+        ra.meta[kMetaPairs] = pairs;
+        ra.meta[kMetaActive] = rt.n_tiles;
+        ra.meta[kMetaZeroSlots] = slots - pairs;
+        ra.meta[kMetaPairTiles] = rt.n_tiles;
+        ra.meta[kMetaMaxRows] = mx;
+    }
+}
+
+// RPL > 0: route here, with that many logits per lane; RPL = 0: another kernel has.
+template <int RPL>
+constexpr int kTableSlots = RPL > 0 ? kRouteHereTokens * kMaxTopK : kStreamSlots;
 
 // GEMM1 + SwiGLU.  Unit = (active expert, 8 features): rows g of the fragment are the 8 gate rows, rows
 // g + 8 the 8 up rows, so a lane's accumulators hold gate and up of the same feature and pair and
@@ -66,19 +185,20 @@ __device__ __forceinline__ void load_route_tables(RouteTables &rt, const int32_t
 constexpr int kUpWarps = 8;
 constexpr int kUpChunk = 4;  // 32-k blocks a warp keeps in flight: 4 x (2 x 512 B of weights)
 
-template <int NT>
+template <int NT, int RPL>
 __global__ void __launch_bounds__(32 * kUpWarps, NT == 1 ? 3 : 2)
-stream_gate_up_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const int32_t *__restrict__ offsets,
-                      const int32_t *__restrict__ tile_expert, const int32_t *__restrict__ pair_token,
-                      const int32_t *__restrict__ meta, int slots, int n_real, int d, int He, __nv_bfloat16 *__restrict__ hmid) {
-    __shared__ RouteTables rt;
-    __shared__ int32_t s_tok[kStreamSlots];
+stream_gate_up_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const RouteArgs ra, int d, int He,
+                      __nv_bfloat16 *__restrict__ hmid) {
+    __shared__ RouteTables<kTableSlots<RPL>> rt;
     __shared__ float part[2][kUpWarps][NT][4][32];
+    if constexpr (RPL > 0) {
+        for (int i = threadIdx.x; i < ra.n_real; i += blockDim.x) rt.mask[i] = 0u;
+        __syncthreads();
+    }
     pdl_wait();
-    pdl_launch_dependents();  // only now: the down kernel reads the routing results before its own wait
-    load_route_tables(rt, tile_expert, offsets, meta, slots, n_real);
-    for (int i = threadIdx.x; i < slots; i += blockDim.x) s_tok[i] = __ldcg(pair_token + i);
-    __syncthreads();
+    pdl_launch_dependents();  // only now: the down kernel reads the logits or the routing results before its own wait
+    if constexpr (RPL > 0) route_here<RPL>(rt, ra);
+    else load_route_tables(rt, ra);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int groups = He / 8, units = rt.n_tiles * groups;
     const int kblocks = d / 32, batches = (kblocks + kUpWarps * kUpChunk - 1) / (kUpWarps * kUpChunk);
@@ -89,7 +209,7 @@ stream_gate_up_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
     auto row_of = [&](int pos0, int n, int col) -> const __nv_bfloat16 * {
-        return col < n ? x + (size_t)s_tok[pos0 + col] * d : nullptr;
+        return col < n ? x + (size_t)rt.tok[pos0 + col] * d : nullptr;
     };
     auto fetch = [&](int u, int batch) {
         const int e = rt.expert[u / groups], f0 = (u % groups) * 8;
@@ -149,6 +269,9 @@ stream_gate_up_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *
         u = nu;
         batch = nb;
     }
+    if constexpr (RPL > 0) {
+        if (blockIdx.x == gridDim.x - 1) publish_route(rt, ra);  // the CTA with the fewest units
+    }
 }
 
 // GEMM2 with the weighted combine of Eq. 1: CTA b owns output features [16 b, 16 b + 16) of every token
@@ -163,22 +286,22 @@ constexpr int kDownWarps = 16, kDownSlices = 4, kDownExperts = kDownWarps / kDow
 constexpr int kDownChunk = 6;
 constexpr int kDownStride = 20;  // floats per pair and slice: 16 features; 20 keeps the fragment stores free of bank conflicts
 
-template <int NT>
+template <int NT, int RPL>
 __global__ void __launch_bounds__(32 * kDownWarps, 1)
-stream_down_combine_kernel(const __nv_bfloat16 *__restrict__ hmid, const __nv_bfloat16 *__restrict__ w, const int32_t *__restrict__ offsets,
-                           const int32_t *__restrict__ tile_expert, const int32_t *__restrict__ inv,
-                           const float *__restrict__ topk_w, const int32_t *__restrict__ meta, const __nv_bfloat16 *__restrict__ x,
-                           int T, int K, int n_real, int d, int He, int copy_experts, __nv_bfloat16 *__restrict__ y,
+stream_down_combine_kernel(const __nv_bfloat16 *__restrict__ hmid, const __nv_bfloat16 *__restrict__ w, const RouteArgs ra,
+                           const __nv_bfloat16 *__restrict__ x, int d, int He, int copy_experts, __nv_bfloat16 *__restrict__ y,
                            __nv_bfloat16 *__restrict__ resid) {
-    __shared__ RouteTables rt;
-    __shared__ int32_t s_inv[kStreamSlots];
-    __shared__ float s_w[kStreamSlots];
+    __shared__ RouteTables<kTableSlots<RPL>> rt;
     extern __shared__ float part[];  // [kDownSlices][slots][kDownStride]
     pdl_launch_dependents();
-    const int slots = T * K;
-    load_route_tables(rt, tile_expert, offsets, meta, slots, n_real);
-    for (int i = threadIdx.x; i < slots; i += blockDim.x) { s_inv[i] = __ldcg(inv + i); s_w[i] = __ldcg(topk_w + i); }
-    __syncthreads();
+    const int T = ra.T, K = ra.K, slots = T * K;
+    if constexpr (RPL > 0) {
+        for (int i = threadIdx.x; i < ra.n_real; i += blockDim.x) rt.mask[i] = 0u;
+        __syncthreads();
+        route_here<RPL>(rt, ra);
+    } else {
+        load_route_tables(rt, ra);
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int slice = warp % kDownSlices, m0 = blockIdx.x * 16;
     const int kblocks = He / 32, batches = (kblocks + kDownSlices * kDownChunk - 1) / (kDownSlices * kDownChunk);
@@ -251,8 +374,8 @@ stream_down_combine_kernel(const __nv_bfloat16 *__restrict__ hmid, const __nv_bf
         const size_t at = (size_t)tok * d + m0 + f;
         float sum = 0.f, zero_mass = 0.f;
         for (int k = 0; k < K; ++k) {
-            const int pos = s_inv[tok * K + k];
-            const float wk = s_w[tok * K + k];
+            const int pos = rt.inv[tok * K + k];
+            const float wk = rt.w[tok * K + k];
             if (pos < 0) { zero_mass += wk; continue; }
             float o = 0.f;
 #pragma unroll
@@ -275,39 +398,65 @@ bool stream_path(const zeda_moe *h, int T) {
     return c.ep_size < 1 && T <= kStreamTokens && T * c.top_k <= kStreamSlots;
 }
 
+bool stream_routes_itself(const zeda_moe *h, int T) { return stream_path(h, T) && T <= kRouteHereTokens; }
+
+namespace {
+
+RouteArgs route_args(const zeda_moe *h, int T) {
+    const zeda_moe_config_t &c = h->cfg;
+    const Workspace &ws = h->ws;
+    return {ws.logits, ws.topk_idx, ws.topk_w, ws.inv, ws.perm, ws.pair_token, ws.counts, ws.offsets, ws.ptile_expert, ws.ptile_row0,
+            ws.meta, T, c.top_k, c.n_real, c.n_real + c.n_zero, c.gate_mode};
+}
+
+template <int NT, int RPL>
+int launch_gate_up(const zeda_moe *h, const __nv_bfloat16 *x, int T, cudaStream_t s) {
+    const zeda_moe_config_t &c = h->cfg;
+    const int slots = T * c.top_k, per_sm = NT == 1 ? 3 : 2;
+    const int units = (slots < c.n_real ? slots : c.n_real) * (c.d_expert / 8);
+    const int grid = units < per_sm * h->sm_count ? units : per_sm * h->sm_count;
+    const cudaError_t e = launch_kernel(h->pdl, stream_gate_up_kernel<NT, RPL>, dim3(grid), dim3(32 * kUpWarps), 0, s, x, h->w_gate_up,
+                                        route_args(h, T), (int)c.d_model, (int)c.d_expert, h->ws.hmid);
+    return e == cudaSuccess ? 1 : -1;
+}
+
+template <int NT, int RPL>
+int launch_down(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y, __nv_bfloat16 *resid, cudaStream_t s) {
+    const zeda_moe_config_t &c = h->cfg;
+    const cudaError_t e = launch_kernel(h->pdl, stream_down_combine_kernel<NT, RPL>, dim3(c.d_model / 16), dim3(32 * kDownWarps),
+                                        down_smem_bytes(T * c.top_k), s, (const __nv_bfloat16 *)h->ws.hmid, h->w_down, route_args(h, T), x,
+                                        (int)c.d_model, (int)c.d_expert, (int)(c.expert_kind == ZEDA_EXPERT_COPY), y, resid);
+    return e == cudaSuccess ? 1 : -1;
+}
+
+template <int NT, int RPL>
+bool prepare_down() {
+    return cudaFuncSetAttribute(stream_down_combine_kernel<NT, RPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                down_smem_bytes(kTableSlots<RPL>)) == cudaSuccess;
+}
+
+}  // namespace
+
 int init_stream_kernels() {
-    const int smem = down_smem_bytes(kStreamSlots);
-    const bool ok = cudaFuncSetAttribute(stream_down_combine_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-                    cudaFuncSetAttribute(stream_down_combine_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+    const bool ok = prepare_down<1, 2>() && prepare_down<1, 4>() && prepare_down<1, 6>() && prepare_down<1, 8>() &&
+                    prepare_down<1, 16>() && prepare_down<2, 0>();
     return ok ? 0 : -1;
 }
 
 int launch_stream_gemm1(const zeda_moe *h, const __nv_bfloat16 *x, int T, cudaStream_t s) {
-    const zeda_moe_config_t &c = h->cfg;
-    const Workspace &ws = h->ws;
-    const int slots = T * c.top_k;
-    auto go = [&](auto kernel, int per_sm) {
-        const int units = (slots < c.n_real ? slots : c.n_real) * (c.d_expert / 8);
-        const int grid = units < per_sm * h->sm_count ? units : per_sm * h->sm_count;
-        return launch_kernel(h->pdl, kernel, dim3(grid), dim3(32 * kUpWarps), 0, s, x, h->w_gate_up, (const int32_t *)ws.offsets,
-                             (const int32_t *)ws.ptile_expert, (const int32_t *)ws.pair_token, (const int32_t *)ws.meta, slots,
-                             (int)c.n_real, (int)c.d_model, (int)c.d_expert, ws.hmid);
-    };
-    const cudaError_t e = T <= 8 ? go(stream_gate_up_kernel<1>, 3) : go(stream_gate_up_kernel<2>, 2);
-    return e == cudaSuccess ? 1 : -1;
+    const int n_cand = h->cfg.n_real + h->cfg.n_zero;
+    if (!stream_routes_itself(h, T)) return launch_gate_up<2, 0>(h, x, T, s);
+#define ZEDA_CALL_UP(R) return launch_gate_up<1, R>(h, x, T, s)
+    ZEDA_RPL_DISPATCH(ZEDA_CALL_UP);
+#undef ZEDA_CALL_UP
 }
 
 int launch_stream_down(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y, __nv_bfloat16 *resid, cudaStream_t s) {
-    const zeda_moe_config_t &c = h->cfg;
-    const Workspace &ws = h->ws;
-    auto go = [&](auto kernel) {
-        return launch_kernel(h->pdl, kernel, dim3(c.d_model / 16), dim3(32 * kDownWarps), down_smem_bytes(T * c.top_k), s,
-                             (const __nv_bfloat16 *)ws.hmid, h->w_down, (const int32_t *)ws.offsets, (const int32_t *)ws.ptile_expert,
-                             (const int32_t *)ws.inv, (const float *)ws.topk_w, (const int32_t *)ws.meta, x, T, (int)c.top_k,
-                             (int)c.n_real, (int)c.d_model, (int)c.d_expert, (int)(c.expert_kind == ZEDA_EXPERT_COPY), y, resid);
-    };
-    const cudaError_t e = T <= 8 ? go(stream_down_combine_kernel<1>) : go(stream_down_combine_kernel<2>);
-    return e == cudaSuccess ? 1 : -1;
+    const int n_cand = h->cfg.n_real + h->cfg.n_zero;
+    if (!stream_routes_itself(h, T)) return launch_down<2, 0>(h, x, T, y, resid, s);
+#define ZEDA_CALL_DOWN(R) return launch_down<1, R>(h, x, T, y, resid, s)
+    ZEDA_RPL_DISPATCH(ZEDA_CALL_DOWN);
+#undef ZEDA_CALL_DOWN
 }
 
 }  // namespace zeda

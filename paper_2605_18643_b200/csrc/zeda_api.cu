@@ -156,7 +156,7 @@ zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_
     if (n < 0) return cuda_fail("router launch", cudaGetLastError());
     mark(1);
     RouteOut none = {};
-    int r = launch_route_from_logits(h, h->ws.logits, T, none, s, n_parts);
+    int r = stream_routes_itself(h, T) ? 0 : launch_route_from_logits(h, h->ws.logits, T, none, s, n_parts);
     if (r < 0) return cuda_fail("routing launch", cudaGetLastError());
     n += r;
     mark(2);

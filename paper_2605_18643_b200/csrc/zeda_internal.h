@@ -147,6 +147,7 @@ int launch_experts_gemm1_pair(const zeda_moe *h, const __nv_bfloat16 *x, const E
 int launch_experts_gemm2_pair(const zeda_moe *h, const ExpertWork &w, __nv_bfloat16 *out, cudaStream_t s);
 // the smallest batches (small_batch.cu): GEMM1, and GEMM2 with the combine (resid given: with the residual update)
 bool stream_path(const zeda_moe *h, int T);
+bool stream_routes_itself(const zeda_moe *h, int T);  // the expert kernels also do the routing: logits -> y
 int init_stream_kernels();
 int launch_stream_gemm1(const zeda_moe *h, const __nv_bfloat16 *x, int T, cudaStream_t s);
 int launch_stream_down(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y, __nv_bfloat16 *resid, cudaStream_t s);

@@ -51,6 +51,9 @@ def test_small_batches_match_the_oracle(T, shape, kind):
         dead = np.nonzero((idx >= wl.E).all(axis=1))[0]
         if dead.size:
             assert int(y[torch.as_tensor(dead, device=dev)].view(torch.int16).abs().max().item()) == 0
-    P = m.last_counters()[0]
-    assert P == int((idx < wl.E).sum())
+    P, U, zero_slots = m.last_counters()[:3]  # what the kernels that route themselves leave in the handle
+    real = idx[idx < wl.E]
+    assert (P, U, zero_slots) == (real.size, np.unique(real).size, idx.size - real.size)
+    share = (idx >= wl.E).mean(axis=1).astype(np.float32)
+    assert np.array_equal(m.token_zero_share(T).cpu().numpy(), share)
     m.close()
