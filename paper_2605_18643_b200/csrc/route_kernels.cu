@@ -547,8 +547,8 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_re
     }
 }
 
-// One CTA.  Column c of the partial sums (n_cand counts, then n_cand probabilities) is shared by as many
-// threads as fit, each adding every n-th CTA's value.
+// One CTA.  A pair of columns of the partial sums (n_cand counts, then n_cand probabilities) is shared by as
+// many threads as fit, each adding every n-th CTA's values, sixteen requested at a time.
 constexpr int kStatFinalThreads = 1024;
 
 __global__ void __launch_bounds__(kStatFinalThreads)
@@ -556,21 +556,29 @@ stats_final_kernel(const float *__restrict__ part, int nblk, int T, int K, int n
                    float *__restrict__ f, float *__restrict__ p_mean, float *__restrict__ out) {
     pdl_launch_dependents();
     pdl_wait();
-    __shared__ float seg[kStatFinalThreads], col[2 * kMaxCand], red[5][kStatFinalThreads / 32];
-    const int cols = 2 * n_cand, segs = max(1, kStatFinalThreads / cols);
+    __shared__ float2 seg[kStatFinalThreads];
+    __shared__ float col[2 * kMaxCand], red[5][kStatFinalThreads / 32];
+    const int cols = 2 * n_cand, segs = kStatFinalThreads / n_cand;  // n_cand pairs of columns
     {
-        const int c = threadIdx.x % cols, s = threadIdx.x / cols;  // (at most 1024 columns)
-        float a = 0.f;
+        const int c = threadIdx.x % n_cand, s = threadIdx.x / n_cand;
+        float2 a = make_float2(0.f, 0.f);
         if (s < segs) {
 #pragma unroll 16
-            for (int b = s; b < nblk; b += segs) a += __ldcg(part + (size_t)b * cols + c);
+            for (int b = s; b < nblk; b += segs) {
+                const float2 v = __ldcg(reinterpret_cast<const float2 *>(part + (size_t)b * cols) + c);
+                a.x += v.x;
+                a.y += v.y;
+            }
         }
         seg[threadIdx.x] = a;
     }
     __syncthreads();
     for (int c = threadIdx.x; c < cols; c += kStatFinalThreads) {
         float a = 0.f;
-        for (int s = 0; s < segs; ++s) a += seg[s * cols + c];
+        for (int s = 0; s < segs; ++s) {
+            const float2 v = seg[s * n_cand + (c >> 1)];
+            a += c & 1 ? v.y : v.x;
+        }
         col[c] = a / T;
         if (c < n_cand) { if (f) f[c] = col[c]; }
         else if (p_mean) p_mean[c - n_cand] = col[c];

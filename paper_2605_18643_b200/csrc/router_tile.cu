@@ -79,7 +79,7 @@ router_logits_tile_kernel(const __grid_constant__ CUtensorMap map_w, const __gri
     // its partial sums to logits + p * T * n_cand and the top-K kernel adds the slices in order.
     const int tok_tiles = (T + kTokTile - 1) / kTokTile;
     const int n_items = tok_tiles * m_tiles * split;
-    k_steps /= split;  // per item
+    auto k_first = [&](int sp) { return sp * k_steps / split; };  // first k-step of slice sp
 
     if (warp == 0) {
         if (lane == 0) {
@@ -87,11 +87,11 @@ router_logits_tile_kernel(const __grid_constant__ CUtensorMap map_w, const __gri
             bool ok = true;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 const int sp = item % split, mt = (item / split) % m_tiles, tt = item / (split * m_tiles);
-                for (int ks = 0; ks < k_steps; ++ks, ++it_count) {
+                for (int ks = k_first(sp); ks < k_first(sp + 1); ++ks, ++it_count) {
                     const uint32_t s = it_count % kStages, ph = (it_count / kStages) & 1u;
                     if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
                     const uint32_t full = bar_full + 8 * s, sa = ring + s * kStageBytes;
-                    const int kc = (sp * k_steps + ks) * kBlockK;
+                    const int kc = ks * kBlockK;
                     mbar_expect_tx(full, kStageBytes);
                     for (int piece = 0; piece < 3; ++piece)
                         tma_load_3d(sa + piece * kTileBytes, &map_w, kc, mt * 128, piece, full);
@@ -110,7 +110,8 @@ router_logits_tile_kernel(const __grid_constant__ CUtensorMap map_w, const __gri
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++tile_count) {
                 if (!mbar_wait(bar_tempty, (tile_count & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
-                for (int ks = 0; ks < k_steps; ++ks, ++it_count) {
+                const int sp = item % split, n_steps = k_first(sp + 1) - k_first(sp);
+                for (int ks = 0; ks < n_steps; ++ks, ++it_count) {
                     const uint32_t s = it_count % kStages, ph = (it_count / kStages) & 1u;
                     if (!mbar_wait(bar_full + 8 * s, ph, abort_flag)) { ok = false; break; }
                     tc_fence_after();
@@ -218,10 +219,13 @@ int router_split_factor(const zeda_moe *h, int T) {
     const int nc_pad = router_split_pad(h->cfg.n_real + h->cfg.n_zero);
     const int items = (T + kTokTile - 1) / kTokTile * (nc_pad / 128);
     const int k_steps = h->cfg.d_model / kBlockK;
-    int split = 1;
-    while (split < kRouterMaxSplit && items * split * 2 <= h->sm_count && k_steps % (split * 2) == 0 &&
-           (long long)T * split * 2 <= router_part_rows(h->cfg.max_tokens))
-        split *= 2;
+    // as many slices as the SMs take (any number: 40 items of 5003 tokens and up to 128 candidates run three
+    // slices of 10 or 11 k-steps each), while the workspace holds them
+    int split = h->sm_count / items;
+    if (split > kRouterMaxSplit) split = kRouterMaxSplit;
+    if (split > k_steps) split = k_steps;
+    while (split > 1 && (long long)T * split > router_part_rows(h->cfg.max_tokens, h->cfg.n_real + h->cfg.n_zero)) --split;
+    if (split < 1) split = 1;
     return split;
 }
 

@@ -79,7 +79,7 @@ size_t carve(const zeda_moe_config_t &c, unsigned char *base, Workspace *ws, int
     w.meta = (int32_t *)take(kMetaCount * 4);
     w.ptile_expert = (int32_t *)take(tiles * 4);
     w.ptile_row0 = (int32_t *)take(tiles * 4);
-    w.logits = (float *)take((size_t)router_part_rows(c.max_tokens) * n_cand * 4);
+    w.logits = (float *)take((size_t)router_part_rows(c.max_tokens, (int)n_cand) * n_cand * 4);
     w.stat_part = (float *)take(nblk_stats * 2 * n_cand * 4);
     // pair buffers carry one tile of slack rows so that a full tile may be read past the last pair
     w.hmid = (__nv_bfloat16 *)take((pair_rows + kPairTileM) * c.d_expert * 2);

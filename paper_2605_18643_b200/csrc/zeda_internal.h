@@ -129,8 +129,9 @@ int router_split_pad(int n_cand);
 int init_router_tile(zeda_moe *h);
 constexpr int kRouterMaxSplit = 8;
 // rows of n_cand floats that the workspace holds for router output (complete logits or their slices)
-inline long long router_part_rows(long long max_tokens) {
-    const long long cap = 9600;  // past this many tokens the unsplit grid covers the SMs already
+inline long long router_part_rows(long long max_tokens, int n_cand) {
+    // slices x tokens that cover 150 SMs with a tile of 128 tokens x 128 candidates each
+    const long long cap = 19200 / ((n_cand + 127) / 128);
     const long long want = kRouterMaxSplit * max_tokens < cap ? kRouterMaxSplit * max_tokens : cap;
     return max_tokens > want ? max_tokens : want;
 }

@@ -107,9 +107,11 @@ class ExpertParallelMoE:
         recv_counts = self.x.counts(expert_counts)
         # the one host synchronisation of the call: the all-to-all needs its split sizes on the host (both
         # directions' counts in one copy)
-        counts = torch.cat((send_counts, recv_counts.reshape(-1))).cpu()
-        send_splits = counts[:self.G].tolist()
-        recv_splits, n_rows = recv_layout(counts[self.G:].view(self.G, -1))
+        counts = torch.cat((send_counts, recv_counts.reshape(-1))).tolist()
+        send_splits = counts[:self.G]
+        n_local = recv_counts.numel() // self.G
+        recv_splits = [sum(counts[self.G + s * n_local:self.G + (s + 1) * n_local]) for s in range(self.G)]  # (recv_layout on host values)
+        n_rows = sum(recv_splits)
         if n_rows > m.cfg.max_recv_pairs:
             raise RuntimeError("rank receives %d pair rows, handle was sized for %d" % (n_rows, m.cfg.max_recv_pairs))
         recv_rows = self.x.rows(send_rows, send_splits, recv_splits)
