@@ -39,8 +39,8 @@ __device__ __forceinline__ void load_slot_table(SlotTable &st, const int32_t *__
         st.pos[k] = -1;
         st.w[k] = 0.f;
         if (k < K) {
-            st.pos[k] = __ldg(inv + (size_t)t * K + k);
-            st.w[k] = __ldg(topk_w + (size_t)t * K + k);
+            st.pos[k] = ld_ordered(inv + (size_t)t * K + k);
+            st.w[k] = __int_as_float(ld_ordered(reinterpret_cast<const int32_t *>(topk_w) + (size_t)t * K + k));
             if (st.pos[k] < 0) st.zero_mass += st.w[k];
         }
     }
@@ -59,13 +59,13 @@ __device__ __forceinline__ void combine_chunk(float (&acc)[8], const SlotTable &
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             if (k0 + k < K && st.pos[k0 + k] >= 0)
-                v[k] = __ldg(reinterpret_cast<const uint4 *>(obuf + (size_t)st.pos[k0 + k] * d) + c);
+                v[k] = __ldcg(reinterpret_cast<const uint4 *>(obuf + (size_t)st.pos[k0 + k] * d) + c);
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             if (k0 + k < K && st.pos[k0 + k] >= 0) fma_bf16x8(acc, st.w[k0 + k], v[k]);
     }
     if (copy_experts && st.zero_mass != 0.f)
-        fma_bf16x8(acc, st.zero_mass, __ldg(reinterpret_cast<const uint4 *>(x + (size_t)t * d) + c));
+        fma_bf16x8(acc, st.zero_mass, __ldcg(reinterpret_cast<const uint4 *>(x + (size_t)t * d) + c));
 }
 
 __global__ void __launch_bounds__(kCombineThreads, 16)
@@ -120,8 +120,8 @@ combine_glue_kernel(const __nv_bfloat16 *__restrict__ obuf, const int32_t *__res
     const bool in = c < d / 8;
     uint4 *rp = reinterpret_cast<uint4 *>(resid + (size_t)t * d) + c;
     const uint4 rv = in ? *rp : make_uint4(0u, 0u, 0u, 0u);
-    const int my_pos = lane < K ? __ldg(inv + (size_t)t * K + lane) : -1;
-    const float my_w = lane < K ? __ldg(topk_w + (size_t)t * K + lane) : 0.f;
+    const int my_pos = lane < K ? __ldcg(inv + (size_t)t * K + lane) : -1;
+    const float my_w = lane < K ? __ldcg(topk_w + (size_t)t * K + lane) : 0.f;
     const unsigned real = __ballot_sync(0xffffffffu, my_pos >= 0);
     float acc[8];
 #pragma unroll
@@ -136,7 +136,7 @@ combine_glue_kernel(const __nv_bfloat16 *__restrict__ obuf, const int32_t *__res
             left &= left - 1u;
             w[r] = __shfl_sync(0xffffffffu, my_w, k);
             const int pos = __shfl_sync(0xffffffffu, my_pos, k);
-            if (r < n && in) v[r] = __ldg(reinterpret_cast<const uint4 *>(obuf + (size_t)pos * d) + c);
+            if (r < n && in) v[r] = __ldcg(reinterpret_cast<const uint4 *>(obuf + (size_t)pos * d) + c);
         }
 #pragma unroll
         for (int r = 0; r < kRowsInFlight; ++r)
@@ -148,7 +148,7 @@ combine_glue_kernel(const __nv_bfloat16 *__restrict__ obuf, const int32_t *__res
             const float w = __shfl_sync(0xffffffffu, my_w, k);
             if (!(real >> k & 1u)) zero_mass += w;
         }
-        if (zero_mass != 0.f && in) fma_bf16x8(acc, zero_mass, __ldg(reinterpret_cast<const uint4 *>(x + (size_t)t * d) + c));
+        if (zero_mass != 0.f && in) fma_bf16x8(acc, zero_mass, __ldcg(reinterpret_cast<const uint4 *>(x + (size_t)t * d) + c));
     }
     const uint32_t ru[4] = {rv.x, rv.y, rv.z, rv.w};
     uint32_t keep[4];  // the updated residual (bf16 pairs)

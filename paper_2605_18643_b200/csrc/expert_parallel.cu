@@ -36,13 +36,13 @@ ep_pack_kernel(__nv_bfloat16 *__restrict__ dst, const __nv_bfloat16 *__restrict_
     const int rows_per_cta = blockDim.x / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int r = blockIdx.x * rows_per_cta + warp; r < n_rows; r += gridDim.x * rows_per_cta) {
-        const uint4 *s = reinterpret_cast<const uint4 *>(src + (size_t)__ldg(idx + r) * d);
+        const uint4 *s = reinterpret_cast<const uint4 *>(src + (size_t)__ldcg(idx + r) * d);
         uint4 *o = reinterpret_cast<uint4 *>(dst + (size_t)r * d);
         for (int c0 = lane; c0 < chunks; c0 += 256) {  // eight loads in flight per lane
             uint4 v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (c0 + 32 * u < chunks) v[u] = __ldg(s + c0 + 32 * u);
+                if (c0 + 32 * u < chunks) v[u] = __ldcg(s + c0 + 32 * u);
 #pragma unroll
             for (int u = 0; u < 8; ++u)
                 if (c0 + 32 * u < chunks) o[c0 + 32 * u] = v[u];
@@ -70,7 +70,7 @@ ep_plan_kernel(const int32_t *__restrict__ recv_counts, int n_ranks, int n_local
     for (int j = threadIdx.x; j < n_local; j += blockDim.x) {
         int total = 0, bef = 0;
         for (int q = 0; q < n_ranks; ++q) {
-            const int c = max(0, __ldg(recv_counts + q * n_local + j));
+            const int c = max(0, __ldcg(recv_counts + q * n_local + j));
             total += c;
             if (q < s) bef += c;
         }
@@ -83,7 +83,7 @@ ep_plan_kernel(const int32_t *__restrict__ recv_counts, int n_ranks, int n_local
         int base = 0;
         for (int j0 = 0; j0 < n_local; j0 += 32) {
             const int j = j0 + threadIdx.x;
-            const int c = j < n_local ? max(0, __ldg(recv_counts + s * n_local + j)) : 0;
+            const int c = j < n_local ? max(0, __ldcg(recv_counts + s * n_local + j)) : 0;
             int sc = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {

@@ -39,7 +39,7 @@ router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restric
             const int i = i0 + u * blockDim.x;
             const int r = i / vec_per_row, c = i % vec_per_row;
             v[u] = make_uint4(0, 0, 0, 0);
-            if (i < kTok * vec_per_row && r < nt) v[u] = __ldg(reinterpret_cast<const uint4 *>(x + (size_t)(t0 + r) * d) + c);
+            if (i < kTok * vec_per_row && r < nt) v[u] = __ldcg(reinterpret_cast<const uint4 *>(x + (size_t)(t0 + r) * d) + c);
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -118,7 +118,7 @@ router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__res
             w[u] = in ? __ldg(reinterpret_cast<const float4 *>(wrow) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int r = 0; r < NT; ++r)
-                xv[r][u] = in && t0 + r < T ? __ldg(reinterpret_cast<const uint2 *>(x + (size_t)(t0 + r) * d) + c) : make_uint2(0u, 0u);
+                xv[r][u] = in && t0 + r < T ? __ldcg(reinterpret_cast<const uint2 *>(x + (size_t)(t0 + r) * d) + c) : make_uint2(0u, 0u);
         }
 #pragma unroll
         for (int r = 0; r < NT; ++r) {
@@ -209,7 +209,7 @@ __device__ __forceinline__ void stage_ints(int32_t *__restrict__ dst, const int3
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u) {
             const int i = i0 + u * blockDim.x;
-            v[u] = i < n ? __ldg(src + i) : 0;
+            v[u] = i < n ? __ldcg(src + i) : 0;
         }
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u) {
@@ -424,7 +424,7 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
 #pragma unroll
     for (int u = 0; u < kSlotRegs; ++u) {
         const int i = threadIdx.x + kScanThreads * u;
-        const int e = i < n_slots ? __ldg(topk_idx + s0 + i) : -1;
+        const int e = i < n_slots ? __ldcg(topk_idx + s0 + i) : -1;
         e_reg[u] = (unsigned)e >= (unsigned)n_real ? -1 : e;
     }
     // column sums of the CTA histograms: staged slab by slab with independent coalesced loads (a

@@ -31,7 +31,7 @@ residual_rmsnorm_kernel(__nv_bfloat16 *__restrict__ r, const __nv_bfloat16 *__re
             const uint32_t au[4] = {a.x, a.y, a.z, a.w};
             uint32_t bu[4] = {0, 0, 0, 0};
             if (y) {
-                const uint4 b = __ldg(reinterpret_cast<const uint4 *>(y + row + 8 * c));
+                const uint4 b = __ldcg(reinterpret_cast<const uint4 *>(y + row + 8 * c));
                 bu[0] = b.x; bu[1] = b.y; bu[2] = b.z; bu[3] = b.w;
             }
             uint4 o;

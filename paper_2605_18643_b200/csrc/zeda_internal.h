@@ -175,12 +175,21 @@ void note_launch_error(cudaError_t e);
 // The kernels of one forward pass are launched back to back on one stream.  Launched with the
 // attribute below, a kernel may start (launch latency, barrier and TMEM set-up) while its
 // predecessor is still draining; it touches no global memory until pdl_wait() returns, which is
-// when the predecessor has completed and its writes are visible.  Each kernel calls
+// when the predecessor has completed and its writes are visible.  What a predecessor in the stream has
+// written is read by plain or ld.cg loads, not by __ldg: the compiler takes the latter to be invariant
+// while the kernel runs and may move it in front of the wait.  Each kernel calls
 // pdl_launch_dependents() first thing so that its successor is released as early as possible.
 // Without the attribute both calls do nothing.
 #if defined(__CUDACC__)
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// a load through L1 that stays behind the wait
+__device__ __forceinline__ int32_t ld_ordered(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.global.ca.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 
 __device__ __forceinline__ float swiglu(float g, float u) { return __fdividef(g * u, 1.f + __expf(-g)); }
 
