@@ -23,9 +23,10 @@ constexpr int kRouterUnroll = 8;  // 16-byte weight loads a lane keeps in flight
 __global__ void __launch_bounds__(256)
 router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w,
                      const float *__restrict__ router_bias, int T, int d, int n_cand,
-                     int cand_per_cta, float *__restrict__ logits) {
+                     int cand_per_cta, float *__restrict__ logits, int32_t *__restrict__ hist, int n_hist) {
     pdl_launch_dependents();
     pdl_wait();
+    clear_hist(hist, n_hist);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(smem_raw);  // [kTok][d]
     const int t0 = blockIdx.x * kTok;
@@ -99,12 +100,14 @@ constexpr int kFewUnroll = 4;
 template <int NT>
 __global__ void __launch_bounds__(kFewThreads)
 router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w,
-                         const float *__restrict__ router_bias, int T, int d, int n_cand, float *__restrict__ logits) {
+                         const float *__restrict__ router_bias, int T, int d, int n_cand, float *__restrict__ logits,
+                         int32_t *__restrict__ hist, int n_hist) {
     pdl_launch_dependents();
     const int j = blockIdx.x, t0 = blockIdx.y * NT;
     const float *wrow = router_w + (size_t)j * d;
     for (int i = threadIdx.x; i < d / 32; i += kFewThreads) asm volatile("prefetch.global.L2 [%0];" ::"l"(wrow + 32 * i));
     pdl_wait();
+    clear_hist(hist, n_hist);
     float acc[NT];
 #pragma unroll
     for (int r = 0; r < NT; ++r) acc[r] = 0.f;
@@ -149,8 +152,7 @@ router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__res
 
 // block_hist (optional): pass 1 of the counting sort done here.  Every slot on a normal expert adds 1
 // to its entry of the histogram of its block of kSortTokens tokens (integer adds: the counts do not
-// depend on their order).  The histograms must be zero on entry; the placement kernel that consumes
-// them zeroes them again.
+// depend on their order).  The histograms must be zero on entry: the call's router kernel clears them.
 template <int RPL>
 __global__ void __launch_bounds__(256)
 topk_gate_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
@@ -199,25 +201,6 @@ slot_hist_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real,
 // counts, exclusive offsets, P, U, and the work lists of the expert kernels.
 // ---------------------------------------------------------------------------------------------
 constexpr int kScanSlabInts = 8192;  // 32 KB of CTA histograms per slab of the expert scan
-
-// Copies n ints from global to shared memory with sixteen loads in flight per thread: a plain
-// load-store loop issues its loads one L2 round trip after another (the store waits for the load).
-__device__ __forceinline__ void stage_ints(int32_t *__restrict__ dst, const int32_t *__restrict__ src, int n) {
-    constexpr int kInFlight = 16;
-    for (int i0 = threadIdx.x; i0 < n; i0 += kInFlight * blockDim.x) {
-        int32_t v[kInFlight];
-#pragma unroll
-        for (int u = 0; u < kInFlight; ++u) {
-            const int i = i0 + u * blockDim.x;
-            v[u] = i < n ? __ldcg(src + i) : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < kInFlight; ++u) {
-            const int i = i0 + u * blockDim.x;
-            if (i < n) dst[i] = v[u];
-        }
-    }
-}
 
 __global__ void __launch_bounds__(512)
 expert_scan_kernel(int32_t *__restrict__ block_hist, int nblk, int n_real, int total_slots,
@@ -330,7 +313,6 @@ route_small_kernel(const float *__restrict__ logits, int n_parts, int T, int n_r
 // memory.  No atomics decide a position, so the order is (expert, token) ascending every run.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPlaceWarps = 8;
-constexpr int kFoldMaxBlocks = 256;  // up to this many CTA histograms the placement CTAs scan them themselves
 
 __global__ void __launch_bounds__(kPlaceWarps * 32)
 slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real,
@@ -395,27 +377,28 @@ slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real
 // once, so a slot's rank among its CTA's pairs of the expert is a popcount over a bit mask of the CTA's
 // tokens (one shared-memory atomicOr per slot instead of two passes of match.any over them).  CTA 0
 // also publishes counts, offsets and the counters; the tile list is filled by all CTAs, a share each.
-// What bounds it is the chain of dependent steps, not the data: 7.4 us for 2 CTAs before, as for 64.
+// What bounds it is the chain of dependent steps, not the data: of the 5.5 us that a CTA took, 1.4 (2 blocks)
+// to 3.2 (64) went to staging and summing the histograms in shared memory and 1 to the fence of a ticket by
+// which the last CTA cleared them.
 // ---------------------------------------------------------------------------------------------
 constexpr int kScanThreads = 256;
 constexpr int kMaskWords = kSortTokens / 32;
 
 __global__ void __launch_bounds__(kScanThreads)
 slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real, int nblk,
-                       int32_t *__restrict__ block_hist, int32_t *__restrict__ counts,
+                       const int32_t *__restrict__ block_hist, int32_t *__restrict__ counts,
                        int32_t *__restrict__ offsets, int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                        const WorkLists wl, int tile_rows, int32_t *__restrict__ perm, int32_t *__restrict__ perm_user,
                        int32_t *__restrict__ inv, int32_t *__restrict__ pair_token) {
     __shared__ ScanShared sh;
-    __shared__ int s_ticket;
-    extern __shared__ __align__(16) int32_t place_smem[];  // base[n_real], token masks [n_real][kMaskWords], a histogram slab [kScanSlabInts]
-    int32_t *base = place_smem;
-    const int pad = (n_real + 3) & ~3;  // the masks are read as 16 bytes
-    uint32_t *mask = reinterpret_cast<uint32_t *>(base + pad);
-    int32_t *slab = base + pad + kMaskWords * pad;
+    extern __shared__ __align__(16) uint32_t place_smem[];  // token masks [n_real][kMaskWords], then base[n_real]
+    uint32_t *mask = place_smem;
+    int32_t *base = reinterpret_cast<int32_t *>(mask + kMaskWords * n_real);
     pdl_launch_dependents();
     for (int i = threadIdx.x; i < n_real * kMaskWords; i += blockDim.x) mask[i] = 0u;
     for (int e = threadIdx.x; e < n_real; e += blockDim.x) { base[e] = 0; sh.cnt[e] = 0; }
+    const uint32_t inv_k = (65536u + K - 1) / K;  // i / K = i * inv_k >> 16 for i < kSortTokens * kMaxTopK
+    __syncthreads();
     pdl_wait();
     // slot s0 + threadIdx.x + kScanThreads * u in e_reg[u], -1 for zero-expert slots and beyond the end
     constexpr int kSlotRegs = kSortTokens * kMaxTopK / kScanThreads;
@@ -427,50 +410,37 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
         const int e = i < n_slots ? __ldcg(topk_idx + s0 + i) : -1;
         e_reg[u] = (unsigned)e >= (unsigned)n_real ? -1 : e;
     }
-    // column sums of the CTA histograms: staged slab by slab with independent coalesced loads (a
-    // per-thread loop over global memory would be one L2 round trip after another); with fewer experts
-    // than threads, several threads share a column
-    const int slab_blocks = max(1, kScanSlabInts / n_real);
-    const int col_parts = max(1, (int)blockDim.x / n_real);
-    for (int b0 = 0; b0 < nblk; b0 += slab_blocks) {
-        const int nb = min(slab_blocks, nblk - b0);
-        __syncthreads();
-        stage_ints(slab, block_hist + (size_t)b0 * n_real, nb * n_real);
-        __syncthreads();
-        for (int i = threadIdx.x; i < n_real * col_parts; i += blockDim.x) {
-            const int e = i % n_real;
-            int before = 0, total = 0;
-#pragma unroll 4
-            for (int b = i / n_real; b < nb; b += col_parts) {
-                const int c = slab[b * n_real + e];
-                total += c;
-                if (b0 + b < (int)blockIdx.x) before += c;
-            }
-            if (total) {
-                atomicAdd(&base[e], before);
-                atomicAdd(&sh.cnt[e], total);
+    // Column sums of the CTA histograms, straight from global memory, sixteen blocks requested at a time;
+    // with fewer experts than threads, several threads share a column.
+    const int col_parts = max(1, kScanThreads / n_real);
+    const int part0 = threadIdx.x / n_real;
+    for (int e = threadIdx.x - part0 * n_real; e < n_real && part0 < col_parts; e += kScanThreads) {
+        int before = 0, total = 0;
+        for (int b0 = part0; b0 < nblk; b0 += 16 * col_parts) {
+            int c[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) c[q] = b0 + q * col_parts < nblk ? __ldcg(block_hist + (size_t)(b0 + q * col_parts) * n_real + e) : 0;
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                total += c[q];
+                if (b0 + q * col_parts < (int)blockIdx.x) before += c[q];
             }
         }
+        atomicAdd(&base[e], before);
+        atomicAdd(&sh.cnt[e], total);
     }
 #pragma unroll
     for (int u = 0; u < kSlotRegs; ++u) {
-        const int tok = (threadIdx.x + kScanThreads * u) / K;
+        const uint32_t tok = (threadIdx.x + kScanThreads * u) * inv_k >> 16;
         if (e_reg[u] >= 0) atomicOr(mask + e_reg[u] * kMaskWords + (tok >> 5), 1u << (tok & 31));
     }
     __syncthreads();
-    // The histograms go back to zero for the next call's top-K kernel: the CTA that is last to have
-    // read them (a ticket, nobody waits; looked at only when this CTA's own work is done) clears them
-    // and the ticket counter.
-    if (threadIdx.x == blockDim.x - 1) {
-        __threadfence();
-        s_ticket = atomicAdd(meta + kMetaHistTicket, 1);
-    }
     finish_expert_scan(sh, n_real, T * K, counts, offsets, n_pairs_out, meta, wl, blockIdx.x == 0, blockIdx.x, gridDim.x, tile_rows);
 #pragma unroll
     for (int u = 0; u < kSlotRegs; ++u) {
         const int i = threadIdx.x + kScanThreads * u;
         if (i >= n_slots) break;
-        const int e = e_reg[u], s = s0 + i, tok = i / K;
+        const int e = e_reg[u], s = s0 + i, tok = i * inv_k >> 16;
         int p = -1;
         if (e >= 0) {
             const uint4 m = *reinterpret_cast<const uint4 *>(mask + e * kMaskWords);
@@ -481,14 +451,9 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
                 p += __popc(q < (tok >> 5) ? w[q] : q == (tok >> 5) ? w[q] & ((1u << (tok & 31)) - 1u) : 0u);
             perm[p] = s;
             if (perm_user) perm_user[p] = s;
-            pair_token[p] = s / K;
+            pair_token[p] = blockIdx.x * kSortTokens + tok;
         }
         inv[s] = p;
-    }
-    __syncthreads();
-    if (s_ticket == (int)gridDim.x - 1) {
-        for (int i = threadIdx.x; i < nblk * n_real; i += blockDim.x) block_hist[i] = 0;
-        if (threadIdx.x == 0) meta[kMetaHistTicket] = 0;
     }
 }
 
@@ -634,18 +599,6 @@ int init_route_kernels(const zeda_moe *h) {
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(router_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return -1;
-    // placement CTAs: static scan state plus (per-warp positions, bases, a histogram slab) pass 48 KB
-    // together when there are many experts
-    const int stats_smem = (int)sizeof(float) * (kStatWarps + 1) * kMaxCand;
-    bool ok = cudaFuncSetAttribute(topk_stats_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
-    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
-    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
-    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
-    ok = ok && cudaFuncSetAttribute(topk_stats_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem) == cudaSuccess;
-    if (!ok) return -1;
-    const int place_smem = (int)sizeof(int32_t) * ((kMaskWords + 1) * kMaxCand + kScanSlabInts);
-    if (cudaFuncSetAttribute(slot_scan_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem) != cudaSuccess)
-        return -1;
     return 0;
 }
 
@@ -662,7 +615,7 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
     if (T <= kFewTokens) {
         auto go = [&](auto kernel, int per_cta) {
             return launch_kernel(h->pdl, kernel, dim3(n_cand, (T + per_cta - 1) / per_cta), dim3(kFewThreads), 0, s, x, h->router_w,
-                                 h->router_bias, T, d, n_cand, logits);
+                                 h->router_bias, T, d, n_cand, logits, h->ws.block_hist, hist_ints(h, T));
         };
         const cudaError_t e = T == 1   ? go(router_logits_few_kernel<1>, 1)
                               : T == 2 ? go(router_logits_few_kernel<2>, 2)
@@ -678,7 +631,7 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
     const int per = (n_cand + splits - 1) / splits;
     const size_t smem = (size_t)kTok * d * sizeof(__nv_bfloat16);
     const cudaError_t e = launch_kernel(h->pdl, router_logits_kernel, dim3(tiles, (n_cand + per - 1) / per), dim3(256), smem, s,
-                                        x, h->router_w, h->router_bias, T, d, n_cand, per, logits);
+                                        x, h->router_w, h->router_bias, T, d, n_cand, per, logits, h->ws.block_hist, hist_ints(h, T));
     return e == cudaSuccess ? 1 : -1;
 }
 
@@ -704,10 +657,12 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         // up to kFoldMaxBlocks sort blocks the top-K kernel counts the slots itself and one more launch
         // scans and places; beyond, histogram, scan and placement are kernels of their own
         const bool fold = nblk <= kFoldMaxBlocks;
-        const int pad = (c.n_real + 3) & ~3;
+        const int topk_warps = T <= 8 * h->sm_count ? 2 : 8;  // the loads of a few tokens spread over all SMs
         int32_t *hist_in_topk = fold ? ws.block_hist : nullptr;
+        // no router kernel has cleared the histograms in front of a caller's own logits
+        if (fold && logits != ws.logits && cudaMemsetAsync(ws.block_hist, 0, sizeof(int32_t) * nblk * c.n_real, s) != cudaSuccess) return -1;
 #define ZEDA_CALL_TOPK(R) \
-    launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + 7) / 8), dim3(256), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
+    launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
                   c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
 #define ZEDA_CALL_STATS(R) \
     launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps), \
@@ -719,8 +674,8 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
 #undef ZEDA_CALL_STATS
         if (fold) {
             launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk), dim3(kScanThreads),
-                          sizeof(int32_t) * ((kMaskWords + 1) * pad + kScanSlabInts), s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
-                          nblk, ws.block_hist, ws.counts, ws.offsets, out.n_pairs, ws.meta, wl, tile_rows, ws.perm,
+                          sizeof(int32_t) * (kMaskWords + 1) * c.n_real, s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
+                          nblk, (const int32_t *)ws.block_hist, ws.counts, ws.offsets, out.n_pairs, ws.meta, wl, tile_rows, ws.perm,
                           out.perm, ws.inv, ws.pair_token);
             launches = 2;
         } else {

@@ -47,7 +47,7 @@ split_router_kernel(const float *__restrict__ w, int n_cand, int nc_pad, int d, 
 __global__ void __launch_bounds__(kThreads, 1)
 router_logits_tile_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                           const float *__restrict__ bias, int T, int n_cand, int m_tiles, int k_steps, int split,
-                          int32_t *__restrict__ meta, float *__restrict__ logits) {
+                          int32_t *__restrict__ meta, float *__restrict__ logits, int32_t *__restrict__ hist, int n_hist) {
     pdl_launch_dependents();
     extern __shared__ __align__(1024) unsigned char router_smem[];
     __shared__ __align__(8) unsigned long long bars[2 * kStages + 2];
@@ -132,6 +132,7 @@ router_logits_tile_kernel(const __grid_constant__ CUtensorMap map_w, const __gri
             if (!ok) { if (!*abort_flag) atomicExch(&meta[kMetaError], 5); s_abort = 1; }
         }
     } else {
+        for (int i = blockIdx.x * 128 + (threadIdx.x - 64); i < n_hist; i += gridDim.x * 128) hist[i] = 0;  // idle until the first tile is done
         const int q = warp & 3;
         uint32_t tile_count = 0;
         bool ok = true;
@@ -244,7 +245,7 @@ int launch_router_logits_tile(const zeda_moe *h, const __nv_bfloat16 *x, int T, 
     const int grid = n_items < h->sm_count ? n_items : h->sm_count;
     const cudaError_t e = launch_kernel(h->pdl, router_logits_tile_kernel, dim3(grid), dim3(kThreads), kSmemBytes, s,
                                         rm->w_split, map_x, h->router_bias, T, n_cand, m_tiles, c.d_model / kBlockK,
-                                        split, h->ws.meta, logits);
+                                        split, h->ws.meta, logits, h->ws.block_hist, hist_ints(h, T));
     return e == cudaSuccess ? 1 : -1;
 }
 

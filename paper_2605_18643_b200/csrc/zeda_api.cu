@@ -273,10 +273,6 @@ zeda_status_t zeda_moe_create(const zeda_moe_config_t *cfg, const float *router_
     }
     e = cudaMemset(h->ws.meta, 0, kMetaCount * 4);
     if (e != cudaSuccess) { delete h; return cuda_fail("cudaMemset(meta)", e); }
-    // the block histograms of the counting sort are zero between calls (the top-K kernel adds into them,
-    // the placement kernel clears them)
-    e = cudaMemset(h->ws.block_hist, 0, hist_bytes(*cfg));
-    if (e != cudaSuccess) { delete h; return cuda_fail("cudaMemset(block_hist)", e); }
     e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { delete h; return cuda_fail("cudaDeviceSynchronize", e); }
     *out = h;
@@ -563,10 +559,6 @@ zeda_status_t zeda_moe_clear_error(zeda_moe_t *h, void *stream) {
     cudaError_t e = cudaSetDevice(h->cfg.device);
     if (e != cudaSuccess) return cuda_fail("cudaSetDevice", e);
     e = cudaMemsetAsync(h->ws.meta + kMetaError, 0, sizeof(int32_t), static_cast<cudaStream_t>(stream));
-    if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync", e);
-    // a call that failed between its top-K and placement kernels leaves counts in the block histograms
-    e = cudaMemsetAsync(h->ws.block_hist, 0, hist_bytes(h->cfg), static_cast<cudaStream_t>(stream));
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->ws.meta + kMetaHistTicket, 0, sizeof(int32_t), static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync", e);
     return ZEDA_OK;
 }

@@ -30,7 +30,6 @@ enum MetaSlot {
     kMetaPairTiles = 7,  // entries of the expert kernels' tile list
     kMetaNextItem1 = 8,  // next unclaimed work item of the GEMM1 kernel (reset by the routing pass)
     kMetaNextItem2 = 9,  // the same for GEMM2
-    kMetaHistTicket = 10,  // placement CTAs that have read the block histograms (the last one clears them)
     kMetaCount = 16
 };
 
@@ -111,6 +110,21 @@ struct zeda_moe {
 };
 
 namespace zeda {
+
+// Block histograms of the counting sort for a call of T tokens, as far as the top-K pass counts into them
+// (more blocks have a histogram kernel of their own): the router kernel of the call sets them to zero.
+constexpr int kFoldMaxBlocks = 256;
+inline int hist_ints(const zeda_moe *h, int T) {
+    const int nblk = (T + kSortTokens - 1) / kSortTokens;
+    return nblk <= kFoldMaxBlocks ? nblk * h->cfg.n_real : 0;
+}
+#if defined(__CUDACC__)
+// by all CTAs of a one- or two-dimensional grid
+__device__ __forceinline__ void clear_hist(int32_t *__restrict__ hist, int n) {
+    const int cta = blockIdx.y * gridDim.x + blockIdx.x;
+    for (int i = cta * blockDim.x + threadIdx.x; i < n; i += gridDim.x * gridDim.y * blockDim.x) hist[i] = 0;
+}
+#endif
 
 // ---- launchers (each returns the number of kernels it enqueued, or <0 on a launch error) ----
 int init_route_kernels(const zeda_moe *h);
