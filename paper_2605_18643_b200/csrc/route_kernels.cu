@@ -527,13 +527,13 @@ stats_final_kernel(const float *__restrict__ part, int nblk, int T, int K, int n
     {
         const int c = threadIdx.x % n_cand, s = threadIdx.x / n_cand;
         float2 a = make_float2(0.f, 0.f);
-        if (s < segs) {
-#pragma unroll 16
-            for (int b = s; b < nblk; b += segs) {
-                const float2 v = __ldcg(reinterpret_cast<const float2 *>(part + (size_t)b * cols) + c);
-                a.x += v.x;
-                a.y += v.y;
-            }
+        for (int b0 = s < segs ? s : nblk; b0 < nblk; b0 += 16 * segs) {
+            float2 v[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+                v[q] = b0 + q * segs < nblk ? __ldcg(reinterpret_cast<const float2 *>(part + (size_t)(b0 + q * segs) * cols) + c) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) { a.x += v[q].x; a.y += v[q].y; }
         }
         seg[threadIdx.x] = a;
     }
