@@ -466,15 +466,20 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
 // 192 candidates and the final pass, a chain of loads per candidate, 19 us.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kStatTokens = 64;
-constexpr int kStatWarps = 32;
+// Warps of a CTA by the logits per lane: sixteen logits a lane do not fit the 64 registers of a thread of 32 warps.
+// The CTA's probabilities, a row of candidates per warp, and its counts need no more shared memory than every launch may have.
+template <int RPL>
+constexpr int kStatWarps = RPL <= 8 ? 32 : 16;
+static_assert((kStatWarps<8> + 1) * 256 <= 12288 && (kStatWarps<16> + 1) * kMaxCand <= 12288, "no opt-in to more than 48 KB is made for the kernel");
 
 template <int RPL>
-__global__ void __launch_bounds__(32 * kStatWarps)
+__global__ void __launch_bounds__(32 * kStatWarps<RPL>)
 topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
                   int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist, float *__restrict__ part) {
     pdl_launch_dependents();
-    extern __shared__ float sm[];  // [kStatWarps][n_cand] probabilities, then [n_cand] counts
-    int32_t *cnt = reinterpret_cast<int32_t *>(sm + kStatWarps * n_cand);
+    constexpr int kWarps = kStatWarps<RPL>;
+    extern __shared__ float sm[];  // [kWarps][n_cand] probabilities, then [n_cand] counts
+    int32_t *cnt = reinterpret_cast<int32_t *>(sm + kWarps * n_cand);
     for (int i = threadIdx.x; i < n_cand; i += blockDim.x) cnt[i] = 0;
     __syncthreads();
     pdl_wait();
@@ -483,7 +488,7 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_re
     float acc[RPL];
 #pragma unroll
     for (int r = 0; r < RPL; ++r) acc[r] = 0.f;
-    for (int t = t0 + warp; t < t1; t += kStatWarps) {
+    for (int t = t0 + warp; t < t1; t += kWarps) {
         int my_idx;
         float my_w, v[RPL], m, den;
         topk_gate_token<RPL, 3>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
@@ -504,7 +509,7 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_re
     for (int j = threadIdx.x; j < n_cand; j += blockDim.x) {
         float p = 0.f;
 #pragma unroll 8
-        for (int w = 0; w < kStatWarps; ++w) p += sm[w * n_cand + j];
+        for (int w = 0; w < kWarps; ++w) p += sm[w * n_cand + j];
         part[(size_t)blockIdx.x * 2 * n_cand + j] = (float)cnt[j];
         part[(size_t)blockIdx.x * 2 * n_cand + n_cand + j] = p;
         // pass 1 of the counting sort, as in the top-K kernel above
@@ -665,8 +670,8 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
                   c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
 #define ZEDA_CALL_STATS(R) \
-    launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps), \
-                  sizeof(float) * (kStatWarps + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
+    launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
+                  sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
                   ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
         if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
         else ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);

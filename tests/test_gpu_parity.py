@@ -282,6 +282,25 @@ def test_routing_statistics(zeda):
     m.close()
 
 
+@pytest.mark.parametrize("T,E,Z,K", [(40, 300, 72, 16), (600, 300, 73, 16), (40, 384, 128, 16), (600, 384, 128, 16),
+                                     (33, 301, 72, 5), (33000, 8, 5, 2)])
+def test_routing_statistics_over_the_range_of_candidates(zeda, T, E, Z, K):
+    # up to the interface's 512 candidates (372 and 373: either side of 48 KB for 33 rows of n_cand floats), odd
+    # candidate counts (a pair of columns then straddles counts and probabilities), more than 256 sort blocks
+    wl = inputs.make_layer("stats", T=T, d=64 if T > 1000 else 256, He=64, E=E, Z=Z, K=K, seed=23, zero_fraction=0.4)
+    dev = torch.device("cuda:0")
+    m = zeda.from_workload(wl, dev)
+    x = wl.x.to(dev)
+    f, p, o = m.stats(x)
+    l, idx, *_ = oracle_route(wl)
+    s = oracle.stats(l, idx, E, Z, alpha=1.0, group_w=1.0)
+    assert np.allclose(f.cpu().numpy(), s["f"], rtol=1e-5, atol=1e-7)
+    assert np.allclose(p.cpu().numpy(), s["P"], rtol=1e-4, atol=1e-7)
+    assert np.isclose(float(o[0]), s["r_ze"], rtol=1e-5) and np.isclose(float(o[1]) * (E + Z) / K, s["L_A"], rtol=1e-4)
+    assert np.array_equal(m.token_zero_share(T).cpu().numpy(), oracle.token_zero_share(idx, E).astype(np.float32))
+    m.close()
+
+
 def test_per_token_zero_share(zeda):
     # the decode recipe spreads the per-token zero share over 0..100 %
     wl = inputs.decode()
