@@ -130,7 +130,7 @@ zeda_status_t check_call(zeda_moe_t *h, const void *in, int32_t T, const char *i
 int route_into(zeda_moe_t *h, const __nv_bfloat16 *x, const float *logits_in, int T, const RouteOut &out, cudaStream_t s,
                float *stat_part = nullptr) {
     int n = 0, n_parts = 1;
-    h->last_routed_tokens = T;
+    h->last_routed_tokens = 0;  // until every launch is in the stream, the handle holds no batch's routing
     const float *logits = logits_in;
     if (!logits) {
         int r = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts);
@@ -140,6 +140,7 @@ int route_into(zeda_moe_t *h, const __nv_bfloat16 *x, const float *logits_in, in
     }
     int r = launch_route_from_logits(h, logits, T, out, s, n_parts, stat_part);
     if (r < 0) return r;
+    h->last_routed_tokens = T;
     return n + r;
 }
 
@@ -150,7 +151,7 @@ zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_
     const bool prof = h->profiling;
     auto mark = [&](int i) { if (prof) cudaEventRecord(h->ev[i], s); };
     mark(0);
-    h->last_routed_tokens = T;
+    h->last_routed_tokens = 0;
     int n_parts = 1;
     int n = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts, split_T);
     if (n < 0) return cuda_fail("router launch", cudaGetLastError());
@@ -164,6 +165,7 @@ zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_
     if (stream_path(h, T)) {  // the down projection and the combine are one kernel: its time counts as GEMM2
         r = launch_stream_gemm1(h, x, T, s);
         if (r < 0) return cuda_fail("expert GEMM1 launch", cudaGetLastError());
+        h->last_routed_tokens = T;  // (this kernel may have been the one that routes)
         n += r;
         mark(3);
         r = launch_stream_down(h, x, T, y, resid, s);
@@ -177,6 +179,7 @@ zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_
         h->last_launches = n + r;
         return ZEDA_OK;
     }
+    h->last_routed_tokens = T;
     const ExpertWork work = {ws.counts, ws.offsets, ws.ptile_expert, ws.ptile_row0, ws.pair_token, T * h->cfg.top_k, tile_rows_for(h, T)};
     r = launch_experts_gemm1_pair(h, x, work, s);
     if (r < 0) return cuda_fail("expert GEMM1 launch", cudaGetLastError());

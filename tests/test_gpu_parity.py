@@ -318,6 +318,36 @@ def test_per_token_zero_share(zeda):
     m.close()
 
 
+def test_a_call_that_fails_leaves_no_routing_to_read(zeda):
+    # A launch into the legacy stream is refused by the runtime while another (blocking) stream is being captured:
+    # an error code on the host, nothing runs.  The handle must not pass off older ids as that call's routing.
+    import ctypes
+    wl = inputs.tiny(seed=9, T=64)
+    dev = torch.device("cuda:0")
+    m = zeda.from_workload(wl, dev)
+    x = wl.x.to(dev)
+    for T in (24, 8, 16):  # the routing pass; the expert kernels that route themselves; those that do not
+        m.route(x)
+        y = torch.empty_like(x[:T])
+        torch.cuda.synchronize()
+        cu, stream, graph = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_void_p()
+        assert cu.cuStreamCreate(ctypes.byref(stream), 0) == 0
+        assert cu.cuStreamBeginCapture_v2(stream, 2) == 0
+        st = zeda.lib.zeda_moe_forward(m._h, x.data_ptr(), T, y.data_ptr(), None)
+        text = zeda.last_error()
+        cu.cuStreamEndCapture(stream, ctypes.byref(graph))
+        assert cu.cuStreamDestroy_v2(stream) == 0
+        assert st == zeda.ERR_CUDA and "launch" in text
+        for n in (T, wl.T):
+            with pytest.raises(zeda.ZedaError) as e:
+                m.token_zero_share(n)
+            assert e.value.status == zeda.ERR_INVALID_ARG
+    m.route(x)
+    _, idx, *_ = oracle_route(wl)
+    assert np.array_equal(m.token_zero_share(wl.T).cpu().numpy(), oracle.token_zero_share(idx, wl.E).astype(np.float32))
+    m.close()
+
+
 def test_tensor_core_router_path(zeda):
     # T >= 256 sends the router GEMM to the tensor cores (three-way bf16 split of the fp32 rows)
     for T in (256, 1000):
