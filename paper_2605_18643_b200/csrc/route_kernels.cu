@@ -189,7 +189,7 @@ slot_hist_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real,
     const int s0 = blockIdx.x * kSortTokens * K;
     const int s1 = min(T * K, s0 + kSortTokens * K);
     for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-        const int e = topk_idx[s];
+        const int e = __ldcg(topk_idx + s);
         if ((unsigned)e < (unsigned)n_real) atomicAdd(&hist[e], 1);  // zero experts and ids < 0 are dropped
     }
     __syncthreads();
@@ -588,7 +588,13 @@ token_zero_share_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int 
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     int zero = 0;
-    for (int k = 0; k < K; ++k) zero += topk_idx[(size_t)t * K + k] >= n_real ? 1 : 0;
+    for (int k0 = 0; k0 < K; k0 += 8) {  // eight loads in flight
+        int e[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) e[u] = __ldcg(topk_idx + (size_t)t * K + min(k0 + u, K - 1));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) zero += k0 + u < K && e[u] >= n_real ? 1 : 0;
+    }
     out[t] = (float)zero / (float)K;
 }
 

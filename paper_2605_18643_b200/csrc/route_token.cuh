@@ -28,7 +28,8 @@ __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, i
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
         const int j = r * 32 + lane;
-        v[r] = (j < n_cand) ? row[j] : -INFINITY;
+        const float a = __ldcg(row + min(j, n_cand - 1));
+        v[r] = j < n_cand ? a : -INFINITY;
     }
     for (int p = 1; p < n_parts; p += PB) {
         float a[PB][RPL];
@@ -37,7 +38,7 @@ __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, i
 #pragma unroll
             for (int r = 0; r < RPL; ++r) {
                 const int j = r * 32 + lane;
-                a[q][r] = p + q < n_parts && j < n_cand ? row[(p + q) * part_stride + j] : 0.f;
+                a[q][r] = ldcg_if(p + q < n_parts && j < n_cand, row + (p + q) * part_stride + j, 0.f);
             }
 #pragma unroll
         for (int q = 0; q < PB; ++q)

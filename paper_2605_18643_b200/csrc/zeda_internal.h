@@ -191,16 +191,25 @@ void note_launch_error(cudaError_t e);
 // The kernels of one forward pass are launched back to back on one stream.  Launched with the
 // attribute below, a kernel may start (launch latency, barrier and TMEM set-up) while its
 // predecessor is still draining; it touches no global memory until pdl_wait() returns, which is
-// when the predecessor has completed and its writes are visible.  What a predecessor in the stream has
-// written is read by plain or ld.cg loads, not by __ldg: the compiler takes the latter to be invariant
-// while the kernel runs and may move it in front of the wait.  Each kernel calls
-// pdl_launch_dependents() first thing so that its successor is released as early as possible.
+// when the predecessor has completed and its writes are visible.  What a kernel in front has written is read
+// by volatile loads (__ldcg and those below), which the compiler keeps behind the wait.  It need not do that
+// for __ldg, nor for a plain load through a __restrict__ parameter (of const data it is the same non-coherent
+// load), and it did not: a placement pass met ids that were not written yet.
+// Each kernel calls pdl_launch_dependents() first thing so that its successor is released as early as possible.
+// The GEMM1 kernels do so behind their own wait: the routing results are complete when GEMM2 starts, which reads
+// them in front of its wait, past L1 (ld.cg), where an older line could be.
 // Without the attribute both calls do nothing.
 #if defined(__CUDACC__)
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// a load through L1 that stays behind the wait
+// *p, or `other` where `on` is false, as one predicated load
+__device__ __forceinline__ float ldcg_if(bool on, const float *p, float other) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.cg.f32 %0, [%1];\n\t}" : "+f"(other) : "l"(p), "r"((unsigned)on));
+    return other;
+}
+
+// a load through L1, behind the wait only: for lines that all threads of a CTA read
 __device__ __forceinline__ int32_t ld_ordered(const int32_t *p) {
     int32_t v;
     asm volatile("ld.global.ca.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");

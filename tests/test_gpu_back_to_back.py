@@ -1,0 +1,89 @@
+"""Calls in a row on one handle, on inputs that route differently and without a host synchronisation in between:
+each kernel is launched while the one in front still runs, and must read what that one writes and not what
+the call before has left in the same buffers.  (On a repeated input stale results are the right ones.)"""
+import pytest
+import torch
+
+from paper_2605_18643_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+SHAPE = dict(d=512, He=256, E=64, Z=32, K=8)
+
+
+class Call:
+    """One call with outputs of its own, made ahead so that nothing stands between the calls in the stream."""
+
+    def __init__(self, zeda, m, use, x):
+        lib, h, T, stream = zeda.lib, m._h, x.shape[0], torch.cuda.current_stream().cuda_stream
+        if use == "forward":
+            self.out = [torch.empty_like(x)]
+            self.run = lambda: m.forward(x, self.out[0])
+        elif use == "residual":
+            self.out = [x.flip(1).contiguous(), torch.empty_like(x)]
+            self.run = lambda: m.forward_residual(x, *self.out)
+        elif use == "stats":
+            n = m.E + m.Z
+            self.out = [torch.empty(k, device=x.device) for k in (n, n, 4, T)]
+
+            def run():
+                p = [t.data_ptr() for t in self.out]
+                assert lib.zeda_moe_stats(h, x.data_ptr(), T, p[0], p[1], p[2], stream) == zeda.OK
+                assert lib.zeda_moe_token_zero_share(h, T, p[3], stream) == zeda.OK
+            self.run = run
+        else:
+            o = m._route_outputs(T)
+            self.out = [o[k] for k in ("topk_idx", "topk_w", "counts", "offsets", "perm", "n_pairs")]
+            self.run = lambda: self._ok(lib.zeda_route(h, x.data_ptr(), T, *[t.data_ptr() for t in self.out], stream), zeda)
+
+    @staticmethod
+    def _ok(status, zeda):
+        assert status == zeda.OK
+
+    def same(self, other):
+        return all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(self.out, other.out))
+
+
+def check(zeda, m, plan):
+    """plan: list of (key, use, x).  Every call of the row gives the bits of a call of the same key on its own."""
+    alone, row = {}, []
+    for key, use, x in plan:
+        row.append((key, Call(zeda, m, use, x)))
+        if key not in alone:
+            alone[key] = Call(zeda, m, use, x)
+            torch.cuda.synchronize()
+            alone[key].run()
+            torch.cuda.synchronize()
+    for _, c in row:
+        c.run()
+    torch.cuda.synchronize()
+    for i, (key, c) in enumerate(row):
+        assert c.same(alone[key]), (i, key)
+    m.last_counters()  # no device-side failure recorded
+    return alone
+
+
+@pytest.fixture(scope="module")
+def layer():
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("back_to_back", T=2048, seed=41, zero_fraction=0.5, **SHAPE)
+    xs = [wl.x.to("cuda:0"), inputs.replica_tokens(wl, 7).to("cuda:0")]
+    return zeda, wl, xs
+
+
+@pytest.mark.parametrize("use", ["forward", "residual", "stats", "route"])
+@pytest.mark.parametrize("T", [1, 8, 16, 129, 300, 777, 2048])
+def test_alternating_inputs_give_the_bits_of_single_calls(layer, T, use):
+    zeda, wl, xs = layer
+    m = zeda.from_workload(wl, max_tokens=2048)
+    alone = check(zeda, m, [(i % 2, use, xs[i % 2][:T].contiguous()) for i in range(20)])
+    assert not alone[0].same(alone[1])
+    m.close()
+
+
+def test_batch_sizes_and_uses_in_any_order(layer):
+    zeda, wl, xs = layer
+    m = zeda.from_workload(wl, max_tokens=2048)
+    order = [(T, use) for T in (2048, 1, 300, 16, 1, 777, 8, 129, 40, 2048, 9, 160) for use in ("forward", "stats", "residual", "route")]
+    check(zeda, m, [((T, use, i % 2), use, xs[i % 2][:T].contiguous()) for i, (T, use) in enumerate(order)])
+    m.close()

@@ -57,3 +57,34 @@ def test_small_batches_match_the_oracle(T, shape, kind):
     share = (idx >= wl.E).mean(axis=1).astype(np.float32)
     assert np.array_equal(m.token_zero_share(T).cpu().numpy(), share)
     m.close()
+
+
+@pytest.mark.parametrize("T", [1, 8, 16])
+def test_small_batches_in_a_graph_and_without_dependent_launch(T):
+    # the expert kernels here read the routing results in front of their wait for the kernel before them
+    from paper_2605_18643_b200 import zeda
+    wl = layer(T)
+    dev = torch.device("cuda:0")
+    xs = [wl.x.to(dev), inputs.replica_tokens(wl, 3).to(dev)]
+    plain = zeda.from_workload(wl, dev, flags=zeda.FLAG_NO_DEPENDENT_LAUNCH)
+    want = [plain.forward(x).view(torch.int16) for x in xs]
+    torch.cuda.synchronize()
+    m = zeda.from_workload(wl, dev)
+    for x, w in zip(xs, want):
+        assert torch.equal(m.forward(x).view(torch.int16), w)
+    x, y, y2 = xs[0].clone(), torch.empty_like(xs[0]), torch.empty_like(xs[0])
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):  # two calls: the second starts under the first
+        m.forward(x, y)
+        m.forward(y, y2)
+    for src in (1, 0, 1):
+        x.copy_(xs[src])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y.view(torch.int16), want[src])
+        assert torch.equal(y2.view(torch.int16), plain.forward(y.clone()).view(torch.int16))
+    del graph
+    m.close()
+    plain.close()
