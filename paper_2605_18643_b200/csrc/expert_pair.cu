@@ -73,15 +73,21 @@ struct StageBytes {
     static constexpr int value = kSingle > kDouble ? kSingle : kDouble;
 };
 
+// The routing results: GEMM1 reads them behind its wait (through L1: the items of a tile read the same lines),
+// GEMM2 in front of it.
+template <int MODE>
+__device__ __forceinline__ int32_t ld_route(const int32_t *p) { return MODE == 1 ? ld_ordered(p) : __ldcg(p); }
+
+template <int MODE>
 __device__ __forceinline__ Item load_item(long long item, int m_blocks, int tile_rows, const int32_t *tile_expert,
                                           const int32_t *tile_row0, const int32_t *counts, const int32_t *offsets) {
     Item it;
     const int tile = (int)(item / m_blocks);
     it.mb = (int)(item % m_blocks);
-    it.e = tile_expert[tile];
-    const int r0 = tile_row0[tile];
-    it.n = min(tile_rows, counts[it.e] - r0);
-    it.pos0 = offsets[it.e] + r0;
+    it.e = ld_route<MODE>(tile_expert + tile);
+    const int r0 = ld_route<MODE>(tile_row0 + tile);
+    it.n = min(tile_rows, ld_route<MODE>(counts + it.e) - r0);
+    it.pos0 = ld_route<MODE>(offsets + it.e) + r0;
     return it;
 }
 
@@ -407,7 +413,7 @@ expert_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
     } else if (warp == (MODE == 1 ? 3 : 2)) {
         // ------------------------------------------------------------------ item scheduler (leader CTA)
         if (leader) {
-            const long long n_items = (long long)meta[kMetaPairTiles] * m_blocks;
+            const long long n_items = (long long)__ldcg(meta + kMetaPairTiles) * m_blocks;
             int32_t *counter = meta + (MODE == 1 ? kMetaNextItem1 : kMetaNextItem2);
             const uint32_t peer_queue = mapa(smem_u32(s_items), 1);
             const volatile int *prod_seq = &s_prod_seq;
@@ -431,7 +437,7 @@ expert_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
                         const long long item = atomicAdd(counter, 1);
                         end = item >= n_items;
                         if (end) break;
-                        it = load_item(item, m_blocks, tile_rows, tile_expert, tile_row0, counts, offsets);
+                        it = load_item<MODE>(item, m_blocks, tile_rows, tile_expert, tile_row0, counts, offsets);
                         // the odd block of a narrow tile belongs to the double item of the block before it
                         if (!(DBL_ROWS > 0 && it.n <= DBL_ROWS && (it.mb & 1))) break;
                     }
@@ -470,8 +476,8 @@ expert_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             for (int i = 0; i < HALF_MAX / 16; ++i) {
                 const int rb = brow0 + rsub + 16 * i;
                 // padding rows read token 0: their columns are never stored
-                const int tok = (rsub + 16 * i < half && rb < it.n) ? pair_token[it.pos0 + rb] : 0;
-                src[i] = x + (size_t)tok * x_ld + chunk * 8;
+                const int tok = ld_route<MODE>(pair_token + it.pos0 + min(rb, it.n - 1));
+                src[i] = x + (size_t)(rsub + 16 * i < half && rb < it.n ? tok : 0) * x_ld + chunk * 8;
             }
             for (int ks = 0; ks < k_steps; ++ks, ++it_count) {
                 const uint32_t s = it_count % STAGES, ph = (it_count / STAGES) & 1u;
@@ -547,11 +553,11 @@ expert_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             } else {
                 const int row0 = 256 * mb + 128 * (int)rank + 32 * q;  // first of this warp's 32 output features
                 const bool r_ok = row0 < out_rows;
-                int target = SCATTER && lane < it.n ? pair_token[it.pos0 + lane] : 0;  // of row c0 + lane
+                int target = SCATTER ? __ldcg(pair_token + it.pos0 + min(lane, it.n - 1)) : 0;  // of row c0 + lane
                 for (int c0 = 0; c0 < it.n; c0 += 32) {
                     float v[32];
                     const int target_now = target;
-                    if (SCATTER) target = c0 + 32 + lane < it.n ? pair_token[it.pos0 + c0 + 32 + lane] : 0;
+                    if (SCATTER) target = __ldcg(pair_token + it.pos0 + min(c0 + 32 + lane, it.n - 1));
                     tmem_ld32(t0 + c0, v);
                     if (last_sub && c0 + 32 >= it.n) {
                         tc_fence_before();
