@@ -27,11 +27,11 @@ ep_pack_kernel(__nv_bfloat16 *__restrict__ dst, const __nv_bfloat16 *__restrict_
     pdl_wait();
     if (blockIdx.x == 0) {
         for (int r = threadIdx.x; r < n_ranks; r += blockDim.x)
-            send_counts[r] = offsets[(r + 1) * n_local] - offsets[r * n_local];
+            send_counts[r] = __ldcg(offsets + (r + 1) * n_local) - __ldcg(offsets + r * n_local);
         if (expert_counts)
-            for (int e = threadIdx.x; e < n_ranks * n_local; e += blockDim.x) expert_counts[e] = counts[e];
+            for (int e = threadIdx.x; e < n_ranks * n_local; e += blockDim.x) expert_counts[e] = __ldcg(counts + e);
     }
-    const int n_rows = min(max_rows, *n_rows_dev);
+    const int n_rows = min(max_rows, __ldcg(n_rows_dev));
     const int chunks = d / 8;
     const int rows_per_cta = blockDim.x / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -87,3 +87,33 @@ def test_batch_sizes_and_uses_in_any_order(layer):
     order = [(T, use) for T in (2048, 1, 300, 16, 1, 777, 8, 129, 40, 2048, 9, 160) for use in ("forward", "stats", "residual", "route")]
     check(zeda, m, [((T, use, i % 2), use, xs[i % 2][:T].contiguous()) for i, (T, use) in enumerate(order)])
     m.close()
+
+
+@pytest.mark.parametrize("T", [40, 300, 2048])
+def test_expert_parallel_calls_in_a_row(layer, T):
+    zeda, wl, xs = layer
+    dev = torch.device("cuda:0")
+    m = zeda.ZedaMoE(wl.router_w.to(dev), wl.router_bias.to(dev), wl.w_gate_up.to(dev), wl.w_down.to(dev), wl.E, wl.Z, wl.K, T,
+                     ep_size=1, max_recv_pairs=T * wl.K)
+    xs = [x[:T].contiguous() for x in xs]
+
+    def run(x, n_rows):
+        send_rows, send_counts, counts = m.ep_dispatch(x)
+        if n_rows is None:
+            n_rows = int(send_counts.sum())
+        rows = m.ep_experts(send_rows, counts.view(1, -1), n_rows)
+        return n_rows, [send_rows, send_counts, counts, m.ep_combine(x, rows)]
+
+    alone = []
+    for x in xs:
+        alone.append(run(x, None))
+        torch.cuda.synchronize()
+    got = [run(xs[i % 2], alone[i % 2][0]) for i in range(20)]
+    torch.cuda.synchronize()
+    for i, (P, out) in enumerate(got):
+        want = alone[i % 2][1]
+        assert torch.equal(out[0][:P].view(torch.int16), want[0][:P].view(torch.int16)), i
+        assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(out[1:], want[1:])), i
+    assert not torch.equal(alone[0][1][3], alone[1][1][3])
+    m.last_counters()
+    m.close()
