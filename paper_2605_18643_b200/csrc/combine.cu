@@ -119,7 +119,7 @@ combine_glue_kernel(const __nv_bfloat16 *__restrict__ obuf, const int32_t *__res
     const int t = blockIdx.x, c = threadIdx.x, lane = threadIdx.x & 31;
     const bool in = c < d / 8;
     uint4 *rp = reinterpret_cast<uint4 *>(resid + (size_t)t * d) + c;
-    const uint4 rv = in ? *rp : make_uint4(0u, 0u, 0u, 0u);
+    const uint4 rv = in ? __ldcg(rp) : make_uint4(0u, 0u, 0u, 0u);
     const int my_pos = lane < K ? __ldcg(inv + (size_t)t * K + lane) : -1;
     const float my_w = lane < K ? __ldcg(topk_w + (size_t)t * K + lane) : 0.f;
     const unsigned real = __ballot_sync(0xffffffffu, my_pos >= 0);

@@ -39,6 +39,10 @@ __device__ __forceinline__ uint4 ld_weights(const __nv_bfloat16 *p) {
 // activations come from the kernel before: straight from L2
 __device__ __forceinline__ uint4 ld_rows(const __nv_bfloat16 *p) { return __ldcg(reinterpret_cast<const uint4 *>(p)); }
 
+__device__ __forceinline__ float ld_value(const __nv_bfloat16 *p) {
+    return __uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short *>(p)) << 16);
+}
+
 constexpr uint4 kZero4 = {0u, 0u, 0u, 0u};
 static_assert(kStreamTokens <= 16, "the kernels are instantiated for up to two column tiles of 8 pair rows");
 
@@ -382,9 +386,9 @@ stream_down_combine_kernel(const __nv_bfloat16 *__restrict__ hmid, const __nv_bf
             for (int q = 0; q < kDownSlices; ++q) o += part[((size_t)q * slots + pos) * kDownStride + f];
             sum = fmaf(wk, __bfloat162float(__float2bfloat16_rn(o)), sum);
         }
-        if (copy_experts && zero_mass != 0.f) sum = fmaf(zero_mass, __bfloat162float(x[at]), sum);
+        if (copy_experts && zero_mass != 0.f) sum = fmaf(zero_mass, ld_value(x + at), sum);
         const __nv_bfloat16 out = __float2bfloat16_rn(sum);
-        if (resid) resid[at] = __float2bfloat16_rn(__bfloat162float(resid[at]) + __bfloat162float(out));
+        if (resid) resid[at] = __float2bfloat16_rn(ld_value(resid + at) + __bfloat162float(out));
         else y[at] = out;
     }
 }

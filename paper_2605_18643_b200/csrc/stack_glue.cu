@@ -27,7 +27,7 @@ residual_rmsnorm_kernel(__nv_bfloat16 *__restrict__ r, const __nv_bfloat16 *__re
     for (int i = 0; i < kGlueChunks; ++i) {
         const int c = threadIdx.x + i * kGlueThreads;
         if (c < chunks) {
-            const uint4 a = *reinterpret_cast<const uint4 *>(r + row + 8 * c);
+            const uint4 a = __ldcg(reinterpret_cast<const uint4 *>(r + row + 8 * c));
             const uint32_t au[4] = {a.x, a.y, a.z, a.w};
             uint32_t bu[4] = {0, 0, 0, 0};
             if (y) {
