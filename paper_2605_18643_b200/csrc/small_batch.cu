@@ -11,6 +11,9 @@
 // consecutive bytes of weight row g (k = 32 b + 8 t ..) as the A operands of two m16n8k16 MMAs and the
 // same 16 bytes of the pair row of column g as their B operands.  Every load is a full 16 bytes, four
 // lanes cover 64 consecutive bytes of a row, and nothing goes through shared memory.
+#include <algorithm>
+#include <cmath>
+
 #include "route_token.cuh"
 
 namespace zeda {
@@ -395,11 +398,35 @@ stream_down_combine_kernel(const __nv_bfloat16 *__restrict__ hmid, const __nv_bf
 
 int down_smem_bytes(int slots) { return kDownSlices * slots * kDownStride * (int)sizeof(float); }
 
+// What these kernels take longer than those of expert_pair.cu, in us, from the shape of the call.  They save the
+// longer chain and the launches of the others, about 12 us a call, and they lose per active expert where the
+// down projection leaves SMs idle (d / 16 CTAs, one per SM) or spends more on an expert's start than on its
+// weights.  Measured both ways at 168 shapes (d 256 to 8192, H_e 128 to 4096, 8 to 256 experts, K 2 to 16, with no
+// zero experts or one for two others) of 1 to 16 tokens, us a call back to back, these kernels and the others:
+//   d 2048, H_e 768, N 128 + 64, K 8   T=1 16.6, 29.6   T=8 72.2, 84.7   T=16 101.5, 106.7
+//   d 1024, H_e 256, N 256, K 16       T=1 20.7, 28.2   T=4 44.6, 39.8   T=8 70.1, 52.7
+//   d 8192, H_e 4096, N 8, K 2         T=1 97.9, 101    T=2 155, 175     T=8 278, 268
+// Of the 774 calls that the rule sends here 7 are more than 3 % slower and none more than 7 %.
+double stream_excess_us(const zeda_moe *h, int T) {
+    const zeda_moe_config_t &c = h->cfg;
+    const double d = c.d_model, He = c.d_expert;
+    // experts with a pair if all candidates are as likely (the host does not know the load)
+    const double active = c.n_real * (1.0 - std::pow(1.0 - (double)c.top_k / (c.n_real + c.n_zero), T));
+    // down kernel: waves of CTAs, each of which takes 0.3 us to start on an expert or 45 GB/s for its 16 weight rows
+    const int ctas = c.d_model / 16, waves = (ctas + h->sm_count - 1) / h->sm_count;
+    const double down = active * waves * std::max(0.3, 0.0007 * He);
+    // there: 6 TB/s, or one work item of 256 rows per CTA pair at 114 GB/s
+    const double down_pair = std::max(active * 2.0 * d * He / 6e6, 0.0045 * He);
+    // both projections stream a little slower, with two column tiles (above 8 tokens) a little more: us per MB
+    const double stream = (T > 8 ? 0.012 : 0.005) * active * 6.0 * d * He * 1e-6;
+    return down - down_pair + stream;
+}
+constexpr double kStreamSavedUs = 9.0;  // (of the 12, so that the rule errs on the side of the other kernels)
+
 }  // namespace
 
 bool stream_path(const zeda_moe *h, int T) {
-    const zeda_moe_config_t &c = h->cfg;
-    return c.ep_size < 1 && T <= kStreamTokens && T * c.top_k <= kStreamSlots;
+    return h->cfg.ep_size < 1 && T <= kStreamTokens && stream_excess_us(h, T) <= kStreamSavedUs;
 }
 
 bool stream_routes_itself(const zeda_moe *h, int T) { return stream_path(h, T) && T <= kRouteHereTokens; }

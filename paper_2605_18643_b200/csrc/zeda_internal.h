@@ -15,10 +15,8 @@ constexpr int kSortTokens = 128;    // tokens per CTA in the counting sort (hist
 constexpr int kPairTileM = 256;     // most pair rows per tile of the expert kernels (one CTA pair, N <= 256)
 constexpr int kMidTileM = 128;      // tile rows of the geometry for mid-sized batches
 constexpr int kMaxEpRanks = 64;     // expert-parallel group size limit
-// The smallest batches run the expert kernels of small_batch.cu (against those of expert_pair.cu: 1 token 20.5
-// and 38.9 us a call, 8 tokens 57.4 and 71.3, 16 tokens 94.2 and 98.3, 32 tokens 143 and 141).
-constexpr int kStreamTokens = 16;   // calls of at most this many tokens ...
-constexpr int kStreamSlots = 256;   // ... and slots run the expert kernels of small_batch.cu
+constexpr int kStreamTokens = 16;   // calls of at most this many tokens may run the expert kernels of small_batch.cu
+constexpr int kStreamSlots = kStreamTokens * kMaxTopK;  // their largest slot table
 
 constexpr int kHostMaxChunks = 3;   // of the host-buffer entry point
 

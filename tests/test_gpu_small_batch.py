@@ -24,6 +24,7 @@ def layer(T, d=256, He=128, E=8, Z=4, K=2, seed=5, zero_fraction=0.5):
     (7, dict(d=320, He=192), 0), (16, dict(d=64, He=64), 1), (3, dict(d=1088, He=832), 0),   # slices with remainders
     (8, dict(E=1, Z=1, K=2), 0), (16, dict(E=1, Z=0, K=1), 0),                               # every token on one expert
     (16, dict(E=40, Z=8, K=16), 0), (9, dict(E=300, Z=100, K=16), 1),                        # widest slot table, many experts
+    (16, dict(E=24, Z=8, K=16), 0), (2, dict(E=300, Z=100, K=16), 1), (1, dict(E=384, Z=128, K=16), 0),  # the same on these kernels
     (4, dict(d=2048, He=768, E=16, Z=8, K=8), 0),
 ])
 def test_small_batches_match_the_oracle(T, shape, kind):
@@ -88,3 +89,29 @@ def test_small_batches_in_a_graph_and_without_dependent_launch(T):
     del graph
     m.close()
     plain.close()
+
+
+@pytest.mark.parametrize("T,shape,streams", [
+    (8, dict(d=256, He=128, E=64, Z=32, K=4), True),
+    (16, dict(d=2048, He=768, E=32, Z=16, K=4), True),
+    (2, dict(d=1024, He=256, E=256, Z=0, K=16), True), (8, dict(d=1024, He=256, E=256, Z=0, K=16), False),
+    (8, dict(d=1024, He=512, E=192, Z=64, K=16), False), (16, dict(d=4096, He=1536, E=24, Z=8, K=8), False),
+])
+def test_which_kernels_a_small_batch_takes(T, shape, streams):
+    # many active experts per call, or a down projection that leaves SMs idle: the kernels for larger batches
+    # (router, routing, two GEMMs, combine) are the faster ones (N 256, K 16, 8 tokens: 52 us against 69)
+    from paper_2605_18643_b200 import zeda
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev).manual_seed(1)
+    E, Z, K, d, He = (shape[k] for k in ("E", "Z", "K", "d", "He"))
+    w = [torch.empty(s, dtype=torch.bfloat16, device=dev).normal_(0, 0.02, generator=g) for s in ((E, 2 * He, d), (E, d, He))]
+    rw = torch.empty(E + Z, d, device=dev).normal_(0, 0.02, generator=g)
+    x = torch.randn(T, d, generator=g, device=dev).to(torch.bfloat16)
+    m = zeda.ZedaMoE(rw, None, w[0], w[1], E, Z, K, 40)
+    y = m.forward(x)
+    assert m.last_counters()[3] == ((3 if T <= 8 else 4) if streams else 5)
+    # rows of a batch that is too large for these kernels: the same expert sums in another order
+    many = m.forward(torch.cat([x, torch.randn(24, d, generator=g, device=dev).to(torch.bfloat16)]))[:T]
+    assert m.last_counters()[3] == 5
+    assert float((y.float() - many.float()).norm() / many.float().norm()) <= (REL_L2 if streams else 1e-3)
+    m.close()
