@@ -91,8 +91,10 @@ router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restric
 // 192 SM-wide bursts instead of 24; the reduction axis is split over four warps.  NT tokens per CTA, all
 // of their loads in flight at once.  The row is asked into L2 before the wait for the kernel in front (a
 // prefetch only: its values are read after the wait).
-constexpr int kTileRouterTokens = 160;  // from here on the tensor-core router (128 tokens: 11 us on the CUDA cores, 193: 15; the tensor-core kernel
-                                      // takes 11 and leaves the top-K pass more slices to add)
+// From kTileRouterTokens on the tensor-core router.  Its accumulators are fp32 too, but against 64 bits its logits
+// are off by 2.1e-6 of their root mean square at d 2048 (1.0e-6 at 1024, 9e-6 at 8192), these kernels' by 1.6e-7:
+// below, where they take 15 us at 193 tokens and 20 at 255 against 11 and more slices to add, they are kept.
+constexpr int kTileRouterTokens = 256;
 constexpr int kFewTokens = 32;  // calls of at most this many tokens
 constexpr int kFewThreads = 128;
 constexpr int kFewUnroll = 4;

@@ -359,12 +359,37 @@ def test_tensor_core_router_path(zeda):
                                      (700, 3, 2, 1), (1153, 512, 0, 3)])
 def test_routing_at_the_edges_of_its_kernels(zeda, T, E, Z, K):
     # sort blocks of 128 tokens with one token over, expert counts that are no multiple of 4 or above the
-    # threads of the placement pass, the switch between the two routers at 160 tokens
+    # threads of the placement pass
     wl = inputs.make_layer("edges", T=T, d=192, He=64, E=E, Z=Z, K=K, seed=21, zero_fraction=0.4 if Z else None)
     m = zeda.from_workload(wl)
     l, idx, w, counts, offsets, perm, P = oracle_route(wl)
     for _ in range(2):  # the second call finds the histograms that the first has cleared
         check_route(m.route(wl.x.to("cuda:0")), idx, w, counts, offsets, perm, P)
+    m.close()
+
+
+@pytest.mark.parametrize("T,d", [(33, 192), (128, 2048), (160, 2048), (193, 8192), (255, 2048), (255, 1088)])
+def test_router_logits_below_the_tensor_core_router_are_fp32_sums(zeda, T, d):
+    # Up to 255 tokens: fp32 FMAs, 32 partial sums a logit.  Bound: each is a chain of d / 32 FMAs and five
+    # additions follow, every one of relative error 2^-24 on a sum of at most the logit's sum of magnitudes; as
+    # the errors' signs are random, their square root counts (four times that here).  Tensor-core accumulators are
+    # off by more than ten times as much.
+    wl = inputs.make_layer("fp32_router", T=T, d=d, He=64, E=40, Z=24, K=4, seed=24)
+    m = zeda.from_workload(wl)
+    x = wl.x.to("cuda:0")
+    got = m.router_logits(x).double().cpu()
+    w, xd = wl.router_w.double(), wl.x.double()
+    want = xd @ w.t() + (0.0 if wl.router_bias is None else wl.router_bias.double())
+    size = torch.sqrt(xd.pow(2) @ w.t().pow(2))  # root of the summed squares: the size of a random-sign partial sum
+    err = (got - want).abs() / size
+    assert float(err.max()) <= 4 * 2.0 ** -24 * (d / 32 + 5) ** 0.5
+    n = min(T, 128)  # a token's logits do not depend on the batch
+    assert torch.equal(m.router_logits(x)[:n], m.router_logits(x[:n].contiguous()))
+    o = m.route(x)
+    p = torch.softmax(want, 1)
+    w_ref = p.gather(1, o["topk_idx"].long().cpu())
+    w_ref /= w_ref.sum(1, keepdim=True)
+    assert float(((o["topk_w"].double().cpu() - w_ref) / w_ref).abs().max()) <= 4e-6
     m.close()
 
 
