@@ -12,7 +12,6 @@ struct ScanShared {
     int32_t cnt[kMaxCand];
     int32_t off[kMaxCand + 1];
     int32_t ptile[kMaxCand + 1];  // exclusive scan of the experts' tile counts
-    int4 chunk[kMaxCand / 32];    // per 32 experts: pairs, tiles, active experts, most pairs of one expert
 };
 
 // From per-expert pair counts in sh.cnt: exclusive offsets, P, U, and the tile list of the expert
@@ -24,53 +23,51 @@ __device__ __forceinline__ void finish_expert_scan(ScanShared &sh, int n_real, i
                                                    int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                                                    const WorkLists &wl, bool write_global = true,
                                                    int list_part = 0, int list_parts = 1, int tile_rows = kPairTileM) {
-    // every warp scans chunks of 32 experts with shuffle prefix sums (a single warp walking all chunks is a
-    // chain of 4 x 17 dependent shuffles for 128 experts); the chunk totals are then added up by every thread
-    const int lane = threadIdx.x & 31, n_chunks = (n_real + 31) / 32;
-    for (int ch = threadIdx.x >> 5; ch < n_chunks; ch += blockDim.x >> 5) {
-        const int i = 32 * ch + lane;
-        const int c = (i < n_real) ? sh.cnt[i] : 0;
-        const int pt = (c + tile_rows - 1) / tile_rows;
-        int so = c, sp = pt;
+    static_assert((kPairTileM & (kPairTileM - 1)) == 0 && (kMidTileM & (kMidTileM - 1)) == 0, "tile heights are powers of two");
+    const int tile_shift = 31 - __clz(tile_rows);
+    // One warp, each lane a run of consecutive experts: one shuffle prefix sum whatever n_real is.  (All warps over
+    // chunks of 32 experts and their totals behind one more barrier: 0.3 us longer up to 64 experts.)
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x, run = (n_real + 31) / 32, e0 = min(n_real, lane * run), e1 = min(n_real, e0 + run);
+        int pairs = 0, tiles = 0, active = 0, max_rows = 0;
+#pragma unroll 4
+        for (int e = e0; e < e1; ++e) {
+            const int c = sh.cnt[e];
+            pairs += c;
+            tiles += (c + tile_rows - 1) >> tile_shift;
+            active += c > 0 ? 1 : 0;
+            max_rows = max(max_rows, c);
+        }
+        int so = pairs, sp = tiles;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int a = __shfl_up_sync(kFull, so, o);
             const int q = __shfl_up_sync(kFull, sp, o);
             if (lane >= o) { so += a; sp += q; }
         }
-        const int active = __popc(__ballot_sync(kFull, c > 0)), mx = __reduce_max_sync(kFull, c);
-        if (i < n_real) {
-            sh.off[i] = so - c;
-            sh.ptile[i] = sp - pt;
+        int off = so - pairs, first = sp - tiles;
+#pragma unroll 4
+        for (int e = e0; e < e1; ++e) {
+            const int c = sh.cnt[e];
+            sh.off[e] = off;
+            sh.ptile[e] = first;
+            off += c;
+            first += (c + tile_rows - 1) >> tile_shift;
         }
-        if (lane == 31) sh.chunk[ch] = make_int4(so, sp, active, mx);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i <= n_real; i += blockDim.x) {  // entry n_real: the totals
-        int off = 0, tiles = 0, active = 0, max_rows = 0;
-        const int before = i < n_real ? i >> 5 : n_chunks;
-        for (int ch = 0; ch < before; ++ch) {
-            const int4 v = sh.chunk[ch];
-            off += v.x;
-            tiles += v.y;
-            active += v.z;
-            max_rows = max(max_rows, v.w);
-        }
-        if (i < n_real) {
-            sh.off[i] += off;
-            sh.ptile[i] += tiles;
-        } else {
-            sh.off[n_real] = off;
-            sh.ptile[n_real] = tiles;
+        active = __reduce_add_sync(kFull, active);
+        max_rows = __reduce_max_sync(kFull, max_rows);
+        if (lane == 31) {
+            sh.off[n_real] = so;
+            sh.ptile[n_real] = sp;
             if (write_global) {
-                meta[kMetaPairs] = off;
+                meta[kMetaPairs] = so;
                 meta[kMetaActive] = active;
-                meta[kMetaZeroSlots] = total_slots - off;
-                meta[kMetaPairTiles] = tiles;
+                meta[kMetaZeroSlots] = total_slots - so;
+                meta[kMetaPairTiles] = sp;
                 meta[kMetaMaxRows] = max_rows;
                 meta[kMetaNextItem1] = 0;
                 meta[kMetaNextItem2] = 0;
-                if (n_pairs_out) *n_pairs_out = off;
+                if (n_pairs_out) *n_pairs_out = so;
             }
         }
     }
