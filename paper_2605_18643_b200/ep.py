@@ -37,11 +37,12 @@ def send_counts_from_offsets(offsets: torch.Tensor, n_real: int, ep_size: int) -
     return [int(o[(r + 1) * n_local] - o[r * n_local]) for r in range(ep_size)]
 
 
-def recv_layout(recv_counts: torch.Tensor):
-    """From recv_counts [G, n_local] (rows from source s for local expert j): rows per source and the
-    total.  The received buffer holds source 0's block, then source 1's, ...; each block is in its
-    sender's (expert, token) order."""
-    per_source = [int(v) for v in recv_counts.sum(dim=1).tolist()]
+def recv_layout(recv_counts):
+    """From recv_counts [G, n_local] (rows from source s for local expert j; a tensor or nested lists): rows
+    per source and the total.  The received buffer holds source 0's block, then source 1's, ...; each block is
+    in its sender's (expert, token) order."""
+    rows = recv_counts.tolist() if isinstance(recv_counts, torch.Tensor) else recv_counts
+    per_source = [sum(row) for row in rows]
     return per_source, sum(per_source)
 
 
@@ -110,8 +111,7 @@ class ExpertParallelMoE:
         counts = torch.cat((send_counts, recv_counts.reshape(-1))).tolist()
         send_splits = counts[:self.G]
         n_local = recv_counts.numel() // self.G
-        recv_splits = [sum(counts[self.G + s * n_local:self.G + (s + 1) * n_local]) for s in range(self.G)]  # (recv_layout on host values)
-        n_rows = sum(recv_splits)
+        recv_splits, n_rows = recv_layout([counts[i:i + n_local] for i in range(self.G, len(counts), n_local)])
         if n_rows > m.cfg.max_recv_pairs:
             raise RuntimeError("rank receives %d pair rows, handle was sized for %d" % (n_rows, m.cfg.max_recv_pairs))
         recv_rows = self.x.rows(send_rows, send_splits, recv_splits)

@@ -105,6 +105,73 @@ def test_two_gloo_ranks_dispatch_compute_and_return():
             assert res[a]["send"][b] == res[b]["recv_splits"][a]
 
 
+FORWARD_WORKER = r'''
+import json, os, sys
+sys.path.insert(0, %(root)r)
+import numpy as np
+import torch
+import torch.distributed as dist
+import oracle
+from paper_2605_18643_b200 import ep, inputs
+
+rank = int(os.environ["RANK"]); G = int(os.environ["WORLD_SIZE"])
+dist.init_process_group(backend="gloo")
+layer = inputs.tiny(seed=22, T=60, E=8, Z=4, K=3)
+x = inputs.replica_tokens(layer, 5 + rank)[:60 - 23 * rank].contiguous()
+E, Z, K, d = layer.E, layer.Z, layer.K, layer.d
+n_local, T = E // G, x.shape[0]
+wgu, wd = inputs.bits(layer.w_gate_up), inputs.bits(layer.w_down)
+y_ref, idx, w = oracle.forward(inputs.bits(x), layer.router_w.numpy(), layer.router_bias.numpy(), wgu, wd, E, Z, K)
+counts, offsets, perm, P = oracle.compact(idx, E)
+
+
+class Moe:
+    """The three device phases of a rank in the oracle's arithmetic; forward does the rest."""
+    class cfg:
+        ep_size, max_recv_pairs = G, 10 ** 6
+
+    def ep_dispatch(self, xs):
+        rows = torch.full((T * K, d), float("nan"), dtype=torch.bfloat16)  # behind the pairs: not to be sent
+        rows[:P] = xs[torch.from_numpy(perm // K).long()]
+        send = torch.tensor(ep.send_counts_from_offsets(torch.from_numpy(offsets), E, G), dtype=torch.int32)
+        return rows, send, torch.from_numpy(counts.astype(np.int32))
+
+    def ep_experts(self, rows, recv_counts, n_rows):
+        assert rows.shape[0] >= n_rows == int(recv_counts.sum()) and recv_counts.shape == (G, n_local)
+        out, row = torch.empty((max(n_rows, 1), d), dtype=torch.float64), 0
+        for s in range(G):
+            for j in range(n_local):
+                for _ in range(int(recv_counts[s, j])):
+                    e = rank * n_local + j
+                    out[row] = torch.from_numpy(oracle.expert(inputs.bits(rows[row:row + 1])[0], wgu[e], wd[e]))
+                    row += 1
+        return out
+
+    def ep_combine(self, xs, back, out):
+        y = np.zeros((T, d))
+        for p in range(P):
+            y[perm[p] // K] += w[perm[p] // K, perm[p] %% K] * back[p].numpy()
+        return y
+
+
+y = ep.ExpertParallelMoE(Moe(), ep.TorchDistExchange()).forward(x)
+dist.barrier()
+print(json.dumps({"err": float(np.max(np.abs(y - y_ref))), "P": int(P), "size": float(np.max(np.abs(y_ref)))}))
+dist.destroy_process_group()
+'''
+
+
+def test_two_gloo_ranks_run_the_forward():
+    port = 35600 + os.getpid() % 2000
+    procs = [subprocess.Popen([sys.executable, "-c", FORWARD_WORKER % {"root": ROOT}], env=_env(r, 2, port),
+                              stdout=subprocess.PIPE, stderr=subprocess.PIPE, text=True) for r in range(2)]
+    outs = [p.communicate(timeout=600) for p in procs]
+    assert all(p.returncode == 0 for p in procs), outs
+    for o in outs:
+        r = json.loads(o[0].strip().splitlines()[-1])
+        assert r["P"] > 0 and r["size"] > 0 and r["err"] < 1e-12  # same fp64 arithmetic, other order only
+
+
 def test_plan_functions_on_small_cases():
     import torch
     sys.path.insert(0, ROOT)
