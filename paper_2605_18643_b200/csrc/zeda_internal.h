@@ -45,7 +45,7 @@ struct Workspace {
     int32_t *meta;         // [kMetaCount]
     int32_t *ptile_expert; // [maxTiles] tiles of at most kPairTileM pair rows of one expert
     int32_t *ptile_row0;   // [maxTiles] first row of the tile within its expert
-    float *logits;         // [maxT*(N+N_Z)]
+    float *logits;         // [router_part_rows(maxT)*(N+N_Z)]: complete logits or up to eight slices of them
     float *stat_part;      // [nblk_stats * 2 * (N+N_Z)]
     __nv_bfloat16 *hmid;   // [maxT*K, He]
     __nv_bfloat16 *obuf;   // [maxT*K, d] (not on expert-parallel handles: their results go to the caller's buffer)

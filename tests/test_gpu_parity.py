@@ -363,7 +363,7 @@ def test_routing_at_the_edges_of_its_kernels(zeda, T, E, Z, K):
     wl = inputs.make_layer("edges", T=T, d=192, He=64, E=E, Z=Z, K=K, seed=21, zero_fraction=0.4 if Z else None)
     m = zeda.from_workload(wl)
     l, idx, w, counts, offsets, perm, P = oracle_route(wl)
-    for _ in range(2):  # the second call finds the histograms that the first has cleared
+    for _ in range(2):  # each call clears the histograms that the call before it has filled
         check_route(m.route(wl.x.to("cuda:0")), idx, w, counts, offsets, perm, P)
     m.close()
 
@@ -411,9 +411,9 @@ def test_no_candidate_is_taken_twice_whatever_the_logits(zeda, T):
 
 @pytest.mark.parametrize("T,max_tokens", [(300, 300), (2500, 2500), (2500, 9000), (5000, 5000), (300, 20000)])
 def test_router_with_sliced_reduction_axis(zeda, T, max_tokens):
-    # mid-sized batches cut the router's reduction axis into 2 or 4 slices (as many as keep the grid
-    # within the SMs and the slices within the workspace); the top-K kernel adds them.  Routing from
-    # x must equal both the oracle's and the routing from the complete logits.
+    # mid-sized batches cut the router's reduction axis into up to eight slices (as many as keep the grid
+    # within the SMs); the top-K pass adds them, that of the statistics too.  Routing from x must equal
+    # both the oracle's and the routing from the complete logits.
     wl = inputs.tiny(seed=12, T=T, d=512, E=96, Z=40, K=4)
     dev = torch.device("cuda:0")
     m = zeda.from_workload(wl, dev, max_tokens=max_tokens)
@@ -423,11 +423,46 @@ def test_router_with_sliced_reduction_axis(zeda, T, max_tokens):
     check_route(a, idx, w, counts, offsets, perm, P)
     b = m.route_from_logits(m.router_logits(x))
     assert torch.equal(a["topk_idx"], b["topk_idx"]) and torch.equal(a["perm"], b["perm"])
-    # the statistics read complete logits, whichever way the routing before them got its own
     f, p, _ = m.stats(x)
     s = oracle.stats(l, idx, wl.E, wl.Z, alpha=1.0, group_w=1.0)
     assert np.allclose(f.cpu().numpy(), s["f"], rtol=1e-5, atol=1e-7)
     assert np.allclose(p.cpu().numpy(), s["P"], rtol=1e-4, atol=1e-7)
+    m.close()
+
+
+@pytest.mark.parametrize("T,split", [(1270, 7), (1790, 5), (2550, 3)])
+def test_router_slices_of_unequal_length(zeda, T, split):
+    # 32 k-steps in 7, 5 or 3 slices (136 candidates: two candidate tiles)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert sms // ((T + 127) // 128 * 2) == split and 32 % split  # the slices that the router takes for this size
+    wl = inputs.make_layer("slices", T=T, d=2048, He=64, E=96, Z=40, K=4, seed=25, zero_fraction=0.4)
+    m = zeda.from_workload(wl)
+    x = wl.x.to("cuda:0")
+    l, idx, w, counts, offsets, perm, P = oracle_route(wl)
+    check_route(m.route(x), idx, w, counts, offsets, perm, P)
+    f, p, _ = m.stats(x)
+    s = oracle.stats(l, idx, wl.E, wl.Z, alpha=1.0, group_w=1.0)
+    assert np.allclose(f.cpu().numpy(), s["f"], rtol=1e-5, atol=1e-7)
+    assert np.allclose(p.cpu().numpy(), s["P"], rtol=1e-4, atol=1e-7)
+    m.close()
+
+
+def test_routing_from_given_logits_behind_other_calls(zeda):
+    # no router runs in front of a caller's own logits: the call itself clears the histograms that calls before
+    # it have left, of its own kind, of a routing from x, of a larger batch
+    base = inputs.tiny(seed=26, T=900)
+    m = zeda.from_workload(base)
+    x = base.x.to("cuda:0")
+    for T, before in ((300, "nothing"), (300, "itself"), (300, "route"), (900, "itself"), (140, "itself"), (900, "route"), (130, "route")):
+        wl = copy.copy(base)
+        wl.x, wl.T = base.x[:T].contiguous(), T
+        l, idx, w, counts, offsets, perm, P = oracle_route(wl)
+        logits = torch.from_numpy(l).to("cuda:0")
+        if before == "itself":
+            m.route_from_logits(logits)
+        elif before == "route":
+            m.route(x)
+        check_route(m.route_from_logits(logits), idx, w, counts, offsets, perm, P)
     m.close()
 
 
