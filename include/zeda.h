@@ -208,6 +208,8 @@ zeda_status_t zeda_moe_last_counters(zeda_moe_t *h, int64_t out[4], void *stream
  * records CUDA events on its stream between the stages; zeda_moe_stage_ms synchronises on the
  * events of the last forward call (blocking) and returns the elapsed milliseconds of
  * {router logits, top-K + counting sort, expert GEMM1 + SwiGLU, expert GEMM2, combine}.
+ * Small batches whose down projection and combine are one kernel report it as GEMM2 (and up to 8 tokens the
+ * routing as part of GEMM1, whose kernel does it); a forward_host call reports its last chunk.
  * Enabling creates host-side event objects only (no device memory). */
 enum { ZEDA_STAGE_ROUTER = 0, ZEDA_STAGE_SORT = 1, ZEDA_STAGE_GEMM1 = 2, ZEDA_STAGE_GEMM2 = 3,
        ZEDA_STAGE_COMBINE = 4, ZEDA_STAGE_COUNT = 5 };

@@ -419,14 +419,16 @@ zeda_status_t zeda_moe_forward_host(zeda_moe_t *h, const void *x_host, int32_t T
              cudaMemcpyAsync(yh + at[i] * row, ys + (size_t)at[i] * h->cfg.d_model, (at[i + 1] - at[i]) * row, cudaMemcpyDeviceToHost,
                              h->copy_out) == cudaSuccess;
     if (!ok || cudaEventRecord(done, h->copy_out) != cudaSuccess) return cuda_fail("copy of y to the host", cudaGetLastError());
+    zeda_status_t routed = ZEDA_OK;
     if (three) {  // the handle keeps the second half's routing: routed again under the copies back
         RouteOut none = {};
         const int n = route_into(h, xs + (size_t)T0 * h->cfg.d_model, nullptr, T - T0, none, s);
-        if (n < 0) return cuda_fail("routing launch", cudaGetLastError());
-        h->last_launches += n;
+        if (n < 0) routed = cuda_fail("routing launch", cudaGetLastError());
+        else h->last_launches += n;
     }
-    e = cudaEventSynchronize(done);
+    e = cudaEventSynchronize(done);  // (also behind a failed launch: the copies write the caller's buffer)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (routed != ZEDA_OK) return routed;
     if (e != cudaSuccess) return cuda_fail("cudaStreamSynchronize", e);
     return ZEDA_OK;
 }
