@@ -52,9 +52,9 @@ ep_pack_kernel(__nv_bfloat16 *__restrict__ dst, const __nv_bfloat16 *__restrict_
 
 // grid (source rank s, share of its rows).  Every CTA sums the count matrix (it is small), runs the expert scan
 // (CTA 0 publishes counts, offsets and counters; the tile list is filled by all CTAs, a share each)
-// and then maps its share of its source's rows (one CTA for all of 16,000 rows took 18 us, 33 take 5): received row = rows of earlier sources + rows of this source
-// for earlier experts + i; sorted position = expert offset + rows of earlier sources for the same
-// expert + i.
+// and then maps its share of its source's rows (one CTA for all of 16,000 rows took 18 us, 33 take 5):
+// received row = rows of earlier sources + rows of this source for earlier experts + i; sorted position =
+// expert offset + rows of earlier sources for the same expert + i.
 __global__ void __launch_bounds__(512)
 ep_plan_kernel(const int32_t *__restrict__ recv_counts, int n_ranks, int n_local, int n_rows,
                int32_t *__restrict__ counts, int32_t *__restrict__ offsets, int32_t *__restrict__ meta,

@@ -348,8 +348,9 @@ zeda_status_t zeda_moe_forward_residual(zeda_moe_t *h, const void *x, int32_t T,
 // The host-buffer entry point cuts large batches into chunks, so that the copy of a chunk runs under the
 // layer of the one before and the copies back under the layers behind; each chunk reads the experts'
 // weights again.  Below 4096 tokens a second pass over the weights costs more than the copies it hides.
-// A third chunk pays from 8192 tokens on (Zipf load, 75 of 128 experts active: 1211 -> 1068 us a call; an
-// even load, where a third pass over all weights costs most, stands even there and loses 5 % at 7168).
+// A third chunk pays from 8192 tokens on: 1234 -> 1189 us a call of 8192 tokens where every expert is active and
+// a third pass over all weights costs most, 2377 -> 2128 of 16384, 4594 -> 4075 of 32768; Zipf load 1273 -> 1176,
+// 2404 -> 2100, 4676 -> 4127.  At 7168 an even load loses 5 %.
 // Equal chunks: with a quarter, a half and a quarter the copies back queue up behind the half (1216 us).
 static const int kHostSplitMinTokens = 4096, kHostThreeChunksMinTokens = 8192;
 
