@@ -91,10 +91,9 @@ router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restric
 // 192 SM-wide bursts instead of 24; the reduction axis is split over four warps.  NT tokens per CTA, all
 // of their loads in flight at once.  The row is asked into L2 before the wait for the kernel in front (a
 // prefetch only: its values are read after the wait).
-// From kTileRouterTokens on the tensor-core router.  Its accumulators are fp32 too, but against 64 bits its logits
+// From kTileRouterTokens on the tensor-core routers.  Their accumulators are fp32 too, but against 64 bits its logits
 // are off by 2.1e-6 of their root mean square at d 2048 (1.0e-6 at 1024, 9e-6 at 8192), these kernels' by 1.6e-7:
 // below, where they take 15 us at 193 tokens and 20 at 255 against 11 and more slices to add, they are kept.
-constexpr int kTileRouterTokens = 256;
 constexpr int kFewTokens = 32;  // calls of at most this many tokens
 constexpr int kFewThreads = 128;
 constexpr int kFewUnroll = 4;
@@ -494,7 +493,7 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_re
     for (int t = t0 + warp; t < t1; t += kWarps) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL, 3>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
+        topk_gate_token<RPL, 3, true>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
                              v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
@@ -616,8 +615,13 @@ int init_route_kernels(const zeda_moe *h) {
     return 0;
 }
 
-int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s, int *n_parts, int split_T) {
+int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s, int *n_parts, int split_T,
+                         float *stat_part) {
     if (n_parts) *n_parts = 1;
+    if (n_parts && pair_router_path(h, split_T > T ? split_T : T)) {
+        *n_parts = 0;
+        return launch_router_topk_pair(h, x, T, split_T, hist_ints(h, T) ? h->ws.block_hist : nullptr, stat_part, s);
+    }
     // large batches: the GEMM goes to the tensor cores (exact three-way bf16 split of the weights)
     if (T >= kTileRouterTokens && h->router_maps) {
         const int split = n_parts ? router_split_factor(h, split_T > T ? split_T : T) : 1;
@@ -675,7 +679,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         const int topk_warps = T <= 8 * h->sm_count ? 2 : 8;  // the loads of a few tokens spread over all SMs
         int32_t *hist_in_topk = fold ? ws.block_hist : nullptr;
         // no router kernel has cleared the histograms in front of a caller's own logits
-        if (fold && logits != ws.logits) e = cudaMemsetAsync(ws.block_hist, 0, sizeof(int32_t) * nblk * c.n_real, s);
+        if (fold && n_parts && logits != ws.logits) e = cudaMemsetAsync(ws.block_hist, 0, sizeof(int32_t) * nblk * c.n_real, s);
         if (e != cudaSuccess) return -1;
 #define ZEDA_CALL_TOPK(R) \
     e = launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
@@ -684,7 +688,8 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     e = launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
                   sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
                   ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
-        if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
+        if (n_parts == 0) launches = 3;  // the router has chosen already
+        else if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
         else ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);
 #undef ZEDA_CALL_TOPK
 #undef ZEDA_CALL_STATS
@@ -694,7 +699,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
                               sizeof(int32_t) * (kMaskWords + 1) * c.n_real, s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
                               nblk, (const int32_t *)ws.block_hist, ws.counts, ws.offsets, out.n_pairs, ws.meta, wl, tile_rows, ws.perm,
                               out.perm, ws.inv, ws.pair_token);
-            launches = 2;
+            launches -= 2;
         } else {
             e = launch_kernel(h->pdl, slot_hist_kernel, dim3(nblk), dim3(256), sizeof(int32_t) * c.n_real, s,
                               (const int32_t *)ws.topk_idx, T, K, c.n_real, ws.block_hist);
@@ -722,8 +727,8 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
 int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s) {
     const zeda_moe_config_t &c = h->cfg;
     const cudaError_t e = launch_kernel(h->pdl, stats_final_kernel, dim3(1), dim3(kStatFinalThreads), 0, s, (const float *)h->ws.stat_part,
-                                        (T + kStatTokens - 1) / kStatTokens, T, (int)c.top_k, (int)c.n_real, (int)(c.n_real + c.n_zero),
-                                        f, p_mean, out);
+                                        pair_router_path(h, T) ? pair_router_stat_blocks(h, T) : (T + kStatTokens - 1) / kStatTokens, T,
+                                        (int)c.top_k, (int)c.n_real, (int)(c.n_real + c.n_zero), f, p_mean, out);
     return e == cudaSuccess ? 1 : -1;
 }
 

@@ -66,7 +66,8 @@ size_t carve(const zeda_moe_config_t &c, unsigned char *base, Workspace *ws, int
     const size_t n_local = ep ? (size_t)c.n_real / c.ep_size : (size_t)c.n_real;
     const size_t pair_rows = ep ? (size_t)c.max_recv_pairs : slots;
     const size_t ep_tiles = pair_rows / kMidTileM + n_local + 1;
-    const size_t nblk_stats = (c.max_tokens + 63) / 64;
+    size_t nblk_stats = (c.max_tokens + 63) / 64;
+    if (nblk_stats < kPairRouterMaxSliced) nblk_stats = kPairRouterMaxSliced;
     Workspace w;
     w.topk_idx = (int32_t *)take(slots * 4);
     w.topk_w = (float *)take(slots * 4);
@@ -133,7 +134,7 @@ int route_into(zeda_moe_t *h, const __nv_bfloat16 *x, const float *logits_in, in
     h->last_routed_tokens = 0;  // until every launch is in the stream, the handle holds no batch's routing
     const float *logits = logits_in;
     if (!logits) {
-        int r = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts);
+        int r = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts, 0, stat_part);
         if (r < 0) return r;
         n += r;
         logits = h->ws.logits;
@@ -260,6 +261,7 @@ zeda_status_t zeda_moe_create(const zeda_moe_config_t *cfg, const float *router_
     h->pair_rows = cfg->ep_size >= 1 ? cfg->max_recv_pairs : cfg->max_tokens * cfg->top_k;
     h->pmaps = nullptr;
     h->router_maps = nullptr;
+    h->pair_router = nullptr;
     h->profiling = false;
     h->profiled_last = false;
     for (auto &ev : h->ev) ev = nullptr;
@@ -269,8 +271,9 @@ zeda_status_t zeda_moe_create(const zeda_moe_config_t *cfg, const float *router_
     if (init_route_kernels(h) < 0) { delete h; return cuda_fail("kernel set-up", cudaGetLastError()); }
     if (init_stream_kernels() < 0) { delete h; return cuda_fail("kernel set-up", cudaGetLastError()); }
     if (init_pair_kernels(h) < 0) { delete h; return ZEDA_ERR_CUDA; }
-    if (init_router_tile(h) < 0) {
+    if (init_router_tile(h) < 0 || init_router_pair(h) < 0) {
         if (h->pmaps) free(h->pmaps);
+        if (h->router_maps) free(h->router_maps);
         delete h;
         return cuda_fail("router set-up", cudaGetLastError());
     }
@@ -345,6 +348,12 @@ zeda_status_t zeda_moe_forward_residual(zeda_moe_t *h, const void *x, int32_t T,
                           static_cast<cudaStream_t>(stream), static_cast<__nv_bfloat16 *>(r), eps);
 }
 
+// Whether the router adds up the reduction axis alike for calls of a and of b tokens.
+static bool same_router_slices(const zeda_moe *h, int a, int b) {
+    if (pair_router_path(h, a) != pair_router_path(h, b)) return false;
+    return pair_router_path(h, a) ? pair_router_slices(h, a) == pair_router_slices(h, b) : router_split_factor(h, a) == router_split_factor(h, b);
+}
+
 // The host-buffer entry point cuts large batches into chunks, so that the copy of a chunk runs under the
 // layer of the one before and the copies back under the layers behind; each chunk reads the experts'
 // weights again.  Below 4096 tokens a second pass over the weights costs more than the copies it hides.
@@ -388,7 +397,7 @@ zeda_status_t zeda_moe_forward_host(zeda_moe_t *h, const void *x_host, int32_t T
     // where the router slices its reduction axis alike for both halves: the chunks take over that slicing,
     // and nothing else of a token's result depends on the tokens around it.
     const int T0 = (T / 2 + 255) / 256 * 256;  // first token of the second half
-    const bool three = T >= kHostThreeChunksMinTokens && router_split_factor(h, T0) == router_split_factor(h, T - T0);
+    const bool three = T >= kHostThreeChunksMinTokens && same_router_slices(h, T0, T - T0);
     const int chunks = three ? kHostMaxChunks : 2;
     int at[kHostMaxChunks + 1] = {0};  // first token of each chunk
     for (int i = 1; i < chunks; ++i) at[i] = (int)(((long long)T * i / chunks + 255) / 256 * 256);
@@ -612,6 +621,7 @@ zeda_status_t zeda_moe_destroy(zeda_moe_t *h) {
     if (h->copy_out) cudaStreamDestroy(h->copy_out);
     if (h->pmaps) free(h->pmaps);
     if (h->router_maps) free(h->router_maps);
+    if (h->pair_router) free(h->pair_router);
     delete h;
     return st;
 }

@@ -18,6 +18,14 @@ constexpr int kMaxEpRanks = 64;     // expert-parallel group size limit
 constexpr int kStreamTokens = 16;   // calls of at most this many tokens may run the expert kernels of small_batch.cu
 constexpr int kStreamSlots = kStreamTokens * kMaxTopK;  // their largest slot table
 
+constexpr int kTileRouterTokens = 256;     // calls of at least this many tokens have their logits from the tensor cores
+// From so many tokens on (and up to so many candidates) the router with top-K.  Below, its tiles of 256 tokens make more
+// than three slices of the reduction axis, whose exchange takes what the second kernel did: one layer of 777 tokens
+// 227.9 us with the logits' own kernel and 228.3 with it, 2048 tokens 256.3 and 257.1; 4096 314.3 and 311.3, 5003
+// 290.0 and 285.6, 8192 442.4 and 434.9.
+constexpr int kPairRouterTokens = 4096;
+constexpr int kPairRouterMaxCand = 256;
+constexpr int kPairRouterMaxSliced = 160;  // its CTAs where it slices the reduction axis (bounds the statistics' buffer)
 constexpr int kHostMaxChunks = 3;   // of the host-buffer entry point
 
 // Device-resident counters of one call.
@@ -100,6 +108,7 @@ struct zeda_moe {
     int last_launches;
     void *pmaps;  // host-side tensor maps of the expert kernels (owned)
     void *router_maps;  // host-side tensor map of the split router weights (owned)
+    void *pair_router;  // the same for the router with top-K, NULL where it does not take the shape (owned)
     bool profiling;
     bool profiled_last;
     int last_routed_tokens;  // T of the most recent routing pass on this handle
@@ -130,17 +139,24 @@ __device__ __forceinline__ void clear_hist(int32_t *__restrict__ hist, int n) {
 int init_route_kernels(const zeda_moe *h);
 // With n_parts == nullptr the logits are complete.  Otherwise the router may cut the reduction axis
 // into *n_parts slices (mid-sized batches on the tensor-core path): slice p then lies at
-// logits + p * T * n_cand, and launch_route_from_logits adds the slices in order.
+// logits + p * T * n_cand, and launch_route_from_logits adds the slices in order.  Where the router with top-K takes the
+// call, no logits are written and *n_parts is 0: the slots' ids and weights and the block histograms are there already.
 // split_T: the number of tokens that the slicing is decided by, if not T (a call that is one part of a
 // batch gives the batch's, so that its logits are the batch's bits).
 int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s,
-                         int *n_parts = nullptr, int split_T = 0);
+                         int *n_parts = nullptr, int split_T = 0, float *stat_part = nullptr);
 int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s,
                              int n_parts = 1, float *stat_part = nullptr);
 // The statistics of the last routing pass, which was given ws.stat_part to leave its partial sums in.
 int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s);
 int router_split_pad(int n_cand);
 int init_router_tile(zeda_moe *h);
+int init_router_pair(zeda_moe *h);  // behind init_router_tile, which splits the router rows
+bool pair_router_path(const zeda_moe *h, int T);
+int pair_router_slices(const zeda_moe *h, int T);
+int pair_router_stat_blocks(const zeda_moe *h, int T);  // CTAs that leave partial sums of the statistics
+int launch_router_topk_pair(const zeda_moe *h, const __nv_bfloat16 *x, int T, int split_T, int32_t *block_hist, float *stat_part,
+                            cudaStream_t s);
 constexpr int kRouterMaxSplit = 8;
 // rows of n_cand floats that the workspace holds for router output (complete logits or their slices)
 inline long long router_part_rows(long long max_tokens, int n_cand) {
