@@ -102,13 +102,14 @@ template <int NT>
 __global__ void __launch_bounds__(kFewThreads)
 router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w,
                          const float *__restrict__ router_bias, int T, int d, int n_cand, float *__restrict__ logits,
-                         int32_t *__restrict__ hist, int n_hist) {
+                         int32_t *__restrict__ hist, int n_hist, int32_t *__restrict__ meta) {
     pdl_launch_dependents();
     const int j = blockIdx.x, t0 = blockIdx.y * NT;
     const float *wrow = router_w + (size_t)j * d;
     for (int i = threadIdx.x; i < d / 32; i += kFewThreads) asm volatile("prefetch.global.L2 [%0];" ::"l"(wrow + 32 * i));
     pdl_wait();
     clear_hist(hist, n_hist);
+    if (j == 0 && t0 == 0 && threadIdx.x == 0) meta[kMetaRouted] = 0;
     float acc[NT];
 #pragma unroll
     for (int r = 0; r < NT; ++r) acc[r] = 0.f;
@@ -633,7 +634,7 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
     if (T <= kFewTokens) {
         auto go = [&](auto kernel, int per_cta) {
             return launch_kernel(h->pdl, kernel, dim3(n_cand, (T + per_cta - 1) / per_cta), dim3(kFewThreads), 0, s, x, h->router_w,
-                                 h->router_bias, T, d, n_cand, logits, h->ws.block_hist, hist_ints(h, T));
+                                 h->router_bias, T, d, n_cand, logits, h->ws.block_hist, hist_ints(h, T), h->ws.meta);
         };
         const cudaError_t e = T == 1   ? go(router_logits_few_kernel<1>, 1)
                               : T == 2 ? go(router_logits_few_kernel<2>, 2)

@@ -38,6 +38,7 @@ enum MetaSlot {
     kMetaPairTiles = 7,  // entries of the expert kernels' tile list
     kMetaNextItem1 = 8,  // next unclaimed work item of the GEMM1 kernel (reset by the routing pass)
     kMetaNextItem2 = 9,  // the same for GEMM2
+    kMetaRouted = 10,    // smallest batches: the routing tables of the call are in the workspace (the router clears it)
     kMetaCount = 16
 };
 
