@@ -25,7 +25,12 @@ __device__ __forceinline__ float warp_sum(float v) {
 // ballot, and a shift in the lane that held it; and where a warp has several tokens it takes two at a time.  The
 // largest logit is the first round's, and the denominator, which normalised weights do not need (it cancels), is
 // summed for the raw softmax and the statistics only.
-constexpr int kSortedLogits = 8;  // logits per lane up to which they are sorted (more would take longer to sort than the rounds)
+// Two logits a lane (up to 64 candidates) are not sorted: a maximum over them and a second warp reduction, for the
+// lowest id, are less work than the ballot and the shuffle (routing pass of 64 candidates, us, sorted and not: K 8, 1500
+// tokens 18.2, 15.0; 2048 tokens 20.2, 16.6; K 16, 2048 tokens 25.1, 19.0), and more than eight would take longer to
+// sort than the rounds.
+template <int RPL>
+constexpr bool kSortedLogits = RPL > 2 && RPL <= 8;
 
 template <int RPL, int N, bool DEN = false>
 __device__ __forceinline__ void topk_gate_select(const float (&v)[N][RPL], int n_real, int n_cand, int K, int gate_mode, int lane,
@@ -47,7 +52,7 @@ __device__ __forceinline__ void topk_gate_select(const float (&v)[N][RPL], int n
         m[n] = 0.f;
     }
     auto logit_of = [](unsigned k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k); };
-    if constexpr (RPL <= kSortedLogits) {
+    if constexpr (kSortedLogits<RPL>) {
         // the lane's keys in falling order (equal ones by rising id: neighbours change places only where the second is
         // larger), and which of its registers they came from, four bits each
         unsigned from[N];
