@@ -386,8 +386,6 @@ int init_router_pair(zeda_moe *h) {
     return 0;
 }
 
-bool pair_router_path(const zeda_moe *h, int T) { return h->pair_router && T >= kPairRouterTokens; }
-
 // As many slices as the clusters of all tiles are resident with at a time.
 int pair_router_slices(const zeda_moe *h, int T) {
     const PairRouterMaps *rm = static_cast<const PairRouterMaps *>(h->pair_router);
@@ -395,6 +393,39 @@ int pair_router_slices(const zeda_moe *h, int T) {
     int s = kMaxSlices;
     while (s > 1 && (s > k_steps || tiles > rm->max_clusters[s] || 2 * s * tiles > kPairRouterMaxSliced)) --s;
     return s;
+}
+
+// What this kernel saves over the candidate-major router with a top-K pass behind it, in us, from the shape of the
+// call.  Both go in waves: there of (128 tokens x 128 candidates) items over the SMs, here of clusters.  Fitted to the
+// routing pass both ways at 2,197 shapes (4096 to 65,536 tokens, d 256 to 8192, 16 to 256 candidates, K 2 to 16); us,
+// there and here, d 2048 and K 8:
+//    96 candidates   T=4096 22.2, 19.4   T=8448 30.9, 23.3   T=8449 31.0, 33.4 (one slice)   T=9473 37.4, 33.2
+//   128              T=4096 22.6, 21.8   T=8448 32.3, 26.5   T=8449 32.3, 37.9   T=12288 42.6, 38.9   T=20000 71.7, 72.7
+//   192              T=4096 27.4, 27.0   T=8448 39.2, 33.8   T=8449 39.2, 47.3   T=9473 55.9, 47.1    T=20000 93.2, 92.5
+//   256              T=4096 29.4, 33.4   T=4737 36.3, 34.7   T=8449 43.7, 59.8   T=9473 61.7, 59.7    T=20000 102.9, 117.6
+double pair_router_saves_us(const zeda_moe *h, int T) {
+    const PairRouterMaps *rm = static_cast<const PairRouterMaps *>(h->pair_router);
+    const int n_cand = h->cfg.n_real + h->cfg.n_zero;
+    const double k_steps = h->cfg.d_model / kBlockK, K = h->cfg.top_k;
+    const int items = (T + 127) / 128 * ((n_cand + 127) / 128), split = router_split_factor(h, T);
+    const int waves_there = (items * split + h->sm_count - 1) / h->sm_count;
+    const double topk_there = 0.001 * T * (0.12 + 0.029 * K) + 3.7;  // with its launch
+    const double there = waves_there * (0.33 * k_steps / split + 7.2) + topk_there;
+    const int slices = pair_router_slices(h, T), tiles = (T + 2 * kTokens - 1) / (2 * kTokens), fit = rm->max_clusters[slices];
+    const int waves = fit > 0 ? (tiles + fit - 1) / fit : tiles;
+    const int turns = ((kTokens + slices - 1) / slices + kTogether * kWarps - 1) / (kTogether * kWarps);  // of a warp's tokens
+    const double topk = turns * (0.39 + 0.126 * K + 0.66 * ((n_cand + 63) / 64));
+    return there - waves * (0.00167 * rm->n_cols * k_steps / slices + 5.9 + topk);
+}
+
+// Where it saves anything, and 2 us in two ranges where the fit is that far off.  Of the 1,568 shapes that this sends
+// here 22 are more than 2 % slower than there (11 % at most, 5632 tokens of many candidates and short rows), of the others
+// 93 would be more than 4 % faster here.
+bool pair_router_path(const zeda_moe *h, int T) {
+    if (!h->pair_router || T < kPairRouterTokens) return false;
+    const int n_cand = h->cfg.n_real + h->cfg.n_zero;
+    const bool margin = (pair_router_slices(h, T) == 1 && n_cand <= 64) || (h->cfg.d_model < 2048 && n_cand > 128);
+    return pair_router_saves_us(h, T) > (margin ? 2.0 : 0.0);
 }
 
 int pair_router_stat_blocks(const zeda_moe *h, int T) { return (T + 2 * kTokens - 1) / (2 * kTokens) * 2 * pair_router_slices(h, T); }

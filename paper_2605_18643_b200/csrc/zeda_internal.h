@@ -19,10 +19,9 @@ constexpr int kStreamTokens = 16;   // calls of at most this many tokens may run
 constexpr int kStreamSlots = kStreamTokens * kMaxTopK;  // their largest slot table
 
 constexpr int kTileRouterTokens = 256;     // calls of at least this many tokens have their logits from the tensor cores
-// From so many tokens on (and up to so many candidates) the router with top-K.  Below, its tiles of 256 tokens make more
-// than three slices of the reduction axis, whose exchange takes what the second kernel did: one layer of 777 tokens
-// 227.9 us with the logits' own kernel and 228.3 with it, 2048 tokens 256.3 and 257.1; 4096 314.3 and 311.3, 5003
-// 290.0 and 285.6, 8192 442.4 and 434.9.
+// From so many tokens on, up to so many candidates and where pair_router_path says so, the router with top-K.  Below,
+// tiles of 256 tokens would need up to eight slices of the reduction axis to cover the SMs: measured with them, one layer
+// of 777 tokens took 227.9 us with the logits' own kernel and 228.3 with it, 2048 tokens 256.3 and 257.1.  It has three.
 constexpr int kPairRouterTokens = 4096;
 constexpr int kPairRouterMaxCand = 256;
 constexpr int kPairRouterMaxSliced = 160;  // its CTAs where it slices the reduction axis (bounds the statistics' buffer)

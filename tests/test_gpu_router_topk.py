@@ -36,6 +36,29 @@ def test_router_with_top_k(T, d, E, Z, K, gate):
     m.close()
 
 
+@pytest.mark.parametrize("T,d,E,Z,K,gate,chooses", [
+    (4400, 320, 65, 32, 7, 2, True),      # three slices, of one, two and two k-steps
+    (5632, 128, 68, 32, 8, 1, True),      # two slices of one k-step
+    (8448, 1024, 100, 60, 8, 0, True),    # as many tiles as two slices take
+    (8449, 1024, 100, 60, 8, 0, False),   # one more: one slice would take longer than the two kernels
+    (9472, 1024, 100, 60, 8, 0, False),   # the most tokens whose logits are one wave there
+    (9473, 1024, 100, 60, 8, 0, True),    # one slice; a last tile of one token
+    (4096, 1024, 192, 64, 8, 0, False),   # many candidates
+    (33000, 256, 100, 30, 3, 2, True),    # more sort blocks than the router counts, two waves of one slice
+])
+def test_which_router_takes_a_call(T, d, E, Z, K, gate, chooses):
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("router", T=T, d=d, He=64, E=E, Z=Z, K=K, seed=33, zero_fraction=0.4)
+    m = zeda.from_workload(wl, gate_mode=gate)
+    x = wl.x.to("cuda:0")
+    _, idx, w, counts, offsets, perm, P = oracle_route(wl, gate)
+    check_route(m.route(x), idx, w, counts, offsets, perm, P)
+    m.forward(x)
+    place = 1 if T <= 256 * 128 else 3
+    assert m.last_counters()[3] == (1 if chooses else 2) + place + 3
+    m.close()
+
+
 @pytest.mark.parametrize("T", [7, 60, 300])
 @pytest.mark.parametrize("E,Z,K", [(40, 17, 16), (100, 28, 8), (150, 42, 8), (200, 50, 16), (300, 200, 16)])
 def test_selection_among_equal_logits(T, E, Z, K):
