@@ -654,6 +654,29 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
     return e == cudaSuccess ? 1 : -1;
 }
 
+// Top-K and routing weights of T tokens from n_parts >= 1 slices of their logits, and pass 1 of the counting sort where it
+// counts there (hist_ints).
+int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, float *stat_part, cudaStream_t s) {
+    const zeda_moe_config_t &c = h->cfg;
+    const int n_cand = c.n_real + c.n_zero, K = c.top_k;
+    const Workspace &ws = h->ws;
+    const int topk_warps = T <= 8 * h->sm_count ? 2 : 8;  // the loads of a few tokens spread over all SMs
+    int32_t *hist_in_topk = hist_ints(h, T) ? ws.block_hist : nullptr;
+    cudaError_t e = cudaSuccess;
+#define ZEDA_CALL_TOPK(R) \
+    e = launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
+              c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
+#define ZEDA_CALL_STATS(R) \
+    e = launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
+              sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
+              ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
+    if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
+    else ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);
+#undef ZEDA_CALL_TOPK
+#undef ZEDA_CALL_STATS
+    return e == cudaSuccess ? 1 : -1;
+}
+
 int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s, int n_parts,
                              float *stat_part) {
     const zeda_moe_config_t &c = h->cfg;
@@ -677,24 +700,11 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         // up to kFoldMaxBlocks sort blocks the top-K kernel counts the slots itself and one more launch
         // scans and places; beyond, histogram, scan and placement are kernels of their own
         const bool fold = nblk <= kFoldMaxBlocks;
-        const int topk_warps = T <= 8 * h->sm_count ? 2 : 8;  // the loads of a few tokens spread over all SMs
-        int32_t *hist_in_topk = fold ? ws.block_hist : nullptr;
         // no router kernel has cleared the histograms in front of a caller's own logits
         if (fold && n_parts && logits != ws.logits) e = cudaMemsetAsync(ws.block_hist, 0, sizeof(int32_t) * nblk * c.n_real, s);
         if (e != cudaSuccess) return -1;
-#define ZEDA_CALL_TOPK(R) \
-    e = launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
-                  c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
-#define ZEDA_CALL_STATS(R) \
-    e = launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
-                  sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
-                  ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
-        if (n_parts == 0) launches = 3;  // the router has chosen already
-        else if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
-        else ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);
-#undef ZEDA_CALL_TOPK
-#undef ZEDA_CALL_STATS
-        if (e != cudaSuccess) return -1;
+        if (n_parts == 0) launches = 3;  // the slots are chosen already
+        else if (launch_topk(h, logits, n_parts, T, stat_part, s) < 0) return -1;
         if (fold) {
             e = launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk), dim3(kScanThreads),
                               sizeof(int32_t) * (kMaskWords + 1) * c.n_real, s, (const int32_t *)ws.topk_idx, T, K, c.n_real,

@@ -145,16 +145,52 @@ int route_into(zeda_moe_t *h, const __nv_bfloat16 *x, const float *logits_in, in
     return n + r;
 }
 
+// Whether the router adds up the reduction axis alike for calls of a and of b tokens.
+bool same_router_slices(const zeda_moe *h, int a, int b) {
+    if (pair_router_path(h, a) != pair_router_path(h, b)) return false;
+    return pair_router_path(h, a) ? pair_router_slices(h, a) == pair_router_slices(h, b) : router_split_factor(h, a) == router_split_factor(h, b);
+}
+
+// The batches that a chunk of the host-buffer call belongs to: its first `cut` tokens (a multiple of kSortTokens) to one of
+// `first` tokens, the others to one of `rest`.  Its tokens are routed as in calls of those batches.
+struct ChunkOf {
+    int cut, first, rest;
+};
+
+// The router's part of a call of T tokens, as launch_router_logits; of a chunk whose two batches the router treats
+// differently, slots of both parts are chosen apart (*n_parts = 0) and placed together behind.
+int launch_router(const zeda_moe *h, const __nv_bfloat16 *x, int T, const ChunkOf *of, cudaStream_t s, int *n_parts) {
+    if (!of || of->cut == 0 || of->cut >= T || same_router_slices(h, of->first, of->rest))
+        return launch_router_logits(h, x, T, h->ws.logits, s, n_parts, !of ? 0 : of->cut > 0 ? of->first : of->rest);
+    int n = 0;
+    for (int at = 0; at < T; at = at ? T : of->cut) {
+        zeda_moe part = *h;  // the same handle, with the part's slots and histogram blocks in front
+        part.ws.topk_idx += (size_t)at * h->cfg.top_k;
+        part.ws.topk_w += (size_t)at * h->cfg.top_k;
+        part.ws.block_hist += (size_t)(at / kSortTokens) * h->cfg.n_real;
+        const int tokens = at ? T - at : of->cut;
+        int r = launch_router_logits(&part, x + (size_t)at * h->cfg.d_model, tokens, h->ws.logits, s, n_parts, at ? of->rest : of->first);
+        if (r < 0) return r;
+        n += r;
+        if (*n_parts == 0) continue;  // the router has chosen
+        r = launch_topk(&part, h->ws.logits, *n_parts, tokens, nullptr, s);
+        if (r < 0) return r;
+        n += r;
+    }
+    *n_parts = 0;
+    return n;
+}
+
 // With resid given, the call ends in the fused combine + glue pass: resid <- bf16(resid + y) and
 // the normalised residual goes where y would have gone.
 zeda_status_t forward_device(zeda_moe_t *h, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y, cudaStream_t s,
-                             __nv_bfloat16 *resid = nullptr, float eps = 0.f, int split_T = 0) {
+                             __nv_bfloat16 *resid = nullptr, float eps = 0.f, const ChunkOf *of = nullptr) {
     const bool prof = h->profiling;
     auto mark = [&](int i) { if (prof) cudaEventRecord(h->ev[i], s); };
     mark(0);
     h->last_routed_tokens = 0;
     int n_parts = 1;
-    int n = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts, split_T);
+    int n = launch_router(h, x, T, of, s, &n_parts);
     if (n < 0) return cuda_fail("router launch", cudaGetLastError());
     mark(1);
     RouteOut none = {};
@@ -348,12 +384,6 @@ zeda_status_t zeda_moe_forward_residual(zeda_moe_t *h, const void *x, int32_t T,
                           static_cast<cudaStream_t>(stream), static_cast<__nv_bfloat16 *>(r), eps);
 }
 
-// Whether the router adds up the reduction axis alike for calls of a and of b tokens.
-static bool same_router_slices(const zeda_moe *h, int a, int b) {
-    if (pair_router_path(h, a) != pair_router_path(h, b)) return false;
-    return pair_router_path(h, a) ? pair_router_slices(h, a) == pair_router_slices(h, b) : router_split_factor(h, a) == router_split_factor(h, b);
-}
-
 // The host-buffer entry point cuts large batches into chunks, so that the copy of a chunk runs under the
 // layer of the one before and the copies back under the layers behind; each chunk reads the experts'
 // weights again.  Below 4096 tokens a second pass over the weights costs more than the copies it hides.
@@ -393,11 +423,12 @@ zeda_status_t zeda_moe_forward_host(zeda_moe_t *h, const void *x_host, int32_t T
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
         if (e != cudaSuccess) return cuda_fail("stream / event creation", e);
     }
-    // The result is that of the batch's two halves as calls of their own.  Three chunks give the same bits
-    // where the router slices its reduction axis alike for both halves: the chunks take over that slicing,
-    // and nothing else of a token's result depends on the tokens around it.
+    // The result is that of the batch's two halves as calls of their own.  Three chunks give the same bits: their
+    // tokens take over the halves' routers and slices, the middle chunk's in two parts where these differ, and
+    // nothing else of a token's result depends on the tokens around it.  (Two chunks where the halves differ and
+    // three: 8400 tokens 1264, 1240 us a call; 9300 1389, 1288; 11,400 1659, 1474; 17,000 2439, 2138.)
     const int T0 = (T / 2 + 255) / 256 * 256;  // first token of the second half
-    const bool three = T >= kHostThreeChunksMinTokens && same_router_slices(h, T0, T - T0);
+    const bool three = T >= kHostThreeChunksMinTokens;
     const int chunks = three ? kHostMaxChunks : 2;
     int at[kHostMaxChunks + 1] = {0};  // first token of each chunk
     for (int i = 1; i < chunks; ++i) at[i] = (int)(((long long)T * i / chunks + 255) / 256 * 256);
@@ -418,7 +449,8 @@ zeda_status_t zeda_moe_forward_host(zeda_moe_t *h, const void *x_host, int32_t T
     for (int i = 0; i < chunks; ++i) {
         const size_t off = (size_t)at[i] * h->cfg.d_model;
         if (cudaStreamWaitEvent(s, copied[i], 0) != cudaSuccess) return cuda_fail("cudaStreamWaitEvent", cudaGetLastError());
-        const zeda_status_t st = forward_device(h, xs + off, at[i + 1] - at[i], ys + off, s, nullptr, 0.f, three ? T0 : 0);
+        const ChunkOf of = {at[i] < T0 ? T0 - at[i] : 0, T0, T - T0};
+        const zeda_status_t st = forward_device(h, xs + off, at[i + 1] - at[i], ys + off, s, nullptr, 0.f, &of);
         if (st != ZEDA_OK) return st;
         launches += h->last_launches;
         if (cudaEventRecord(computed[i], s) != cudaSuccess) return cuda_fail("cudaEventRecord", cudaGetLastError());

@@ -147,6 +147,7 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
                          int *n_parts = nullptr, int split_T = 0, float *stat_part = nullptr);
 int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s,
                              int n_parts = 1, float *stat_part = nullptr);
+int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, float *stat_part, cudaStream_t s);
 // The statistics of the last routing pass, which was given ws.stat_part to leave its partial sums in.
 int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s);
 int router_split_pad(int n_cand);

@@ -265,6 +265,28 @@ def test_host_buffer_entry_point_chunk_counts(zeda, T):
     m.close()
 
 
+@pytest.mark.parametrize("T,launches", [
+    (8200, 21),   # halves of 4352 and 3848 tokens: the router with top-K, and the other in two slices
+    (11400, 18),  # 5888 and 5512: two slices and three
+    (12000, 17),  # 6144 and 5856: both two, where a chunk of 4000 tokens would have the other router
+    (17000, 20),  # 8704 and 8296: the other router in one slice, and the router with top-K
+])
+def test_host_buffer_entry_point_where_the_halves_have_other_routers(zeda, T, launches):
+    # three chunks all the same (the launches are theirs), the middle one's tokens chosen as in their half
+    wl = inputs.make_layer("host_halves", T=T, d=2048, He=64, E=128, Z=64, K=8, seed=19)
+    dev = torch.device("cuda:0")
+    m = zeda.from_workload(wl, dev)
+    x = wl.x.to(dev)
+    T0 = (T // 2 + 255) // 256 * 256
+    want = torch.cat([m.forward(x[:T0].contiguous()), m.forward(x[T0:].contiguous())]).cpu()
+    share, counters = m.token_zero_share(T - T0).cpu(), m.last_counters()[:3]
+    host = wl.x.pin_memory()
+    for _ in range(2):
+        assert torch.equal(want.view(torch.int16), m.forward_host(host).view(torch.int16))
+        assert torch.equal(m.token_zero_share(T - T0).cpu(), share) and m.last_counters() == counters + (launches,)
+    m.close()
+
+
 def test_routing_statistics(zeda):
     wl = inputs.tiny(seed=9, T=200)
     dev = torch.device("cuda:0")
