@@ -81,6 +81,34 @@ def test_alternating_inputs_give_the_bits_of_single_calls(layer, T, use):
     m.close()
 
 
+@pytest.fixture(scope="module")
+def large_layer():
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("back_to_back", T=9473, d=1024, He=64, E=64, Z=32, K=8, seed=42, zero_fraction=0.5)
+    return zeda, wl, [wl.x.to("cuda:0"), inputs.replica_tokens(wl, 7).to("cuda:0")]
+
+
+@pytest.mark.parametrize("use", ["forward", "residual", "stats", "route"])
+@pytest.mark.parametrize("T", [4096, 5633, 8449, 9473])
+def test_alternating_large_batches_give_the_bits_of_single_calls(large_layer, T, use):
+    # the router with top-K in three slices, two and one, and between them a size that the other router takes
+    zeda, wl, xs = large_layer
+    m = zeda.from_workload(wl)
+    alone = check(zeda, m, [(i % 2, use, xs[i % 2][:T].contiguous()) for i in range(20)])
+    assert not alone[0].same(alone[1])
+    m.forward(xs[0][:T].contiguous())
+    assert m.last_counters()[3] == (6 if T == 8449 else 5)
+    m.close()
+
+
+def test_large_batches_in_any_order(large_layer):
+    zeda, wl, xs = large_layer
+    m = zeda.from_workload(wl)
+    order = [(T, use) for T in (9473, 8449, 300, 4096, 8, 5633, 9473, 4095, 5003) for use in ("forward", "stats", "residual", "route")]
+    check(zeda, m, [((T, use, i % 2), use, xs[i % 2][:T].contiguous()) for i, (T, use) in enumerate(order)])
+    m.close()
+
+
 def test_batch_sizes_and_uses_in_any_order(layer):
     zeda, wl, xs = layer
     m = zeda.from_workload(wl, max_tokens=2048)

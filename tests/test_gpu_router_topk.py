@@ -71,3 +71,70 @@ def test_selection_among_equal_logits(T, E, Z, K):
     idx, w = oracle.route(l, E, Z, K, 0)
     check_route(m.route_from_logits(torch.from_numpy(l).to("cuda:0")), idx, w, *oracle.compact(idx, E))
     m.close()
+
+
+@pytest.mark.parametrize("T,d,E,Z,K,rows", [
+    (4097, 1024, 28, 12, 16, 20),    # each row twice, in other lanes
+    (4800, 1024, 70, 30, 8, 32),     # up to four times in one lane
+    (4737, 1024, 100, 60, 16, 40),   # in other lanes and registers
+    (5633, 2048, 180, 70, 8, 32),
+    (9473, 2048, 100, 60, 8, 20),    # one slice
+])
+def test_router_with_top_k_among_equal_logits_and_nan_tokens(T, d, E, Z, K, rows):
+    # a few router rows repeated: the logits of their candidates are equal, bit for bit; every seventh token is NaN
+    from paper_2605_18643_b200 import zeda
+    n = E + Z
+    wl = inputs.make_layer("equal", T=T + 256, d=d, He=64, E=E, Z=Z, K=K, seed=34, zero_fraction=None)
+    wl.router_w = wl.router_w[torch.arange(n) % rows].contiguous()
+    # logits of other rows are further apart than the fp32 sums are exact (4e-6 at these sizes)
+    top = torch.topk(wl.x.float() @ wl.router_w[:rows].t(), min(K, rows - 1) + 1, dim=1).values
+    wl.x = wl.x[(top[:, :-1] - top[:, 1:]).amin(dim=1) > 5e-5][:T].contiguous()
+    wl.T = wl.x.shape[0]
+    assert wl.T == T
+    nan = np.arange(T) % 7 == 3
+    x = wl.x.to("cuda:0")
+    x[torch.from_numpy(nan).to(x.device)] = float("nan")
+    _, idx, w, *_ = oracle_route(wl)
+    idx[nan] = np.arange(K)  # equal keys throughout: the lowest ids
+    m = zeda.from_workload(wl)
+    m.forward(x)
+    assert m.last_counters()[3] == 5  # the router that also chooses
+    o = m.route(x)
+    counts, offsets, perm, P = oracle.compact(idx, E)
+    got = o["topk_w"].cpu().numpy()
+    assert np.isnan(got[nan]).all()
+    o["topk_w"][torch.from_numpy(nan).to(x.device)] = torch.from_numpy(w[nan]).float().to(x.device)
+    check_route(o, idx, w, counts, offsets, perm, P)
+    m.close()
+
+
+@pytest.mark.parametrize("T", [4097, 8448, 9473])
+def test_router_with_top_k_in_a_graph_and_without_dependent_launch(T):
+    # it fetches router rows in front of its wait for the kernel before it, and clears its own histograms
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("router", T=T, d=1024, He=64, E=64, Z=32, K=8, seed=35)
+    dev = torch.device("cuda:0")
+    xs = [wl.x.to(dev), inputs.replica_tokens(wl, 3).to(dev)]
+    plain = zeda.from_workload(wl, dev, flags=zeda.FLAG_NO_DEPENDENT_LAUNCH)
+    want = [plain.forward(x).view(torch.int16) for x in xs]
+    torch.cuda.synchronize()
+    m = zeda.from_workload(wl, dev)
+    for i in (0, 1, 0):
+        assert torch.equal(m.forward(xs[i]).view(torch.int16), want[i])
+    assert m.last_counters()[3] == 5
+    x, y, y2 = xs[0].clone(), torch.empty_like(xs[0]), torch.empty_like(xs[0])
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):  # two calls: the second starts under the first
+        m.forward(x, y)
+        m.forward(y, y2)
+    for src in (1, 0, 1):
+        x.copy_(xs[src])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y.view(torch.int16), want[src])
+        assert torch.equal(y2.view(torch.int16), plain.forward(y.clone()).view(torch.int16))
+    del graph
+    m.close()
+    plain.close()

@@ -60,6 +60,33 @@ def test_small_batches_match_the_oracle(T, shape, kind):
     m.close()
 
 
+@pytest.mark.parametrize("He,K", [(128, 4), (1024, 2)])
+@pytest.mark.parametrize("E,Z,gate", [(32, 32, 0), (64, 64, 1), (100, 60, 2), (150, 100, 0), (200, 200, 1)])
+def test_down_kernel_fetches_the_routing_or_repeats_it(E, Z, gate, He, K):
+    # Launched in stream order the down kernel always finds gate/up's tables.  With dependent launch it starts as gate/up's
+    # CTAs leave, and where these have little to do (H_e 128) nearly all of its CTAs are there before the tables and
+    # route for themselves.  Copy experts: the routing weights of zero slots count too.
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("routed", T=8, d=1024, He=He, E=E, Z=Z, K=K, seed=36, zero_fraction=0.5)
+    xs = [wl.x.to("cuda:0"), inputs.replica_tokens(wl, 5).to("cuda:0")]
+    kw = dict(gate_mode=gate, expert_kind=zeda.EXPERT_COPY)
+    plain = zeda.from_workload(wl, flags=zeda.FLAG_NO_DEPENDENT_LAUNCH, **kw)
+    m = zeda.from_workload(wl, **kw)
+    for T in (1, 2, 5, 8):
+        x = [a[:T].contiguous() for a in xs]
+        want = [plain.forward(a) for a in x]
+        assert plain.last_counters()[3] == 3 and not torch.equal(want[0], want[1])
+        got = [torch.empty_like(x[0]) for _ in range(20)]
+        torch.cuda.synchronize()
+        for i, y in enumerate(got):  # no synchronisation in between
+            m.forward(x[i % 2], y)
+        torch.cuda.synchronize()
+        for i, y in enumerate(got):
+            assert torch.equal(y.view(torch.int16), want[i % 2].view(torch.int16)), (T, i)
+    m.close()
+    plain.close()
+
+
 @pytest.mark.parametrize("T", [1, 8, 16])
 def test_small_batches_in_a_graph_and_without_dependent_launch(T):
     # the expert kernels here read the routing results in front of their wait for the kernel before them
