@@ -85,17 +85,17 @@ __device__ __forceinline__ void load_route_tables(RouteTables<SLOTS> &rt, const 
     __syncthreads();
 }
 
-// Up to kRouteHereTokens tokens every CTA routes them itself, from the logits: one warp per token and a
-// scan over bit masks take about as long as fetching another kernel's results, and the call has one
-// kernel fewer in its chain (one token: 24.9 -> 15.7 us a call back to back, 8 tokens: 53.7 -> 52.7).  All
-// CTAs arrive at the same tables.
+// Up to kRouteHereTokens tokens every gate/up CTA routes them itself, from the logits: one warp per token (no loop: with
+// sixteen logits a lane it spilled) and a scan over bit masks take no longer than a routing kernel in front, and the call
+// has one kernel fewer in its chain (one token: 24.9 -> 15.7 us a call back to back, 8 tokens: 53.7 -> 52.7).  All CTAs
+// arrive at the same tables.
 constexpr int kRouteHereTokens = 8;
 
 template <int RPL, int SLOTS>
 __device__ __forceinline__ void route_here(RouteTables<SLOTS> &rt, const RouteArgs &ra) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const int n_chunks = (ra.n_real + 31) / 32;
-    for (int t = warp; t < ra.T; t += n_warps) {
+    if (const int t = warp; t < ra.T) {
         int my_idx;
         float my_w, v[RPL], m, den;
         topk_gate_token<RPL>(ra.logits + (size_t)t * ra.n_cand, 1, 0, ra.n_real, ra.n_cand, ra.K, ra.gate_mode, lane, v, m, den, my_idx, my_w);
@@ -178,12 +178,12 @@ __device__ __forceinline__ void publish_route(const RouteTables<SLOTS> &rt, cons
         ra.meta[kMetaPairTiles] = rt.n_tiles;
         ra.meta[kMetaMaxRows] = mx;
     }
-    __threadfence();
-    __syncthreads();
+    __syncthreads();  // the CTA's stores come before the release that follows it
     if (threadIdx.x == 0) asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(ra.meta + kMetaRouted) : "memory");
 }
 
-// Whether the tables above are there; every thread that reads them asks for itself.
+// Whether the tables above are there, for one thread of a CTA to ask; the barrier behind it passes its acquire on to the
+// others (each asking for itself takes 0.2 us longer).
 __device__ __forceinline__ bool route_published(const RouteArgs &ra) {
     int32_t v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ra.meta + kMetaRouted) : "memory");
@@ -303,8 +303,10 @@ stream_gate_up_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *
 // Up to kRouteHereTokens tokens the routing is gate/up's: it has left its tables long before its last CTAs leave the SMs
 // to these, and fetching them takes 1 us where routing takes 3 (us for four layers, routing here and fetching: 1 token
 // 81.9, 77.0; 2 tokens 109.2, 104.1; 4 tokens 151.0, 146.3; 8 tokens 224.8, 220.3).  A CTA that is here before them does
-// not wait: it routes for itself and arrives at the same tables.
+// not wait: it routes for itself and arrives at the same tables.  That is nearly every CTA where gate/up's have little to
+// do (no pair at all, or H_e 128), for the price of the look at the flag, at most 1 % of such a call.
 constexpr int kDownWarps = 16, kDownSlices = 4, kDownExperts = kDownWarps / kDownSlices;
+static_assert(kUpWarps >= kRouteHereTokens && kDownWarps >= kRouteHereTokens, "a warp per token");
 constexpr int kDownChunk = 6;
 constexpr int kDownStride = 20;  // floats per pair and slice: 16 features; 20 keeps the fragment stores free of bank conflicts
 
@@ -319,7 +321,7 @@ stream_down_combine_kernel(const __nv_bfloat16 *__restrict__ hmid, const __nv_bf
     const int T = ra.T, K = ra.K, slots = T * K;
     if constexpr (RPL > 0) {
         for (int i = threadIdx.x; i < ra.n_real; i += blockDim.x) rt.mask[i] = 0u;
-        if (__syncthreads_and(route_published(ra))) load_route_tables(rt, ra);
+        if (__syncthreads_or(threadIdx.x == 0 && route_published(ra))) load_route_tables(rt, ra);
         else route_here<RPL>(rt, ra);
     } else {
         load_route_tables(rt, ra);
