@@ -12,13 +12,13 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("T,d,E,Z,K,gate", [
-    (4096, 64, 20, 12, 4, 0),      # one k-step, 32 candidates
+    (4096, 64, 20, 12, 4, 0),      # one k-step, 32 candidates (the other router)
     (4097, 192, 65, 32, 16, 2),    # three slices of one k-step, 97 candidates, one token in the last tile
-    (4400, 320, 129, 0, 1, 0),     # slices of unequal length, 129 candidates
-    (5632, 128, 100, 61, 8, 1),    # as many tiles as three slices take, fewer k-steps than that
+    (4400, 320, 129, 0, 1, 0),     # 129 candidates (the other router)
+    (5632, 128, 100, 61, 8, 1),    # the same, fewer k-steps than slices
     (5700, 256, 33, 0, 5, 2),      # two accumulators of the large products
-    (8449, 192, 200, 55, 8, 0),    # one slice, 255 candidates, an empty half tile
-    (33000, 64, 160, 96, 3, 0),    # 256 candidates, more sort blocks than the router counts
+    (8449, 192, 200, 55, 8, 0),    # 255 candidates (the other router)
+    (33000, 64, 160, 96, 3, 0),    # 256 candidates, more sort blocks than the router counts (the other router)
 ])
 def test_router_with_top_k(T, d, E, Z, K, gate):
     from paper_2605_18643_b200 import zeda
@@ -45,6 +45,9 @@ def test_router_with_top_k(T, d, E, Z, K, gate):
     (9473, 1024, 100, 60, 8, 0, True),    # one slice; a last tile of one token
     (4096, 1024, 192, 64, 8, 0, False),   # many candidates
     (33000, 256, 100, 30, 3, 2, True),    # more sort blocks than the router counts, two waves of one slice
+    (18000, 64, 20, 12, 2, 0, True),      # one k-step, 32 candidates
+    (4737, 2048, 200, 55, 8, 1, True),    # 255 candidates, an odd count; a last half tile of one token
+    (5003, 2048, 150, 60, 3, 0, True),    # 210 candidates: 224 columns
 ])
 def test_which_router_takes_a_call(T, d, E, Z, K, gate, chooses):
     from paper_2605_18643_b200 import zeda
