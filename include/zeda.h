@@ -131,9 +131,10 @@ zeda_status_t zeda_route_from_logits(zeda_moe_t *h, const float *logits, int32_t
                                      void *stream);
 
 /* Test entry: the fp32 router logits x * router_w^T + bias, dev [T, N+N_Z].  zeda_route and
- * zeda_moe_forward compute the same sums, for mid-sized batches (256 <= T, up to a few thousand
- * tokens) in two to eight slices of the reduction axis that are added afterwards: their logits can
- * differ from these in the last bits (fp32 addition order), never in the exact products. */
+ * zeda_moe_forward add up the same exact products, from 256 tokens on in another order: mid-sized
+ * batches in up to eight slices of the reduction axis that are added afterwards, most batches of 4096
+ * tokens and more (up to 256 candidates) in another kernel, which keeps no logits, in one to three.
+ * Their logits can differ from these in the last bits at any T >= 256, never in the products. */
 zeda_status_t zeda_router_logits(zeda_moe_t *h, const void *x, int32_t T, float *logits, void *stream);
 
 /* Layer forward, Eq. 1 (Eq. 7 / Appendix B through the configured modes).
@@ -209,7 +210,8 @@ zeda_status_t zeda_moe_last_counters(zeda_moe_t *h, int64_t out[4], void *stream
  * events of the last forward call (blocking) and returns the elapsed milliseconds of
  * {router logits, top-K + counting sort, expert GEMM1 + SwiGLU, expert GEMM2, combine}.
  * Small batches whose down projection and combine are one kernel report it as GEMM2 (and up to 8 tokens the
- * routing as part of GEMM1, whose kernel does it); a forward_host call reports its last chunk.
+ * routing as part of GEMM1, whose kernel does it); batches whose router also chooses (most from 4096 tokens on)
+ * report the top-K as part of the router; a forward_host call reports its last chunk.
  * Enabling creates host-side event objects only (no device memory). */
 enum { ZEDA_STAGE_ROUTER = 0, ZEDA_STAGE_SORT = 1, ZEDA_STAGE_GEMM1 = 2, ZEDA_STAGE_GEMM2 = 3,
        ZEDA_STAGE_COMBINE = 4, ZEDA_STAGE_COUNT = 5 };

@@ -119,7 +119,7 @@ __device__ __forceinline__ void topk_gate_select(const float (&v)[N][RPL], int n
                 if (k == 0) m[n] = logit_of(gm);
             }
     }
-    // a NaN among the logits, selected or not, is one in every weight
+    // a NaN among the logits, selected or not, is one in every weight (in Eq. 7's, whose sum is then not above 0, a zero)
 #pragma unroll
     for (int n = 0; n < N; ++n) {
         bool bad = false;
