@@ -265,15 +265,16 @@ def test_host_buffer_entry_point_chunk_counts(zeda, T):
     m.close()
 
 
-@pytest.mark.parametrize("T,launches", [
-    (8200, 21),   # halves of 4352 and 3848 tokens: the router with top-K, and the other in two slices
-    (11400, 18),  # 5888 and 5512: two slices and three
-    (12000, 17),  # 6144 and 5856: both two, where a chunk of 4000 tokens would have the other router
-    (17000, 20),  # 8704 and 8296: the other router in one slice, and the router with top-K
+@pytest.mark.parametrize("T,d,E,launches", [
+    (8200, 2048, 128, 21),   # halves of 4352 and 3848 tokens: the router with top-K, and the other in two slices
+    (9472, 128, 96, 23),     # 4864 and 4608: the other router in one slice and in two
+    (11400, 2048, 128, 18),  # 5888 and 5512: two slices and three
+    (12000, 2048, 128, 17),  # 6144 and 5856: both two, where a chunk of 4000 tokens would have the other router
+    (17000, 2048, 128, 20),  # 8704 and 8296: the other router in one slice, and the router with top-K
 ])
-def test_host_buffer_entry_point_where_the_halves_have_other_routers(zeda, T, launches):
+def test_host_buffer_entry_point_where_the_halves_have_other_routers(zeda, T, d, E, launches):
     # three chunks all the same (the launches are theirs), the middle one's tokens chosen as in their half
-    wl = inputs.make_layer("host_halves", T=T, d=2048, He=64, E=128, Z=64, K=8, seed=19)
+    wl = inputs.make_layer("host_halves", T=T, d=d, He=64, E=E, Z=64, K=8, seed=19)
     dev = torch.device("cuda:0")
     m = zeda.from_workload(wl, dev)
     x = wl.x.to(dev)
