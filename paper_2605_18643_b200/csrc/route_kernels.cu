@@ -93,7 +93,7 @@ router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restric
 // prefetch only: its values are read after the wait).
 // From kTileRouterTokens on the tensor-core routers.  Their accumulators are fp32 too, but against 64 bits its logits
 // are off by 2.1e-6 of their root mean square at d 2048 (1.0e-6 at 1024, 9e-6 at 8192), these kernels' by 1.6e-7:
-// below, where they take 15 us at 193 tokens and 20 at 255 against 11 and more slices to add, they are kept.
+// below, the CUDA cores keep them.
 constexpr int kFewTokens = 32;  // calls of at most this many tokens
 constexpr int kFewThreads = 128;
 constexpr int kFewUnroll = 4;
@@ -152,12 +152,161 @@ router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__res
     }
 }
 
+// Sliced router of 33 to 255 tokens: kSliceTokens x kSliceCand logits per CTA over a slice of the reduction axis, each of its
+// eight warps over an eighth of the slice, 8 x 4 logits per lane.  A warp copies what it needs into shared memory by itself,
+// all of it at once (its router rows before the wait for the kernel in front: they are the caller's constants), so a CTA
+// waits for memory once; the products then take 16 loads of 16 bytes per 256 fused multiply-adds.  (The kernel above, a warp
+// per candidate row and 8 tokens, converts every x value once per candidate and waits for each row.)  Sums are fp32, of runs
+// of 16 products, then of the runs, the warps and, in the top-K pass, the slices; the bias comes behind them.
+constexpr int kSliceTokens = 32, kSliceCand = 32, kSliceWarps = 8;
+constexpr int kSliceRedLd = 40;   // floats between the tokens of a warp's sums: the lanes of a store hit all banks
+constexpr int kSliceRun = 2;      // octets of products added up before they go to the total
+constexpr int kSliceMinPart = 256;  // elements of the reduction axis that make a slice worth it
+constexpr int kSliceMaxParts = 7;   // with the bias as many as the top-K pass requests at a time (8 where they would not fit otherwise)
+constexpr int kSliceMinModel = 1024, kSliceMinLogits = 4000;   // d, and T x candidates
+constexpr long long kSliceMinProducts = 12600000;              // T x candidates x d
+constexpr int kSliceMaxSmem = 200 * 1024;
+
+// Bytes between the rows of a warp's operands of `octets` groups of eight elements: odd multiples of 16, so that rows next
+// to one another lie in different banks.
+__host__ __device__ constexpr int slice_x_stride(int octets) { return 16 * (octets | 1); }
+__host__ __device__ constexpr int slice_w_stride(int octets) { return 32 * octets + 16; }
+__host__ __device__ constexpr int slice_warp_octets(int d, int parts) { return ((d / 8 + parts - 1) / parts + kSliceWarps - 1) / kSliceWarps; }
+
+size_t slice_smem(int d, int parts) {
+    const int n = slice_warp_octets(d, parts);
+    const size_t operands = (size_t)kSliceWarps * (kSliceTokens * slice_x_stride(n) + kSliceCand * slice_w_stride(n));
+    const size_t sums = (size_t)kSliceWarps * kSliceTokens * kSliceRedLd * sizeof(float);
+    return operands > sums ? operands : sums;
+}
+
+__global__ void __launch_bounds__(32 * kSliceWarps, 1)
+router_logits_slice_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w, int T, int d, int n_cand,
+                           float *__restrict__ logits, int32_t *__restrict__ hist, int n_hist) {
+    pdl_launch_dependents();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int j0 = blockIdx.x * kSliceCand, t0 = blockIdx.y * kSliceTokens, part = blockIdx.z, parts = gridDim.z;
+    const int o0 = d / 8 * part / parts, o1 = d / 8 * (part + 1) / parts;
+    const int q0 = o0 + (o1 - o0) * warp / kSliceWarps, n = o0 + (o1 - o0) * (warp + 1) / kSliceWarps - q0;  // this warp's octets, 4 to 16
+    const int octets = slice_warp_octets(d, parts);
+    const int xs = slice_x_stride(octets), ws = slice_w_stride(octets);
+    unsigned char *xb = smem_raw + warp * (kSliceTokens * xs + kSliceCand * ws), *wb = xb + kSliceTokens * xs;
+    auto copy16 = [](void *dst, const void *src) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+    };
+    const int rows_w = min(kSliceCand, n_cand - j0), rows_x = min(kSliceTokens, T - t0);
+    {
+        const uint32_t inv = (1u << 20) / (2 * n) + 1;  // i / (2 n) = i * inv >> 20 for the i below
+        for (int i = lane; i < rows_w * 2 * n; i += 32) {
+            const int r = i * inv >> 20, c = i - r * 2 * n;
+            copy16(wb + r * ws + 16 * c, router_w + (size_t)(j0 + r) * d + 8 * q0 + 4 * c);
+        }
+    }
+    pdl_wait();
+    {
+        const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        for (int i = cta * blockDim.x + threadIdx.x; i < n_hist; i += gridDim.x * gridDim.y * gridDim.z * blockDim.x) hist[i] = 0;
+    }
+    {
+        const uint32_t inv = (1u << 20) / n + 1;
+        for (int i = lane; i < rows_x * n; i += 32) {
+            const int r = i * inv >> 20, c = i - r * n;
+            copy16(xb + r * xs + 16 * c, x + (size_t)(t0 + r) * d + 8 * (q0 + c));
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    // lane: tokens tg + 4 i, candidates cg + 8 j (rows beyond the call's hold what was there: their sums are not stored)
+    const int tg = lane >> 3, cg = lane & 7;
+    float acc[8][4], tot[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = tot[i][j] = 0.f;
+    for (int q = 0; q < n; ++q) {
+        uint4 xv[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) xv[i] = *reinterpret_cast<const uint4 *>(xb + (tg + 4 * i) * xs + 16 * q);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float4 w[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4 *>(wb + (cg + 8 * j) * ws + 32 * q + 16 * h);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t lo = h ? xv[i].z : xv[i].x, hi = h ? xv[i].w : xv[i].y;
+                const float x0 = __uint_as_float(lo << 16), x1 = __uint_as_float(lo & 0xffff0000u);
+                const float x2 = __uint_as_float(hi << 16), x3 = __uint_as_float(hi & 0xffff0000u);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc[i][j] = fmaf(w[j].x, x0, acc[i][j]);
+                    acc[i][j] = fmaf(w[j].y, x1, acc[i][j]);
+                    acc[i][j] = fmaf(w[j].z, x2, acc[i][j]);
+                    acc[i][j] = fmaf(w[j].w, x3, acc[i][j]);
+                }
+            }
+        }
+        if ((q + 1) % kSliceRun == 0 || q + 1 == n) {  // (uniform)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { tot[i][j] += acc[i][j]; acc[i][j] = 0.f; }
+        }
+    }
+    __syncthreads();  // the operands have been read: their room takes the warps' sums
+    float *red = reinterpret_cast<float *>(smem_raw);  // [kSliceWarps][kSliceTokens][kSliceRedLd]
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) red[(warp * kSliceTokens + tg + 4 * i) * kSliceRedLd + cg + 8 * j] = tot[i][j];
+    __syncthreads();
+    const int r = threadIdx.x >> 3, c = (threadIdx.x & 7) * 4;  // four candidates of a token per thread
+    float4 v[kSliceWarps];
+#pragma unroll
+    for (int q = 0; q < kSliceWarps; ++q) v[q] = *reinterpret_cast<const float4 *>(red + (q * kSliceTokens + r) * kSliceRedLd + c);
+#pragma unroll
+    for (int o = 1; o < kSliceWarps; o *= 2)
+#pragma unroll
+        for (int q = 0; q < kSliceWarps; q += 2 * o) v[q] = make_float4(v[q].x + v[q + o].x, v[q].y + v[q + o].y, v[q].z + v[q + o].z, v[q].w + v[q + o].w);
+    if (r >= rows_x) return;
+    float *out = logits + ((size_t)part * T + t0 + r) * n_cand + j0;
+    const float s[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (c + j < rows_w) out[c + j] = s[j];
+}
+
+// Slices of the reduction axis for a call of T tokens by that kernel, 0 where the one above takes the call: as many as give
+// every SM at most one CTA, but no fewer than fit its shared memory.  Routing pass, us, by the kernel above and by this:
+//   d 2048, 192 candidates   T=33 13.8, 11.2    T=64 13.2, 11.4    T=128 15.7, 12.7   T=193 20.2, 15.9   T=255 27.0, 16.7
+//   d 2048, 96               T=33 11.2, 11.9    T=64 11.9, 12.2    T=96 13.7, 12.1    T=193 15.3, 11.7   T=255 15.3, 12.3
+//   d 1024, 96               T=33 9.3, 10.8     T=64 10.1, 11.0    T=128 11.2, 11.7   T=129 12.6, 11.5   T=255 13.2, 11.8
+//   d 2048, 12               T=33 8.9, 9.7      T=128 9.3, 10.1    T=255 11.0, 10.4
+//   d 8192, 400              T=33 39.2, 36.6    T=128 103.5, 51.5  T=255 171, 85
+//   d 2048, 512              T=33 20.6, 19.3    T=128 34.6, 25.7   T=129 31.3, 35.1   T=160 40.2, 33.9
+// So few logits stay there, and calls (the last row's 129 tokens) whose last wave here would be a handful of CTAs.  The
+// weights' distance from 64 bits, 2-norms: d 1024 1.0e-7 and 9.3e-8, d 2048 1.6e-7 and 1.3e-7, d 8192 5e-7 and 2.6e-7.
+int router_slices(const zeda_moe *h, int T) {
+    const int d = h->cfg.d_model, n_cand = h->cfg.n_real + h->cfg.n_zero;
+    if (T <= kFewTokens || T >= kTileRouterTokens || d < kSliceMinModel || T * n_cand < kSliceMinLogits ||
+        (long long)T * n_cand * d < kSliceMinProducts)
+        return 0;
+    const int tiles = ((T + kSliceTokens - 1) / kSliceTokens) * ((n_cand + kSliceCand - 1) / kSliceCand);
+    int parts = h->sm_count / tiles;
+    if (parts > d / kSliceMinPart) parts = d / kSliceMinPart;
+    parts = parts < 1 ? 1 : parts > kSliceMaxParts ? kSliceMaxParts : parts;
+    while (parts < kRouterMaxSplit && slice_smem(d, parts) > kSliceMaxSmem) ++parts;
+    const int ctas = tiles * parts;
+    return ctas > h->sm_count && 10 * ctas <= 11 * h->sm_count ? 0 : parts;
+}
+
 // block_hist (optional): pass 1 of the counting sort done here.  Every slot on a normal expert adds 1
 // to its entry of the histogram of its block of kSortTokens tokens (integer adds: the counts do not
 // depend on their order).  The histograms must be zero on entry: the call's router kernel clears them.
 template <int RPL>
 __global__ void __launch_bounds__(256)
-topk_gate_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
+topk_gate_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
                  int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist) {
     pdl_launch_dependents();
     pdl_wait();
@@ -166,7 +315,7 @@ topk_gate_kernel(const float *__restrict__ logits, int n_parts, int T, int n_rea
     if (t >= T) return;
     int my_idx;
     float my_w, v[RPL], m, den;
-    topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
+    topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
                          v, m, den, my_idx, my_w);
     if (lane < K) {
         topk_idx[(size_t)t * K + lane] = my_idx;
@@ -254,7 +403,7 @@ constexpr int kSmallThreads = 32 * (kSmallTokens / kSmallCluster);  // one warp 
 // CLUSTER = 1: up to 16 tokens fit one CTA, which saves the cluster's launch and barriers.
 template <int RPL, int CLUSTER>
 __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kSmallThreads)
-route_small_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
+route_small_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
                    int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ counts,
                    int32_t *__restrict__ offsets, int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                    const WorkLists wl, int tile_rows, int32_t *__restrict__ perm,
@@ -275,7 +424,7 @@ route_small_kernel(const float *__restrict__ logits, int n_parts, int T, int n_r
     if (t < T) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
+        topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
             topk_w[(size_t)t * K + lane] = my_w;
@@ -477,7 +626,7 @@ static_assert((kStatWarps<8> + 1) * 256 <= 12288 && (kStatWarps<16> + 1) * kMaxC
 
 template <int RPL>
 __global__ void __launch_bounds__(32 * kStatWarps<RPL>)
-topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
+topk_stats_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
                   int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist, float *__restrict__ part) {
     pdl_launch_dependents();
     constexpr int kWarps = kStatWarps<RPL>;
@@ -494,7 +643,7 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_re
     for (int t = t0 + warp; t < t1; t += kWarps) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL, 3, true>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
+        topk_gate_token<RPL, 3, true>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
                              v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
@@ -613,6 +762,7 @@ int init_route_kernels(const zeda_moe *h) {
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(router_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return -1;
+    if (cudaFuncSetAttribute(router_logits_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceMaxSmem) != cudaSuccess) return -1;
     return 0;
 }
 
@@ -642,6 +792,12 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
                                        : go(router_logits_few_kernel<8>, 8);
         return e == cudaSuccess ? 1 : -1;
     }
+    if (const int parts = n_parts ? router_slices(h, T) : 0) {
+        *n_parts = parts;
+        const cudaError_t e = launch_kernel(h->pdl, router_logits_slice_kernel, dim3((n_cand + kSliceCand - 1) / kSliceCand, (T + kSliceTokens - 1) / kSliceTokens, parts),
+                                            dim3(32 * kSliceWarps), slice_smem(d, parts), s, x, h->router_w, T, d, n_cand, logits, h->ws.block_hist, hist_ints(h, T));
+        return e == cudaSuccess ? 1 : -1;
+    }
     // split the candidates over grid.y until the grid covers the SMs about twice
     int splits = 1;
     const int max_splits = (n_cand + 7) / 8;
@@ -654,6 +810,13 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
     return e == cudaSuccess ? 1 : -1;
 }
 
+namespace {
+// what the top-K pass has to add to the sum of its slices: the bias, if they are the sliced router's
+const float *bias_of_slices(const zeda_moe *h, const float *logits, int T) {
+    return logits == h->ws.logits && router_slices(h, T) > 0 ? h->router_bias : nullptr;
+}
+}  // namespace
+
 // Top-K and routing weights of T tokens from n_parts >= 1 slices of their logits, and pass 1 of the counting sort where it
 // counts there (hist_ints).
 int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, float *stat_part, cudaStream_t s) {
@@ -662,13 +825,14 @@ int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, floa
     const Workspace &ws = h->ws;
     const int topk_warps = T <= 8 * h->sm_count ? 2 : 8;  // the loads of a few tokens spread over all SMs
     int32_t *hist_in_topk = hist_ints(h, T) ? ws.block_hist : nullptr;
+    const float *late_bias = bias_of_slices(h, logits, T);
     cudaError_t e = cudaSuccess;
 #define ZEDA_CALL_TOPK(R) \
-    e = launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
+    e = launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, \
               c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
 #define ZEDA_CALL_STATS(R) \
     e = launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
-              sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
+              sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, c.gate_mode, \
               ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
     if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
     else ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);
@@ -687,11 +851,12 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     cudaError_t e = cudaSuccess;  // of the latest launch: nothing is launched behind one that failed
     const WorkLists wl = {ws.ptile_expert, ws.ptile_row0};
     const int tile_rows = tile_rows_for(h, T);
+    const float *late_bias = bias_of_slices(h, logits, T);
     if (!stat_part && T <= kSmallTokens && c.n_real <= kSmallThreads) {
         const bool one_cta = T <= kSmallTokens / kSmallCluster;
 #define ZEDA_CALL_SMALL(R)                                                                                         \
     e = launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1> : route_small_kernel<R, kSmallCluster>,            \
-        dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
+        dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
         ws.meta, wl, tile_rows, ws.perm, out.perm, ws.inv, ws.pair_token)
         ZEDA_RPL_DISPATCH(ZEDA_CALL_SMALL);
 #undef ZEDA_CALL_SMALL

@@ -1,0 +1,44 @@
+"""The sliced router of 33 to 255 tokens at the edges of its tiles and slices, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_18643_b200 import inputs
+from test_gpu_parity import check_route, oracle_route
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,d,E,Z,K,gate", [
+    (33, 2048, 140, 60, 8, 0),     # a second tile of one token, a last candidate tile of eight
+    (64, 1088, 200, 32, 16, 2),    # four slices of 34 groups of eight elements: warps of four and of five
+    (65, 2048, 128, 64, 8, 1),     # seven slices, unequal: with the bias as many as the top-K pass requests at a time
+    (128, 8192, 33, 0, 5, 0),      # eight slices, the fullest shared memory; a last candidate tile of one
+    (129, 4096, 300, 100, 8, 0),   # as many slices as fit the shared memory, two waves
+    (255, 2048, 40, 23, 4, 1),     # an odd number of candidates
+    (129, 2048, 384, 128, 8, 0),   # a second wave of a few CTAs (the other router)
+    (65, 2048, 64, 32, 4, 0),      # the fewest products of this router
+    (64, 2048, 64, 32, 4, 0),      # (the other one's)
+    (255, 960, 40, 24, 4, 0),
+])
+@pytest.mark.parametrize("bias", [0.0, 50.0])
+def test_router_of_33_to_255_tokens(T, d, E, Z, K, gate, bias):
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("slices", T=T, d=d, He=64, E=E, Z=Z, K=K, seed=37, zero_fraction=0.4 if Z else None)
+    # a bias far above the logits: it has to be added once, behind the slices (a sum that carries it loses the logits' last bits)
+    b = torch.zeros(E + Z) if wl.router_bias is None else wl.router_bias.clone()
+    wl.router_bias = b + bias
+    m = zeda.from_workload(wl, gate_mode=gate)
+    x = wl.x.to("cuda:0")
+    l, idx, w, counts, offsets, perm, P = oracle_route(wl, gate)
+    # the logits' error: sums of fp32 products (2e-6 at most at these sizes) and one rounding of a logit of the bias' size
+    tol = 2e-6 + 2.0 ** -24 * (bias + np.abs(l).max())
+    top = -np.sort(-l.astype(np.float64), axis=1)[:, :K + 1]
+    assert float((top[:, :-1] - top[:, 1:]).min()) > 4 * tol  # so that the choice is the oracle's
+    for _ in range(2):  # each call clears the histograms that the call before it has filled
+        o = m.route(x)
+        assert np.array_equal(o["topk_idx"].cpu().numpy(), idx)
+        # a weight is a ratio of exponentials of logits: its relative error is at most the errors of two logits, and rounding
+        assert np.allclose(o["topk_w"].cpu().numpy(), w, rtol=2 * tol + 1e-6, atol=1e-30)
+        check_route(dict(o, topk_w=torch.from_numpy(np.ascontiguousarray(w))), idx, w, counts, offsets, perm, P)
+    m.close()
