@@ -521,6 +521,98 @@ slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real
     }
 }
 
+// Routing statistics, final sums by one CTA: adds up what the CTAs of the top-K pass have left in `part` (per CTA n_cand
+// selection counts, then n_cand sums of probabilities) in a fixed order.  A group of neighbouring columns (four where the
+// rows allow 16-byte loads) is shared by as many threads as fit, each adding every n-th row, sixteen requested at a time
+// and added up pairwise.
+struct StatsJob {
+    const float *part;
+    int rows;  // of part
+    float *f, *p_mean, *out;
+};
+
+__device__ __forceinline__ float4 add_columns(const float4 &a, const float4 &b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ float2 add_columns(const float2 &a, const float2 &b) { return make_float2(a.x + b.x, a.y + b.y); }
+
+constexpr int kStatFinalThreads = 256;
+
+struct StatsShared {
+    float col[2 * kMaxCand];
+    float red[5][kStatFinalThreads / 32];
+};
+
+template <typename V>
+__device__ __forceinline__ void sum_stat_columns(const StatsJob &job, int cols, float *col) {
+    constexpr int kDeep = 16;
+    const int groups = cols / (int)(sizeof(V) / sizeof(float)), segs = max(1, kStatFinalThreads / groups), seg = threadIdx.x / groups;
+    for (int c0 = 0; c0 < groups; c0 += kStatFinalThreads) {  // (more than one turn only where each group has one thread)
+        const int c = segs > 1 ? threadIdx.x - seg * groups : c0 + threadIdx.x;
+        const bool on = segs > 1 ? seg < segs : c < groups;
+        V a = {};
+        if (on)
+            for (int b0 = segs > 1 ? seg : 0; b0 < job.rows; b0 += kDeep * segs) {
+                V v[kDeep];
+#pragma unroll
+                for (int q = 0; q < kDeep; ++q)
+                    v[q] = b0 + q * segs < job.rows ? __ldcg(reinterpret_cast<const V *>(job.part + (size_t)(b0 + q * segs) * cols) + c) : V{};
+#pragma unroll
+                for (int o = kDeep / 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int q = 0; q < o; ++q) v[q] = add_columns(v[q], v[q + o]);
+                a = add_columns(a, v[0]);
+            }
+        for (int s = 0; s < segs; ++s) {  // the shares of a group in order
+            if (on && (segs == 1 || seg == s)) {
+                V *dst = reinterpret_cast<V *>(col) + c;
+                *dst = s == 0 ? a : add_columns(*dst, a);
+            }
+            __syncthreads();
+        }
+    }
+}
+
+__device__ __forceinline__ void stats_final(const StatsJob &job, int T, int K, int n_real, int n_cand, StatsShared &sh) {
+    if (n_cand % 2 == 0) sum_stat_columns<float4>(job, 2 * n_cand, sh.col);
+    else sum_stat_columns<float2>(job, 2 * n_cand, sh.col);
+    float sums[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int j = threadIdx.x; j < n_cand; j += kStatFinalThreads) {
+        const float fj = sh.col[j] / T, pj = sh.col[n_cand + j] / T;
+        if (job.f) job.f[j] = fj;
+        if (job.p_mean) job.p_mean[j] = pj;
+        const bool real = j < n_real;
+        const float add[5] = {fj * pj, real ? fj : 0.f, real ? pj : 0.f, real ? 0.f : fj, real ? 0.f : pj};
+#pragma unroll
+        for (int i = 0; i < 5; ++i) sums[i] += add[i];
+    }
+    if (!job.out) return;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const float s = warp_sum(sums[i]);
+        if ((threadIdx.x & 31) == 0) sh.red[i][threadIdx.x >> 5] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        float tot[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) tot[i] = warp_sum(threadIdx.x < kStatFinalThreads / 32 ? sh.red[i][threadIdx.x] : 0.f);
+        if (threadIdx.x == 0) {
+            job.out[0] = tot[3] / K;
+            job.out[1] = tot[0];
+            job.out[2] = tot[1] * tot[2];
+            job.out[3] = tot[3] * tot[4];
+        }
+    }
+}
+
+// as a kernel of its own, where the placement is no single kernel (more than kFoldMaxBlocks blocks of the counting sort)
+__global__ void __launch_bounds__(kStatFinalThreads)
+stats_final_kernel(const StatsJob job, int T, int K, int n_real, int n_cand) {
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ __align__(16) StatsShared sh;
+    stats_final(job, T, K, n_real, n_cand, sh);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Counting sort, passes 2 + 3 in one launch (used while the CTA histograms are few): every CTA
 // sums the histogram columns itself (pairs of each expert in earlier CTAs, and in all CTAs), scans
@@ -531,6 +623,8 @@ slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real
 // What bounds it is the chain of dependent steps, not the data: of the 5.5 us that a CTA took, 1.4 (2 blocks)
 // to 3.2 (64) went to staging and summing the histograms in shared memory and 1 to the fence of a ticket by
 // which the last CTA cleared them.
+// A statistics call adds one CTA, which takes the final sums beside the placement instead of behind it (8192 tokens of 192
+// candidates: 44.2 -> 40.8 us a call).
 // ---------------------------------------------------------------------------------------------
 constexpr int kScanThreads = 256;
 constexpr int kMaskWords = kSortTokens / 32;
@@ -540,7 +634,15 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
                        const int32_t *__restrict__ block_hist, int32_t *__restrict__ counts,
                        int32_t *__restrict__ offsets, int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                        const WorkLists wl, int tile_rows, int32_t *__restrict__ perm, int32_t *__restrict__ perm_user,
-                       int32_t *__restrict__ inv, int32_t *__restrict__ pair_token) {
+                       int32_t *__restrict__ inv, int32_t *__restrict__ pair_token, const StatsJob job, int n_cand) {
+    static_assert(kStatFinalThreads == kScanThreads, "one CTA size for both");
+    if ((int)blockIdx.x == nblk) {
+        __shared__ __align__(16) StatsShared stats;
+        pdl_launch_dependents();
+        pdl_wait();
+        stats_final(job, T, K, n_real, n_cand, stats);
+        return;
+    }
     __shared__ ScanShared sh;
     extern __shared__ __align__(16) uint32_t place_smem[];  // token masks [n_real][kMaskWords], then base[n_real]
     uint32_t *mask = place_smem;
@@ -586,7 +688,7 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
         if (e_reg[u] >= 0) atomicOr(mask + e_reg[u] * kMaskWords + (tok >> 5), 1u << (tok & 31));
     }
     __syncthreads();
-    finish_expert_scan(sh, n_real, T * K, counts, offsets, n_pairs_out, meta, wl, blockIdx.x == 0, blockIdx.x, gridDim.x, tile_rows);
+    finish_expert_scan(sh, n_real, T * K, counts, offsets, n_pairs_out, meta, wl, blockIdx.x == 0, blockIdx.x, nblk, tile_rows);
 #pragma unroll
     for (int u = 0; u < kSlotRegs; ++u) {
         const int i = threadIdx.x + kScanThreads * u;
@@ -666,67 +768,6 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, const float *__
         part[(size_t)blockIdx.x * 2 * n_cand + n_cand + j] = p;
         // pass 1 of the counting sort, as in the top-K kernel above
         if (block_hist && j < n_real && cnt[j]) atomicAdd(block_hist + (size_t)(t0 / kSortTokens) * n_real + j, cnt[j]);
-    }
-}
-
-// One CTA.  A pair of columns of the partial sums (n_cand counts, then n_cand probabilities) is shared by as
-// many threads as fit, each adding every n-th CTA's values, sixteen requested at a time.
-constexpr int kStatFinalThreads = 1024;
-
-__global__ void __launch_bounds__(kStatFinalThreads)
-stats_final_kernel(const float *__restrict__ part, int nblk, int T, int K, int n_real, int n_cand,
-                   float *__restrict__ f, float *__restrict__ p_mean, float *__restrict__ out) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ float2 seg[kStatFinalThreads];
-    __shared__ float col[2 * kMaxCand], red[5][kStatFinalThreads / 32];
-    const int cols = 2 * n_cand, segs = kStatFinalThreads / n_cand;  // n_cand pairs of columns
-    {
-        const int c = threadIdx.x % n_cand, s = threadIdx.x / n_cand;
-        float2 a = make_float2(0.f, 0.f);
-        for (int b0 = s < segs ? s : nblk; b0 < nblk; b0 += 16 * segs) {
-            float2 v[16];
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-                v[q] = b0 + q * segs < nblk ? __ldcg(reinterpret_cast<const float2 *>(part + (size_t)(b0 + q * segs) * cols) + c) : make_float2(0.f, 0.f);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) { a.x += v[q].x; a.y += v[q].y; }
-        }
-        seg[threadIdx.x] = a;
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < cols; c += kStatFinalThreads) {
-        float a = 0.f;
-        for (int s = 0; s < segs; ++s) {
-            const float2 v = seg[s * n_cand + (c >> 1)];
-            a += c & 1 ? v.y : v.x;
-        }
-        col[c] = a / T;
-        if (c < n_cand) { if (f) f[c] = col[c]; }
-        else if (p_mean) p_mean[c - n_cand] = col[c];
-    }
-    __syncthreads();
-    if (!out) return;
-    const int j = threadIdx.x;
-    const float fj = j < n_cand ? col[j] : 0.f, pj = j < n_cand ? col[n_cand + j] : 0.f;
-    const bool real = j < n_real;
-    const float sums[5] = {fj * pj, real ? fj : 0.f, real ? pj : 0.f, real ? 0.f : fj, real ? 0.f : pj};
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const float s = warp_sum(sums[i]);
-        if ((j & 31) == 0) red[i][j >> 5] = s;
-    }
-    __syncthreads();
-    if (j < 32) {
-        float tot[5];
-#pragma unroll
-        for (int i = 0; i < 5; ++i) tot[i] = warp_sum(red[i][j]);
-        if (j == 0) {
-            out[0] = tot[3] / K;
-            out[1] = tot[0];
-            out[2] = tot[1] * tot[2];
-            out[3] = tot[3] * tot[4];
-        }
     }
 }
 
@@ -842,7 +883,7 @@ int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, floa
 }
 
 int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s, int n_parts,
-                             float *stat_part) {
+                             const StatsOut *stats) {
     const zeda_moe_config_t &c = h->cfg;
     const int n_cand = c.n_real + c.n_zero, K = c.top_k;
     const Workspace &ws = h->ws;
@@ -852,7 +893,10 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     const WorkLists wl = {ws.ptile_expert, ws.ptile_row0};
     const int tile_rows = tile_rows_for(h, T);
     const float *late_bias = bias_of_slices(h, logits, T);
-    if (!stat_part && T <= kSmallTokens && c.n_real <= kSmallThreads) {
+    float *stat_part = stats ? ws.stat_part : nullptr;
+    StatsJob job = {};
+    if (stats) job = {stat_part, n_parts == 0 ? pair_router_stat_blocks(h, T) : (T + kStatTokens - 1) / kStatTokens, stats->f, stats->p_mean, stats->out};
+    if (!stats && T <= kSmallTokens && c.n_real <= kSmallThreads) {
         const bool one_cta = T <= kSmallTokens / kSmallCluster;
 #define ZEDA_CALL_SMALL(R)                                                                                         \
     e = launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1> : route_small_kernel<R, kSmallCluster>,            \
@@ -871,10 +915,10 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         if (n_parts == 0) launches = 3;  // the slots are chosen already
         else if (launch_topk(h, logits, n_parts, T, stat_part, s) < 0) return -1;
         if (fold) {
-            e = launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk), dim3(kScanThreads),
+            e = launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk + (stats ? 1 : 0)), dim3(kScanThreads),
                               sizeof(int32_t) * (kMaskWords + 1) * c.n_real, s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
                               nblk, (const int32_t *)ws.block_hist, ws.counts, ws.offsets, out.n_pairs, ws.meta, wl, tile_rows, ws.perm,
-                              out.perm, ws.inv, ws.pair_token);
+                              out.perm, ws.inv, ws.pair_token, job, n_cand);
             launches -= 2;
         } else {
             e = launch_kernel(h->pdl, slot_hist_kernel, dim3(nblk), dim3(256), sizeof(int32_t) * c.n_real, s,
@@ -886,6 +930,10 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
             e = launch_kernel(false, slot_place_kernel, dim3(nblk), dim3(kPlaceWarps * 32), sizeof(int32_t) * kPlaceWarps * c.n_real, s,
                               (const int32_t *)ws.topk_idx, T, K, c.n_real, (const int32_t *)ws.block_hist, (const int32_t *)ws.offsets,
                               ws.perm, out.perm, ws.inv, ws.pair_token);
+            if (stats && e == cudaSuccess) {
+                e = launch_kernel(h->pdl, stats_final_kernel, dim3(1), dim3(kStatFinalThreads), 0, s, job, T, K, c.n_real, n_cand);
+                ++launches;
+            }
         }
     }
     if (e != cudaSuccess) return -1;
@@ -898,14 +946,6 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     copy(out.counts, ws.counts, c.n_real);
     copy(out.offsets, ws.offsets, c.n_real + 1);
     return e == cudaSuccess ? launches : -1;
-}
-
-int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s) {
-    const zeda_moe_config_t &c = h->cfg;
-    const cudaError_t e = launch_kernel(h->pdl, stats_final_kernel, dim3(1), dim3(kStatFinalThreads), 0, s, (const float *)h->ws.stat_part,
-                                        pair_router_path(h, T) ? pair_router_stat_blocks(h, T) : (T + kStatTokens - 1) / kStatTokens, T,
-                                        (int)c.top_k, (int)c.n_real, (int)(c.n_real + c.n_zero), f, p_mean, out);
-    return e == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace zeda

@@ -127,19 +127,19 @@ zeda_status_t check_call(zeda_moe_t *h, const void *in, int32_t T, const char *i
 }
 
 // Routing into the workspace (+ optional user copies); returns launches or <0.
-// stat_part: where a statistics call wants the partial sums of its top-K pass.
+// stats: where a statistics call wants its results; the top-K pass leaves their partial sums in the workspace.
 int route_into(zeda_moe_t *h, const __nv_bfloat16 *x, const float *logits_in, int T, const RouteOut &out, cudaStream_t s,
-               float *stat_part = nullptr) {
+               const StatsOut *stats = nullptr) {
     int n = 0, n_parts = 1;
     h->last_routed_tokens = 0;  // until every launch is in the stream, the handle holds no batch's routing
     const float *logits = logits_in;
     if (!logits) {
-        int r = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts, 0, stat_part);
+        int r = launch_router_logits(h, x, T, h->ws.logits, s, &n_parts, 0, stats ? h->ws.stat_part : nullptr);
         if (r < 0) return r;
         n += r;
         logits = h->ws.logits;
     }
-    int r = launch_route_from_logits(h, logits, T, out, s, n_parts, stat_part);
+    int r = launch_route_from_logits(h, logits, T, out, s, n_parts, stats);
     if (r < 0) return r;
     h->last_routed_tokens = T;
     return n + r;
@@ -546,11 +546,10 @@ zeda_status_t zeda_moe_stats(zeda_moe_t *h, const void *x, int32_t T, float *f, 
     if (st != ZEDA_OK || T == 0) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     RouteOut none = {};
-    int n = route_into(h, static_cast<const __nv_bfloat16 *>(x), nullptr, T, none, s, h->ws.stat_part);
+    const StatsOut stats = {f, p_mean, out};
+    int n = route_into(h, static_cast<const __nv_bfloat16 *>(x), nullptr, T, none, s, &stats);
     if (n < 0) return cuda_fail("routing launch", cudaGetLastError());
-    int r = launch_stats_final(h, T, f, p_mean, out, s);
-    if (r < 0) return cuda_fail("stats launch", cudaGetLastError());
-    h->last_launches = n + r;
+    h->last_launches = n;
     return ZEDA_OK;
 }
 

@@ -91,6 +91,10 @@ struct RouteOut {  // where one routing pass writes (user buffers or workspace)
     int32_t *n_pairs;  // optional extra copy of P
 };
 
+struct StatsOut {  // where a statistics call wants its results (each may be NULL)
+    float *f, *p_mean, *out;
+};
+
 }  // namespace zeda
 
 struct zeda_moe {
@@ -146,10 +150,8 @@ int init_route_kernels(const zeda_moe *h);
 int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float *logits, cudaStream_t s,
                          int *n_parts = nullptr, int split_T = 0, float *stat_part = nullptr);
 int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, const RouteOut &out, cudaStream_t s,
-                             int n_parts = 1, float *stat_part = nullptr);
+                             int n_parts = 1, const StatsOut *stats = nullptr);
 int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, float *stat_part, cudaStream_t s);
-// The statistics of the last routing pass, which was given ws.stat_part to leave its partial sums in.
-int launch_stats_final(const zeda_moe *h, int T, float *f, float *p_mean, float *out, cudaStream_t s);
 int router_split_pad(int n_cand);
 int init_router_tile(zeda_moe *h);
 int init_router_pair(zeda_moe *h);  // behind init_router_tile, which splits the router rows
