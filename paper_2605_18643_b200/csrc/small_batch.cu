@@ -146,6 +146,33 @@ __device__ __forceinline__ void route_here(RouteTables<SLOTS> &rt, const RouteAr
     __syncthreads();
 }
 
+// The same for one token, as far as gate/up reads it: the active experts, their positions and the token.  A warp has the
+// whole choice in its lanes, so the scan over bit masks and all but one of the barriers drop out, and the weights, which
+// only the down kernel needs, are left to the CTA that publishes the tables.
+template <int RPL, int SLOTS>
+__device__ __forceinline__ void route_one_token(RouteTables<SLOTS> &rt, const RouteArgs &ra) {
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int my_idx;
+        float my_w, v[RPL], m, den;
+        topk_gate_token<RPL>(ra.logits, 1, 0, nullptr, ra.n_real, ra.n_cand, ra.K, ZEDA_GATE_TOPK_NORM, lane, v, m, den, my_idx, my_w);
+        const bool real = lane < ra.K && my_idx < ra.n_real;
+        const int id = real ? my_idx : kMaxCand;
+        int pos = 0;
+#pragma unroll
+        for (int k = 0; k < kMaxTopK; ++k) pos += __shfl_sync(kFull, id, k) < id ? 1 : 0;  // (slots beyond K hold no expert)
+        if (real) {
+            rt.expert[pos] = id;
+            rt.off[id] = pos;
+            rt.off[id + 1] = pos + 1;  // (the next expert's too, if it is active)
+            rt.tok[pos] = 0;
+        }
+        const int n = __popc(__ballot_sync(kFull, real));
+        if (lane == 0) rt.n_tiles = n;
+    }
+    __syncthreads();
+}
+
 // What the routing pass leaves in the workspace, by one CTA; then the flag that says so.
 template <int SLOTS>
 __device__ __forceinline__ void publish_route(const RouteTables<SLOTS> &rt, const RouteArgs &ra) {
@@ -215,8 +242,10 @@ stream_gate_up_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *
     pdl_wait();
     pdl_launch_dependents();  // only now: the down kernel reads the logits or the routing results before its own wait
     if constexpr (RPL > 0) {
-        route_here<RPL>(rt, ra);
-        if (blockIdx.x == gridDim.x - 1) publish_route(rt, ra);  // the CTA with the fewest units
+        const bool publish = blockIdx.x == gridDim.x - 1;  // the CTA with the fewest units
+        if (ra.T == 1 && !publish) route_one_token<RPL>(rt, ra);
+        else route_here<RPL>(rt, ra);
+        if (publish) publish_route(rt, ra);
     } else {
         load_route_tables(rt, ra);
     }

@@ -1,0 +1,41 @@
+"""The final sums of the routing statistics at the edges of their column groups, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2605_18643_b200 import inputs
+from test_gpu_parity import oracle_route
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,E,Z,K", [
+    (40, 3, 2, 2),        # odd: pairs of columns, many threads per group
+    (1100, 200, 101, 4),  # odd and more groups than threads: two turns
+    (700, 340, 172, 8),   # as many groups of four as threads
+    (4500, 5, 5, 3),      # more rows than one turn of a group's threads takes
+])
+def test_final_sums_of_the_statistics(T, E, Z, K):
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("stats", T=T, d=64, He=64, E=E, Z=Z, K=K, seed=43, zero_fraction=0.4)
+    m = zeda.from_workload(wl)
+    x = wl.x.to("cuda:0")
+    l, idx, *_ = oracle_route(wl)
+    s = oracle.stats(l, idx, E, Z, alpha=1.0, group_w=1.0)
+    # counts are whole numbers and exact in fp32; a probability is an fp32 exponential of a logit that is off by up to 2e-5
+    f_ref, p_ref = s["f"], s["P"]
+    for _ in range(2):
+        f, p, o = m.stats(x)
+        f, p, o = (t.cpu().numpy().astype(np.float64) for t in (f, p, o))
+        assert np.allclose(f, f_ref, rtol=2e-7, atol=0) and np.allclose(p, p_ref, rtol=5e-5, atol=1e-9)
+        want = [f_ref[E:].sum() / K, (f_ref * p_ref).sum(), f_ref[:E].sum() * p_ref[:E].sum(), f_ref[E:].sum() * p_ref[E:].sum()]
+        assert np.allclose(o, want, rtol=1e-4, atol=1e-9)
+    # each result may be left out
+    out = torch.empty(4, device=x.device)
+    stream = torch.cuda.current_stream().cuda_stream
+    assert zeda.lib.zeda_moe_stats(m._h, x.data_ptr(), T, None, None, out.data_ptr(), stream) == zeda.OK
+    assert np.array_equal(out.cpu().numpy().astype(np.float64), o)
+    assert zeda.lib.zeda_moe_stats(m._h, x.data_ptr(), T, None, None, None, stream) == zeda.OK
+    m.last_counters()
+    m.close()
