@@ -18,82 +18,89 @@ __device__ __forceinline__ void fma_bf16x8(float (&acc)[8], float w, const uint4
     }
 }
 
-// One CTA per token, kCombineThreads threads, each owning every kCombineThreads-th 16-byte chunk of
-// the row (small CTAs: many tokens in flight per SM hide the dependent slot-table and row loads).
-constexpr int kCombineThreads = 64;
-
-// The token's slot table: positions of its surviving slots in the expert outputs (-1 for a zero slot),
-// the gate weights, and the summed weight of the zero slots.
-struct SlotTable {
-    int32_t pos[kMaxTopK];
-    float w[kMaxTopK];
-    float zero_mass;
-};
-
-__device__ __forceinline__ void load_slot_table(SlotTable &st, const int32_t *__restrict__ inv,
-                                                const float *__restrict__ topk_w, int t, int K) {
-    // every thread reads the table itself (K <= 16 entries, one cache line each way)
-    st.zero_mass = 0.f;
-#pragma unroll
-    for (int k = 0; k < kMaxTopK; ++k) {
-        st.pos[k] = -1;
-        st.w[k] = 0.f;
-        if (k < K) {
-            st.pos[k] = ld_ordered(inv + (size_t)t * K + k);
-            st.w[k] = __int_as_float(ld_ordered(reinterpret_cast<const int32_t *>(topk_w) + (size_t)t * K + k));
-            if (st.pos[k] < 0) st.zero_mass += st.w[k];
-        }
-    }
-}
-
-// 16-byte chunk c of y[t] in fp32: the sum of Eq. 1 in slot order.
-__device__ __forceinline__ void combine_chunk(float (&acc)[8], const SlotTable &st, const __nv_bfloat16 *__restrict__ obuf,
-                                              const __nv_bfloat16 *__restrict__ x, int t, int c, int K, int d,
-                                              int copy_experts) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
-#pragma unroll
-    for (int k0 = 0; k0 < kMaxTopK; k0 += 8) {  // eight row loads are issued before the first use
-        if (k0 >= K) break;
-        uint4 v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (k0 + k < K && st.pos[k0 + k] >= 0)
-                v[k] = __ldcg(reinterpret_cast<const uint4 *>(obuf + (size_t)st.pos[k0 + k] * d) + c);
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (k0 + k < K && st.pos[k0 + k] >= 0) fma_bf16x8(acc, st.w[k0 + k], v[k]);
-    }
-    if (copy_experts && st.zero_mass != 0.f)
-        fma_bf16x8(acc, st.zero_mass, __ldcg(reinterpret_cast<const uint4 *>(x + (size_t)t * d) + c));
-}
-
-__global__ void __launch_bounds__(kCombineThreads, 16)
-combine_kernel(const __nv_bfloat16 *__restrict__ obuf, const int32_t *__restrict__ inv,
-               const float *__restrict__ topk_w, const __nv_bfloat16 *__restrict__ x, int K, int d,
-               int copy_experts, __nv_bfloat16 *__restrict__ y) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int t = blockIdx.x;
-    SlotTable st;
-    load_slot_table(st, inv, topk_w, t, K);
-    for (int c = blockIdx.y * kCombineThreads + threadIdx.x; c < d / 8; c += gridDim.y * kCombineThreads) {
-        float acc[8];
-        combine_chunk(acc, st, obuf, x, t, c, K, d, copy_experts);
-        uint4 o;
-        uint32_t *ou = reinterpret_cast<uint32_t *>(&o);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const __nv_bfloat162 b = __floats2bfloat162_rn(acc[2 * i], acc[2 * i + 1]);
-            ou[i] = *reinterpret_cast<const uint32_t *>(&b);
-        }
-        reinterpret_cast<uint4 *>(y + (size_t)t * d)[c] = o;
-    }
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&b);
+}
+
+__device__ __forceinline__ uint4 pack_bf16x8(const float (&a)[8]) {
+    return make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]), pack_bf16(a[6], a[7]));
+}
+
+// A warp's share of a token's row: P * 32 16-byte chunks from chunk c0 on, chunk c0 + 32 p + lane in acc[p] (those beyond the
+// row stay zero).  Lane k holds slot k: its position in the expert outputs (-1 for a zero slot) and its weight.  Only the
+// surviving slots are walked, in slot order, ROWS at a time: P * ROWS loads of 16 bytes per lane in flight.
+template <int P, int ROWS>
+__device__ __forceinline__ void combine_chunks(float (&acc)[P][8], const __nv_bfloat16 *__restrict__ obuf, const int32_t *__restrict__ inv,
+                                               const float *__restrict__ topk_w, const __nv_bfloat16 *__restrict__ x, int t, int c0, int K,
+                                               int d, int copy_experts, int lane) {
+    const int my_pos = lane < K ? __ldcg(inv + (size_t)t * K + lane) : -1;
+    const float my_w = lane < K ? __ldcg(topk_w + (size_t)t * K + lane) : 0.f;
+    const unsigned real = __ballot_sync(0xffffffffu, my_pos >= 0);
+    const int c = c0 + lane, chunks = d / 8;
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[p][i] = 0.f;
+    for (unsigned left = real; left;) {  // (uniform over the warp)
+        uint4 v[ROWS][P];
+        float w[ROWS];
+        const int n = __popc(left);
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const int k = r < n ? __ffs(left) - 1 : 0;
+            left &= left - 1u;
+            w[r] = __shfl_sync(0xffffffffu, my_w, k);
+            const int pos = __shfl_sync(0xffffffffu, my_pos, k);
+            const uint4 *row = reinterpret_cast<const uint4 *>(obuf + (size_t)pos * d) + c;
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                if (r < n && c + 32 * p < chunks) v[r][p] = __ldcg(row + 32 * p);
+        }
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                if (r < n && c + 32 * p < chunks) fma_bf16x8(acc[p], w[r], v[r][p]);
+    }
+    if (!copy_experts) return;
+    float zero_mass = 0.f;  // the summed weight of the zero slots
+    for (int k = 0; k < K; ++k) {
+        const float w = __shfl_sync(0xffffffffu, my_w, k);
+        if (!(real >> k & 1u)) zero_mass += w;
+    }
+    if (zero_mass == 0.f) return;
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+        if (c + 32 * p < chunks) fma_bf16x8(acc[p], zero_mass, __ldcg(reinterpret_cast<const uint4 *>(x + (size_t)t * d) + c + 32 * p));
+}
+
+// A warp per CHUNKS * 32 chunks of a token, four warps per CTA.  Bound by the reads in flight: with every thread holding the
+// slot table itself and eight loads predicated by slot, of which the zero slots' were none, 64 threads had a token's chunks
+// one after the other.  Combine stage, us, before and now: 777 tokens of the Qwen-shaped layer 10.1 -> 8.3, 2048 tokens
+// 14.3 -> 11.9, 8192 tokens of Zipf load 42.8 -> 37.3, of the static layer 60.4 -> 58.3; 5003 tokens of the GLM-shaped
+// layer 24.5 -> 16.6.  (One chunk per lane: 10.0, 14.4, 46, 60.5, 27; four: 10.2, 19.3, 52.7, 95, 23.5.)
+// Where the warps are few all the same, one chunk per lane and eight slots at a time: twice the warps, half the round trips.
+constexpr int kCombineThreads = 128;
+constexpr int kFewWarps = 8;  // of two chunks per lane, per SM
+
+template <int CHUNKS, int ROWS>
+__global__ void __launch_bounds__(kCombineThreads, 7)
+combine_kernel(const __nv_bfloat16 *__restrict__ obuf, const int32_t *__restrict__ inv,
+               const float *__restrict__ topk_w, const __nv_bfloat16 *__restrict__ x, int T, int K, int d, int pieces,
+               int copy_experts, __nv_bfloat16 *__restrict__ y) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int id = blockIdx.x * (kCombineThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int t = id / pieces, c0 = (id - t * pieces) * 32 * CHUNKS;
+    if (t >= T) return;
+    float acc[CHUNKS][8];
+    combine_chunks<CHUNKS, ROWS>(acc, obuf, inv, topk_w, x, t, c0, K, d, copy_experts, lane);
+#pragma unroll
+    for (int p = 0; p < CHUNKS; ++p) {
+        const int c = c0 + 32 * p + lane;
+        if (c < d / 8) reinterpret_cast<uint4 *>(y + (size_t)t * d)[c] = pack_bf16x8(acc[p]);
+    }
 }
 
 // The combine fused with the glue between stacked layers: instead of storing y the CTA forms
@@ -191,13 +198,14 @@ int launch_combine(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat
 int launch_combine_rows(const zeda_moe *h, const __nv_bfloat16 *rows, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y,
                         cudaStream_t s) {
     const zeda_moe_config_t &c = h->cfg;
-    // small batches spread a row over several CTAs so that the grid still covers the SMs
-    const int chunks = c.d_model / 8;
-    int gy = 1;
-    // (777 tokens: 12.2 us with one CTA per row, 10.3 with more; 2048 tokens: 14.4, 15.2)
-    while (T * gy < 8 * h->sm_count && gy * kCombineThreads < chunks) gy *= 2;
-    const cudaError_t e = launch_kernel(h->pdl, combine_kernel, dim3(T, gy), dim3(kCombineThreads), 0, s, rows, (const int32_t *)h->ws.inv,
-                                        (const float *)h->ws.topk_w, x, c.top_k, c.d_model, (int)(c.expert_kind == ZEDA_EXPERT_COPY), y);
+    auto go = [&](auto kernel, int per_warp) {
+        const int pieces = (c.d_model / 8 + per_warp - 1) / per_warp, per_cta = kCombineThreads / 32;
+        return launch_kernel(h->pdl, kernel, dim3(((long long)T * pieces + per_cta - 1) / per_cta), dim3(kCombineThreads), 0, s, rows,
+                             (const int32_t *)h->ws.inv, (const float *)h->ws.topk_w, x, T, c.top_k, c.d_model, pieces,
+                             (int)(c.expert_kind == ZEDA_EXPERT_COPY), y);
+    };
+    const bool few = (long long)T * (c.d_model / 8) < 64ll * kFewWarps * h->sm_count;
+    const cudaError_t e = few ? go(combine_kernel<1, 8>, 32) : go(combine_kernel<2, 4>, 64);
     return e == cudaSuccess ? 1 : -1;
 }
 
