@@ -304,7 +304,7 @@ int router_slices(const zeda_moe *h, int T) {
 // block_hist (optional): pass 1 of the counting sort done here.  Every slot on a normal expert adds 1
 // to its entry of the histogram of its block of kSortTokens tokens (integer adds: the counts do not
 // depend on their order).  The histograms must be zero on entry: the call's router kernel clears them.
-template <int RPL>
+template <int RPL, bool LATE>
 __global__ void __launch_bounds__(256)
 topk_gate_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
                  int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist) {
@@ -315,7 +315,7 @@ topk_gate_kernel(const float *__restrict__ logits, int n_parts, const float *__r
     if (t >= T) return;
     int my_idx;
     float my_w, v[RPL], m, den;
-    topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
+    topk_gate_token<RPL, LATE>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
                          v, m, den, my_idx, my_w);
     if (lane < K) {
         topk_idx[(size_t)t * K + lane] = my_idx;
@@ -401,7 +401,7 @@ constexpr int kSmallCluster = 8;
 constexpr int kSmallThreads = 32 * (kSmallTokens / kSmallCluster);  // one warp per token
 
 // CLUSTER = 1: up to 16 tokens fit one CTA, which saves the cluster's launch and barriers.
-template <int RPL, int CLUSTER>
+template <int RPL, int CLUSTER, bool LATE>
 __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kSmallThreads)
 route_small_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
                    int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ counts,
@@ -424,7 +424,7 @@ route_small_kernel(const float *__restrict__ logits, int n_parts, const float *_
     if (t < T) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
+        topk_gate_token<RPL, LATE>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
             topk_w[(size_t)t * K + lane] = my_w;
@@ -523,8 +523,9 @@ slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real
 
 // Routing statistics, final sums by one CTA: adds up what the CTAs of the top-K pass have left in `part` (per CTA n_cand
 // selection counts, then n_cand sums of probabilities) in a fixed order.  A group of neighbouring columns (four where the
-// rows allow 16-byte loads) is shared by as many threads as fit, each adding every n-th row, sixteen requested at a time
-// and added up pairwise.
+// rows allow 16-byte loads) is shared by as many threads as fit, each adding every n-th row, 32 requested at a time and
+// added up pairwise (8192 tokens of 192 candidates: 45.3 us a call with the sums behind the placement, 43.5 beside it with
+// sixteen rows at a time, 36.8 with 32).
 struct StatsJob {
     const float *part;
     int rows;  // of part
@@ -543,7 +544,7 @@ struct StatsShared {
 
 template <typename V>
 __device__ __forceinline__ void sum_stat_columns(const StatsJob &job, int cols, float *col) {
-    constexpr int kDeep = 16;
+    constexpr int kDeep = 32;
     const int groups = cols / (int)(sizeof(V) / sizeof(float)), segs = max(1, kStatFinalThreads / groups), seg = threadIdx.x / groups;
     for (int c0 = 0; c0 < groups; c0 += kStatFinalThreads) {  // (more than one turn only where each group has one thread)
         const int c = segs > 1 ? threadIdx.x - seg * groups : c0 + threadIdx.x;
@@ -623,12 +624,12 @@ stats_final_kernel(const StatsJob job, int T, int K, int n_real, int n_cand) {
 // What bounds it is the chain of dependent steps, not the data: of the 5.5 us that a CTA took, 1.4 (2 blocks)
 // to 3.2 (64) went to staging and summing the histograms in shared memory and 1 to the fence of a ticket by
 // which the last CTA cleared them.
-// A statistics call adds one CTA, which takes the final sums beside the placement instead of behind it (8192 tokens of 192
-// candidates: 44.2 -> 40.8 us a call).
+// A statistics call (STATS) adds one CTA, which takes the final sums beside the placement instead of behind it.
 // ---------------------------------------------------------------------------------------------
 constexpr int kScanThreads = 256;
 constexpr int kMaskWords = kSortTokens / 32;
 
+template <bool STATS>
 __global__ void __launch_bounds__(kScanThreads)
 slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real, int nblk,
                        const int32_t *__restrict__ block_hist, int32_t *__restrict__ counts,
@@ -636,7 +637,7 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
                        const WorkLists wl, int tile_rows, int32_t *__restrict__ perm, int32_t *__restrict__ perm_user,
                        int32_t *__restrict__ inv, int32_t *__restrict__ pair_token, const StatsJob job, int n_cand) {
     static_assert(kStatFinalThreads == kScanThreads, "one CTA size for both");
-    if ((int)blockIdx.x == nblk) {
+    if (STATS && (int)blockIdx.x == nblk) {
         __shared__ __align__(16) StatsShared stats;
         pdl_launch_dependents();
         pdl_wait();
@@ -726,7 +727,7 @@ template <int RPL>
 constexpr int kStatWarps = RPL <= 8 ? 32 : 16;
 static_assert((kStatWarps<8> + 1) * 256 <= 12288 && (kStatWarps<16> + 1) * kMaxCand <= 12288, "no opt-in to more than 48 KB is made for the kernel");
 
-template <int RPL>
+template <int RPL, bool LATE>
 __global__ void __launch_bounds__(32 * kStatWarps<RPL>)
 topk_stats_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
                   int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist, float *__restrict__ part) {
@@ -745,7 +746,7 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, const float *__
     for (int t = t0 + warp; t < t1; t += kWarps) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL, 3, true>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
+        topk_gate_token<RPL, LATE, 3, true>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
                              v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
@@ -869,10 +870,10 @@ int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, floa
     const float *late_bias = bias_of_slices(h, logits, T);
     cudaError_t e = cudaSuccess;
 #define ZEDA_CALL_TOPK(R) \
-    e = launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, \
+    e = launch_kernel(h->pdl, late_bias ? topk_gate_kernel<R, true> : topk_gate_kernel<R, false>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, \
               c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
 #define ZEDA_CALL_STATS(R) \
-    e = launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
+    e = launch_kernel(h->pdl, late_bias ? topk_stats_kernel<R, true> : topk_stats_kernel<R, false>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
               sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, c.gate_mode, \
               ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
     if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
@@ -899,7 +900,8 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     if (!stats && T <= kSmallTokens && c.n_real <= kSmallThreads) {
         const bool one_cta = T <= kSmallTokens / kSmallCluster;
 #define ZEDA_CALL_SMALL(R)                                                                                         \
-    e = launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1> : route_small_kernel<R, kSmallCluster>,            \
+    e = launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1, false>                                             \
+                              : late_bias ? route_small_kernel<R, kSmallCluster, true> : route_small_kernel<R, kSmallCluster, false>, \
         dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
         ws.meta, wl, tile_rows, ws.perm, out.perm, ws.inv, ws.pair_token)
         ZEDA_RPL_DISPATCH(ZEDA_CALL_SMALL);
@@ -915,7 +917,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
         if (n_parts == 0) launches = 3;  // the slots are chosen already
         else if (launch_topk(h, logits, n_parts, T, stat_part, s) < 0) return -1;
         if (fold) {
-            e = launch_kernel(h->pdl, slot_scan_place_kernel, dim3(nblk + (stats ? 1 : 0)), dim3(kScanThreads),
+            e = launch_kernel(h->pdl, stats ? slot_scan_place_kernel<true> : slot_scan_place_kernel<false>, dim3(nblk + (stats ? 1 : 0)), dim3(kScanThreads),
                               sizeof(int32_t) * (kMaskWords + 1) * c.n_real, s, (const int32_t *)ws.topk_idx, T, K, c.n_real,
                               nblk, (const int32_t *)ws.block_hist, ws.counts, ws.offsets, out.n_pairs, ws.meta, wl, tile_rows, ws.perm,
                               out.perm, ws.inv, ws.pair_token, job, n_cand);
