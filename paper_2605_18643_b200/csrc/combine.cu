@@ -80,18 +80,18 @@ __device__ __forceinline__ void combine_chunks(float (&acc)[P][8], const __nv_bf
 // one after the other.  Combine stage, us, before and now: 777 tokens of the Qwen-shaped layer 10.1 -> 8.3, 2048 tokens
 // 14.3 -> 11.9, 8192 tokens of Zipf load 42.8 -> 37.3, of the static layer 60.4 -> 58.3; 5003 tokens of the GLM-shaped
 // layer 24.5 -> 16.6.  (One chunk per lane: 10.0, 14.4, 46, 60.5, 27; four: 10.2, 19.3, 52.7, 95, 23.5.)
-// Where the warps are few all the same, one chunk per lane and eight slots at a time: twice the warps, half the round trips.
-constexpr int kCombineThreads = 128;
+// Where the warps are few all the same, one chunk per lane and eight slots at a time: twice the warps, half the round trips,
+// and CTAs of two warps.
 constexpr int kFewWarps = 8;  // of two chunks per lane, per SM
 
-template <int CHUNKS, int ROWS>
-__global__ void __launch_bounds__(kCombineThreads, 7)
+template <int CHUNKS, int ROWS, int THREADS>
+__global__ void __launch_bounds__(THREADS, 896 / THREADS)
 combine_kernel(const __nv_bfloat16 *__restrict__ obuf, const int32_t *__restrict__ inv,
                const float *__restrict__ topk_w, const __nv_bfloat16 *__restrict__ x, int T, int K, int d, int pieces,
                int copy_experts, __nv_bfloat16 *__restrict__ y) {
     pdl_launch_dependents();
     pdl_wait();
-    const int id = blockIdx.x * (kCombineThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int id = blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int t = id / pieces, c0 = (id - t * pieces) * 32 * CHUNKS;
     if (t >= T) return;
     float acc[CHUNKS][8];
@@ -198,14 +198,14 @@ int launch_combine(const zeda_moe *h, const __nv_bfloat16 *x, int T, __nv_bfloat
 int launch_combine_rows(const zeda_moe *h, const __nv_bfloat16 *rows, const __nv_bfloat16 *x, int T, __nv_bfloat16 *y,
                         cudaStream_t s) {
     const zeda_moe_config_t &c = h->cfg;
-    auto go = [&](auto kernel, int per_warp) {
-        const int pieces = (c.d_model / 8 + per_warp - 1) / per_warp, per_cta = kCombineThreads / 32;
-        return launch_kernel(h->pdl, kernel, dim3(((long long)T * pieces + per_cta - 1) / per_cta), dim3(kCombineThreads), 0, s, rows,
+    auto go = [&](auto kernel, int per_warp, int threads) {
+        const int pieces = (c.d_model / 8 + per_warp - 1) / per_warp, per_cta = threads / 32;
+        return launch_kernel(h->pdl, kernel, dim3(((long long)T * pieces + per_cta - 1) / per_cta), dim3(threads), 0, s, rows,
                              (const int32_t *)h->ws.inv, (const float *)h->ws.topk_w, x, T, c.top_k, c.d_model, pieces,
                              (int)(c.expert_kind == ZEDA_EXPERT_COPY), y);
     };
     const bool few = (long long)T * (c.d_model / 8) < 64ll * kFewWarps * h->sm_count;
-    const cudaError_t e = few ? go(combine_kernel<1, 8>, 32) : go(combine_kernel<2, 4>, 64);
+    const cudaError_t e = few ? go(combine_kernel<1, 8, 64>, 32, 64) : go(combine_kernel<2, 4, 128>, 64, 128);
     return e == cudaSuccess ? 1 : -1;
 }
 
