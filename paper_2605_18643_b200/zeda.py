@@ -267,8 +267,8 @@ class ZedaMoE:
         G = max(1, self.cfg.ep_size)
         if send_rows is None:
             send_rows = torch.empty((T * self.K, self.d), dtype=torch.bfloat16, device=self.device)
-        send_counts = torch.empty(G, dtype=torch.int32, device=self.device)
-        expert_counts = torch.empty(self.E, dtype=torch.int32, device=self.device)
+        counts = torch.empty(G + self.E, dtype=torch.int32, device=self.device)  # side by side, so that one copy can take both
+        send_counts, expert_counts = counts[:G], counts[G:]
         _check(lib.zeda_ep_dispatch(self._h, _ptr(x), T, _ptr(send_rows), _ptr(send_counts), _ptr(expert_counts),
                                     _stream(self.device)))
         return send_rows, send_counts, expert_counts
