@@ -81,8 +81,9 @@ __device__ __forceinline__ void combine_chunks(float (&acc)[P][8], const __nv_bf
 // 14.3 -> 11.9, 8192 tokens of Zipf load 42.8 -> 37.3, of the static layer 60.4 -> 58.3; 5003 tokens of the GLM-shaped
 // layer 24.5 -> 16.6.  (One chunk per lane: 10.0, 14.4, 46, 60.5, 27; four: 10.2, 19.3, 52.7, 95, 23.5.)
 // Where the warps are few all the same, one chunk per lane and eight slots at a time: twice the warps, half the round trips,
-// and CTAs of two warps.
-constexpr int kFewWarps = 8;  // of two chunks per lane, per SM
+// and CTAs of two warps (40 tokens of the GLM-shaped layer, us a call: 164.1 before, 163.3 so, 1.2 longer in CTAs of four;
+// 193 tokens of the Qwen-shaped one, the stage: 8.1 with two chunks, 7.5 so; from 777 tokens on two chunks win, above).
+constexpr int kFewWarps = 8;  // of two chunks per lane, per SM: the line lies at 296 tokens of d 2048
 
 template <int CHUNKS, int ROWS, int THREADS>
 __global__ void __launch_bounds__(THREADS, 896 / THREADS)
