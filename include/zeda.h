@@ -131,11 +131,12 @@ zeda_status_t zeda_route_from_logits(zeda_moe_t *h, const float *logits, int32_t
                                      void *stream);
 
 /* Test entry: the fp32 router logits x * router_w^T + bias, dev [T, N+N_Z].  zeda_route and
- * zeda_moe_forward add up the same products, from 33 tokens on in another order: batches of up to
- * 4095 tokens in up to eight slices of the reduction axis that are added afterwards, most batches of
- * 4096 tokens and more (up to 256 candidates) in another kernel, which keeps no logits, in one to three.
- * Their logits can differ from these in the last bits at any T >= 33, never in the products; by how much
- * depends on the batch's size, while these depend on the token alone up to T = 255. */
+ * zeda_moe_forward route by the same bits up to 255 tokens, where a token's logits do not depend on
+ * the batch (they can differ in the last bits between batches of up to 32 tokens and larger ones).
+ * From 256 tokens on they add up the same exact products in another order: mid-sized
+ * batches in up to eight slices of the reduction axis that are added afterwards, most batches of 4096
+ * tokens and more (up to 256 candidates) in another kernel, which keeps no logits, in one to three.
+ * Their logits can differ from these in the last bits at any T >= 256, never in the products. */
 zeda_status_t zeda_router_logits(zeda_moe_t *h, const void *x, int32_t T, float *logits, void *stream);
 
 /* Layer forward, Eq. 1 (Eq. 7 / Appendix B through the configured modes).

@@ -13,86 +13,14 @@ namespace zeda {
 namespace {
 
 // ---------------------------------------------------------------------------------------------
-// Router logits, CUDA-core version: l[t, j] = <x_t, W_r[j]> + b[j] in fp32.
-// One CTA = kTok tokens (bf16 rows staged in shared memory) x a slice of the candidates; one warp
-// per candidate row, lanes striding the feature axis with 16-byte loads.
+// Router logits on the CUDA cores, up to 255 tokens: l[t, j] = <x_t, W_r[j]> + b[j] in fp32.
 // ---------------------------------------------------------------------------------------------
-constexpr int kTok = 8;
-constexpr int kRouterUnroll = 8;  // 16-byte weight loads a lane keeps in flight
-
-__global__ void __launch_bounds__(256)
-router_logits_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w,
-                     const float *__restrict__ router_bias, int T, int d, int n_cand,
-                     int cand_per_cta, float *__restrict__ logits, int32_t *__restrict__ hist, int n_hist) {
-    pdl_launch_dependents();
-    pdl_wait();
-    clear_hist(hist, n_hist);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(smem_raw);  // [kTok][d]
-    const int t0 = blockIdx.x * kTok;
-    const int nt = min(kTok, T - t0);
-    const int vec_per_row = d / 8;
-    // eight 16-byte loads in flight per thread (a plain load-store loop waits for each load in turn)
-    for (int i0 = threadIdx.x; i0 < kTok * vec_per_row; i0 += 8 * blockDim.x) {
-        uint4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * blockDim.x;
-            const int r = i / vec_per_row, c = i % vec_per_row;
-            v[u] = make_uint4(0, 0, 0, 0);
-            if (i < kTok * vec_per_row && r < nt) v[u] = __ldcg(reinterpret_cast<const uint4 *>(x + (size_t)(t0 + r) * d) + c);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * blockDim.x;
-            if (i < kTok * vec_per_row) reinterpret_cast<uint4 *>(xs + (size_t)(i / vec_per_row) * d)[i % vec_per_row] = v[u];
-        }
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j_begin = blockIdx.y * cand_per_cta;
-    const int j_end = min(n_cand, j_begin + cand_per_cta);
-    for (int j = j_begin + warp; j < j_end; j += 8) {
-        float acc[kTok];
-#pragma unroll
-        for (int r = 0; r < kTok; ++r) acc[r] = 0.f;
-        const float4 *wrow = reinterpret_cast<const float4 *>(router_w + (size_t)j * d);
-        for (int c4 = lane; c4 < d / 4; c4 += 32 * kRouterUnroll) {
-            float4 w[kRouterUnroll];
-#pragma unroll
-            for (int u = 0; u < kRouterUnroll; ++u)  // independent 16-byte loads in flight per lane
-                w[u] = (c4 + 32 * u < d / 4) ? __ldg(wrow + c4 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int u = 0; u < kRouterUnroll; ++u) {
-                if (c4 + 32 * u < d / 4) {
-#pragma unroll
-                    for (int r = 0; r < kTok; ++r) {
-                        const uint2 xv = reinterpret_cast<const uint2 *>(xs + (size_t)r * d)[c4 + 32 * u];
-                        const float x0 = __uint_as_float(xv.x << 16), x1 = __uint_as_float(xv.x & 0xffff0000u);
-                        const float x2 = __uint_as_float(xv.y << 16), x3 = __uint_as_float(xv.y & 0xffff0000u);
-                        acc[r] = fmaf(w[u].x, x0, acc[r]);
-                        acc[r] = fmaf(w[u].y, x1, acc[r]);
-                        acc[r] = fmaf(w[u].z, x2, acc[r]);
-                        acc[r] = fmaf(w[u].w, x3, acc[r]);
-                    }
-                }
-            }
-        }
-        const float b = router_bias ? __ldg(router_bias + j) : 0.f;
-#pragma unroll
-        for (int r = 0; r < kTok; ++r) {
-            const float s = warp_sum(acc[r]);
-            if (lane == 0 && r < nt) logits[(size_t)(t0 + r) * n_cand + j] = s + b;
-        }
-    }
-}
-
 // Few tokens: one candidate row per CTA, so that the rows (1.5 MB for 192 candidates of 2048) are read by
 // 192 SM-wide bursts instead of 24; the reduction axis is split over four warps.  NT tokens per CTA, all
 // of their loads in flight at once.  The row is asked into L2 before the wait for the kernel in front (a
 // prefetch only: its values are read after the wait).
 // From kTileRouterTokens on the tensor-core routers.  Their accumulators are fp32 too, but against 64 bits its logits
-// are off by 2.1e-6 of their root mean square at d 2048 (1.0e-6 at 1024, 9e-6 at 8192), these kernels' by 1.6e-7:
+// are off by 2.1e-6 of their root mean square at d 2048 (1.0e-6 at 1024, 9e-6 at 8192), these kernels' by 1.1e-7:
 // below, the CUDA cores keep them.
 constexpr int kFewTokens = 32;  // calls of at most this many tokens
 constexpr int kFewThreads = 128;
@@ -152,161 +80,209 @@ router_logits_few_kernel(const __nv_bfloat16 *__restrict__ x, const float *__res
     }
 }
 
-// Sliced router of 33 to 255 tokens: kSliceTokens x kSliceCand logits per CTA over a slice of the reduction axis, each of its
-// eight warps over an eighth of the slice, 8 x 4 logits per lane.  A warp copies what it needs into shared memory by itself,
-// all of it at once (its router rows before the wait for the kernel in front: they are the caller's constants), so a CTA
-// waits for memory once; the products then take 16 loads of 16 bytes per 256 fused multiply-adds.  (The kernel above, a warp
-// per candidate row and 8 tokens, converts every x value once per candidate and waits for each row.)  Sums are fp32, of runs
-// of 16 products, then of the runs, the warps and, in the top-K pass, the slices; the bias comes behind them.
-constexpr int kSliceTokens = 32, kSliceCand = 32, kSliceWarps = 8;
-constexpr int kSliceRedLd = 40;   // floats between the tokens of a warp's sums: the lanes of a store hit all banks
-constexpr int kSliceRun = 2;      // octets of products added up before they go to the total
-constexpr int kSliceMinPart = 256;  // elements of the reduction axis that make a slice worth it
-constexpr int kSliceMaxParts = 7;   // with the bias as many as the top-K pass requests at a time (8 where they would not fit otherwise)
-constexpr int kSliceMinModel = 1024, kSliceMinLogits = 4000;   // d, and T x candidates
-constexpr long long kSliceMinProducts = 12600000;              // T x candidates x d
-constexpr int kSliceMaxSmem = 200 * 1024;
+// Router of 33 to 255 tokens: 4 TL x kTileCand logits per cluster of CTAS CTAs, TL x 4 logits per lane.
+// The sum of a logit is the same additions in every form, so that a token's logits do not depend on its batch: 32 chains
+// (chain c: elements 4 c to 4 c + 3 of every 128), each in runs of kRunSteps x 4 products that are added up one behind the
+// other, then the chains pairwise, neighbours first, then the bias.  A warp takes a chain, a CTA kWarps of them; it sends
+// the sum of its chains, through distributed shared memory, to the CTA of the cluster that finishes the token.
+// What bounds it is shared memory and the fused multiply-adds alike (TL + 4 loads per 16 TL of them), on an SM's 8 or 4
+// warps, behind one wait for memory: a CTA asks for the first two stages of its operands at once, its router rows (the
+// caller's constants) in front of the wait for the kernel before.  The loop is short because a call meets its instructions
+// cold (unrolled by four, 64 tokens 0.9 us longer).
+//
+// Which form takes a call: that of the least work per SM.  CTAs have an SM each (where two of a cluster share one while
+// others have none, a call of 160 tokens takes 4 us longer), so the clusters that run at a time are few (33 of four CTAs, 15
+// of eight), and a second wave of them costs as much as the first: tiles are as tall as one wave needs, eight CTAs where
+// those fit.  A wave takes TL times 2 (eight CTAs) or 3 (four: twice the chains per SM, on twice the warps).  A layer with
+// small experts (weights beyond L2), us, by the forms <8,8>, <8,10>, <4,8>, <4,10>, <4,12>, <4,14>, <4,16>, and by one that
+// had a warp per candidate row and 8 tokens:
+//   d 2048, 192 candidates   T=33   55.3  56.0  56.8  57.7  60.1  61.1  61.1,  59.1
+//                            T=80   70.8  66.1  67.3  68.1  69.8  70.7  71.9,  67.4
+//                            T=160  73.2  74.2  69.8  71.1  72.8  73.7  74.5,  76.5
+//                            T=193  79.1  74.4  77.6  70.8  72.7  74.1  74.9,  76.6
+//                            T=240  84.9  80.5  77.4  79.5  72.8  74.2  75.0,  84.1
+//                            T=255  84.9  80.8  77.5  79.3  82.6  74.4  74.7,  84.1
+//   d 2048, 512              T=64  111.8 113.7 102.4 103.4 105.2 106.2 107.1, 107.9
+//                            T=255 187.7 187.4 169.0 171.7 170.3 171.5 163.1, 178.3
+//   d 8192, 300              T=33  190.8 177.7 183.6 186.6 192.9 196.4 199.5, 187.8
+//   d 512, 64                T=33   41.9  42.6  42.2  42.9  43.5  43.8  44.2,  43.0
+// (Eight CTAs and taller tiles never cost less than four and 32 tokens.)
+constexpr int kChains = 32, kRunSteps = 4;
 
-// Bytes between the rows of a warp's operands of `octets` groups of eight elements: odd multiples of 16, so that rows next
-// to one another lie in different banks.
-__host__ __device__ constexpr int slice_x_stride(int octets) { return 16 * (octets | 1); }
-__host__ __device__ constexpr int slice_w_stride(int octets) { return 32 * octets + 16; }
-__host__ __device__ constexpr int slice_warp_octets(int d, int parts) { return ((d / 8 + parts - 1) / parts + kSliceWarps - 1) / kSliceWarps; }
-
-size_t slice_smem(int d, int parts) {
-    const int n = slice_warp_octets(d, parts);
-    const size_t operands = (size_t)kSliceWarps * (kSliceTokens * slice_x_stride(n) + kSliceCand * slice_w_stride(n));
-    const size_t sums = (size_t)kSliceWarps * kSliceTokens * kSliceRedLd * sizeof(float);
-    return operands > sums ? operands : sums;
+// Two fp32 numbers side by side, and the same operation on both at once: each as by itself, bit for bit.
+using F32x2 = unsigned long long;
+__device__ __forceinline__ F32x2 f32x2(uint32_t lo, uint32_t hi) { return (F32x2)hi << 32 | lo; }
+__device__ __forceinline__ void fma_f32x2(F32x2 &acc, float a, F32x2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(f32x2(__float_as_uint(a), __float_as_uint(a))), "l"(b));
 }
+__device__ __forceinline__ void add_f32x2(F32x2 &acc, F32x2 a) { asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(a)); }
 
-__global__ void __launch_bounds__(32 * kSliceWarps, 1)
-router_logits_slice_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w, int T, int d, int n_cand,
-                           float *__restrict__ logits, int32_t *__restrict__ hist, int n_hist) {
+template <int CTAS, int TL>
+struct RouterCluster {
+    static constexpr int kCtas = CTAS, kTileTokens = 4 * TL, kTileCand = 32;
+    static constexpr int kWarps = kChains / CTAS, kThreads = 32 * kWarps;
+    static constexpr int kSteps = 8, kStage = 128 * kSteps;  // of a chain per stage; elements of a row
+    // bytes between rows: odd multiples of 16, so that rows next to one another lie in different banks
+    static constexpr int kXLd = 8 * kWarps * kSteps + 16, kWLd = 16 * kWarps * kSteps + 16;
+    static constexpr int kBuffer = kTileTokens * kXLd + kTileCand * kWLd;
+    static constexpr int kRedLd = 40;                // floats between the tokens of a chain's sums: the lanes of a store hit all banks
+    static constexpr int kOwn = kTileTokens / CTAS;  // tokens that a CTA finishes
+    static constexpr int kUsed = 2 * kBuffer + kTileTokens * kTileCand * (int)sizeof(float);
+    // more than half of an SM's shared memory: CTAs of a cluster that share an SM, while others have none, take twice as long
+    static constexpr int kSmem = kUsed > 120 * 1024 ? kUsed : 120 * 1024;
+    static_assert(kSteps % kRunSteps == 0, "no run of products crosses a stage");
+    static_assert(kWarps * kTileTokens * kRedLd * 4 <= 2 * kBuffer, "the sums take the operands' room");
+};
+
+template <int CTAS, int TL>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(RouterCluster<CTAS, TL>::kThreads, 1)
+router_logits_cluster_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ router_w, const float *__restrict__ router_bias,
+                             int T, int d, int n_cand, float *__restrict__ logits, int32_t *__restrict__ hist, int n_hist) {
+    using C = RouterCluster<CTAS, TL>;
     pdl_launch_dependents();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j0 = blockIdx.x * kSliceCand, t0 = blockIdx.y * kSliceTokens, part = blockIdx.z, parts = gridDim.z;
-    const int o0 = d / 8 * part / parts, o1 = d / 8 * (part + 1) / parts;
-    const int q0 = o0 + (o1 - o0) * warp / kSliceWarps, n = o0 + (o1 - o0) * (warp + 1) / kSliceWarps - q0;  // this warp's octets, 4 to 16
-    const int octets = slice_warp_octets(d, parts);
-    const int xs = slice_x_stride(octets), ws = slice_w_stride(octets);
-    unsigned char *xb = smem_raw + warp * (kSliceTokens * xs + kSliceCand * ws), *wb = xb + kSliceTokens * xs;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    extern __shared__ __align__(16) unsigned char smem_raw[];  // two stages of tokens and router rows, then the sums received
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = blockIdx.x % CTAS;
+    const int j0 = blockIdx.x / CTAS * C::kTileCand, t0 = blockIdx.y * C::kTileTokens;
+    const int rows_w = min(C::kTileCand, n_cand - j0), rows_x = min(C::kTileTokens, T - t0);
+    const int n_stages = (d + C::kStage - 1) / C::kStage;
     auto copy16 = [](void *dst, const void *src) {
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
     };
-    const int rows_w = min(kSliceCand, n_cand - j0), rows_x = min(kSliceTokens, T - t0);
-    {
-        const uint32_t inv = (1u << 20) / (2 * n) + 1;  // i / (2 n) = i * inv >> 20 for the i below
-        for (int i = lane; i < rows_w * 2 * n; i += 32) {
-            const int r = i * inv >> 20, c = i - r * 2 * n;
-            copy16(wb + r * ws + 16 * c, router_w + (size_t)(j0 + r) * d + 8 * q0 + 4 * c);
-        }
-    }
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    // Of every 128 elements of a row the CTA takes its chains' 4 x kWarps.  (Rows beyond the call's and elements beyond the
+    // row are not copied: the former's sums are not stored, the latter are not multiplied.)
+    auto copy_w = [&](int stage) {
+        unsigned char *dst = smem_raw + (stage & 1) * C::kBuffer + C::kTileTokens * C::kXLd;
+        constexpr int kPieces = C::kSteps * C::kWarps;  // of 16 bytes, of a row
+        const int piece = threadIdx.x % kPieces;
+        const int col = stage * C::kStage + 128 * (piece / C::kWarps) + 4 * (rank * C::kWarps + piece % C::kWarps);
+        if (col < d)
+#pragma unroll
+            for (int r = threadIdx.x / kPieces; r < C::kTileCand; r += C::kThreads / kPieces)
+                if (r < rows_w) copy16(dst + r * C::kWLd + 16 * piece, router_w + (size_t)(j0 + r) * d + col);
+    };
+    auto copy_x = [&](int stage) {  // (two chains to a piece: d is a multiple of 64, so both are in the row or neither)
+        unsigned char *dst = smem_raw + (stage & 1) * C::kBuffer;
+        constexpr int kPairs = C::kWarps / 2, kPieces = C::kSteps * kPairs;
+        const int piece = threadIdx.x % kPieces;
+        const int col = stage * C::kStage + 128 * (piece / kPairs) + 4 * rank * C::kWarps + 8 * (piece % kPairs);
+        if (col < d)
+#pragma unroll
+            for (int r = threadIdx.x / kPieces; r < C::kTileTokens; r += C::kThreads / kPieces)
+                if (r < rows_x) copy16(dst + r * C::kXLd + 16 * piece, x + (size_t)(t0 + r) * d + col);
+    };
+    copy_w(0);
+    if (n_stages > 1) copy_w(1);
+    commit();
     pdl_wait();
-    {
-        const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        for (int i = cta * blockDim.x + threadIdx.x; i < n_hist; i += gridDim.x * gridDim.y * gridDim.z * blockDim.x) hist[i] = 0;
-    }
-    {
-        const uint32_t inv = (1u << 20) / n + 1;
-        for (int i = lane; i < rows_x * n; i += 32) {
-            const int r = i * inv >> 20, c = i - r * n;
-            copy16(xb + r * xs + 16 * c, x + (size_t)(t0 + r) * d + 8 * (q0 + c));
-        }
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncwarp();
-    // lane: tokens tg + 4 i, candidates cg + 8 j (rows beyond the call's hold what was there: their sums are not stored)
+    clear_hist(hist, n_hist);
+    copy_x(0);
+    commit();
+    if (n_stages > 1) copy_x(1);
+    commit();
+    // lane: tokens tg + 4 i, candidates cg + 8 j
     const int tg = lane >> 3, cg = lane & 7;
-    float acc[8][4], tot[8][4];
+    F32x2 acc[TL / 2][4], tot[TL / 2][4];  // of tokens tg + 4 i and tg + 4 (i + TL / 2)
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < TL / 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = tot[i][j] = 0.f;
-    for (int q = 0; q < n; ++q) {
-        uint4 xv[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) xv[i] = *reinterpret_cast<const uint4 *>(xb + (tg + 4 * i) * xs + 16 * q);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int j = 0; j < 4; ++j) acc[i][j] = tot[i][j] = 0;
+    for (int stage = 0; stage < n_stages; ++stage) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");  // all but the next stage's
+        __syncthreads();
+        const unsigned char *xb = smem_raw + (stage & 1) * C::kBuffer + 8 * warp;
+        const unsigned char *wb = smem_raw + (stage & 1) * C::kBuffer + C::kTileTokens * C::kXLd + 16 * warp;
+        const int left = d - stage * C::kStage - 4 * (rank * C::kWarps + warp);  // of the row, from the chain's next element on
+        const int steps = min(C::kSteps, (left + 127) / 128);
+#pragma unroll 1  // (a short loop: a call meets its instructions cold)
+        for (int u = 0; u < steps; ++u) {
+            uint2 xv[TL];
             float4 w[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4 *>(wb + (cg + 8 * j) * ws + 32 * q + 16 * h);
+            for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4 *>(wb + (cg + 8 * j) * C::kWLd + 16 * C::kWarps * u);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const uint32_t lo = h ? xv[i].z : xv[i].x, hi = h ? xv[i].w : xv[i].y;
-                const float x0 = __uint_as_float(lo << 16), x1 = __uint_as_float(lo & 0xffff0000u);
-                const float x2 = __uint_as_float(hi << 16), x3 = __uint_as_float(hi & 0xffff0000u);
+            for (int i = 0; i < TL; ++i) xv[i] = *reinterpret_cast<const uint2 *>(xb + (tg + 4 * i) * C::kXLd + 8 * C::kWarps * u);
+#pragma unroll
+            for (int i = 0; i < TL / 2; ++i) {
+                const uint2 a = xv[i], b = xv[i + TL / 2];
+                const F32x2 x0 = f32x2(a.x << 16, b.x << 16), x1 = f32x2(a.x & 0xffff0000u, b.x & 0xffff0000u);
+                const F32x2 x2 = f32x2(a.y << 16, b.y << 16), x3 = f32x2(a.y & 0xffff0000u, b.y & 0xffff0000u);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    acc[i][j] = fmaf(w[j].x, x0, acc[i][j]);
-                    acc[i][j] = fmaf(w[j].y, x1, acc[i][j]);
-                    acc[i][j] = fmaf(w[j].z, x2, acc[i][j]);
-                    acc[i][j] = fmaf(w[j].w, x3, acc[i][j]);
+                    fma_f32x2(acc[i][j], w[j].x, x0);
+                    fma_f32x2(acc[i][j], w[j].y, x1);
+                    fma_f32x2(acc[i][j], w[j].z, x2);
+                    fma_f32x2(acc[i][j], w[j].w, x3);
                 }
             }
-        }
-        if ((q + 1) % kSliceRun == 0 || q + 1 == n) {  // (uniform)
+            if ((u + 1) % kRunSteps == 0 || u + 1 == steps) {  // (uniform over the warp)
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < TL / 2; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) { tot[i][j] += acc[i][j]; acc[i][j] = 0.f; }
+                    for (int j = 0; j < 4; ++j) { add_f32x2(tot[i][j], acc[i][j]); acc[i][j] = 0; }
+            }
         }
+        __syncthreads();  // the stage has been read: its room takes another, or the sums
+        if (stage + 2 < n_stages) {
+            copy_w(stage + 2);
+            copy_x(stage + 2);
+        }
+        commit();
     }
-    __syncthreads();  // the operands have been read: their room takes the warps' sums
-    float *red = reinterpret_cast<float *>(smem_raw);  // [kSliceWarps][kSliceTokens][kSliceRedLd]
+    float *red = reinterpret_cast<float *>(smem_raw);  // [kWarps][kTileTokens][kRedLd]
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < TL; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) red[(warp * kSliceTokens + tg + 4 * i) * kSliceRedLd + cg + 8 * j] = tot[i][j];
+        for (int j = 0; j < 4; ++j)
+            red[(warp * C::kTileTokens + tg + 4 * i) * C::kRedLd + cg + 8 * j] = __uint_as_float((uint32_t)(tot[i % (TL / 2)][j] >> (i < TL / 2 ? 0 : 32)));
     __syncthreads();
-    const int r = threadIdx.x >> 3, c = (threadIdx.x & 7) * 4;  // four candidates of a token per thread
-    float4 v[kSliceWarps];
+    auto cluster = cooperative_groups::this_cluster();
+    float *got = reinterpret_cast<float *>(smem_raw + 2 * C::kBuffer);  // [CTAS][kOwn][kTileCand]
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // (every CTA of the cluster has started)
+    for (int i = threadIdx.x; i < C::kTileTokens * C::kTileCand / 4; i += C::kThreads) {  // four candidates of a token
+        const int t = i / (C::kTileCand / 4), c = i % (C::kTileCand / 4) * 4;
+        float4 v[C::kWarps];
 #pragma unroll
-    for (int q = 0; q < kSliceWarps; ++q) v[q] = *reinterpret_cast<const float4 *>(red + (q * kSliceTokens + r) * kSliceRedLd + c);
+        for (int q = 0; q < C::kWarps; ++q) v[q] = *reinterpret_cast<const float4 *>(red + (q * C::kTileTokens + t) * C::kRedLd + c);
 #pragma unroll
-    for (int o = 1; o < kSliceWarps; o *= 2)
+        for (int o = 1; o < C::kWarps; o *= 2)
 #pragma unroll
-        for (int q = 0; q < kSliceWarps; q += 2 * o) v[q] = make_float4(v[q].x + v[q + o].x, v[q].y + v[q + o].y, v[q].z + v[q + o].z, v[q].w + v[q + o].w);
-    if (r >= rows_x) return;
-    float *out = logits + ((size_t)part * T + t0 + r) * n_cand + j0;
-    const float s[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+            for (int q = 0; q < C::kWarps; q += 2 * o) v[q] = make_float4(v[q].x + v[q + o].x, v[q].y + v[q + o].y, v[q].z + v[q + o].z, v[q].w + v[q + o].w);
+        *reinterpret_cast<float4 *>(cluster.map_shared_rank(got, t / C::kOwn) + (rank * C::kOwn + t % C::kOwn) * C::kTileCand + c) = v[0];
+    }
+    cluster.sync();
+    for (int own = warp; own < C::kOwn; own += C::kWarps) {  // a token per warp, a candidate per lane
+        const int r = rank * C::kOwn + own;
+        float v[CTAS];
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-        if (c + j < rows_w) out[c + j] = s[j];
+        for (int q = 0; q < CTAS; ++q) v[q] = got[(q * C::kOwn + own) * C::kTileCand + lane];
+#pragma unroll
+        for (int o = 1; o < CTAS; o *= 2)
+#pragma unroll
+            for (int q = 0; q < CTAS; q += 2 * o) v[q] += v[q + o];
+        if (r < rows_x && lane < rows_w) logits[(size_t)(t0 + r) * n_cand + j0 + lane] = v[0] + (router_bias ? __ldg(router_bias + j0 + lane) : 0.f);
+    }
 }
 
-// Slices of the reduction axis for a call of T tokens by that kernel, 0 where the one above takes the call: as many as give
-// every SM at most one CTA, but no fewer than fit its shared memory.  Routing pass, us, by the kernel above and by this:
-//   d 2048, 192 candidates   T=33 13.8, 11.2    T=64 13.2, 11.4    T=128 15.7, 12.7   T=193 20.2, 15.9   T=255 27.0, 16.7
-//   d 2048, 96               T=33 11.2, 11.9    T=64 11.9, 12.2    T=96 13.7, 12.1    T=193 15.3, 11.7   T=255 15.3, 12.3
-//   d 1024, 96               T=33 9.3, 10.8     T=64 10.1, 11.0    T=128 11.2, 11.7   T=129 12.6, 11.5   T=255 13.2, 11.8
-//   d 2048, 12               T=33 8.9, 9.7      T=128 9.3, 10.1    T=255 11.0, 10.4
-//   d 8192, 400              T=33 39.2, 36.6    T=128 103.5, 51.5  T=255 171, 85
-//   d 2048, 512              T=33 20.6, 19.3    T=128 34.6, 25.7   T=129 31.3, 35.1   T=160 40.2, 33.9
-// So few logits stay there, and calls (the last row's 129 tokens) whose last wave here would be a handful of CTAs.  The
-// weights' distance from 64 bits, 2-norms: d 1024 1.0e-7 and 9.3e-8, d 2048 1.6e-7 and 1.3e-7, d 8192 5e-7 and 2.6e-7.
-int router_slices(const zeda_moe *h, int T) {
-    const int d = h->cfg.d_model, n_cand = h->cfg.n_real + h->cfg.n_zero;
-    if (T <= kFewTokens || T >= kTileRouterTokens || d < kSliceMinModel || T * n_cand < kSliceMinLogits ||
-        (long long)T * n_cand * d < kSliceMinProducts)
-        return 0;
-    const int tiles = ((T + kSliceTokens - 1) / kSliceTokens) * ((n_cand + kSliceCand - 1) / kSliceCand);
-    int parts = h->sm_count / tiles;
-    if (parts > d / kSliceMinPart) parts = d / kSliceMinPart;
-    parts = parts < 1 ? 1 : parts > kSliceMaxParts ? kSliceMaxParts : parts;
-    while (parts < kRouterMaxSplit && slice_smem(d, parts) > kSliceMaxSmem) ++parts;
-    const int ctas = tiles * parts;
-    return ctas > h->sm_count && 10 * ctas <= 11 * h->sm_count ? 0 : parts;
+// The forms; of equal cost the later one takes a call.
+template <typename F>
+void each_router_form(F f) {
+    f(RouterCluster<8, 8>(), router_logits_cluster_kernel<8, 8>);
+    f(RouterCluster<8, 10>(), router_logits_cluster_kernel<8, 10>);
+    f(RouterCluster<4, 8>(), router_logits_cluster_kernel<4, 8>);
+    f(RouterCluster<4, 10>(), router_logits_cluster_kernel<4, 10>);
+    f(RouterCluster<4, 12>(), router_logits_cluster_kernel<4, 12>);
+    f(RouterCluster<4, 14>(), router_logits_cluster_kernel<4, 14>);
+    f(RouterCluster<4, 16>(), router_logits_cluster_kernel<4, 16>);
 }
 
 // block_hist (optional): pass 1 of the counting sort done here.  Every slot on a normal expert adds 1
 // to its entry of the histogram of its block of kSortTokens tokens (integer adds: the counts do not
 // depend on their order).  The histograms must be zero on entry: the call's router kernel clears them.
-template <int RPL, bool LATE>
+template <int RPL>
 __global__ void __launch_bounds__(256)
-topk_gate_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
+topk_gate_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
                  int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist) {
     pdl_launch_dependents();
     pdl_wait();
@@ -315,7 +291,7 @@ topk_gate_kernel(const float *__restrict__ logits, int n_parts, const float *__r
     if (t >= T) return;
     int my_idx;
     float my_w, v[RPL], m, den;
-    topk_gate_token<RPL, LATE>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
+    topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
                          v, m, den, my_idx, my_w);
     if (lane < K) {
         topk_idx[(size_t)t * K + lane] = my_idx;
@@ -401,9 +377,9 @@ constexpr int kSmallCluster = 8;
 constexpr int kSmallThreads = 32 * (kSmallTokens / kSmallCluster);  // one warp per token
 
 // CLUSTER = 1: up to 16 tokens fit one CTA, which saves the cluster's launch and barriers.
-template <int RPL, int CLUSTER, bool LATE>
+template <int RPL, int CLUSTER>
 __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kSmallThreads)
-route_small_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
+route_small_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
                    int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ counts,
                    int32_t *__restrict__ offsets, int32_t *__restrict__ n_pairs_out, int32_t *__restrict__ meta,
                    const WorkLists wl, int tile_rows, int32_t *__restrict__ perm,
@@ -424,7 +400,7 @@ route_small_kernel(const float *__restrict__ logits, int n_parts, const float *_
     if (t < T) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL, LATE>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
+        topk_gate_token<RPL>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane, v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
             topk_w[(size_t)t * K + lane] = my_w;
@@ -727,9 +703,9 @@ template <int RPL>
 constexpr int kStatWarps = RPL <= 8 ? 32 : 16;
 static_assert((kStatWarps<8> + 1) * 256 <= 12288 && (kStatWarps<16> + 1) * kMaxCand <= 12288, "no opt-in to more than 48 KB is made for the kernel");
 
-template <int RPL, bool LATE>
+template <int RPL>
 __global__ void __launch_bounds__(32 * kStatWarps<RPL>)
-topk_stats_kernel(const float *__restrict__ logits, int n_parts, const float *__restrict__ late_bias, int T, int n_real, int n_cand, int K, int gate_mode,
+topk_stats_kernel(const float *__restrict__ logits, int n_parts, int T, int n_real, int n_cand, int K, int gate_mode,
                   int32_t *__restrict__ topk_idx, float *__restrict__ topk_w, int32_t *__restrict__ block_hist, float *__restrict__ part) {
     pdl_launch_dependents();
     constexpr int kWarps = kStatWarps<RPL>;
@@ -746,7 +722,7 @@ topk_stats_kernel(const float *__restrict__ logits, int n_parts, const float *__
     for (int t = t0 + warp; t < t1; t += kWarps) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL, LATE, 3, true>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, late_bias, n_real, n_cand, K, gate_mode, lane,
+        topk_gate_token<RPL, 3, true>(logits + (size_t)t * n_cand, n_parts, (size_t)T * n_cand, n_real, n_cand, K, gate_mode, lane,
                              v, m, den, my_idx, my_w);
         if (lane < K) {
             topk_idx[(size_t)t * K + lane] = my_idx;
@@ -799,12 +775,27 @@ int launch_token_zero_share(const zeda_moe *h, int T, float *out, cudaStream_t s
     return e == cudaSuccess ? 1 : -1;
 }
 
-int init_route_kernels(const zeda_moe *h) {
-    const size_t smem = (size_t)kTok * h->cfg.d_model * sizeof(__nv_bfloat16);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(router_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return -1;
-    if (cudaFuncSetAttribute(router_logits_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceMaxSmem) != cudaSuccess) return -1;
+int init_route_kernels(zeda_moe *h) {
+    cudaError_t e = cudaSuccess;
+    each_router_form([&](auto form, auto kernel) {
+        using C = decltype(form);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
+        if (e != cudaSuccess) return;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(C::kCtas);
+        cfg.blockDim = dim3(C::kThreads);
+        cfg.dynamicSmemBytes = C::kSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = C::kCtas;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int &clusters = C::kCtas == 8 ? h->router_clusters8 : h->router_clusters4;
+        if (!clusters) e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+        if (e == cudaSuccess && clusters < 1) clusters = 1;
+    });
+    if (e != cudaSuccess) return -1;
     return 0;
 }
 
@@ -816,13 +807,12 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
         return launch_router_topk_pair(h, x, T, split_T, hist_ints(h, T) ? h->ws.block_hist : nullptr, stat_part, s);
     }
     // large batches: the GEMM goes to the tensor cores (exact three-way bf16 split of the weights)
-    if (T >= kTileRouterTokens && h->router_maps) {
+    if (T >= kTileRouterTokens) {
         const int split = n_parts ? router_split_factor(h, split_T > T ? split_T : T) : 1;
         if (n_parts) *n_parts = split;
         return launch_router_logits_tile(h, x, T, logits, split, s);
     }
     const int d = h->cfg.d_model, n_cand = h->cfg.n_real + h->cfg.n_zero;
-    const int tiles = (T + kTok - 1) / kTok;
     if (T <= kFewTokens) {
         auto go = [&](auto kernel, int per_cta) {
             return launch_kernel(h->pdl, kernel, dim3(n_cand, (T + per_cta - 1) / per_cta), dim3(kFewThreads), 0, s, x, h->router_w,
@@ -834,30 +824,26 @@ int launch_router_logits(const zeda_moe *h, const __nv_bfloat16 *x, int T, float
                                        : go(router_logits_few_kernel<8>, 8);
         return e == cudaSuccess ? 1 : -1;
     }
-    if (const int parts = n_parts ? router_slices(h, T) : 0) {
-        *n_parts = parts;
-        const cudaError_t e = launch_kernel(h->pdl, router_logits_slice_kernel, dim3((n_cand + kSliceCand - 1) / kSliceCand, (T + kSliceTokens - 1) / kSliceTokens, parts),
-                                            dim3(32 * kSliceWarps), slice_smem(d, parts), s, x, h->router_w, T, d, n_cand, logits, h->ws.block_hist, hist_ints(h, T));
-        return e == cudaSuccess ? 1 : -1;
-    }
-    // split the candidates over grid.y until the grid covers the SMs about twice
-    int splits = 1;
-    const int max_splits = (n_cand + 7) / 8;
-    while (tiles * splits < 2 * h->sm_count && splits < max_splits) splits *= 2;
-    if (splits > max_splits) splits = max_splits;
-    const int per = (n_cand + splits - 1) / splits;
-    const size_t smem = (size_t)kTok * d * sizeof(__nv_bfloat16);
-    const cudaError_t e = launch_kernel(h->pdl, router_logits_kernel, dim3(tiles, (n_cand + per - 1) / per), dim3(256), smem, s,
-                                        x, h->router_w, h->router_bias, T, d, n_cand, per, logits, h->ws.block_hist, hist_ints(h, T));
+    // the form of the least work per SM (at the kernel)
+    int best = 0, of_best = 0, at = 0;
+    auto tiles = [](int n, int per) { return (n + per - 1) / per; };
+    each_router_form([&](auto form, auto) {
+        using C = decltype(form);
+        const int clusters = tiles(n_cand, C::kTileCand) * tiles(T, C::kTileTokens), wave = C::kCtas == 8 ? h->router_clusters8 : h->router_clusters4;
+        const int cost = tiles(clusters, wave) * C::kTileTokens * (C::kCtas == 8 ? 2 : 3);
+        if (at == 0 || cost <= of_best) { best = at; of_best = cost; }
+        ++at;
+    });
+    cudaError_t e = cudaSuccess;
+    at = 0;
+    each_router_form([&](auto form, auto kernel) {
+        using C = decltype(form);
+        if (at++ == best)
+            e = launch_kernel(h->pdl, kernel, dim3(tiles(n_cand, C::kTileCand) * C::kCtas, tiles(T, C::kTileTokens)), dim3(C::kThreads), C::kSmem, s, x,
+                              h->router_w, h->router_bias, T, d, n_cand, logits, h->ws.block_hist, hist_ints(h, T));
+    });
     return e == cudaSuccess ? 1 : -1;
 }
-
-namespace {
-// what the top-K pass has to add to the sum of its slices: the bias, if they are the sliced router's
-const float *bias_of_slices(const zeda_moe *h, const float *logits, int T) {
-    return logits == h->ws.logits && router_slices(h, T) > 0 ? h->router_bias : nullptr;
-}
-}  // namespace
 
 // Top-K and routing weights of T tokens from n_parts >= 1 slices of their logits, and pass 1 of the counting sort where it
 // counts there (hist_ints).
@@ -867,14 +853,13 @@ int launch_topk(const zeda_moe *h, const float *logits, int n_parts, int T, floa
     const Workspace &ws = h->ws;
     const int topk_warps = T <= 8 * h->sm_count ? 2 : 8;  // the loads of a few tokens spread over all SMs
     int32_t *hist_in_topk = hist_ints(h, T) ? ws.block_hist : nullptr;
-    const float *late_bias = bias_of_slices(h, logits, T);
     cudaError_t e = cudaSuccess;
 #define ZEDA_CALL_TOPK(R) \
-    e = launch_kernel(h->pdl, late_bias ? topk_gate_kernel<R, true> : topk_gate_kernel<R, false>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, \
+    e = launch_kernel(h->pdl, topk_gate_kernel<R>, dim3((T + topk_warps - 1) / topk_warps), dim3(32 * topk_warps), 0, s, logits, n_parts, T, c.n_real, n_cand, K, \
               c.gate_mode, ws.topk_idx, ws.topk_w, hist_in_topk)
 #define ZEDA_CALL_STATS(R) \
-    e = launch_kernel(h->pdl, late_bias ? topk_stats_kernel<R, true> : topk_stats_kernel<R, false>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
-              sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, c.gate_mode, \
+    e = launch_kernel(h->pdl, topk_stats_kernel<R>, dim3((T + kStatTokens - 1) / kStatTokens), dim3(32 * kStatWarps<R>), \
+              sizeof(float) * (kStatWarps<R> + 1) * n_cand, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, \
               ws.topk_idx, ws.topk_w, hist_in_topk, stat_part)
     if (stat_part) ZEDA_RPL_DISPATCH(ZEDA_CALL_STATS);
     else ZEDA_RPL_DISPATCH(ZEDA_CALL_TOPK);
@@ -893,16 +878,14 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
     cudaError_t e = cudaSuccess;  // of the latest launch: nothing is launched behind one that failed
     const WorkLists wl = {ws.ptile_expert, ws.ptile_row0};
     const int tile_rows = tile_rows_for(h, T);
-    const float *late_bias = bias_of_slices(h, logits, T);
     float *stat_part = stats ? ws.stat_part : nullptr;
     StatsJob job = {};
     if (stats) job = {stat_part, n_parts == 0 ? pair_router_stat_blocks(h, T) : (T + kStatTokens - 1) / kStatTokens, stats->f, stats->p_mean, stats->out};
     if (!stats && T <= kSmallTokens && c.n_real <= kSmallThreads) {
         const bool one_cta = T <= kSmallTokens / kSmallCluster;
 #define ZEDA_CALL_SMALL(R)                                                                                         \
-    e = launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1, false>                                             \
-                              : late_bias ? route_small_kernel<R, kSmallCluster, true> : route_small_kernel<R, kSmallCluster, false>, \
-        dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, n_parts, late_bias, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
+    e = launch_kernel(h->pdl, one_cta ? route_small_kernel<R, 1> : route_small_kernel<R, kSmallCluster>,            \
+        dim3(one_cta ? 1 : kSmallCluster), dim3(kSmallThreads), 0, s, logits, n_parts, T, c.n_real, n_cand, K, c.gate_mode, ws.topk_idx, ws.topk_w, ws.counts, ws.offsets, out.n_pairs,   \
         ws.meta, wl, tile_rows, ws.perm, out.perm, ws.inv, ws.pair_token)
         ZEDA_RPL_DISPATCH(ZEDA_CALL_SMALL);
 #undef ZEDA_CALL_SMALL

@@ -167,10 +167,10 @@ __device__ __forceinline__ void topk_gate_select(const float (&v)[N][RPL], int n
 
 // The same with the token's logits read from memory (and returned in v), one token.
 // The row may arrive as n_parts partial sums, part_stride floats apart; they are added in order, PB slices
-// requested at a time (one slice after another is a chain of L2 round trips); with LATE, late_bias behind them.
-template <int RPL, bool LATE = false, int PB = (RPL <= 8 ? 7 : 3), bool DEN = false>
+// requested at a time (one slice after another is a chain of L2 round trips).
+template <int RPL, int PB = (RPL <= 8 ? 7 : 3), bool DEN = false>
 __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, int n_parts, size_t part_stride,
-                                                const float *__restrict__ late_bias, int n_real, int n_cand, int K, int gate_mode, int lane,
+                                                int n_real, int n_cand, int K, int gate_mode, int lane,
                                                 float (&v)[RPL], float &m, float &den, int &my_idx, float &my_w) {
     float u[1][RPL], mm[1], dd[1], w[1];
     int idx[1];
@@ -180,21 +180,20 @@ __device__ __forceinline__ void topk_gate_token(const float *__restrict__ row, i
         const float a = __ldcg(row + min(j, n_cand - 1));
         u[0][r] = j < n_cand ? a : -INFINITY;
     }
-    const int n_add = n_parts + (LATE ? 1 : 0);
-    for (int p = 1; p < n_add; p += PB) {
+    for (int p = 1; p < n_parts; p += PB) {
         float a[PB][RPL];
 #pragma unroll
         for (int q = 0; q < PB; ++q)
 #pragma unroll
             for (int r = 0; r < RPL; ++r) {
                 const int j = r * 32 + lane;
-                a[q][r] = ldcg_if(p + q < n_add && j < n_cand, (!LATE || p + q < n_parts ? row + (p + q) * part_stride : late_bias) + j, 0.f);
+                a[q][r] = ldcg_if(p + q < n_parts && j < n_cand, row + (p + q) * part_stride + j, 0.f);
             }
 #pragma unroll
         for (int q = 0; q < PB; ++q)
 #pragma unroll
             for (int r = 0; r < RPL; ++r)
-                if (p + q < n_add) u[0][r] += a[q][r];
+                if (p + q < n_parts) u[0][r] += a[q][r];
     }
     topk_gate_select<RPL, 1, DEN>(u, n_real, n_cand, K, gate_mode, lane, mm, dd, idx, w);
 #pragma unroll

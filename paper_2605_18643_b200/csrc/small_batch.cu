@@ -98,7 +98,7 @@ __device__ __forceinline__ void route_here(RouteTables<SLOTS> &rt, const RouteAr
     if (const int t = warp; t < ra.T) {
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL>(ra.logits + (size_t)t * ra.n_cand, 1, 0, nullptr, ra.n_real, ra.n_cand, ra.K, ra.gate_mode, lane, v, m, den, my_idx, my_w);
+        topk_gate_token<RPL>(ra.logits + (size_t)t * ra.n_cand, 1, 0, ra.n_real, ra.n_cand, ra.K, ra.gate_mode, lane, v, m, den, my_idx, my_w);
         if (lane < ra.K) {
             rt.idx[t * ra.K + lane] = my_idx;
             rt.w[t * ra.K + lane] = my_w;
@@ -155,7 +155,7 @@ __device__ __forceinline__ void route_one_token(RouteTables<SLOTS> &rt, const Ro
         const int lane = threadIdx.x;
         int my_idx;
         float my_w, v[RPL], m, den;
-        topk_gate_token<RPL>(ra.logits, 1, 0, nullptr, ra.n_real, ra.n_cand, ra.K, ZEDA_GATE_TOPK_NORM, lane, v, m, den, my_idx, my_w);
+        topk_gate_token<RPL>(ra.logits, 1, 0, ra.n_real, ra.n_cand, ra.K, ZEDA_GATE_TOPK_NORM, lane, v, m, den, my_idx, my_w);
         const bool real = lane < ra.K && my_idx < ra.n_real;
         const int id = real ? my_idx : kMaxCand;
         int pos = 0;

@@ -106,6 +106,7 @@ struct zeda_moe {
     const __nv_bfloat16 *w_down;
     zeda::Workspace ws;
     int sm_count;
+    int router_clusters8, router_clusters4;  // clusters of 8 and of 4 CTAs of the router of 33 to 255 tokens that run at a time
     int max_tiles;
     int n_local;    // experts whose weights this handle holds (n_real unless expert-parallel)
     int pair_rows;  // capacity of the pair buffers (max_tokens * top_k, or max_recv_pairs)
@@ -140,7 +141,7 @@ __device__ __forceinline__ void clear_hist(int32_t *__restrict__ hist, int n) {
 #endif
 
 // ---- launchers (each returns the number of kernels it enqueued, or <0 on a launch error) ----
-int init_route_kernels(const zeda_moe *h);
+int init_route_kernels(zeda_moe *h);
 // With n_parts == nullptr the logits are complete.  Otherwise the router may cut the reduction axis
 // into *n_parts slices (mid-sized batches on the tensor-core path): slice p then lies at
 // logits + p * T * n_cand, and launch_route_from_logits adds the slices in order.  Where the router with top-K takes the

@@ -1,4 +1,4 @@
-"""The sliced router of 33 to 255 tokens at the edges of its tiles and slices, against the oracle."""
+"""The router of 33 to 255 tokens at the edges of its tiles, stages and waves, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -11,21 +11,24 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("T,d,E,Z,K,gate", [
     (33, 2048, 140, 60, 8, 0),     # a second tile of one token, a last candidate tile of eight
-    (64, 1088, 200, 32, 16, 2),    # four slices of 34 groups of eight elements: warps of four and of five
-    (65, 2048, 128, 64, 8, 1),     # seven slices, unequal: with the bias as many as the top-K pass requests at a time
-    (128, 8192, 33, 0, 5, 0),      # eight slices, the fullest shared memory; a last candidate tile of one
-    (129, 4096, 300, 100, 8, 0),   # as many slices as fit the shared memory, two waves
+    (64, 1088, 200, 32, 16, 2),    # a last stage of 64 elements: chains of nine steps and of eight
+    (65, 2048, 128, 64, 8, 1),     # tiles of 40 tokens by eight CTAs
+    (128, 8192, 33, 0, 5, 0),      # eight stages; a last candidate tile of one
+    (129, 4096, 300, 100, 8, 0),   # two waves of tiles of 32 tokens by four CTAs
     (255, 2048, 40, 23, 4, 1),     # an odd number of candidates
-    (129, 2048, 384, 128, 8, 0),   # a second wave of a few CTAs (the other router)
-    (65, 2048, 64, 32, 4, 0),      # the fewest products of this router
-    (64, 2048, 64, 32, 4, 0),      # (the other one's)
+    (129, 2048, 384, 128, 8, 0),   # two waves of tiles of 40 tokens
+    (65, 2048, 64, 32, 4, 0),      # a last tile of one token
+    (64, 2048, 64, 32, 4, 0),      # full tiles
     (255, 960, 40, 24, 4, 0),
+    (224, 2048, 128, 64, 8, 0),    # tiles of 48 tokens
+    (241, 2048, 128, 64, 8, 2),    # tiles of 56 tokens
+    (128, 1088, 300, 101, 16, 0),  # tiles of 64 tokens
 ])
 @pytest.mark.parametrize("bias", [0.0, 50.0])
 def test_router_of_33_to_255_tokens(T, d, E, Z, K, gate, bias):
     from paper_2605_18643_b200 import zeda
     wl = inputs.make_layer("slices", T=T, d=d, He=64, E=E, Z=Z, K=K, seed=37, zero_fraction=0.4 if Z else None)
-    # a bias far above the logits: it has to be added once, behind the slices (a sum that carries it loses the logits' last bits)
+    # a bias far above the logits: it has to be added once, behind the products (a sum that carries it loses the logits' last bits)
     b = torch.zeros(E + Z) if wl.router_bias is None else wl.router_bias.clone()
     wl.router_bias = b + bias
     m = zeda.from_workload(wl, gate_mode=gate)
