@@ -75,15 +75,19 @@ __device__ __forceinline__ void combine_chunks(float (&acc)[P][8], const __nv_bf
         if (c + 32 * p < chunks) fma_bf16x8(acc[p], zero_mass, __ldcg(reinterpret_cast<const uint4 *>(x + (size_t)t * d) + c + 32 * p));
 }
 
-// A warp per CHUNKS * 32 chunks of a token, four warps per CTA.  Bound by the reads in flight: with every thread holding the
+// A warp per CHUNKS * 32 chunks of a token.  Bound by the reads in flight: with every thread holding the
 // slot table itself and eight loads predicated by slot, of which the zero slots' were none, 64 threads had a token's chunks
-// one after the other.  Combine stage, us, before and now: 777 tokens of the Qwen-shaped layer 10.1 -> 8.3, 2048 tokens
-// 14.3 -> 11.9, 8192 tokens of Zipf load 42.8 -> 37.3, of the static layer 60.4 -> 58.3; 5003 tokens of the GLM-shaped
-// layer 24.5 -> 16.6.  (One chunk per lane: 10.0, 14.4, 46, 60.5, 27; four: 10.2, 19.3, 52.7, 95, 23.5.)
-// Where the warps are few all the same, one chunk per lane and eight slots at a time: twice the warps, half the round trips,
-// and CTAs of two warps (40 tokens of the GLM-shaped layer, us a call: 164.1 before, 163.3 so, 1.2 longer in CTAs of four;
-// 193 tokens of the Qwen-shaped one, the stage: 8.1 with two chunks, 7.5 so; from 777 tokens on two chunks win, above).
-constexpr int kFewWarps = 8;  // of two chunks per lane, per SM: the line lies at 296 tokens of d 2048
+// one after the other.  Combine stage, us, before and now (two chunks per lane, four warps per CTA): 777 tokens of the
+// Qwen-shaped layer 10.1 -> 8.3, 2048 tokens 14.3 -> 11.9, 8192 tokens of Zipf load 42.8 -> 37.3, of the static layer
+// 60.4 -> 58.3; 5003 tokens of the GLM-shaped layer 24.5 -> 16.6.  (One chunk per lane: 10.0, 14.4, 46, 60.5, 27; four:
+// 10.2, 19.3, 52.7, 95, 23.5.)
+// Where the warps are few, one chunk per lane and eight slots at a time: twice the warps, half the round trips, and CTAs of
+// two warps (40 tokens of the GLM-shaped layer, us a call: 164.1 before, 163.3 so, 1.2 longer in CTAs of four).  A call of
+// the Qwen-shaped layer, us, so and with two chunks: 300 tokens 208.4, 209.1; 400 tokens 209.2, 210.3; 500 tokens 210.2,
+// 212.1; 600 tokens 212.4, 213.4; 777 tokens 218.3, 218.4; 1000 tokens 225.4, 224.8.  With experts of H_e 128 600 tokens
+// 74.5, 75.6; 1000 tokens 78.4, 77.7; at d 1024 (H_e 256) 600 tokens 64.5, 66.0; 1200 tokens 68.1, 69.3.
+// At d 4096 (GLM-shaped) 300 tokens 95.7, 95.4; 368 tokens 96.4, 95.5; rows of up to 256 elements are one warp's either way.
+constexpr int kFewWarps = 16;  // of two chunks per lane, per SM: the line lies at 592 tokens of d 2048
 
 template <int CHUNKS, int ROWS, int THREADS>
 __global__ void __launch_bounds__(THREADS, 896 / THREADS)
@@ -205,7 +209,7 @@ int launch_combine_rows(const zeda_moe *h, const __nv_bfloat16 *rows, const __nv
                              (const int32_t *)h->ws.inv, (const float *)h->ws.topk_w, x, T, c.top_k, c.d_model, pieces,
                              (int)(c.expert_kind == ZEDA_EXPERT_COPY), y);
     };
-    const bool few = (long long)T * (c.d_model / 8) < 64ll * kFewWarps * h->sm_count;
+    const bool few = (long long)T * ((c.d_model / 8 + 63) / 64) < (long long)kFewWarps * h->sm_count;
     const cudaError_t e = few ? go(combine_kernel<1, 8, 64>, 32, 64) : go(combine_kernel<2, 4, 128>, 64, 128);
     return e == cudaSuccess ? 1 : -1;
 }
