@@ -101,6 +101,32 @@ def test_alternating_large_batches_give_the_bits_of_single_calls(large_layer, T,
     m.close()
 
 
+@pytest.fixture(scope="module")
+def long_rows():
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("back_to_back", T=255, d=3136, He=64, E=64, Z=32, K=8, seed=44, zero_fraction=0.5)
+    return zeda, wl, [wl.x.to("cuda:0"), inputs.replica_tokens(wl, 7).to("cuda:0")]
+
+
+@pytest.mark.parametrize("use", ["forward", "stats", "route"])
+@pytest.mark.parametrize("T", [40, 129, 255])
+def test_alternating_inputs_whose_rows_pass_through_shared_memory_in_stages(long_rows, T, use):
+    # the router of 33 to 255 tokens: router rows asked for in front of its wait, and four stages in the room of two
+    zeda, wl, xs = long_rows
+    m = zeda.from_workload(wl)
+    alone = check(zeda, m, [(i % 2, use, xs[i % 2][:T].contiguous()) for i in range(20)])
+    assert not alone[0].same(alone[1])
+    m.close()
+
+
+def test_batches_around_the_router_on_clusters_in_any_order(long_rows):
+    zeda, wl, xs = long_rows
+    m = zeda.from_workload(wl)
+    order = [(T, use) for T in (255, 32, 33, 129, 1, 65, 254, 193, 8, 97) for use in ("forward", "stats", "route")]
+    check(zeda, m, [((T, use, i % 2), use, xs[i % 2][:T].contiguous()) for i, (T, use) in enumerate(order)])
+    m.close()
+
+
 def test_large_batches_in_any_order(large_layer):
     zeda, wl, xs = large_layer
     m = zeda.from_workload(wl)

@@ -45,3 +45,34 @@ def test_router_of_33_to_255_tokens(T, d, E, Z, K, gate, bias):
         assert np.allclose(o["topk_w"].cpu().numpy(), w, rtol=2 * tol + 1e-6, atol=1e-30)
         check_route(dict(o, topk_w=torch.from_numpy(np.ascontiguousarray(w))), idx, w, counts, offsets, perm, P)
     m.close()
+
+
+@pytest.mark.parametrize("T", [33, 129, 255])
+def test_router_of_33_to_255_tokens_in_a_graph_and_without_dependent_launch(T):
+    # it asks for router rows in front of its wait for the kernel before it
+    from paper_2605_18643_b200 import zeda
+    wl = inputs.make_layer("slices", T=T, d=2112, He=64, E=64, Z=32, K=8, seed=38, zero_fraction=0.4)
+    dev = torch.device("cuda:0")
+    xs = [wl.x.to(dev), inputs.replica_tokens(wl, 3).to(dev)]
+    plain = zeda.from_workload(wl, dev, flags=zeda.FLAG_NO_DEPENDENT_LAUNCH)
+    want = [plain.forward(x).view(torch.int16) for x in xs]
+    torch.cuda.synchronize()
+    m = zeda.from_workload(wl, dev)
+    for i in (0, 1, 0):
+        assert torch.equal(m.forward(xs[i]).view(torch.int16), want[i])
+    x, y, y2 = xs[0].clone(), torch.empty_like(xs[0]), torch.empty_like(xs[0])
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):  # two calls: the second starts under the first
+        m.forward(x, y)
+        m.forward(y, y2)
+    for src in (1, 0, 1):
+        x.copy_(xs[src])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y.view(torch.int16), want[src])
+        assert torch.equal(y2.view(torch.int16), plain.forward(y.clone()).view(torch.int16))
+    del graph
+    m.close()
+    plain.close()
