@@ -10,15 +10,20 @@ from test_gpu_parity import oracle_route
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("T,E,Z,K", [
-    (40, 3, 2, 2),        # odd: pairs of columns, many threads per group
-    (1100, 200, 101, 4),  # odd and more groups than threads: two turns
-    (700, 340, 172, 8),   # as many groups of four as threads
-    (4500, 5, 5, 3),      # more rows than one turn of a group's threads takes
+@pytest.mark.parametrize("T,E,Z,K,d", [
+    (40, 3, 2, 2, 64),        # odd: pairs of columns, many threads per group
+    (1100, 200, 101, 4, 64),  # odd and more groups than threads: two turns
+    (700, 340, 172, 8, 64),   # as many groups of four as threads
+    (4500, 5, 5, 3, 64),      # 51 threads per group
+    (4500, 200, 312, 8, 64),  # a thread per group of four, 71 rows: three turns of 32
+    (3000, 200, 55, 8, 64),   # the same with pairs, 47 rows: two turns
+    (33, 128, 64, 8, 2048),   # few tokens of long rows: one row, and four
+    (193, 128, 64, 8, 2048),
+    (255, 150, 73, 8, 1088),  # (eight logits a lane)
 ])
-def test_final_sums_of_the_statistics(T, E, Z, K):
+def test_final_sums_of_the_statistics(T, E, Z, K, d):
     from paper_2605_18643_b200 import zeda
-    wl = inputs.make_layer("stats", T=T, d=64, He=64, E=E, Z=Z, K=K, seed=43, zero_fraction=0.4)
+    wl = inputs.make_layer("stats", T=T, d=d, He=64, E=E, Z=Z, K=K, seed=43, zero_fraction=0.4)
     m = zeda.from_workload(wl)
     x = wl.x.to("cuda:0")
     l, idx, *_ = oracle_route(wl)
