@@ -501,7 +501,8 @@ slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real
 // selection counts, then n_cand sums of probabilities) in a fixed order.  A group of neighbouring columns (four where the
 // rows allow 16-byte loads) is shared by as many threads as fit, each adding every n-th row, 32 requested at a time and
 // added up pairwise (8192 tokens of 192 candidates: 45.3 us a call with the sums behind the placement, 43.5 beside it with
-// sixteen rows at a time, 36.8 with 32).
+// sixteen rows at a time, 36.8 with 32), then the threads of a group pairwise (one after the other, 8192 tokens of 12
+// candidates took 15.0 us, so 13.7).
 struct StatsJob {
     const float *part;
     int rows;  // of part
@@ -511,18 +512,20 @@ struct StatsJob {
 __device__ __forceinline__ float4 add_columns(const float4 &a, const float4 &b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 __device__ __forceinline__ float2 add_columns(const float2 &a, const float2 &b) { return make_float2(a.x + b.x, a.y + b.y); }
 
-constexpr int kStatFinalThreads = 256;
+constexpr int kStatFinalThreads = 256, kStatFinalDeep = 32;        // beside the placement
+constexpr int kStatManyRowsThreads = 1024, kStatManyRowsDeep = 8;  // as a kernel of its own, for more rows
 
+template <int THREADS>
 struct StatsShared {
     float col[2 * kMaxCand];
-    float red[5][kStatFinalThreads / 32];
+    float4 share[THREADS];
+    float red[5][THREADS / 32];
 };
 
-template <typename V>
-__device__ __forceinline__ void sum_stat_columns(const StatsJob &job, int cols, float *col) {
-    constexpr int kDeep = 32;
-    const int groups = cols / (int)(sizeof(V) / sizeof(float)), segs = max(1, kStatFinalThreads / groups), seg = threadIdx.x / groups;
-    for (int c0 = 0; c0 < groups; c0 += kStatFinalThreads) {  // (more than one turn only where each group has one thread)
+template <typename V, int THREADS, int kDeep>
+__device__ __forceinline__ void sum_stat_columns(const StatsJob &job, int cols, float *col, float4 *share) {
+    const int groups = cols / (int)(sizeof(V) / sizeof(float)), segs = max(1, THREADS / groups), seg = threadIdx.x / groups;
+    for (int c0 = 0; c0 < groups; c0 += THREADS) {  // (more than one turn only where each group has one thread)
         const int c = segs > 1 ? threadIdx.x - seg * groups : c0 + threadIdx.x;
         const bool on = segs > 1 ? seg < segs : c < groups;
         V a = {};
@@ -538,21 +541,26 @@ __device__ __forceinline__ void sum_stat_columns(const StatsJob &job, int cols, 
                     for (int q = 0; q < o; ++q) v[q] = add_columns(v[q], v[q + o]);
                 a = add_columns(a, v[0]);
             }
-        for (int s = 0; s < segs; ++s) {  // the shares of a group in order
-            if (on && (segs == 1 || seg == s)) {
-                V *dst = reinterpret_cast<V *>(col) + c;
-                *dst = s == 0 ? a : add_columns(*dst, a);
-            }
+        // the shares of a group, those of the upper half of its threads onto the lower half's
+        V *mine = reinterpret_cast<V *>(share) + threadIdx.x;
+        for (int n = segs; n > 1;) {
+            const int half = (n + 1) / 2;
+            if (on && seg >= half && seg < n) *mine = a;
             __syncthreads();
+            if (on && seg + half < n) a = add_columns(a, mine[half * groups]);
+            n = half;
         }
+        if (on && (segs == 1 || seg == 0)) reinterpret_cast<V *>(col)[c] = a;
+        __syncthreads();
     }
 }
 
-__device__ __forceinline__ void stats_final(const StatsJob &job, int T, int K, int n_real, int n_cand, StatsShared &sh) {
-    if (n_cand % 2 == 0) sum_stat_columns<float4>(job, 2 * n_cand, sh.col);
-    else sum_stat_columns<float2>(job, 2 * n_cand, sh.col);
+template <int THREADS, int DEEP>
+__device__ __forceinline__ void stats_final(const StatsJob &job, int T, int K, int n_real, int n_cand, StatsShared<THREADS> &sh) {
+    if (n_cand % 2 == 0) sum_stat_columns<float4, THREADS, DEEP>(job, 2 * n_cand, sh.col, sh.share);
+    else sum_stat_columns<float2, THREADS, DEEP>(job, 2 * n_cand, sh.col, sh.share);
     float sums[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int j = threadIdx.x; j < n_cand; j += kStatFinalThreads) {
+    for (int j = threadIdx.x; j < n_cand; j += THREADS) {
         const float fj = sh.col[j] / T, pj = sh.col[n_cand + j] / T;
         if (job.f) job.f[j] = fj;
         if (job.p_mean) job.p_mean[j] = pj;
@@ -571,7 +579,7 @@ __device__ __forceinline__ void stats_final(const StatsJob &job, int T, int K, i
     if (threadIdx.x < 32) {
         float tot[5];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) tot[i] = warp_sum(threadIdx.x < kStatFinalThreads / 32 ? sh.red[i][threadIdx.x] : 0.f);
+        for (int i = 0; i < 5; ++i) tot[i] = warp_sum(threadIdx.x < THREADS / 32 ? sh.red[i][threadIdx.x] : 0.f);
         if (threadIdx.x == 0) {
             job.out[0] = tot[3] / K;
             job.out[1] = tot[0];
@@ -581,13 +589,15 @@ __device__ __forceinline__ void stats_final(const StatsJob &job, int T, int K, i
     }
 }
 
-// as a kernel of its own, where the placement is no single kernel (more than kFoldMaxBlocks blocks of the counting sort)
-__global__ void __launch_bounds__(kStatFinalThreads)
+// As a kernel of its own, where the placement is no single kernel (more than kFoldMaxBlocks blocks of the counting sort): more
+// than 512 rows, for which 32 warps take less time than eight with four times the requests (a call of 33,000 tokens of 192
+// candidates 142.5 us with eight, 138.9 so; 65,536 tokens of 512 candidates 587, 559).
+__global__ void __launch_bounds__(kStatManyRowsThreads)
 stats_final_kernel(const StatsJob job, int T, int K, int n_real, int n_cand) {
     pdl_launch_dependents();
     pdl_wait();
-    __shared__ __align__(16) StatsShared sh;
-    stats_final(job, T, K, n_real, n_cand, sh);
+    __shared__ __align__(16) StatsShared<kStatManyRowsThreads> sh;
+    stats_final<kStatManyRowsThreads, kStatManyRowsDeep>(job, T, K, n_real, n_cand, sh);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -614,10 +624,10 @@ slot_scan_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n
                        int32_t *__restrict__ inv, int32_t *__restrict__ pair_token, const StatsJob job, int n_cand) {
     static_assert(kStatFinalThreads == kScanThreads, "one CTA size for both");
     if (STATS && (int)blockIdx.x == nblk) {
-        __shared__ __align__(16) StatsShared stats;
+        __shared__ __align__(16) StatsShared<kStatFinalThreads> stats;
         pdl_launch_dependents();
         pdl_wait();
-        stats_final(job, T, K, n_real, n_cand, stats);
+        stats_final<kStatFinalThreads, kStatFinalDeep>(job, T, K, n_real, n_cand, stats);
         return;
     }
     __shared__ ScanShared sh;
@@ -916,7 +926,7 @@ int launch_route_from_logits(const zeda_moe *h, const float *logits, int T, cons
                               (const int32_t *)ws.topk_idx, T, K, c.n_real, (const int32_t *)ws.block_hist, (const int32_t *)ws.offsets,
                               ws.perm, out.perm, ws.inv, ws.pair_token);
             if (stats && e == cudaSuccess) {
-                e = launch_kernel(h->pdl, stats_final_kernel, dim3(1), dim3(kStatFinalThreads), 0, s, job, T, K, c.n_real, n_cand);
+                e = launch_kernel(h->pdl, stats_final_kernel, dim3(1), dim3(kStatManyRowsThreads), 0, s, job, T, K, c.n_real, n_cand);
                 ++launches;
             }
         }

@@ -17,6 +17,8 @@ pytestmark = pytest.mark.gpu
     (4500, 5, 5, 3, 64),      # 51 threads per group
     (4500, 200, 312, 8, 64),  # a thread per group of four, 71 rows: three turns of 32
     (3000, 200, 55, 8, 64),   # the same with pairs, 47 rows: two turns
+    (32800, 7, 4, 2, 64),     # a kernel of its own: pairs, 93 threads a group
+    (32800, 300, 212, 4, 64), # the same, four threads a group
     (33, 128, 64, 8, 2048),   # few tokens of long rows: one row, and four
     (193, 128, 64, 8, 2048),
     (255, 150, 73, 8, 1088),  # (eight logits a lane)
