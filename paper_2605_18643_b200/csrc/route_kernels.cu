@@ -499,8 +499,8 @@ slot_place_kernel(const int32_t *__restrict__ topk_idx, int T, int K, int n_real
 
 // Routing statistics, final sums by one CTA: adds up what the CTAs of the top-K pass have left in `part` (per CTA n_cand
 // selection counts, then n_cand sums of probabilities) in a fixed order.  A group of neighbouring columns (four where the
-// rows allow 16-byte loads) is shared by as many threads as fit, each adding every n-th row, 32 requested at a time and
-// added up pairwise (8192 tokens of 192 candidates: 45.3 us a call with the sums behind the placement, 43.5 beside it with
+// rows allow 16-byte loads) is shared by as many threads as fit, each adding every n-th row, 32 requested at a time (8 in the
+// kernel of its own) and added up pairwise (8192 tokens of 192 candidates: 45.3 us a call with the sums behind the placement, 43.5 beside it with
 // sixteen rows at a time, 36.8 with 32), then the threads of a group pairwise (one after the other, 8192 tokens of 12
 // candidates took 15.0 us, so 13.7).
 struct StatsJob {
